@@ -3,14 +3,18 @@
 // two or four at 64 and 128), sized by the host so that the CTAs spread
 // evenly over the SMs.
 //
-// Same arithmetic as the fused kernel of kc_fwd.cu (double-single phase,
+// The mixed path of the fused kernel of kc_fwd.cu (double-single phase,
 // Sec. 5; Kepler's equation in single precision, Sec. 4.3; Eq. 3 velocity;
-// Kahan sums of the planet velocities and of chi2, Sec. 4.4), laid out for
-// the SMs rather than for a tile:
+// Kahan sums of the planet velocities and of chi2, Sec. 4.4) in the packed
+// two-observation form of kc_pair.cuh, laid out for the SMs rather than for
+// a tile.  Bound by FP32 issue and register ports (68 clocks per warp,
+// planet and observation and sub-partition in steady state).  Measured, us
+// per launch, before (scalar form) and now: 2^20 x 4 x 256 3224 -> 2014, 4096
+// x 4 x 256 back to back 14.3 -> 11.2, 300 x 3 x 101 5.9 -> 4.3.
 //
 //  - A CTA of W warps evaluates W * 32 / G systems (one round).  The host
-//    picks G and W so that the CTAs of the first wave land evenly on the
-//    SMs (for 4096 systems, 27 warps per CTA: one CTA and 27 systems on
+//    picks G and W by a cost model (pick_warp_tile) so that the CTAs land
+//    evenly on the SMs and share their staging (for 4096 systems, 27 warps per CTA: one CTA and 27 systems on
 //    every SM, where tiles of 16 systems leave some SMs with 32 and others
 //    with 16).  Larger batches run many waves; the hardware then overlaps
 //    one CTA's prologue with the work of the others on its SM.
@@ -19,13 +23,15 @@
 //    is used, so the CTA waits for memory once.
 //  - The observations (shared by every system, Sec. 4.1) are converted to
 //    float pairs and staged in shared memory, padded with zero-weight
-//    entries to whole chunks, so the inner loops have no tail.
-//  - Each lane holds a chunk of kChunk observations (their phases and their
-//    compensated velocity sums) in registers and streams the planets over
-//    it: a planet's constants (phase, velocity and the hoisted part of
-//    Mikkola's start, computed once per (system, planet)) are read from
-//    shared memory once per chunk, and the chunk's kChunk Kepler solves are
-//    independent chains for the scheduler to interleave.
+//    entries to whole chunks, so the inner loops have no tail; the last
+//    threads of the CTA stage while the first set the planets up.
+//  - Each lane holds a chunk of kChunk observations (two packed pairs: their
+//    phases and their compensated velocity sums) in registers and streams
+//    the planets over it: a planet's constants (PlanetP, computed once per
+//    (system, planet)) are read from shared memory once per chunk, and the
+//    chunk's Kepler solves are independent chains for the scheduler.
+//  - A CTA whose planets or times leave the short mean anomaly's range takes
+//    the wide one for all its systems (kc_pair.cuh).
 //  - The lanes of a system combine their compensated sums with TwoSum
 //    shuffles, and the warps of a system (G > 32) through a few words of
 //    shared memory; no atomics, no scratch memory.  Splitting a system over
@@ -37,7 +43,7 @@
 //    (griddepcontrol.launch_dependents), so that a following batch's CTAs
 //    are placed on the SMs as this grid's CTAs exit instead of after the
 //    whole grid has completed (back-to-back 4096 x 4 x 256 batches: 14.0 us
-//    each instead of 16.4 us).  The launch asks for it only outside stream
+//    each instead of 16.4 us, with the scalar body).  The launch asks for it only outside stream
 //    capture: as programmatic edges in the DE-MC driver's graph (4096
 //    chains, halves of 2048) it cost a quarter of the generations per
 //    second (2.36e4 against 3.12e4), where back-to-back launches of 1024 to
@@ -50,6 +56,7 @@
 #include "kc_demc.cuh"
 #include "kc_device.cuh"
 #include "kc_internal.h"
+#include "kc_pair.cuh"
 
 namespace kc {
 
@@ -63,21 +70,18 @@ __host__ __device__ inline int round_up(int x, int m) { return (x + m - 1) / m *
 // x rounded up to a multiple of the power of two m (no division)
 __device__ __forceinline__ int round_up_pow2(int x, int m) { return (x + m - 1) & -m; }
 
-// Planet constants of the kernel: phase and velocity (PlanetF) and the
-// hoisted part of Mikkola's start (StartF); 48 bytes, three 16-byte loads.
-struct PlanetW {
-  PlanetF f;
-  StartF m;
-};
-
+// Shared memory: the sin/cos table, the planets' constants, the systems'
+// gamma, the staged observations (one float array per quantity, so that a
+// lane reads the pair of observations it packs as one 8-byte word), and the
+// words that combine a system's warps.
 struct WarpLayout {
-  size_t pl, gam, obs, w, red, total;
+  size_t tab, pl, gam, obs, red, total;
   __host__ __device__ WarpLayout(int spr, int J, int tile, int nwarps) {
-    pl = 0;
-    gam = pl + sizeof(PlanetW) * spr * J;
+    tab = 0;
+    pl = tab + sizeof(AngTab);
+    gam = pl + sizeof(PlanetP) * spr * J;
     obs = align16(gam + sizeof(float) * spr);
-    w = obs + sizeof(float4) * tile;
-    red = align16(w + sizeof(float) * tile);      // G > 32: 3 words per warp
+    red = obs + sizeof(float) * 5 * tile;         // G > 32: 3 words per warp
     total = align16(red + sizeof(float) * 3 * nwarps);
   }
 };
@@ -92,19 +96,17 @@ __host__ __device__ inline int warp_obs_tile(int n_obs, int G) {
 // (system, planet) constants, items spr*J .. spr*(J+1) - 1 the systems'
 // gamma.  p holds the item's parameters (five, or gamma in p[0]); an
 // invalid planet carries e = NaN, which poisons its system.
+// Returns whether the planet's period asks for the wide mean anomaly.
 template <int J>
-__device__ __forceinline__ void setup_item(int i, int spr, int64_t sys0, int64_t n_sys,
+__device__ __forceinline__ bool setup_item(int i, int spr, int64_t sys0, int64_t n_sys,
                                            const double (&p)[5], double t_ref, double t0,
-                                           PlanetW *pl_s, float *gam_s, unsigned long long *dbg) {
-  if (!dbg_ok(dbg, i < spr * (J + 1), kDbgSmem, i)) return;
+                                           PlanetP *pl_s, float *gam_s, unsigned long long *dbg) {
+  if (!dbg_ok(dbg, i < spr * (J + 1), kDbgSmem, i)) return false;
+  bool wide = false;
   if (i < spr * J) {
     const int64_t s = sys0 + i / J;
-    PlanetW q = {};
-    if (s < n_sys) {
-      q.f = planet_setup_mixed(p, t_ref, t0);
-      if (!planet_valid(p[0], p[1], p[2], p[3], p[4])) q.f.e = __int_as_float(0x7fc00000);
-      q.m = kepler_start_setup(q.f.e);
-    }
+    PlanetP q = {};
+    if (s < n_sys) q = planet_setup_pair(p, t_ref, t0, wide);
     pl_s[i] = q;
   } else {
     const int sl = i - spr * J;
@@ -112,6 +114,7 @@ __device__ __forceinline__ void setup_item(int i, int spr, int64_t sys0, int64_t
     if (sys0 + sl < n_sys) g = finite_bits(p[0]) ? d2f(p[0]) : __int_as_float(0x7fc00000);
     gam_s[sl] = g;
   }
+  return wide;
 }
 
 // The item's parameters.  DEMC: the launch evaluates DE-MC proposals; with
@@ -148,6 +151,62 @@ __device__ __forceinline__ void load_item(int i, int spr, int64_t sys0, const Un
   }
 }
 
+// The thread's observations of one staged tile: npad (whole chunks), nk of
+// them real.  The thread takes kChunk observations at a time as kChunk / 2
+// packed pairs.
+template <int J, bool RESID, bool WIDE>
+__device__ __forceinline__ void warp_tile_sum(const float *th_s, int tile, const PlanetP *q,
+                                              const float *tab, float gam, int c, int lg,
+                                              int npad, int nk, Kahan2 &acc, float &rmax,
+                                              unsigned long long *dbg) {
+  constexpr int kPairs = kChunk / 2;
+  const int step = kChunk << lg;
+  for (int base = 2 * c; base < npad; base += step) {
+    if (!dbg_ok(dbg, base + ((kPairs - 1) << (lg + 1)) + 1 < tile, kDbgSmem, base)) break;
+    f32x2 th[kPairs], tl[kPairs];
+    Kahan2 V[kPairs];
+#pragma unroll
+    for (int i = 0; i < kPairs; ++i) {
+      const float *o = th_s + base + (i << (lg + 1));
+      th[i] = *reinterpret_cast<const f32x2 *>(o);
+      tl[i] = *reinterpret_cast<const f32x2 *>(o + tile);
+      V[i].big = dup2(gam);
+      V[i].small = 0;
+    }
+    // two planets per iteration: the second one's constants load while the
+    // first one's chains run (2074 us against 2195 for one at a time on the
+    // 2^20-system sweep; all four at once spill: 2171)
+#pragma unroll 2
+    for (int j = 0; j < J; ++j) {
+      const PlanetP qj = q[j];
+#pragma unroll
+      for (int i = 0; i < kPairs; ++i) {
+        const f32x2 M = mean_anomaly2<WIDE>(th[i], tl[i], qj);
+        const f32x2 m = abs2(M);
+        f32x2 s, cE, E;
+        kepler_pair(m, qj, tab, s, cE, E);
+        if (RESID) {
+          const f32x2 r = fma2(dup2(-qj.e), s, sub2(E, m));
+          const int k = base + (i << (lg + 1));
+          rmax = fmaxf(rmax, k < nk ? fabsf(lo2(r)) : 0.0f);
+          rmax = fmaxf(rmax, k + 1 < nk ? fabsf(hi2(r)) : 0.0f);
+        }
+        velocity_sum(V[i], qj, signed_as(s, M), cE);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kPairs; ++i) {
+      const float *o = th_s + 2 * tile + base + (i << (lg + 1));
+      const f32x2 vh = *reinterpret_cast<const f32x2 *>(o);
+      const f32x2 vl = *reinterpret_cast<const f32x2 *>(o + tile);
+      const f32x2 w = *reinterpret_cast<const f32x2 *>(o + 2 * tile);
+      // residual V - v_obs with the model and the observation as float pairs
+      const f32x2 r = sub2(sub2(V[i].big, vh), add2(V[i].small, vl));
+      kahan_add(acc, mul2(mul2(w, r), r));
+    }
+  }
+}
+
 // RESID: also the per-system max Kepler residual.  DEMC: the batch is a
 // DE-MC step's proposals (a.demc): formed in the prologue, Metropolis
 // decision in the epilogue; plain evaluations contain neither.
@@ -165,10 +224,10 @@ chi2_mixed_warp_kernel(UniformArgs a, int lg, int tile, int ntiles, float *__res
   const int G = 1 << lg;
   const int spr = block >> lg;                   // systems of this CTA
   const WarpLayout L(spr, J, tile, block >> 5);
-  PlanetW *pl_s = reinterpret_cast<PlanetW *>(smem + L.pl);
+  float *tab_s = reinterpret_cast<float *>(smem + L.tab);
+  PlanetP *pl_s = reinterpret_cast<PlanetP *>(smem + L.pl);
   float *gam_s = reinterpret_cast<float *>(smem + L.gam);
-  float4 *obs_s = reinterpret_cast<float4 *>(smem + L.obs);
-  float *w_s = reinterpret_cast<float *>(smem + L.w);
+  float *obs_s = reinterpret_cast<float *>(smem + L.obs);
 
   const int64_t sys0 = (int64_t)blockIdx.x * spr;
   const int nitems = spr * (J + 1);
@@ -180,59 +239,70 @@ chi2_mixed_warp_kernel(UniformArgs a, int lg, int tile, int ntiles, float *__res
   const double t_ref = a.n_obs > 0 ? a.t[0] : a.t0;
   double p[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   if (tid < nitems) load_item<J, DEMC>(tid, spr, sys0, a, p);
-  const bool has0 = tid < nk0 && dbg_ok(a.invalid, tid < a.n_obs, kDbgObs, tid);
-  const bool has1 = tid + block < nk0 && dbg_ok(a.invalid, tid + block < a.n_obs, kDbgObs,
-                                                tid + block);
+  // the observations are staged from the last thread down, so that in a
+  // large CTA other warps convert them than set the planets up
+  const int ob = block - 1 - tid;
+  const bool has0 = ob < nk0 && dbg_ok(a.invalid, ob < a.n_obs, kDbgObs, ob);
+  const bool has1 = ob + block < nk0 && dbg_ok(a.invalid, ob + block < a.n_obs, kDbgObs,
+                                               ob + block);
   double t0v = 0.0, v0v = 0.0, s0v = 1.0, t1v = 0.0, v1v = 0.0, s1v = 1.0;
-  if (has0) { t0v = a.t[tid]; v0v = a.v[tid]; s0v = a.sigma[tid]; }
-  if (has1) { t1v = a.t[tid + block]; v1v = a.v[tid + block]; s1v = a.sigma[tid + block]; }
+  if (has0) { t0v = a.t[ob]; v0v = a.v[ob]; s0v = a.sigma[ob]; }
+  if (has1) { t1v = a.t[ob + block]; v1v = a.v[ob + block]; s1v = a.sigma[ob + block]; }
+  ang_tab_load(tab_s, tid, block);
 
   // the reference time's split, needed by the threads that stage
   Split3 tr3 = {0.0f, 0.0f, 0.0f};
-  if (tid < npad0 || ntiles > 1) tr3 = split3(t_ref);
+  if (ob < npad0 || ntiles > 1) tr3 = split3(t_ref);
   const float jit2 = d2f(a.jitter2);
-  // tau = t - t_ref and v as float pairs, w = 1/(sigma^2 + jitter^2); the
-  // padding up to whole chunks has zero weight (and tau = v = 0)
+  // tau = t - t_ref as (th, tl) and v as float pairs, w = 1/(sigma^2 +
+  // jitter^2); the padding up to whole chunks has zero weight (and tau = v =
+  // 0).  Returns whether the time asks for the wide mean anomaly.
   auto convert = [&](int k, bool real, double t, double v, double sigma) {
-    if (!dbg_ok(a.invalid, k < tile, kDbgSmem, k)) return;
-    float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    float wk = 0.0f;
+    if (!dbg_ok(a.invalid, k < tile, kDbgSmem, k)) return false;
+    float th = 0.0f, tl = 0.0f, vh = 0.0f, vl = 0.0f, wk = 0.0f;
     if (real) {
-      sub_ds(split3(t), tr3, o.x, o.y);
-      split_d(v, o.z, o.w);
+      sub_ds(split3(t), tr3, th, tl);
+      tau_place(th, tl);
+      split_d(v, vh, vl);
       const float sg = d2f(sigma);
       const float var = __fmaf_rn(sg, sg, jit2);
       wk = var > 0.0f ? 1.0f / var : __int_as_float(0x7fc00000);
     }
-    obs_s[k] = o;
-    w_s[k] = wk;
+    obs_s[k] = th;
+    obs_s[tile + k] = tl;
+    obs_s[2 * tile + k] = vh;
+    obs_s[3 * tile + k] = vl;
+    obs_s[4 * tile + k] = wk;
+    return !(fabsf(th) < kPairMaxTau);
   };
 
-  if (tid < nitems) setup_item<J>(tid, spr, sys0, a.n_sys, p, t_ref, a.t0, pl_s, gam_s, a.invalid);
+  bool wide = false;
+  if (tid < nitems)
+    wide = setup_item<J>(tid, spr, sys0, a.n_sys, p, t_ref, a.t0, pl_s, gam_s, a.invalid);
   for (int i = tid + block; i < nitems; i += block) {       // more items than threads
     double q[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     load_item<J, DEMC>(i, spr, sys0, a, q);
-    setup_item<J>(i, spr, sys0, a.n_sys, q, t_ref, a.t0, pl_s, gam_s, a.invalid);
+    wide |= setup_item<J>(i, spr, sys0, a.n_sys, q, t_ref, a.t0, pl_s, gam_s, a.invalid);
   }
-  if (tid < npad0) convert(tid, has0, t0v, v0v, s0v);
-  if (tid + block < npad0) convert(tid + block, has1, t1v, v1v, s1v);
-  for (int k = tid + 2 * block; k < npad0; k += block) {
+  if (ob < npad0) wide |= convert(ob, has0, t0v, v0v, s0v);
+  if (ob + block < npad0) wide |= convert(ob + block, has1, t1v, v1v, s1v);
+  for (int k = ob + 2 * block; k < npad0; k += block) {
     const bool real = k < nk0 && dbg_ok(a.invalid, k < a.n_obs, kDbgObs, k);
-    convert(k, real, real ? a.t[k] : 0.0, real ? a.v[k] : 0.0, real ? a.sigma[k] : 1.0);
+    wide |= convert(k, real, real ? a.t[k] : 0.0, real ? a.v[k] : 0.0, real ? a.sigma[k] : 1.0);
   }
-  __syncthreads();
+  wide = __syncthreads_or(wide);
 
   // ---- the CTA's systems, one per G lanes ----
   int slot = tid >> lg;
   if (!dbg_ok(a.invalid, slot < spr, kDbgSmem, slot)) slot = 0;
   const int c = tid & (G - 1);                   // the thread's place in its system
   const int64_t s = sys0 + slot;
-  const PlanetW *q = pl_s + slot * J;
+  const PlanetP *q = pl_s + slot * J;
   const float gam = gam_s[slot];
   float poison = 0.0f * gam;                     // NaN for an invalid system
 #pragma unroll
-  for (int j = 0; j < J; ++j) poison += 0.0f * q[j].f.e;
-  Kahan acc = {0.0f, 0.0f};
+  for (int j = 0; j < J; ++j) poison += 0.0f * q[j].e;
+  Kahan2 acc2 = {0, 0};
   float rmax = 0.0f;
 
   for (int t = 0; t < ntiles; ++t) {
@@ -241,53 +311,22 @@ chi2_mixed_warp_kernel(UniformArgs a, int lg, int tile, int ntiles, float *__res
     const int npad = round_up_pow2(nk, step);
     if (t > 0) {
       __syncthreads();
+      bool far = false;
       for (int k = tid; k < npad; k += block) {
         const bool real = k < nk && dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k);
-        convert(k, real, real ? a.t[k0 + k] : 0.0, real ? a.v[k0 + k] : 0.0,
-                real ? a.sigma[k0 + k] : 1.0);
+        far |= convert(k, real, real ? a.t[k0 + k] : 0.0, real ? a.v[k0 + k] : 0.0,
+                       real ? a.sigma[k0 + k] : 1.0);
       }
-      __syncthreads();
+      wide |= (bool)__syncthreads_or(far);
     }
-    for (int base = c; base < npad; base += step) {
-      if (!dbg_ok(a.invalid, base + ((kChunk - 1) << lg) < tile, kDbgSmem, base)) break;
-      float th[kChunk], tl[kChunk];
-      Kahan V[kChunk];
-#pragma unroll
-      for (int i = 0; i < kChunk; ++i) {
-        const float2 tt = *reinterpret_cast<const float2 *>(obs_s + base + (i << lg));
-        th[i] = tt.x;
-        tl[i] = tt.y;
-        V[i].big = 0.0f;
-        V[i].small = 0.0f;
-      }
-      // two planets per iteration: the second one's constants load while the
-      // first one's chains run (full unrolling spills at 64 registers)
-#pragma unroll 2
-      for (int j = 0; j < J; ++j) {
-        const PlanetW qj = q[j];
-#pragma unroll
-        for (int i = 0; i < kChunk; ++i) {
-          const float M = mean_anomaly_mixed(th[i], tl[i], qj.f);
-          float sE, cE;
-          const float E = kepler_f32_h(M, qj.f.e, qj.m, sE, cE);
-          if (RESID) {
-            const float r = fabsf((E - M) - qj.f.e * sE);
-            rmax = fmaxf(rmax, base + (i << lg) < nk ? r : 0.0f);
-          }
-          kahan_add(V[i], velocity_h(qj.f, sE, cE));
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < kChunk; ++i) {
-        const int k = base + (i << lg);
-        const float2 vo = *reinterpret_cast<const float2 *>(&obs_s[k].z);
-        // residual V - v_obs with the model and the observation as float pairs
-        const float r = __fadd_rn(__fsub_rn(V[i].big, vo.x),
-                                  __fsub_rn(gam, __fadd_rn(V[i].small, vo.y)));
-        kahan_add(acc, w_s[k] * r * r);
-      }
-    }
+    if (wide)
+      warp_tile_sum<J, RESID, true>(obs_s, tile, q, tab_s, gam, c, lg, npad, nk, acc2, rmax,
+                                    a.invalid);
+    else
+      warp_tile_sum<J, RESID, false>(obs_s, tile, q, tab_s, gam, c, lg, npad, nk, acc2, rmax,
+                                     a.invalid);
   }
+  Kahan acc = kahan_join(acc2);
 
   // combine the system's lanes within each of its warps (G a power of two)
   for (int m = (G < 32 ? G : 32) >> 1; m >= 1; m >>= 1) {
@@ -401,71 +440,91 @@ bool warp_tile_ok(int G, int block) {
   return lanes && block >= 32 && block <= 1024 && !(block & 31) && block % G == 0;
 }
 
-int warp_lanes_for(int n_obs) {
-  if (n_obs >= 32 * kChunk) return 32;
-  if (n_obs >= 16 * kChunk) return 16;
-  return 8;
-}
-
 bool warp_lanes_fit(int G, int n_obs) { return G == 8 || n_obs >= G * kChunk; }
 
-Tile warp_tile(int64_t n_sys, int n_pl, int n_obs, bool multi_warp) {
-  // A grid of one CTA per block / G systems.  When it fits on the device
-  // at once, an SM holds at most ceil(CTAs / n_sm) CTAs; otherwise the
-  // hardware refills the SMs wave after wave and the load per SM is the
-  // total over the SMs.  Pick the shape whose busiest SM carries the least
-  // work (warps x 32 / G: systems' worth of lanes); among equals, the one
-  // with more warps resident per SM (more latency hidden), then the larger
-  // CTA (fewer CTAs share an SM: on the 4096-system batch one CTA of 27
-  // warps per SM ran 18.4 us where three of nine ran 20.5 us, with the
-  // same 27 systems per SM).  With multi_warp, 32 lanes per system and at
-  // least 4 observations per lane at G = 64 or 128, a system split over 2
-  // or 4 warps replaces that shape if its load is lower by more than 1 %,
-  // or within 1 % in fewer waves, or in as many waves with at least as many
-  // warps resident (then the larger CTA).  Back to back on n_obs = 256
-  // (us per launch): 256 systems 6.51 -> 5.24, 512: 6.65 -> 5.41, 1024:
-  // 7.44 -> 6.75, 2048: 9.52 -> 9.23; the 4096-system batch keeps its single
-  // wave of 27-warp CTAs (13.9 against 17.4 for 64 lanes in 28-warp CTAs).
-  const int G0 = warp_lanes_for(n_obs);
-  const int64_t n_sm = sm_count();
-  Tile best{G0, 8 * 32, 0, 3};
-  double best_load = 1e300;
-  int64_t best_warps = 0, best_waves = 0;
-  for (int G : {G0, 64, 128}) {
-    const bool multi = G > 32;
-    if (multi && (!multi_warp || G0 != 32 || !warp_lanes_fit(G, n_obs))) continue;
+// Resident CTAs per SM of `block` threads at the kernel's 64 registers and
+// `smem` bytes: the occupancy API's answer by arithmetic (the choice below
+// asks for 145 shapes).
+static int warp_occupancy(int block, size_t smem, int smem_sm) {
+  const int by_regs = 65536 / (64 * block);
+  const int by_smem = (int)((size_t)smem_sm / (smem + 1024));      // 1 KB reserved per CTA
+  return std::min(std::min(by_regs, 2048 / block), std::min(by_smem, 32));
+}
+
+static Tile pick_warp_tile(int64_t n_sys, int n_pl, int n_obs, bool multi_warp) {
+  // Predicted clocks of one SM for every shape of G lanes per system and W
+  // warps per CTA, the smallest wins.  An SM runs ceil(CTAs / n_sm) CTAs,
+  // each costing its four sub-partitions
+  //  - kEval clocks per warp and planet for every observation of a lane (the
+  //    measured steady state of the packed body), or the body's latency
+  //    shared by the resident warps where they are too few to cover it
+  //    (kChain clocks per chunk of kChunk observations);
+  //  - the prologue's instructions: kSetup clocks per warp of (system,
+  //    planet) items, kStage per warp of staged observations.
+  // Few lanes per system share the staged observations and the planets'
+  // setup among many systems (2^20 x 4 x 256: 1963 us at G = 8 against 2539
+  // at G = 32), many lanes spread a small batch over the SMs (300 x 3 x 101:
+  // 4.3 us at G = 32, 5.1 at 16; 256 x 4 x 256: G = 64); a CTA count just
+  // above a multiple of the SM count leaves most of them idle at the end
+  // (4096 x 4 x 256: 11.3 us in 152 CTAs of 27 warps, 13.2 in 256 of 16).
+  // W counts half as rounded up to whole warps per sub-partition (9-warp
+  // CTAs measured between the two).
+  constexpr double kEval = 68.0, kChain = 560.0, kSetup = 600.0, kStage = 180.0;
+  const int64_t n_sm = sm_count() > 1 ? sm_count() : 152;     // no device: a GB300's shapes
+  int dev = 0, smem_sm = 228 * 1024;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    smem_sm = 228 * 1024;                        // no device: shapes stay valid
+  }
+  Tile best{8, 128, 0, 3};
+  double best_cost = 1e300;
+  for (int G : {8, 16, 32, 64, 128}) {
+    if (G > 32 && (!multi_warp || !warp_lanes_fit(G, n_obs))) continue;
+    const int npad = round_up(n_obs > 0 ? n_obs : 1, G * kChunk);
+    const double chunks = (double)npad / (G * kChunk);
     for (int W = 4; W <= 32; ++W) {
       const int block = 32 * W;
       if (block % G) continue;
-      const int occ = blocks_per_sm(n_pl, 0, block, warp_smem(n_pl, G, block, n_obs));
+      const int occ = warp_occupancy(block, warp_smem(n_pl, G, block, n_obs), smem_sm);
       if (occ < 1) continue;
       const int64_t spc = block / G;                 // systems per CTA
-      const int64_t ctas = (n_sys + spc - 1) / spc;
-      const int64_t cap = n_sm * occ;
-      const int64_t per_sm = (ctas + n_sm - 1) / n_sm;
-      const int64_t resident = ctas <= cap ? per_sm : occ;
-      const double load = (double)per_sm * W * 32.0 / G;
-      const int64_t warps = resident * W;
-      const int64_t waves = (ctas + cap - 1) / cap;
-      bool take;
-      if (!multi) {
-        const bool tie = load <= best_load * (1.0 + 1e-9);
-        take = load < best_load * (1.0 - 1e-9) || (tie && warps >= best_warps);
-      } else {
-        const bool near = load <= best_load * 1.01;
-        take = load < best_load * 0.99 ||
-               (near && (waves < best_waves || (waves == best_waves && warps >= best_warps)));
-      }
-      if (take) {
-        best_load = load;
-        best_warps = warps;
-        best_waves = waves;
+      const int64_t per_sm = ((n_sys + spc - 1) / spc + n_sm - 1) / n_sm;
+      const int resident = (int)std::min<int64_t>(per_sm, occ);
+      const int quads = (W + 3) / 4;                 // warps of the fullest sub-partition
+      const double load = resident == 1 ? quads : 0.5 * (0.25 * W + quads);
+      const double chunk = std::max(kEval * kChunk, kChain / (0.25 * W * resident));
+      const double items = (double)((spc * n_pl + 31) / 32), stage = (double)((npad + 31) / 32);
+      const double cost = (double)per_sm * (load * n_pl * chunks * chunk +
+                                            0.25 * (items * kSetup + stage * kStage));
+      if (cost < best_cost * (1.0 - 1e-9)) {
+        best_cost = cost;
         best = Tile{G, block, 0, 3};
       }
     }
   }
   best.obs_tile = warp_obs_tile(n_obs, best.G);
   return best;
+}
+
+// The choice is the same for every call of a size: remembered, up to a
+// bounded number of sizes.
+Tile warp_tile(int64_t n_sys, int n_pl, int n_obs, bool multi_warp) {
+  typedef std::tuple<int64_t, int, int, int, int> Key;
+  static std::mutex mu;
+  static std::map<Key, Tile> known;
+  const Key key(n_sys, n_pl, n_obs, multi_warp, sm_count());
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = known.find(key);
+    if (it != known.end()) return it->second;
+  }
+  const Tile t = pick_warp_tile(n_sys, n_pl, n_obs, multi_warp);
+  std::lock_guard<std::mutex> lk(mu);
+  if (known.size() >= 256) known.clear();
+  known[key] = t;
+  return t;
 }
 
 cudaError_t launch_chi2_mixed_warp(const UniformArgs &a, const Tile &tile, float *out,

@@ -151,7 +151,6 @@ cudaError_t launch_chi2_mixed(const UniformArgs &a, const Tile &tile, float *out
 // systems; warp_tile picks the shape that spreads the work evenly over the
 // SMs.  Carries a DE-MC step when a.demc.states is set.
 bool warp_tile_ok(int G, int block);
-int warp_lanes_for(int n_obs);
 // G lanes per system give every lane at least 4 observations (G = 8: always)
 bool warp_lanes_fit(int G, int n_obs);
 // The built-in warp tile; multi_warp admits systems split over 2 or 4 warps

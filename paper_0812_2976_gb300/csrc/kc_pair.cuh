@@ -1,0 +1,356 @@
+// kc_pair.cuh -- the mixed path's evaluation of two observations at a time
+// in packed single precision (fma / add / mul .f32x2).
+//
+// What bounds the mixed kernels is FP32 issue and the register file's read
+// ports.  On a GB300 a packed instruction takes the FMA pipe as long as two
+// scalar ones but one issue slot (measured, clocks per warp and SM
+// sub-partition: FFMA 1.04, FFMA2 2.06; with three different registers, or
+// pairs, as operands 1.51 and 3.11), so a packed body leaves slots to the
+// MUFU, integer and shared-memory work: the same body ran the 2^20-system
+// sweep in 2067 us packed and 2221 scalar.  The body itself is cut to about
+// 45 FMA-pipe operations, 40 clocks of MUFU and one shared-memory gather per
+// planet-observation evaluation (before: 68 operations, 44 clocks): 68
+// clocks per warp and sub-partition in steady state, 104 before.
+//
+//  - mean anomaly, 8 operations instead of 13: the observation times and
+//    1/P are split at fixed binary places (2^-6 d and 2^-17 cycles/d), so
+//    that their product is a multiple of 2^-23 cycles and its difference
+//    from the nearest integer of the phase is exact in one FMA;
+//  - Mikkola's cubic start with its quintic correction replaced by a
+//    degree-four fit (below): within 8e-4 rad of the root instead of
+//    3.6e-3, which lets one Newton step (4 operations) stand for Halley's
+//    (9);
+//  - sin/cos of the start from a table at multiples of 2^-8 rad in shared
+//    memory and a rotation by the remainder (8 operations instead of 15);
+//  - the velocity as (A cos E - B sin E)/(1 - e cos E) with its last product
+//    inside the first operation of the compensated planet sum.
+// The whole solve runs on |M| (E is odd in M), with M's sign put back on
+// sin E.
+//
+// Accuracy, a float emulation of both forms over 2^20 draws each (P in 1 ..
+// 4000 d, 4000 d of observations; errors of M in rad, of v in units of K,
+// rms): M 6.9e-8 (scalar form 9.8e-8), v 7.9e-8 for e < 0.3 (9.1e-8),
+// 6.6e-8 for e in 0.3 .. 0.8 (8.2e-8), 5.9e-8 for 0.8 .. 0.95 (8.6e-8),
+// 7.3e-8 for 0.95 .. 0.99 (1.0e-7), 1.3e-7 for 0.99 .. 0.999 (1.4e-7).
+#pragma once
+
+#include "kc_device.cuh"
+
+namespace kc {
+
+// ------------------------------------------------ packed arithmetic
+
+typedef unsigned long long f32x2;      // two floats, the first in the low half
+
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 dup2(float a) { return pack2(a, a); }
+__device__ __forceinline__ float lo2(f32x2 a) {
+  float x, y;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a));
+  return x;
+}
+__device__ __forceinline__ float hi2(f32x2 a) {
+  float x, y;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a));
+  return y;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return pack2(-lo2(a), -hi2(a)); }
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return add2(a, neg2(b)); }
+__device__ __forceinline__ f32x2 rcp2(f32x2 a) {
+  return pack2(rcp_fast(lo2(a)), rcp_fast(hi2(a)));
+}
+
+// Two compensated sums side by side (Kahan, as in kc_device.cuh).
+struct Kahan2 {
+  f32x2 big, small;
+};
+
+// k += x where y = x - k.small is already formed (its subtraction can ride
+// in the FMA that produces x).
+__device__ __forceinline__ void kahan_add_y(Kahan2 &k, f32x2 y) {
+  const f32x2 t = add2(k.big, y);
+  k.small = sub2(sub2(t, k.big), y);
+  k.big = t;
+}
+__device__ __forceinline__ void kahan_add(Kahan2 &k, f32x2 x) { kahan_add_y(k, sub2(x, k.small)); }
+
+// The two sums of a pair as one.
+__device__ __forceinline__ Kahan kahan_join(const Kahan2 &k) {
+  Kahan a = {lo2(k.big), lo2(k.small)};
+  const Kahan b = {hi2(k.big), hi2(k.small)};
+  kahan_merge(a, b);
+  return a;
+}
+
+// ------------------------------------------------ sin/cos table
+
+// sin and cos at k 2^-8 rad, k = 0 .. 1023, rounded to float: 8 KB.  The start
+// of the solve lies in [0, 1.04 pi), below 3.3.  A power of two of entries,
+// so that the index of any start (NaN included, for an invalid planet) is
+// masked into the table.  Two arrays, not (sin, cos) words: two 4-byte
+// gathers land in the halves of the packed registers, where one 8-byte
+// gather per observation needed moves (1995 us against 2067 on the sweep).
+constexpr int kAngTabN = 1024;
+constexpr float kAngRound = 49152.0f;              // 1.5 * 2^15: rounds to 2^-8
+
+struct AngTab {
+  float s[kAngTabN], c[kAngTabN];
+};
+
+// Taylor series about 0 in double: below 2e-15 absolute for x < 4.
+constexpr double ang_series(double x, bool cosine) {
+  double term = cosine ? 1.0 : x, sum = 0.0;
+  for (int n = cosine ? 0 : 1; n < 50; n += 2) {
+    sum += term;
+    term *= -x * x / ((n + 1.0) * (n + 2.0));
+  }
+  return sum;
+}
+constexpr AngTab make_ang_tab() {
+  AngTab t{};
+  for (int k = 0; k < kAngTabN; ++k) {
+    t.s[k] = (float)ang_series(k / 256.0, false);
+    t.c[k] = (float)ang_series(k / 256.0, true);
+  }
+  return t;
+}
+static __device__ const __align__(16) AngTab kAngTab = make_ang_tab();
+
+// The CTA's copy in shared memory (16-byte copies; a barrier must follow).
+__device__ __forceinline__ void ang_tab_load(float *tab, int tid, int nthreads) {
+  const float4 *src = reinterpret_cast<const float4 *>(&kAngTab);
+  for (int i = tid; i < kAngTabN / 2; i += nthreads) reinterpret_cast<float4 *>(tab)[i] = src[i];
+}
+
+// ------------------------------------------------ observation times
+
+// tau = th + tl with th a multiple of 2^-6 d (or tau_hi itself from 2^17 d
+// on, whose last place is no finer) and |tl| <= 2^-7 d.
+constexpr float kTauPlace = 64.0f;
+__device__ __forceinline__ void tau_place(float &hi, float &lo) {
+  const float th = fabsf(hi) < 131072.0f ? rintf(hi * kTauPlace) * (1.0f / kTauPlace) : hi;
+  lo = __fadd_rn(__fsub_rn(hi, th), lo);
+  hi = th;
+}
+
+// Limits of the short form of the mean anomaly (mean_anomaly_pair): 1/P up
+// to 2 cycles/d, |tau| below 2^14 d (45 years).  Beyond them a CTA takes
+// mean_anomaly_wide for all its systems.
+constexpr float kPairMaxFreq = 2.0f;
+constexpr float kPairMaxTau = 16384.0f;
+
+// ------------------------------------------------ per-planet constants
+
+// Phase: n = 1/P rounded; nq its multiple of 2^-17 (n itself above 2^6,
+// whose last place is no finer), nlo the rest; c a multiple of 2^-23, clo the
+// rest, both low parts and n2pi times 2 pi.  Start: bs and q[0..4], below.
+// Velocity: v = (A cos E - B sin E)/(1 - e cos E), A = K cos w (1 - e^2),
+// B = K sqrt(1 - e^2) sin w.
+struct __align__(16) PlanetP {
+  float n, nq, c, nlo2pi;
+  float clo2pi, n2pi, e, bs;
+  float q[4];
+  float q4, A, B, pad;
+};
+
+// The start.  With a = (1 - e)/(4 e + 1/2), the real root of Mikkola's
+// cubic s^3 + 3 a s = M/(4 e + 1/2) is s = sqrt(a) (z - 1/z), z = (b +
+// sqrt(b^2 + 1))^(1/3), b = M bs, bs = 1/((8 e + 1) a^(3/2)); s is close to
+// sin(E/3), and sin E = 3 s - 4 s^3 there.  Instead of correcting s (his
+// -0.078 s^5/(1 + e)), sin E is taken as s (3 + c1 x + c2 x^2 + c3 x^3 +
+// c4 x^4), x = s^2, with c1 .. c4 cubics in e fitted to keep the error of
+// ONE NEWTON STEP small (weighted least squares with the weights iterated
+// towards the largest error, kepler_start_fit.py): the start is within 8e-4
+// rad, the step within 5.1e-9 rad of the root for every 0 <= e < 1 and |M|
+// <= 1.02 pi (as Halley's step from the quintic correction).  Scaled
+// to s' = z - 1/z: E0 = M + s' (q0 + q1 x' + .. + q4 x'^4), q_i = e c_i
+// a^(i + 1/2).
+__device__ __forceinline__ float start_fit(float e, float k0, float k1, float k2, float k3) {
+  return __fmaf_rn(e, __fmaf_rn(e, __fmaf_rn(e, k3, k2), k1), k0);
+}
+
+__device__ __forceinline__ void start_setup(PlanetP &p) {
+  const float e = p.e;
+  const float r = 1.0f / __fmaf_rn(4.0f, e, 0.5f);
+  const float a = fmaxf((1.0f - e) * r, 1e-8f);      // e rounded up to 1: finite
+  const float sa = sqrtf(a);
+  p.bs = 0.5f * r / (a * sa);
+  float f = e * sa;
+  p.q[0] = 3.0f * f;
+  f *= a;
+  p.q[1] = f * start_fit(e, -3.9074f, -0.4550f, 0.5740f, -0.2644f);
+  f *= a;
+  p.q[2] = f * start_fit(e, -0.8507f, 3.2176f, -3.9800f, 1.8248f);
+  f *= a;
+  p.q[3] = f * start_fit(e, 2.1773f, -6.5683f, 8.0450f, -3.7069f);
+  f *= a;
+  p.q4 = f * start_fit(e, -0.8390f, 3.4927f, -4.6815f, 2.2459f);
+}
+
+// Constants of one planet (K, e, w as in planet_setup_mixed).  An invalid
+// planet (checked by the caller) gets e = NaN, which makes its velocities
+// NaN.  wide: set if the period is too short for the short form.
+__device__ __forceinline__ PlanetP planet_setup_pair(const double *p, double t_ref, double t0,
+                                                     bool &wide) {
+  PlanetP q;
+  float n_hi, n_lo, c_hi, c_lo;
+  phase_setup_ds(p[0], p[4], t_ref, t0, n_hi, n_lo, c_hi, c_lo);
+  constexpr float kPlaceN = 131072.0f, kPlaceC = 8388608.0f;          // 2^17, 2^23
+  q.n = n_hi;
+  q.nq = n_hi < 64.0f ? rintf(n_hi * kPlaceN) * (1.0f / kPlaceN) : n_hi;
+  q.nlo2pi = __fadd_rn(__fsub_rn(n_hi, q.nq), n_lo) * kTwoPiF;
+  q.c = rintf(c_hi * kPlaceC) * (1.0f / kPlaceC);
+  q.clo2pi = __fadd_rn(__fsub_rn(c_hi, q.c), c_lo) * kTwoPiF;
+  q.n2pi = n_hi * kTwoPiF;
+  wide = !(n_hi <= kPairMaxFreq);
+  const float ef = d2f(p[2]);
+  q.e = planet_valid(p[0], p[1], p[2], p[3], p[4]) ? ef : __int_as_float(0x7fc00000);
+  start_setup(q);
+  float w_hi, w_lo;
+  split_d(p[3], w_hi, w_lo);
+  float sw, cw;
+  sincosf(w_hi, &sw, &cw);
+  const float sw1 = __fmaf_rn(w_lo, cw, sw);
+  cw = __fmaf_rn(-w_lo, sw, cw);
+  // K cos w b2 and K sin w sqrt(b2), b2 = 1 - e^2 in one rounding, each
+  // product rounded once (its remainder and K's low part carried)
+  float K_hi, K_lo;
+  split_d(p[1], K_hi, K_lo);
+  const float b2 = __fmaf_rn(-ef, ef, 1.0f), b = sqrtf(b2);
+  float u, ue;
+  two_prod(K_hi, cw, u, ue);
+  q.A = __fmaf_rn(u, b2, __fmaf_rn(K_lo, cw, ue) * b2);
+  two_prod(K_hi, sw1, u, ue);
+  q.B = __fmaf_rn(u, b, __fmaf_rn(K_lo, sw1, ue) * b);
+  q.pad = 0.0f;
+  return q;
+}
+
+// ------------------------------------------------ mean anomaly
+
+// M of two observations, |M| <= 1.02 pi.  k is the integer nearest to the
+// phase (up to tl n <= 2^-6 cycles); th nq is a multiple of 2^-23 and its
+// distance from k below 2, so the FMA is exact, and so is the sum with c.
+// The low parts (below 0.1 cycles) add three roundings near 2^-26 rad and
+// the final FMA one: 2.1e-7 rad at worst, 6.9e-8 rms.
+__device__ __forceinline__ f32x2 mean_anomaly_pair(f32x2 th, f32x2 tl, const PlanetP &q) {
+  const f32x2 magic = dup2(kRoundMagic);
+  const f32x2 y = fma2(th, dup2(q.n), dup2(q.c));
+  const f32x2 k = sub2(add2(y, magic), magic);
+  const f32x2 u = add2(fma2(th, dup2(q.nq), neg2(k)), dup2(q.c));
+  const f32x2 lo = fma2(tl, dup2(q.n2pi), fma2(th, dup2(q.nlo2pi), dup2(q.clo2pi)));
+  return fma2(u, dup2(kTwoPiF), lo);
+}
+
+// One observation at any period and time the double-single phase covers
+// (|tau/P| < 2^22): tau as the float pair of its leading 48 bits, the
+// product's FMA remainder kept, every part wrapped before the sum.
+__device__ __forceinline__ float mean_anomaly_wide(float th, float tl, const PlanetP &q) {
+  const float hi = __fadd_rn(th, tl);
+  const float lo = __fsub_rn(tl, __fsub_rn(hi, th));
+  const float p = __fmul_rn(hi, q.nq);
+  const float pe = __fmaf_rn(hi, q.nq, -p);
+  float lc = __fmaf_rn(lo, q.n, pe);
+  lc = __fadd_rn(lc, __fmaf_rn(hi, q.nlo2pi, q.clo2pi) * (float)kInvTwoPi);
+  lc = __fsub_rn(lc, round_small(lc));
+  float u = __fadd_rn(__fsub_rn(p, round_small(p)), q.c);
+  u = __fsub_rn(u, round_small(u));
+  u = __fsub_rn(u, round_small(__fadd_rn(u, lc)));
+  return __fmaf_rn(u, kTwoPiF, lc * kTwoPiF);
+}
+
+template <bool WIDE>
+__device__ __forceinline__ f32x2 mean_anomaly2(f32x2 th, f32x2 tl, const PlanetP &q) {
+  if (WIDE)
+    return pack2(mean_anomaly_wide(lo2(th), lo2(tl), q), mean_anomaly_wide(hi2(th), hi2(tl), q));
+  return mean_anomaly_pair(th, tl, q);
+}
+
+// ------------------------------------------------ Kepler's equation
+
+__device__ __forceinline__ float abs_bits(float x) {
+  return fabsf(x);
+}
+
+// s' = z - 1/z of the start for one |M|.  1/z is the exponential of the
+// negated logarithm: ex2 runs at twice the rate of rcp (4 clocks per warp
+// against 8).
+__device__ __forceinline__ float start_root(float b, float w) {
+  const float l = lg2_fast(b + sqrt_fast(w)) * (1.0f / 3.0f);
+  return ex2_fast(l) - ex2_fast(-l);
+}
+
+// Table index of the angle behind k = angle + kAngRound.
+__device__ __forceinline__ unsigned ang_index(float k) {
+  return __float_as_uint(k) & (kAngTabN - 1);
+}
+
+// Solves E - e sin E = |M| for two mean anomalies: sin E >= 0-signed as for
+// |M| (s, without M's sign), cos E (c) and, for a residual, E.
+// The table's angle a = E0 rounded to 2^-8 is exact in float, and so is b =
+// E0 - a, |b| <= 2^-9: sin b = b and cos b = 1 - b^2/2 to 1.3e-9.
+__device__ __forceinline__ void kepler_pair(f32x2 m, const PlanetP &q, const float *tab, f32x2 &s,
+                                            f32x2 &c, f32x2 &E) {
+  const f32x2 b = mul2(m, dup2(q.bs));
+  const f32x2 w = fma2(b, b, dup2(1.0f));
+  const f32x2 r = pack2(start_root(lo2(b), lo2(w)), start_root(hi2(b), hi2(w)));
+  const f32x2 x = mul2(r, r);
+  f32x2 p = fma2(x, dup2(q.q4), dup2(q.q[3]));
+  p = fma2(x, p, dup2(q.q[2]));
+  p = fma2(x, p, dup2(q.q[1]));
+  p = fma2(x, p, dup2(q.q[0]));
+  const f32x2 E0 = fma2(r, p, m);
+  // sin, cos of E0
+  const f32x2 k = add2(E0, dup2(kAngRound));
+  const f32x2 d0 = sub2(E0, sub2(k, dup2(kAngRound)));
+  const unsigned i0 = ang_index(lo2(k)), i1 = ang_index(hi2(k));
+  const f32x2 S = pack2(tab[i0], tab[i1]), C = pack2(tab[kAngTabN + i0], tab[kAngTabN + i1]);
+  const f32x2 h0 = mul2(d0, dup2(-0.5f));
+  const f32x2 s0 = fma2(d0, fma2(h0, S, C), S);
+  const f32x2 c0 = fma2(d0, fma2(h0, C, neg2(S)), C);
+  // Newton: d = (E0 - e sin E0 - m)/(1 - e cos E0), E = E0 - d
+  const f32x2 ne = dup2(-q.e);
+  const f32x2 f = fma2(ne, s0, sub2(E0, m));
+  const f32x2 d = mul2(f, rcp2(fma2(ne, c0, dup2(1.0f))));
+  const f32x2 h = mul2(d, dup2(-0.5f));
+  s = fma2(d, neg2(fma2(neg2(h), s0, c0)), s0);
+  c = fma2(d, fma2(h, c0, s0), c0);
+  E = sub2(E0, d);
+}
+
+// x with M's sign (x's own kept: an exclusive or).
+__device__ __forceinline__ f32x2 signed_as(f32x2 x, f32x2 M) {
+  const unsigned a = __float_as_uint(lo2(x)) ^ (__float_as_uint(lo2(M)) & 0x80000000u);
+  const unsigned b = __float_as_uint(hi2(x)) ^ (__float_as_uint(hi2(M)) & 0x80000000u);
+  return pack2(__uint_as_float(a), __uint_as_float(b));
+}
+
+__device__ __forceinline__ f32x2 abs2(f32x2 x) { return pack2(abs_bits(lo2(x)), abs_bits(hi2(x))); }
+
+// V += v with sin E already signed.
+__device__ __forceinline__ void velocity_sum(Kahan2 &V, const PlanetP &q, f32x2 s, f32x2 c) {
+  const f32x2 D = fma2(dup2(-q.e), c, dup2(1.0f));
+  const f32x2 num = fma2(dup2(q.A), c, neg2(mul2(dup2(q.B), s)));
+  kahan_add_y(V, fma2(num, rcp2(D), neg2(V.small)));
+}
+
+}  // namespace kc
