@@ -151,6 +151,17 @@ __device__ __forceinline__ double rcp_f64(double x) {
   return fma(r, fma(-x, r, 1.0), r);
 }
 
+// 1/x in double to about an ulp: the same seed and two Newton steps (four
+// FP64 operations instead of the nine of the IEEE division); outside the
+// normal float range the division.
+__device__ __forceinline__ double recip_d(double x) {
+  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  if (ex - 900u > 240u) return 1.0 / x;
+  double r = f2d(rcp_fast(d2f(x)));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
 // sin and cos for |x| <= 3 pi / 2 (the starting values of the
 // single-precision Kepler solve lie within pi + 0.1): x = k pi + r with
 // k = round(x / pi) in {-1, 0, 1} and pi split into two floats (the first
@@ -412,50 +423,6 @@ __device__ __forceinline__ void with_high_e(bool hi, F &&body) {
     body(HiTag<false>{});
 }
 
-// Table-driven sin/cos in double (the table method of Tang, 1989-1991):
-// x = k (2 pi/N) + b with k the nearest integer to x N/(2 pi) (chosen in
-// single precision from x as a float, kf), b reduced in double with 2 pi/N
-// split into two doubles, |b| <= pi/N + 1e-5; sin b and cos b by Taylor
-// series to b^5 and b^6 (truncation below 1e-17 at N = 256); then
-// sin x = S_k cos b + C_k sin b, cos x = C_k cos b - S_k sin b with
-// (S_k, C_k) = (sin, cos)(2 pi k/N) from a table in shared memory
-// (sincos_table_build).  The series' last terms, b^5/120 < 2.4e-12 and
-// b^6/720 < 4.9e-15, enter the combination through one single-precision
-// term each (error below 1e-18): 11 FP64 operations against 21 for
-// sincos_f64.
-constexpr int kSinTabN = 256;
-constexpr double kTabStepHi = 0.02454369260617026;      // RN(2 pi/256)
-constexpr double kTabStepLo = 9.567553118338697e-19;    // 2 pi/256 - hi
-constexpr float kTabInvStepF = 40.74366543152521f;      // 256/(2 pi)
-
-__device__ __forceinline__ void sincos_table_build(double2 *tab, int tid, int nthreads) {
-  for (int i = tid; i < kSinTabN; i += nthreads) {
-    double s, c;
-    sincos_f64(fma((double)i, kTabStepHi, (double)i * kTabStepLo), s, c);
-    tab[i] = make_double2(s, c);
-  }
-}
-
-// xf: x rounded to float (the FP64 path evaluates sin/cos at its
-// single-precision Kepler solution, or within a float ulp of it).
-__device__ __forceinline__ void sincos_tab(double x, float xf, const double2 *tab, double &s,
-                                           double &c) {
-  const float kf = rintf(xf * kTabInvStepF);
-  const double kd = f2d(kf);
-  double b = fma(-kd, kTabStepHi, x);
-  b = fma(-kd, kTabStepLo, b);
-  const double b2 = b * b;
-  const double sb3 = fma(b * b2, -1.0 / 6.0, b);                  // sin b to b^3
-  const double cb4 = fma(b2, fma(b2, 1.0 / 24.0, -0.5), 1.0);     // cos b to b^4
-  const double2 sc = tab[(int)kf & (kSinTabN - 1)];
-  const float bf = d2f(b), b2f = bf * bf;
-  const float sb5 = b2f * b2f * bf * (1.0f / 120.0f);             // b^5/120
-  const float cb6 = -(b2f * b2f * b2f) * (1.0f / 720.0f);         // -b^6/720
-  const float Sf = d2f(sc.x), Cf = d2f(sc.y);
-  s = fma(sc.x, cb4, fma(sc.y, sb3, f2d(__fmaf_rn(Sf, cb6, Cf * sb5))));
-  c = fma(sc.y, cb4, fma(-sc.x, sb3, f2d(__fmaf_rn(Cf, cb6, -(Sf * sb5)))));
-}
-
 // Halley's step -2 f f' / (2 f'^2 - f f'') = -f f' / (f'^2 - f e sin E / 2)
 // for f(E) = E - e sin E - M, in double: 8 FP64 operations (13 FLOPs)
 // against 26 FLOPs for Danby's quartic step.  From the single-precision
@@ -481,29 +448,20 @@ __device__ __forceinline__ double halley_delta_f64(double E, double M, double e,
 // order in that last step.  HI and e > kEccFast: two quartic steps in
 // double instead (the seed's error grows like 1e-7 / (1 - e cos E)).  The
 // single-precision work costs little here: one FP64 instruction takes as
-// long on GB300's FP64 pipe as ~76 FP32 issues.
-// With a table (tab != nullptr, sincos_table_build), sin/cos come from
-// sincos_tab.
+// long on GB300's FP64 pipe as 64 FP32 issues.
 template <bool HI = true>
-__device__ __forceinline__ double kepler_f64(double M, double e, double &sE, double &cE,
-                                             const double2 *tab = nullptr) {
+__device__ __forceinline__ double kepler_f64(double M, double e, double &sE, double &cE) {
   const float Mf = d2f(M), ef = d2f(e);
   float sf, cf;
   const float Ef = kepler_f32(Mf, ef, sf, cf);
   const bool high = HI && ef > kEccFast;
   double E = f2d(Ef);
   double s, c;
-  if (tab)
-    sincos_tab(E, Ef, tab, s, c);
-  else
-    sincos_f64(E, s, c);
+  sincos_f64(E, s, c);
   double d;
   if (high) {
     E += danby_delta_f64(E, M, e, s, c);
-    if (tab)
-      sincos_tab(E, d2f(E), tab, s, c);
-    else
-      sincos_f64(E, s, c);
+    sincos_f64(E, s, c);
     d = danby_delta_f64(E, M, e, s, c);
   } else {
     d = halley_delta_f64(E, M, e, s, c, ef, sf);

@@ -20,6 +20,7 @@
 
 #include "kc_demc.cuh"
 #include "kc_device.cuh"
+#include "kc_f64.cuh"
 #include "kc_internal.h"
 
 namespace kc {
@@ -41,16 +42,20 @@ struct MixedLayout {
   }
 };
 
-struct ObsD {
-  double tau, v, w, pad;
+constexpr size_t kMaxSmem = 227 * 1024;       // of a CTA
+
+struct __align__(16) ObsD {
+  double tau, v, w;
+  float tf, pad;            // tau in single precision
 };
 
+// In shared memory: the planets' constants, the systems' gamma and jitter,
+// the words that combine a system's warps, the staged observations.
 struct F64Layout {
-  size_t tab, pl, gam, s2, red, obs, total;
+  size_t pl, gam, s2, red, obs, total;
   __host__ __device__ F64Layout(int ST, int J, int nwarps, int obs_tile) {
-    tab = 0;                                          // sin/cos table, 4 KB
-    pl = tab + sizeof(double2) * kSinTabN;
-    gam = pl + sizeof(PlanetD) * ST * J;
+    pl = 0;
+    gam = pl + sizeof(PlanetX) * ST * J;
     s2 = gam + sizeof(double) * ST;
     red = align_up(s2 + sizeof(double) * ST, 16);
     obs = align_up(red + sizeof(double) * 2 * nwarps, 16);
@@ -85,14 +90,10 @@ constexpr double kLn2Pi = 1.8378770664093454836;      // ln(2 pi)
 // Inverse variance 1/(sigma_k^2 + sigma_jit^2) (Eq. 5); NaN if not positive.
 __device__ inline double inv_variance(double sigma, double jitter2) {
   const double var = fma(sigma, sigma, jitter2);
-  return (var > 0.0) ? 1.0 / var : __longlong_as_double(0x7ff8000000000000ll);
+  return (var > 0.0) ? recip_d(var) : __longlong_as_double(0x7ff8000000000000ll);
 }
 
 // ------------------------------------------------------------ mixed
-
-// Thread that handles setup item i: items are dealt round-robin over the
-// warps so that the double-precision setup runs on every SM sub-partition.
-__device__ inline int setup_slot(int tid, int nwarps) { return (tid & 31) * nwarps + (tid >> 5); }
 
 // Prepared inputs of the split variant: per-(system, planet) constants,
 // per-system gamma (NaN if invalid) and converted observations, written by
@@ -467,16 +468,23 @@ chi2_mixed_chunk_kernel(UniformArgs a, MixedPrep prep, ChunkScratch cs, int chun
 
 // ------------------------------------------------------------ FP64
 
+// Bound by the FP64 pipe (kc_f64.cuh: 7 FP64 instructions per evaluation and
+// 4 per observation, 64 clocks each).  The sin/cos table (54 KB) is read from
+// global memory through L1, where it stays: copied to shared memory by each
+// CTA it ran the same (4096 x 4 x 256: 110.8 against 111.0 us before the last
+// cuts) and cost small batches the copy (64 x 1 x 32: 8.3 against 10.3 us).
+// The planets' setup, about 45 FP64 instructions of one lane each, is dealt
+// densely to one warp of the CTA (the pipe's cost is per warp, not per
+// lane), another one in each CTA so that no sub-partition takes them all.
 template <int J, bool NLL = false, bool DEMC = false>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, 4)
 chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
                 float *__restrict__ resid_out) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int block = blockDim.x;
   const int ST = block / G;
   const F64Layout L(ST, J, block / 32, obs_tile);
-  double2 *tab_s = reinterpret_cast<double2 *>(smem + L.tab);
-  PlanetD *pl_s = reinterpret_cast<PlanetD *>(smem + L.pl);
+  PlanetX *pl_s = reinterpret_cast<PlanetX *>(smem + L.pl);
   double *gam_s = reinterpret_cast<double *>(smem + L.gam);
   double *s2_s = reinterpret_cast<double *>(smem + L.s2);
   double *red_s = reinterpret_cast<double *>(smem + L.red);
@@ -488,21 +496,24 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
   const double t_ref = a.n_obs > 0 ? a.t[0] : a.t0;
   const double dref = t_ref - a.t0;
   const bool want_resid = resid_out != nullptr;
-  sincos_table_build(tab_s, tid, block);      // read after the tile loop's first barrier
 
-  for (int i = setup_slot(tid, block >> 5); i < ST * J; i += block) {
-    const int sl = i / J, j = i - sl * J;
-    const int64_t s = sys0 + sl;
-    PlanetD q = {};
-    if (s < a.n_sys && dbg_ok(a.invalid, s * npar + 5 * j + 4 < a.n_sys * npar, kDbgParam,
-                              s * npar + 5 * j))
-      q = planet_setup_f64(a.params + s * npar + 5 * j, dref);
-    pl_s[i] = q;
-  }
-  for (int i = tid; i < ST; i += block) {
+  for (int i = block - 1 - tid; i < ST; i += block) {
     const int64_t s = sys0 + i;
     gam_s[i] = s < a.n_sys ? system_gamma(a.params + s * npar, J) : 0.0;
     if (NLL) s2_s[i] = s < a.n_sys ? system_jitter2(a.params + s * npar, J) : 0.0;
+  }
+  int first = tid - 32 * (int)(blockIdx.x % (unsigned)(block >> 5));
+  if (first < 0) first += block;
+  for (int i = first; i < ST * J; i += block) {
+    const int sl = i / J, j = i - sl * J;
+    const int64_t s = sys0 + sl;
+    PlanetX q = {};
+    if (s < a.n_sys && dbg_ok(a.invalid, s * npar + 5 * j + 4 < a.n_sys * npar, kDbgParam,
+                              s * npar + 5 * j)) {
+      double sw, cw, beta;
+      q = planet_setup_x(a.params + s * npar + 5 * j, dref, sw, cw, beta);
+    }
+    pl_s[i] = q;
   }
 
   const int sl = tid / G, c = tid - sl * G;
@@ -511,19 +522,20 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
 
   for (int k0 = 0; k0 < a.n_obs; k0 += obs_tile) {
     const int nk = min(obs_tile, a.n_obs - k0);
-    __syncthreads();
+    if (k0 > 0) __syncthreads();
     for (int k = tid; k < nk; k += block) {
       if (!dbg_ok(a.invalid, k0 + k < a.n_obs && k < obs_tile, kDbgObs, k0 + k)) continue;
       ObsD o;
       o.tau = a.t[k0 + k] - t_ref;
       o.v = a.v[k0 + k];
       o.w = NLL ? a.sigma[k0 + k] * a.sigma[k0 + k] : inv_variance(a.sigma[k0 + k], a.jitter2);
-      o.pad = 0.0;
+      o.tf = d2f(o.tau);
+      o.pad = 0.0f;
       obs_s[k] = o;
     }
     __syncthreads();
     const double gam = gam_s[sl];
-    const PlanetD *q = pl_s + sl * J;
+    const PlanetX *q = pl_s + sl * J;
     bool hi = false;
 #pragma unroll
     for (int j = 0; j < J; ++j) hi = hi || q[j].e > (double)kEccFast;
@@ -531,17 +543,22 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
       constexpr bool HI = decltype(tag)::value;
       for (int k = c; k < nk; k += G) {
         const ObsD o = obs_s[k];
-        double V = gam;
-#pragma unroll
+        double r = gam - o.v;
+        float vh = 0.0f, vl = 0.0f;
+#pragma unroll 1
         for (int j = 0; j < J; ++j) {
-          const PlanetD p = q[j];
-          const double M = mean_anomaly_f64(o.tau, p);
-          double sE, cE;
-          const double E = kepler_f64<HI>(M, p.e, sE, cE, tab_s);
-          if (want_resid) rmax = fmax(rmax, fabs((E - M) - p.e * sE));
-          V = velocity_add_f64(p, sE, cE, V);
+          const PlanetX &p = q[j];
+          if (HI) {
+            double sE, cE, res;
+            r = eval_high(o.tau, o.tf, p, r, sE, cE, res);
+            if (want_resid) rmax = fmax(rmax, res);
+          } else {
+            const EvalX x = solve_x(o.tau, o.tf, p);
+            if (want_resid) rmax = fmax(rmax, resid_x(x, p));
+            velocity_x(x, p, r, vh, vl);
+          }
         }
-        const double r = V - o.v;
+        if (!HI) r = add_pair(r, vh, vl);
         if (NLL) {
           const double var = o.w + s2_s[sl];
           const double wk = var > 0.0 ? 1.0 / var : __longlong_as_double(0x7ff8000000000000ll);
@@ -552,6 +569,7 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
       }
     });
   }
+  if (a.n_obs == 0) __syncthreads();            // gam_s, s2_s written by other threads
 
   const int gw = G < 32 ? G : 32;
   for (int m = gw >> 1; m >= 1; m >>= 1) {
@@ -585,28 +603,53 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
 
 // ------------------------------------------------------------ prediction
 
-// V(t_k) = gamma + sum_j v_j(t_k) in FP64, one thread per (system, obs).
-__global__ void rv_predict_kernel(const double *__restrict__ params, const double *__restrict__ t,
-                                  int64_t n_sys, int J, int n_obs, double t0,
-                                  double *__restrict__ v_out) {
-  const int64_t total = n_sys * (int64_t)n_obs;
+// V(t_k) = gamma + sum_j v_j(t_k) in FP64, G threads per system and `chunk`
+// observations of each of the CTA's systems per CTA.  Bound by the FP64 pipe
+// like chi2 (kc_f64.cuh); the planets are set up once per CTA, where one
+// thread per (system, observation) had repeated the setup at every
+// evaluation (512 x 3 x 1000: 305 us, now 38).
+constexpr int kPredictBlock = 128;
+constexpr int kPredictMinG = 8;
+
+__global__ void __launch_bounds__(kPredictBlock)
+rv_predict_kernel(const double *__restrict__ params, const double *__restrict__ t, int64_t n_sys,
+                  int J, int n_obs, double t0, int G, int chunk, int chunks,
+                  double *__restrict__ v_out) {
+  __shared__ PlanetX pl_s[kPredictBlock / kPredictMinG * KC_MAX_PLANETS];
+  __shared__ double gam_s[kPredictBlock / kPredictMinG];
+  const int tid = threadIdx.x, ST = kPredictBlock / G;
   const int npar = 5 * J + 1;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t s = i / n_obs;
-    const int k = (int)(i - s * n_obs);
-    const double *p = params + s * npar;
-    const double t_ref = t[0];
-    double V = system_gamma(p, J);
-    for (int j = 0; j < J; ++j) {
-      const PlanetD q = planet_setup_f64(p + 5 * j, t_ref - t0);
-      const double M = mean_anomaly_f64(t[k] - t_ref, q);
-      double sE, cE;
-      kepler_f64(M, q.e, sE, cE);
-      V = velocity_add_f64(q, sE, cE, V);
+  const int64_t group = blockIdx.x / chunks;
+  const int k0 = (int)(blockIdx.x - group * chunks) * chunk, k1 = min(n_obs, k0 + chunk);
+  const int64_t sys0 = group * ST;
+  const double t_ref = t[0];
+  for (int i = kPredictBlock - 1 - tid; i < ST; i += kPredictBlock)
+    if (sys0 + i < n_sys) gam_s[i] = system_gamma(params + (sys0 + i) * npar, J);
+  int first = tid - 32 * (int)(blockIdx.x % (kPredictBlock / 32));
+  if (first < 0) first += kPredictBlock;
+  for (int i = first; i < ST * J; i += kPredictBlock) {
+    const int64_t s = sys0 + i / J;
+    PlanetX q = {};
+    if (s < n_sys) {
+      double sw, cw, beta;
+      q = planet_setup_x(params + s * npar + 5 * (i % J), t_ref - t0, sw, cw, beta);
     }
-    v_out[i] = V;
+    pl_s[i] = q;
   }
+  __syncthreads();
+  const int sl = tid / G, c = tid - sl * G;
+  const int64_t s = sys0 + sl;
+  const PlanetX *q = pl_s + sl * J;
+  bool hi = false;
+  for (int j = 0; j < J; ++j) hi = hi || q[j].e > (double)kEccFast;
+  const double gam = s < n_sys ? gam_s[sl] : 0.0;
+  with_high_e(any_high_e(hi), [&](auto tag) {
+    constexpr bool HI = decltype(tag)::value;
+    for (int k = k0 + c; k < k1; k += G) {
+      const double V = model_velocity<HI>(t[k] - t_ref, q, J, gam);
+      if (s < n_sys) v_out[s * n_obs + k] = V;
+    }
+  });
 }
 
 // ------------------------------------------------------------ Kepler only
@@ -698,8 +741,18 @@ size_t smem_chi2_mixed(int n_pl, const Tile &t) {
   return MixedLayout(t.block / t.G, n_pl, t.block / 32, t.obs_tile).total;
 }
 
-size_t smem_chi2_f64(int n_pl, const Tile &t) {
-  return F64Layout(t.block / t.G, n_pl, t.block / 32, t.obs_tile).total;
+// Shared memory of an FP64 launch, and as many observations at a time as fit
+// (wide CTAs of one-thread systems keep up to 2048 planets).
+struct F64Shape {
+  int obs_tile;
+  size_t smem;
+};
+static F64Shape f64_shape(int n_pl, const Tile &t) {
+  F64Shape f{t.obs_tile, 0};
+  auto bytes = [&] { return F64Layout(t.block / t.G, n_pl, t.block / 32, f.obs_tile).total; };
+  while (bytes() > kMaxSmem && f.obs_tile > 32) f.obs_tile = (f.obs_tile + 1) / 2;
+  f.smem = bytes();
+  return f;
 }
 
 #define KC_DISPATCH_J(J, MACRO) \
@@ -874,19 +927,19 @@ cudaError_t launch_chi2_f64(const UniformArgs &a_in, const Tile &tile, double *o
   UniformArgs a = a_in;
   cudaError_t err = form_proposals(a, st);
   if (err != cudaSuccess) return err;
-  const size_t smem = smem_chi2_f64(a.n_pl, tile);
+  const F64Shape f = f64_shape(a.n_pl, tile);
+  const size_t smem = f.smem;
   const int grid = grid_for(a.n_sys, tile.block / tile.G);
 #define KC_LAUNCH(JJ)                                                                      \
   if (a.demc.states) {                                                                     \
     err = set_smem(chi2_f64_kernel<JJ, false, true>, smem);                                \
     if (err == cudaSuccess)                                                                \
-      chi2_f64_kernel<JJ, false, true><<<grid, tile.block, smem, st>>>(a, tile.G,            \
-                                                                      tile.obs_tile, out, resid); \
+      chi2_f64_kernel<JJ, false, true><<<grid, tile.block, smem, st>>>(a, tile.G, f.obs_tile, \
+                                                                      out, resid);         \
   } else {                                                                                 \
     err = set_smem(chi2_f64_kernel<JJ>, smem);                                             \
     if (err == cudaSuccess)                                                                \
-      chi2_f64_kernel<JJ><<<grid, tile.block, smem, st>>>(a, tile.G, tile.obs_tile, out,     \
-                                                          resid);                          \
+      chi2_f64_kernel<JJ><<<grid, tile.block, smem, st>>>(a, tile.G, f.obs_tile, out, resid); \
   }
   KC_DISPATCH_J(a.n_pl, KC_LAUNCH)
 #undef KC_LAUNCH
@@ -930,14 +983,14 @@ cudaError_t launch_nll_mixed(const UniformArgs &a, const Tile &tile, float *out,
 }
 
 cudaError_t launch_nll_f64(const UniformArgs &a, const Tile &tile, double *out, cudaStream_t st) {
-  const size_t smem = smem_chi2_f64(a.n_pl, tile);
+  const F64Shape f = f64_shape(a.n_pl, tile);
+  const size_t smem = f.smem;
   const int grid = grid_for(a.n_sys, tile.block / tile.G);
   cudaError_t err = cudaSuccess;
-#define KC_LAUNCH(JJ)                                                                      \
-  err = set_smem(chi2_f64_kernel<JJ, true>, smem);                                         \
-  if (err == cudaSuccess)                                                                  \
-    chi2_f64_kernel<JJ, true><<<grid, tile.block, smem, st>>>(a, tile.G, tile.obs_tile, out, \
-                                                              nullptr);
+#define KC_LAUNCH(JJ)                                                                       \
+  err = set_smem(chi2_f64_kernel<JJ, true>, smem);                                          \
+  if (err == cudaSuccess)                                                                   \
+    chi2_f64_kernel<JJ, true><<<grid, tile.block, smem, st>>>(a, tile.G, f.obs_tile, out, nullptr);
   KC_DISPATCH_J(a.n_pl, KC_LAUNCH)
 #undef KC_LAUNCH
   if (err != cudaSuccess) return err;
@@ -946,9 +999,17 @@ cudaError_t launch_nll_f64(const UniformArgs &a, const Tile &tile, double *out, 
 
 cudaError_t launch_rv_predict(const double *params, const double *t, int64_t n_sys, int n_pl,
                               int n_obs, double t0, double *v_out, cudaStream_t st) {
-  const int64_t total = n_sys * (int64_t)n_obs;
-  rv_predict_kernel<<<elementwise_grid(total), 256, 0, st>>>(params, t, n_sys, n_pl, n_obs, t0,
-                                                             v_out);
+  int G = kPredictMinG;
+  while (G < kPredictBlock && G < n_obs) G <<= 1;
+  const int64_t groups = (n_sys + kPredictBlock / G - 1) / (kPredictBlock / G);
+  // up to eight observations per thread share a CTA's setup, as long as the
+  // CTAs still fill the SMs four times over
+  int per = 8;
+  while (per > 1 && groups * ((n_obs + per * G - 1) / (per * G)) < (int64_t)sm_count() * 4) per /= 2;
+  const int chunk = per * G, chunks = (n_obs + chunk - 1) / chunk;
+  if (groups * chunks > 0x7fffffff) return cudaErrorInvalidConfiguration;
+  rv_predict_kernel<<<(unsigned)(groups * chunks), kPredictBlock, 0, st>>>(
+      params, t, n_sys, n_pl, n_obs, t0, G, chunk, chunks, v_out);
   return cudaGetLastError();
 }
 

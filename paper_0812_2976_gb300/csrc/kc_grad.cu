@@ -23,6 +23,7 @@
 #include <cmath>
 
 #include "kc_device.cuh"
+#include "kc_f64.cuh"
 #include "kc_internal.h"
 #include "kc_tcgen05.cuh"
 
@@ -93,7 +94,7 @@ constexpr double kLn2PiG = 1.8378770664093454836;      // ln(2 pi)
 
 __device__ inline double inv_variance_g(double sigma, double jitter2) {
   const double var = fma(sigma, sigma, jitter2);
-  return (var > 0.0) ? 1.0 / var : nan_d();
+  return (var > 0.0) ? recip_d(var) : nan_d();
 }
 
 template <typename T>
@@ -133,15 +134,28 @@ struct ObsGD {
   double tau, v, w, dt;    // dt = t - t0
 };
 
+// Staged observation of the FP64 gradient (tf = tau in single precision).
+struct __align__(16) ObsXD {
+  double tau, v, w, dt;    // dt = t - t0
+  float tf, pad;
+  double pad2;
+};
+
+// Planet constants of the FP64 gradient: the solve's, and those of the
+// partials in the form below.
+struct __align__(8) GradPlanetX {
+  PlanetX base;
+  double K, sw, cw, A1, B1, C1, esw, beta, ibeta, n2;
+};
+
 struct F64GradLayout {
-  size_t tab, pl, gam, sj, obs, total;
+  size_t pl, gam, sj, obs, total;
   __host__ __device__ F64GradLayout(int ST, int J, int obs_tile) {
-    tab = 0;                                          // sin/cos table, 4 KB
-    pl = tab + sizeof(double2) * kSinTabN;
-    gam = pl + sizeof(GradPlanetD) * ST * J;
+    pl = 0;
+    gam = pl + sizeof(GradPlanetX) * ST * J;
     sj = gam + sizeof(double) * ST;
     obs = align_up(sj + sizeof(double) * ST, 16);
-    total = align_up(obs + sizeof(ObsGD) * obs_tile, 16);
+    total = align_up(obs + sizeof(ObsXD) * obs_tile, 16);
   }
 };
 
@@ -287,8 +301,38 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
 
 // ------------------------------------------------------------ FP64
 
+// Bound by the FP64 pipe: 27 FP64 instructions per evaluation (kc_f64.cuh's
+// solve 4, sin E, cos E and 1/D 5, the velocity and Q 7, the partials and
+// their sums 11), 105 before.  With
+// y = 1/D, A1 = cos w (1 - e^2), B1 = beta sin w, C1 = beta cos w,
+//   dv/dK  = (A1 cos E - B1 sin E) y = v/K,
+//   Q      = sin(w + f) = (sin w cos E + C1 sin E - e sin w) y,
+//   dv/dw  = -K (Q + e sin w),   dv/dM0 = -K beta Q y^2,
+//   dv/de  = K cos w - K Q y sin E (1/beta + beta y),
+// so the sums over the observations need only those of a v/K, a Q, a Q y^2,
+// a dt Q y^2 and a Q y sin E (1/beta + beta y), a = 2 w r: the per-planet
+// factors, and the parts a alone multiplies (its sum is gamma's gradient),
+// are applied once per system.
+__device__ inline GradPlanetX grad_setup_x(const double *p, double dref) {
+  GradPlanetX g;
+  double sw, cw, beta;
+  g.base = planet_setup_x(p, dref, sw, cw, beta);
+  const double e = p[2];
+  g.K = p[1];
+  g.sw = sw;
+  g.cw = cw;
+  g.A1 = cw * ((1.0 - e) * (1.0 + e));
+  g.B1 = beta * sw;
+  g.C1 = beta * cw;
+  g.esw = e * sw;
+  g.beta = beta;
+  g.ibeta = 1.0 / beta;
+  g.n2 = g.base.inv_P * g.base.inv_P;
+  return g;
+}
+
 template <int J, bool NLL = false>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
 grad_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ chi2_out,
                 double *__restrict__ grad_out) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -296,115 +340,140 @@ grad_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ chi2_ou
   const int block = blockDim.x;
   const int ST = block / G;
   const F64GradLayout L(ST, J, obs_tile);
-  double2 *tab_s = reinterpret_cast<double2 *>(smem + L.tab);
-  GradPlanetD *pl_s = reinterpret_cast<GradPlanetD *>(smem + L.pl);
+  GradPlanetX *pl_s = reinterpret_cast<GradPlanetX *>(smem + L.pl);
   double *gam_s = reinterpret_cast<double *>(smem + L.gam);
   double *sj_s = reinterpret_cast<double *>(smem + L.sj);
-  ObsGD *obs_s = reinterpret_cast<ObsGD *>(smem + L.obs);
+  ObsXD *obs_s = reinterpret_cast<ObsXD *>(smem + L.obs);
 
   const int tid = threadIdx.x;
   const int64_t sys0 = (int64_t)blockIdx.x * ST;
   const double t_ref = a.n_obs > 0 ? a.t[0] : a.t0;
   const double dref = t_ref - a.t0;
-  sincos_table_build(tab_s, tid, block);      // read after the tile loop's first barrier
 
-  for (int i = (tid & 31) * (block >> 5) + (tid >> 5); i < ST * J; i += block) {
-    const int sl = i / J, j = i - sl * J;
-    const int64_t s = sys0 + sl;
-    GradPlanetD q = {};
-    if (s < a.n_sys && dbg_ok(a.invalid, s * NP + 5 * j + 4 < a.n_sys * NP, kDbgParam, s * NP))
-      q = grad_setup_f64(a.params + s * NP + 5 * j, dref);
-    pl_s[i] = q;
-  }
-  for (int i = tid; i < ST; i += block) {
+  for (int i = block - 1 - tid; i < ST; i += block) {
     const int64_t s = sys0 + i;
     gam_s[i] = s < a.n_sys ? system_gamma_g(a.params + s * NP, J) : 0.0;
     if (NLL) sj_s[i] = s < a.n_sys ? system_jitter_g(a.params + s * NP, J) : 0.0;
   }
+  // the planets' setup dealt densely to one warp, another in each CTA
+  int first = tid - 32 * (int)(blockIdx.x % (unsigned)(block >> 5));
+  if (first < 0) first += block;
+  for (int i = first; i < ST * J; i += block) {
+    const int sl = i / J, j = i - sl * J;
+    const int64_t s = sys0 + sl;
+    GradPlanetX q = {};
+    if (s < a.n_sys && dbg_ok(a.invalid, s * NP + 5 * j + 4 < a.n_sys * NP, kDbgParam, s * NP))
+      q = grad_setup_x(a.params + s * NP + 5 * j, dref);
+    pl_s[i] = q;
+  }
 
   const int sl = tid / G, c = tid - sl * G;
   const int64_t s = sys0 + sl;
-  double acc = 0.0;
-  double g[NP];
+  double acc = 0.0, sum_a = 0.0, sum_j = 0.0;
+  double g[5 * J];
 #pragma unroll
-  for (int i = 0; i < NP; ++i) g[i] = 0.0;
+  for (int i = 0; i < 5 * J; ++i) g[i] = 0.0;
 
   for (int k0 = 0; k0 < a.n_obs; k0 += obs_tile) {
     const int nk = min(obs_tile, a.n_obs - k0);
-    __syncthreads();
+    if (k0 > 0) __syncthreads();
     for (int k = tid; k < nk; k += block) {
       if (!dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k)) continue;
-      ObsGD o;
+      ObsXD o;
       const double tk = a.t[k0 + k];
       o.tau = tk - t_ref;
       o.v = a.v[k0 + k];
       o.w = NLL ? a.sigma[k0 + k] * a.sigma[k0 + k] : inv_variance_g(a.sigma[k0 + k], a.jitter2);
       o.dt = tk - a.t0;
+      o.tf = d2f(o.tau);
+      o.pad = 0.0f;
+      o.pad2 = 0.0;
       obs_s[k] = o;
     }
     __syncthreads();
     const double gam = gam_s[sl];
-    const GradPlanetD *q = pl_s + sl * J;
+    const GradPlanetX *q = pl_s + sl * J;
     bool hi = false;
 #pragma unroll
     for (int j = 0; j < J; ++j) hi = hi || q[j].base.e > (double)kEccFast;
     with_high_e(any_high_e(hi), [&](auto tag) {
       constexpr bool HI = decltype(tag)::value;
       for (int k = c; k < nk; k += G) {
-        const ObsGD o = obs_s[k];
-        double sEj[J], cEj[J];
-        double V = gam;
-#pragma unroll
+        const ObsXD o = obs_s[k];
+        double sE[J], dK[J], Q[J], y[J];
+        double r = gam - o.v;
+#pragma unroll (J <= 3 ? J : 1)
         for (int j = 0; j < J; ++j) {
-          const PlanetD p = q[j].base;
-          const double M = mean_anomaly_f64(o.tau, p);
-          kepler_f64<HI>(M, p.e, sEj[j], cEj[j], tab_s);
-          V = velocity_add_f64(p, sEj[j], cEj[j], V);
+          const GradPlanetX &p = q[j];
+          double cE;
+          if (HI) {
+            double res;
+            eval_high(o.tau, o.tf, p.base, 0.0, sE[j], cE, res);
+            y[j] = 1.0 / fma(-p.base.e, cE, 1.0);
+          } else {
+            solved_d(solve_x(o.tau, o.tf, p.base), p.base.e, sE[j], cE, y[j]);
+          }
+          dK[j] = fma(p.A1, cE, -(p.B1 * sE[j])) * y[j];
+          Q[j] = fma(p.C1, sE[j], fma(p.sw, cE, -p.esw)) * y[j];
+          r = fma(p.K, dK[j], r);
         }
-        const double r = V - o.v;
         double a2;
         if (NLL) {
           const double sj = sj_s[sl];
           const double var = fma(sj, sj, o.w);
-          const double wk = var > 0.0 ? 1.0 / var : nan_d();
-          acc += fma(wk * r, r, log(var));
-          a2 = wk * r;
-          g[NP - 1] = fma(sj * wk, fma(-wk * r, r, 1.0), g[NP - 1]);
+          const double wk = var > 0.0 ? recip_d(var) : nan_d();
+          const double wr = wk * r;
+          acc += fma(wr, r, log(var));
+          a2 = wr;
+          sum_j = fma(wk, fma(-wr, r, 1.0), sum_j);
         } else {
-          acc = fma(o.w * r, r, acc);
-          a2 = 2.0 * o.w * r;
+          const double wr = o.w * r;
+          acc = fma(wr, r, acc);
+          a2 = 2.0 * wr;
         }
+        sum_a += a2;
+        const double adt = a2 * o.dt;
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-          const GradPlanetD qj = q[j];
-          Partials<double> d;
-          const double invD = 1.0 / fma(-qj.base.e, cEj[j], 1.0);
-          velocity_partials(qj.base.e, qj.K, qj.cw, qj.sw, qj.base.beta, qj.ibeta, sEj[j], cEj[j],
-                            invD, d);
-          d.dP = d.dM * (-kTwoPi * o.dt * qj.n2);
-          g[5 * j + 0] = fma(a2, d.dP, g[5 * j + 0]);
-          g[5 * j + 1] = fma(a2, d.dK, g[5 * j + 1]);
-          g[5 * j + 2] = fma(a2, d.de, g[5 * j + 2]);
-          g[5 * j + 3] = fma(a2, d.dw, g[5 * j + 3]);
-          g[5 * j + 4] = fma(a2, d.dM, g[5 * j + 4]);
+          const GradPlanetX &p = q[j];
+          const double Qy = Q[j] * y[j], Qyy = Qy * y[j];
+          const double h = fma(p.beta, y[j], p.ibeta);
+          g[5 * j + 0] = fma(adt, Qyy, g[5 * j + 0]);
+          g[5 * j + 1] = fma(a2, dK[j], g[5 * j + 1]);
+          g[5 * j + 2] = fma(a2 * Qy, sE[j] * h, g[5 * j + 2]);
+          g[5 * j + 3] = fma(a2, Q[j], g[5 * j + 3]);
+          g[5 * j + 4] = fma(a2, Qyy, g[5 * j + 4]);
         }
-        g[5 * J] += a2;
       }
     });
   }
+  if (a.n_obs == 0) __syncthreads();            // gam_s, sj_s written by other threads
 
   for (int m = G >> 1; m >= 1; m >>= 1) {
     acc += shfl_xor(acc, m);
+    sum_a += shfl_xor(sum_a, m);
+    if (NLL) sum_j += shfl_xor(sum_j, m);
 #pragma unroll
-    for (int i = 0; i < NP; ++i) g[i] += shfl_xor(g[i], m);
+    for (int i = 0; i < 5 * J; ++i) g[i] += shfl_xor(g[i], m);
   }
   if (c == 0 && s < a.n_sys) {
     const double poison = 0.0 * gam_s[sl] + (NLL ? 0.0 * sj_s[sl] : 0.0);
     const double value = NLL ? 0.5 * (acc + a.n_obs * kLn2PiG) + poison : acc + poison;
     if (chi2_out) chi2_out[s] = value;
     note_invalid(a.invalid, value);
+    double *out = grad_out + s * NP;
 #pragma unroll
-    for (int i = 0; i < NP; ++i) grad_out[s * NP + i] = g[i] + poison;
+    for (int j = 0; j < J; ++j) {
+      const GradPlanetX &p = pl_s[sl * J + j];
+      const double Kb = p.K * p.beta;
+      out[5 * j + 0] = fma(Kb * (kTwoPi * p.n2), g[5 * j + 0], poison);
+      out[5 * j + 1] = g[5 * j + 1] + poison;
+      out[5 * j + 2] = fma(p.K, fma(p.cw, sum_a, -g[5 * j + 2]), poison);
+      out[5 * j + 3] = fma(-p.K, fma(p.esw, sum_a, g[5 * j + 3]), poison);
+      out[5 * j + 4] = fma(-Kb, g[5 * j + 4], poison);
+    }
+    out[5 * J] = sum_a + poison;
+    if (NLL) out[5 * J + 1] = fma(sj_s[sl], sum_j, poison);
   }
 }
 
@@ -1162,10 +1231,31 @@ cudaError_t set_smem(Kern k, size_t bytes) {
 
 }  // namespace
 
-size_t smem_grad(int n_pl, const Tile &t, bool f64) {
-  const int ST = t.block / t.G;
-  return f64 ? F64GradLayout(ST, n_pl, t.obs_tile).total
-             : MixedGradLayout(ST, n_pl, t.obs_tile).total;
+// Launch shape of a gradient tile: as many observations at a time as fit
+// beside the planets of the CTA's systems, and a smaller CTA where the planets
+// alone do not fit (tiles of few threads per system).
+struct GradShape {
+  int block, obs_tile;
+  size_t smem;
+};
+static GradShape grad_shape(int n_pl, const Tile &t, bool f64) {
+  GradShape f{t.block, t.obs_tile, 0};
+  auto bytes = [&] {
+    const int ST = f.block / t.G;
+    return f64 ? F64GradLayout(ST, n_pl, f.obs_tile).total
+               : MixedGradLayout(ST, n_pl, f.obs_tile).total;
+  };
+  constexpr size_t kMax = 227 * 1024;
+  while (bytes() > kMax) {
+    if (f.obs_tile > 32)
+      f.obs_tile = (f.obs_tile + 1) / 2;
+    else if (f.block > 32)
+      f.block = (f.block / 2 + 31) / 32 * 32;
+    else
+      break;
+  }
+  f.smem = bytes();
+  return f;
 }
 
 #define KC_DISPATCH_J(J, MACRO) \
@@ -1184,14 +1274,15 @@ size_t smem_grad(int n_pl, const Tile &t, bool f64) {
 cudaError_t launch_grad_mixed(const UniformArgs &a, const Tile &tile, float *chi2, float *grad,
                               cudaStream_t st, bool nll) {
   if (tile.G > 32) return cudaErrorInvalidValue;
-  const size_t smem = smem_grad(a.n_pl, tile, false);
-  const int ST = tile.block / tile.G;
+  const GradShape f = grad_shape(a.n_pl, tile, false);
+  const size_t smem = f.smem;
+  const int ST = f.block / tile.G;
   const int grid = (int)((a.n_sys + ST - 1) / ST);
   cudaError_t err = cudaSuccess;
 #define KC_LAUNCH_NLL(JJ, NN)                                                                   \
   err = set_smem(grad_mixed_kernel<JJ, NN>, smem);                                              \
   if (err == cudaSuccess)                                                                       \
-    grad_mixed_kernel<JJ, NN><<<grid, tile.block, smem, st>>>(a, tile.G, tile.obs_tile, chi2,     \
+    grad_mixed_kernel<JJ, NN><<<grid, f.block, smem, st>>>(a, tile.G, f.obs_tile, chi2,           \
                                                               grad);
 #define KC_LAUNCH(JJ)                      \
   if (nll) {                               \
@@ -1209,14 +1300,15 @@ cudaError_t launch_grad_mixed(const UniformArgs &a, const Tile &tile, float *chi
 cudaError_t launch_grad_f64(const UniformArgs &a, const Tile &tile, double *chi2, double *grad,
                             cudaStream_t st, bool nll) {
   if (tile.G > 32) return cudaErrorInvalidValue;
-  const size_t smem = smem_grad(a.n_pl, tile, true);
-  const int ST = tile.block / tile.G;
+  const GradShape f = grad_shape(a.n_pl, tile, true);
+  const size_t smem = f.smem;
+  const int ST = f.block / tile.G;
   const int grid = (int)((a.n_sys + ST - 1) / ST);
   cudaError_t err = cudaSuccess;
 #define KC_LAUNCH_NLL(JJ, NN)                                                                 \
   err = set_smem(grad_f64_kernel<JJ, NN>, smem);                                              \
   if (err == cudaSuccess)                                                                     \
-    grad_f64_kernel<JJ, NN><<<grid, tile.block, smem, st>>>(a, tile.G, tile.obs_tile, chi2,     \
+    grad_f64_kernel<JJ, NN><<<grid, f.block, smem, st>>>(a, tile.G, f.obs_tile, chi2,           \
                                                             grad);
 #define KC_LAUNCH(JJ)                      \
   if (nll) {                               \

@@ -176,10 +176,8 @@ cudaError_t launch_kepler_f64(const double *M, const double *e, int64_t n, doubl
 cudaError_t launch_kepler_f32(const float *M, const float *e, int64_t n, float *E,
                               cudaStream_t st);
 
-// Shared-memory bytes a uniform kernel needs for a tile.
-size_t smem_chi2_f64(int n_pl, const Tile &tile);
+// Shared-memory bytes the mixed tile kernel needs for a tile.
 size_t smem_chi2_mixed(int n_pl, const Tile &tile);
-size_t smem_grad(int n_pl, const Tile &tile, bool f64);
 
 // Launch shape for a problem (kc_api.cu): the tuned table, else a heuristic.
 enum class Kind { Chi2F64 = 0, Chi2Mixed = 1, GradF64 = 2, GradMixed = 3, GnMixed = 4 };

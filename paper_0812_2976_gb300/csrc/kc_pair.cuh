@@ -160,18 +160,6 @@ constexpr float kPairMaxTau = 16384.0f;
 
 // ------------------------------------------------ per-planet constants
 
-// Phase: n = 1/P rounded; nq its multiple of 2^-17 (n itself above 2^6,
-// whose last place is no finer), nlo the rest; c a multiple of 2^-23, clo the
-// rest, both low parts and n2pi times 2 pi.  Start: bs and q[0..4], below.
-// Velocity: v = (A cos E - B sin E)/(1 - e cos E), A = K cos w (1 - e^2),
-// B = K sqrt(1 - e^2) sin w.
-struct __align__(16) PlanetP {
-  float n, nq, c, nlo2pi;
-  float clo2pi, n2pi, e, bs;
-  float q[4];
-  float q4, A, B, pad;
-};
-
 // The start.  With a = (1 - e)/(4 e + 1/2), the real root of Mikkola's
 // cubic s^3 + 3 a s = M/(4 e + 1/2) is s = sqrt(a) (z - 1/z), z = (b +
 // sqrt(b^2 + 1))^(1/3), b = M bs, bs = 1/((8 e + 1) a^(3/2)); s is close to
@@ -188,8 +176,12 @@ __device__ __forceinline__ float start_fit(float e, float k0, float k1, float k2
   return __fmaf_rn(e, __fmaf_rn(e, __fmaf_rn(e, k3, k2), k1), k0);
 }
 
-__device__ __forceinline__ void start_setup(PlanetP &p) {
-  const float e = p.e;
+struct StartP {
+  float bs, q[5];
+};
+
+__device__ __forceinline__ StartP start_constants(float e) {
+  StartP p;
   const float r = 1.0f / __fmaf_rn(4.0f, e, 0.5f);
   const float a = fmaxf((1.0f - e) * r, 1e-8f);      // e rounded up to 1: finite
   const float sa = sqrtf(a);
@@ -203,8 +195,21 @@ __device__ __forceinline__ void start_setup(PlanetP &p) {
   f *= a;
   p.q[3] = f * start_fit(e, 2.1773f, -6.5683f, 8.0450f, -3.7069f);
   f *= a;
-  p.q4 = f * start_fit(e, -0.8390f, 3.4927f, -4.6815f, 2.2459f);
+  p.q[4] = f * start_fit(e, -0.8390f, 3.4927f, -4.6815f, 2.2459f);
+  return p;
 }
+
+// Phase: n = 1/P rounded; nq its multiple of 2^-17 (n itself above 2^6,
+// whose last place is no finer), nlo the rest; c a multiple of 2^-23, clo the
+// rest, both low parts and n2pi times 2 pi.  Start: st, above.
+// Velocity: v = (A cos E - B sin E)/(1 - e cos E), A = K cos w (1 - e^2),
+// B = K sqrt(1 - e^2) sin w.
+struct __align__(16) PlanetP {
+  float n, nq, c, nlo2pi;
+  float clo2pi, n2pi, e;
+  StartP st;
+  float A, B, pad;
+};
 
 // Constants of one planet (K, e, w as in planet_setup_mixed).  An invalid
 // planet (checked by the caller) gets e = NaN, which makes its velocities
@@ -224,7 +229,7 @@ __device__ __forceinline__ PlanetP planet_setup_pair(const double *p, double t_r
   wide = !(n_hi <= kPairMaxFreq);
   const float ef = d2f(p[2]);
   q.e = planet_valid(p[0], p[1], p[2], p[3], p[4]) ? ef : __int_as_float(0x7fc00000);
-  start_setup(q);
+  q.st = start_constants(q.e);
   float w_hi, w_lo;
   split_d(p[3], w_hi, w_lo);
   float sw, cw;
@@ -310,14 +315,14 @@ __device__ __forceinline__ unsigned ang_index(float k) {
 // E0 - a, |b| <= 2^-9: sin b = b and cos b = 1 - b^2/2 to 1.3e-9.
 __device__ __forceinline__ void kepler_pair(f32x2 m, const PlanetP &q, const float *tab, f32x2 &s,
                                             f32x2 &c, f32x2 &E) {
-  const f32x2 b = mul2(m, dup2(q.bs));
+  const f32x2 b = mul2(m, dup2(q.st.bs));
   const f32x2 w = fma2(b, b, dup2(1.0f));
   const f32x2 r = pack2(start_root(lo2(b), lo2(w)), start_root(hi2(b), hi2(w)));
   const f32x2 x = mul2(r, r);
-  f32x2 p = fma2(x, dup2(q.q4), dup2(q.q[3]));
-  p = fma2(x, p, dup2(q.q[2]));
-  p = fma2(x, p, dup2(q.q[1]));
-  p = fma2(x, p, dup2(q.q[0]));
+  f32x2 p = fma2(x, dup2(q.st.q[4]), dup2(q.st.q[3]));
+  p = fma2(x, p, dup2(q.st.q[2]));
+  p = fma2(x, p, dup2(q.st.q[1]));
+  p = fma2(x, p, dup2(q.st.q[0]));
   const f32x2 E0 = fma2(r, p, m);
   // sin, cos of E0
   const f32x2 k = add2(E0, dup2(kAngRound));

@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "kc_device.cuh"
+#include "kc_f64.cuh"
 #include "kc_internal.h"
 #include "kc_ragged.h"
 
@@ -108,15 +109,19 @@ __global__ void prep_obs_f64(RaggedDev d, const double *__restrict__ t,
   }
 }
 
-// FP64 model velocities of a ragged batch, one warp per system.
-__global__ void predict_ragged_kernel(const double *__restrict__ params,
+// FP64 model velocities of a ragged batch, one warp per system, its planets
+// set up once by the first lanes.
+__global__ void __launch_bounds__(256)
+predict_ragged_kernel(const double *__restrict__ params,
                                       const int64_t *__restrict__ par_off,
                                       const int32_t *__restrict__ n_pl,
                                       const double *__restrict__ t,
                                       const int64_t *__restrict__ obs_off, int64_t n_sys,
                                       double t0, double *__restrict__ v_out,
                                       unsigned long long *words) {
+  __shared__ PlanetX pl_s[8][KC_MAX_PLANETS];
   const int lane = threadIdx.x & 31;
+  PlanetX *pl = pl_s[threadIdx.x >> 5];
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t s = warp; s < n_sys; s += nwarp) {
@@ -131,16 +136,16 @@ __global__ void predict_ragged_kernel(const double *__restrict__ params,
     const double *p = params + par_off[s];
     const double tr = t[o0];
     const double gam = system_gamma_r(p, J);
-    for (int64_t k = o0 + lane; k < o1; k += 32) {
-      double V = gam;
-      for (int j = 0; j < J; ++j) {
-        const PlanetD q = planet_setup_f64(p + 5 * j, tr - t0);
-        double sE, cE;
-        kepler_f64(mean_anomaly_f64(t[k] - tr, q), q.e, sE, cE);
-        V = velocity_add_f64(q, sE, cE, V);
-      }
-      v_out[k] = V;
+    __syncwarp();
+    if (lane < J) {
+      double sw, cw, beta;
+      pl[lane] = planet_setup_x(p + 5 * lane, tr - t0, sw, cw, beta);
     }
+    __syncwarp();
+    const bool hi = any_high_e(lane < J && pl[lane].e > (double)kEccFast);
+    for (int64_t k = o0 + lane; k < o1; k += 32)
+      v_out[k] = hi ? model_velocity<true>(t[k] - tr, pl, J, gam)
+                    : model_velocity<false>(t[k] - tr, pl, J, gam);
   }
 }
 

@@ -1,4 +1,4 @@
-"""Coefficients of the solve's start in kc_pair.cuh (start_setup).
+"""Coefficients of the solve's start in kc_pair.cuh (start_constants).
 
 With s the real root of Mikkola's (1987) cubic, the start is
 
