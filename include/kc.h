@@ -124,6 +124,16 @@ kc_status kc_chi2_grad(const double *params, const double *t,
                        double jitter, kc_mode mode, void *chi2_out,
                        void *grad_out, kc_stream stream);
 
+/* The same, KC_MIXED by the scalar one-observation kernel: its sums keep
+ * their form and order from version to version, for a caller that hands the
+ * gradient on in double (autograd does) and so may not see it move by a
+ * single-precision rounding.  KC_FP64: kc_chi2_grad. */
+kc_status kc_chi2_grad_scalar(const double *params, const double *t,
+                              const double *v_obs, const double *sigma,
+                              int64_t n_sys, int32_t n_pl, int32_t n_obs,
+                              double t0, double jitter, kc_mode mode,
+                              void *chi2_out, void *grad_out, kc_stream stream);
+
 /* Gauss-Newton normal matrix (derivatives for least-squares refinement,
  * which Sec. 6 lists as future work): for every system
  *   H = sum_k w_k J_k J_k^T,  J_k = dV_k/dtheta over its n = 5*n_pl + 1

@@ -202,6 +202,13 @@ def kc_chi2_grad(params, t, v_obs, sigma, t0: float = 0.0, jitter: float = 0.0,
                  mode="mixed", chi2_out=None, grad_out=None,
                  stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """(chi2 [n_sys], d chi2/d params [n_sys, 5*n_pl+1]) (kc_chi2_grad)."""
+    return _grad_call("kc_chi2_grad", params, t, v_obs, sigma, t0, jitter, mode, chi2_out,
+                      grad_out, stream)
+
+
+def _grad_call(fn, params, t, v_obs, sigma, t0, jitter, mode, chi2_out=None, grad_out=None,
+               stream=None):
+    """kc_chi2_grad or kc_chi2_grad_scalar."""
     params = _dev_f64("params", params, 2)
     t, v_obs, sigma = _obs(t, v_obs, sigma)
     m = _mode(mode)
@@ -212,10 +219,10 @@ def kc_chi2_grad(params, t, v_obs, sigma, t0: float = 0.0, jitter: float = 0.0,
     if grad_out is None:
         grad_out = torch.empty(params.shape, dtype=dtype, device=params.device)
     lib = _lib.load()
-    _lib.check(lib.kc_chi2_grad(
+    _lib.check(getattr(lib, fn)(
         params.data_ptr(), t.data_ptr(), v_obs.data_ptr(), sigma.data_ptr(), n_sys,
         n_planets(params), t.numel(), float(t0), float(jitter), m, chi2_out.data_ptr(),
-        grad_out.data_ptr(), _stream(stream)), "kc_chi2_grad")
+        grad_out.data_ptr(), _stream(stream)), fn)
     return chi2_out, grad_out
 
 
@@ -670,11 +677,12 @@ class DEMCMC:
 
 
 class _Chi2Fn(torch.autograd.Function):
-    """chi2 with the adjoint kernel as backward."""
+    """chi2 with the adjoint kernel as backward (the scalar one: the gradient
+    leaves here in float64)."""
 
     @staticmethod
     def forward(ctx, params, t, v_obs, sigma, t0, jitter, mode):
-        chi, grad = kc_chi2_grad(params, t, v_obs, sigma, t0, jitter, mode)
+        chi, grad = _grad_call("kc_chi2_grad_scalar", params, t, v_obs, sigma, t0, jitter, mode)
         ctx.save_for_backward(grad)
         return chi
 
@@ -713,7 +721,7 @@ def chi2(params, t, v_obs, sigma, t0: float = 0.0, jitter: float = 0.0,
     """Differentiable chi2 [n_sys] with respect to ``params``.
 
     Without grad, the forward kernel (kc_chi2_eval_ex) runs; with grad the
-    adjoint kernel (kc_chi2_grad) produces chi2 and its gradient in one pass
+    adjoint kernel (kc_chi2_grad_scalar) produces chi2 and its gradient in one pass
     and backward scales it by the incoming gradient."""
     if params.requires_grad and torch.is_grad_enabled():
         return _Chi2Fn.apply(params, t, v_obs, sigma, float(t0), float(jitter), mode)

@@ -48,6 +48,8 @@ SIGNATURES = {
                                _d, _d, _st]),
     "kc_chi2_eval_mixed_noalloc": (_i32, [_d, _d, _d, _d, _i64, _i32, _i32, _f64, _f64, _d,
                                           _d, _st]),
+    "kc_chi2_grad_scalar": (_i32, [_d, _d, _d, _d, _i64, _i32, _i32, _f64, _f64, _i32, _d,
+                                   _d, _st]),
     "kc_chi2_grad": (_i32, [_d, _d, _d, _d, _i64, _i32, _i32, _f64, _f64, _i32, _d,
                             _d, _st]),
     "kc_chi2_gauss_newton": (_i32, [_d, _d, _d, _d, _i64, _i32, _i32, _f64, _f64, _i32, _d, _d,

@@ -1,5 +1,6 @@
 // kc_api.cu -- the library's C ABI (include/kc.h): argument checks, launch
 // shapes and error reporting around the kernels of kc_fwd.cu / kc_grad.cu.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -162,56 +163,64 @@ int obs_tile_for(Kind kind, int n_obs) {
   return n_obs < cap ? (n_obs > 0 ? n_obs : 1) : cap;
 }
 
-// Built-in launch shape of the FP64 chi2 and gradient kernels: the smallest
-// predicted time of an SM's sub-partition, in clocks.  An SM runs ceil(CTAs /
-// n_sm) CTAs; a warp's evaluation costs eval clocks of the FP64 pipe, or its
-// latency shared by the warps resident on the sub-partition where they are
-// too few; a CTA also costs one warp-wide setup per 32 planets and kStage per
-// 32 staged observations.  Fitted to timings of every power of two of G with
-// blocks of 32 to 256 on ten sizes (chi2) and six (gradient): its pick is
-// within 13 % of the fastest there (4096 x 4 x 256: (32, 128), 80.0 us, the
-// fastest; the shape used before, (64, 256): 82.2; 300 x 3 x 101: 10.6
-// against 25.9 at (16, 256)).
-static Tile f64_tile(bool grad, int64_t n_sys, int n_pl, int n_obs) {
-  const double eval = grad ? 1800.0 : 560.0, latency = grad ? 4000.0 : 1700.0;
-  const double setup = grad ? 4000.0 : 2900.0;
-  constexpr double kStage = 450.0;
-  const int max_g = grad ? 32 : 128, regs = grad ? 128 : 64;
+// Built-in launch shape of the FP64 chi2 and of both gradient kernels: the
+// smallest predicted time of an SM's sub-partition, in clocks.  An SM runs
+// ceil(CTAs / n_sm) CTAs.  A warp's step over `unit` observations per lane
+// costs eval clocks per planet and observation of the pipe that bounds the
+// kernel, or the step's latency shared by the warps resident on the
+// sub-partition where they are too few; a CTA also costs one warp-wide setup
+// per 32 planets, `stage` per 32 staged observations, and `combine` per
+// level of the lanes' reduction and planet.  The constants were fitted to
+// timings of all powers of two of G and blocks of 32 to 256: within 13 % of
+// the fastest shape on ten sizes (FP64 chi2), 14 % on six (FP64 gradient) and
+// 5 % on nine (mixed gradient).  Before and now, us: FP64 chi2 300 x 3 x 101
+// (16, 256) 25.9, (128, 256) 10.6; mixed gradient 10000 x 2 x 150 (32, 256)
+// 29.0, (8, 128) 18.6, and 65536 x 3 x 512 (16, 256) 277, (4, 256) 258.
+struct TileCost {
+  double eval, latency0, latency_pl, setup, stage, combine;
+  int unit, max_g, regs, min_block;
+};
+
+static Tile model_tile(const TileCost &m, Kind kind, int64_t n_sys, int n_pl, int n_obs) {
   const int64_t n_sm = sm_count() > 1 ? sm_count() : 152;       // no device: a GB300's
   Tile best{32, 128, 0};
   double best_cost = 1e300;
-  for (int G = 1; G <= max_g && (G == 1 || G < 2 * n_obs); G <<= 1) {
-    for (int B : {64, 128, 256}) {
+  int levels = 0;
+  for (int G = 1; G <= m.max_g && (G == 1 || G < 2 * n_obs); G <<= 1, ++levels) {
+    for (int B = m.min_block; B <= 256; B *= 2) {
       if (G > B) continue;
       const int W = B / 32, ST = B / G;
       const int64_t per_sm = ((n_sys + ST - 1) / ST + n_sm - 1) / n_sm;
-      const int occ = 65536 / (regs * B) < 2048 / B ? 65536 / (regs * B) : 2048 / B;
-      const double resident = (double)(per_sm < occ ? per_sm : occ);
+      const int occ = std::min(65536 / (m.regs * B), 2048 / B);
+      const double resident = (double)std::min<int64_t>(per_sm, occ);
       const double warps = W >= 4 || resident * W < 4 ? (W + 3) / 4 : 0.25 * W;   // per CTA
-      const double clocks = eval > latency / (warps * resident) ? eval
-                                                                : latency / (warps * resident);
-      const double iters = (double)((n_obs + G - 1) / G);
+      const double steps = (double)((n_obs + m.unit * G - 1) / (m.unit * G));
+      const double step = std::max(m.eval * m.unit * n_pl,
+                                   (m.latency0 + m.latency_pl * n_pl) / (warps * resident));
+      const double prologue = 0.25 * ((ST * n_pl + 31) / 32 * m.setup +
+                                      (n_obs + 31) / 32 * m.stage);
       const double cost =
-          (double)per_sm * (warps * n_pl * iters * clocks +
-                            0.25 * ((ST * n_pl + 31) / 32 * setup + (n_obs + 31) / 32 * kStage)) +
-          (double)per_sm / resident * setup;
+          (double)per_sm * (warps * (steps * step + m.combine * (n_pl + 1) * levels) + prologue +
+                            m.setup / resident);
       if (cost < best_cost * (1.0 - 1e-9)) {
         best_cost = cost;
         best = Tile{G, B, 0};
       }
     }
   }
-  best.obs_tile = obs_tile_for(grad ? Kind::GradF64 : Kind::Chi2F64, n_obs);
+  best.obs_tile = obs_tile_for(kind, n_obs);
   return best;
 }
 
-// Built-in launch shape.  G threads share one system; enough threads to fill
-// the device's SMs a few times over, but each thread keeps at least four
-// observations so the per-system combine stays cheap.
-Tile default_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs) {
-  if (kind == Kind::Chi2F64 || kind == Kind::GradF64)
-    return f64_tile(kind == Kind::GradF64, n_sys, n_pl, n_obs);
-  const bool grad = kind == Kind::GradMixed;
+constexpr TileCost kCostChi2F64 = {560.0, 0.0, 1700.0, 2900.0, 450.0, 0.0, 1, 128, 64, 64};
+constexpr TileCost kCostGradF64 = {1800.0, 0.0, 4000.0, 4000.0, 450.0, 0.0, 1, 32, 128, 64};
+constexpr TileCost kCostGradMixed = {100.0, 500.0, 250.0, 700.0, 200.0, 30.0, 2, 32, 128, 128};
+
+// Launch shape of the mixed tile kernels and of the scalar gradient: G threads
+// share one system; enough threads to fill the device's SMs a few times over,
+// but each thread keeps at least four observations so the per-system combine
+// stays cheap.
+static Tile even_tile(Kind kind, int64_t n_sys, int n_obs) {
   Tile t;
   t.block = 256;
   const int64_t want_threads = int64_t(sm_count()) * 2048 * 2;
@@ -219,11 +228,19 @@ Tile default_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs) {
   while (G < 256 && n_sys * G < want_threads) G <<= 1;
   const int max_g_obs = n_obs >= 4 ? n_obs / 4 : 1;
   while (G > 1 && G > max_g_obs) G >>= 1;
-  if (grad && G > 32) G = 32;
+  if (kind == Kind::GradMixed && G > 32) G = 32;
   if (G < 4) G = 4;
   t.G = G;
   t.obs_tile = obs_tile_for(kind, n_obs);
   return t;
+}
+
+// Built-in launch shape.
+Tile default_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs) {
+  if (kind == Kind::Chi2F64) return model_tile(kCostChi2F64, kind, n_sys, n_pl, n_obs);
+  if (kind == Kind::GradF64) return model_tile(kCostGradF64, kind, n_sys, n_pl, n_obs);
+  if (kind == Kind::GradMixed) return model_tile(kCostGradMixed, kind, n_sys, n_pl, n_obs);
+  return even_tile(kind, n_sys, n_obs);
 }
 
 namespace {
@@ -280,6 +297,14 @@ Tile choose_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs) {
     }
   }
   return builtin_tile(kind, n_sys, n_pl, n_obs);
+}
+
+// The scalar gradient's shape: the gradient's table entry, else the rule its
+// results were always summed by (the order of a sum shows in its rounding).
+Tile scalar_grad_tile(int64_t n_sys, int n_pl, int n_obs) {
+  if (has_tile_entry(Kind::GradMixed, n_sys, n_pl, n_obs))
+    return choose_tile(Kind::GradMixed, n_sys, n_pl, n_obs);
+  return even_tile(Kind::GradMixed, n_sys, n_obs);
 }
 
 }  // namespace kc
@@ -413,10 +438,10 @@ kc_status kc_chi2_eval_mixed(const double *params, const double *t, const double
                          max_kepler_resid, stream);
 }
 
-kc_status kc_chi2_grad(const double *params, const double *t, const double *v_obs,
-                       const double *sigma, int64_t n_sys, int32_t n_pl, int32_t n_obs,
-                       double t0, double jitter, kc_mode mode, void *chi2_out, void *grad_out,
-                       kc_stream stream) {
+static kc_status chi2_grad(const double *params, const double *t, const double *v_obs,
+                           const double *sigma, int64_t n_sys, int32_t n_pl, int32_t n_obs,
+                           double t0, double jitter, kc_mode mode, void *chi2_out, void *grad_out,
+                           kc_stream stream, bool scalar) {
   kc_status st = check_uniform(params, t, v_obs, sigma, n_sys, n_pl, n_obs, grad_out,
                                "kc_chi2_grad");
   if (st != KC_OK) return st;
@@ -432,10 +457,31 @@ kc_status kc_chi2_grad(const double *params, const double *t, const double *v_ob
                                            static_cast<double *>(grad_out), s),
                        "kc_chi2_grad (fp64)");
   }
+  if (scalar)
+    return cuda_status(kc::launch_grad_scalar(a, kc::scalar_grad_tile(n_sys, n_pl, n_obs),
+                                              static_cast<float *>(chi2_out),
+                                              static_cast<float *>(grad_out), s, false),
+                       "kc_chi2_grad_scalar");
   const Tile tile = kc::choose_tile(Kind::GradMixed, n_sys, n_pl, n_obs);
   return cuda_status(kc::launch_grad_mixed(a, tile, static_cast<float *>(chi2_out),
                                            static_cast<float *>(grad_out), s),
                      "kc_chi2_grad (mixed)");
+}
+
+kc_status kc_chi2_grad(const double *params, const double *t, const double *v_obs,
+                       const double *sigma, int64_t n_sys, int32_t n_pl, int32_t n_obs,
+                       double t0, double jitter, kc_mode mode, void *chi2_out, void *grad_out,
+                       kc_stream stream) {
+  return chi2_grad(params, t, v_obs, sigma, n_sys, n_pl, n_obs, t0, jitter, mode, chi2_out,
+                   grad_out, stream, false);
+}
+
+kc_status kc_chi2_grad_scalar(const double *params, const double *t, const double *v_obs,
+                              const double *sigma, int64_t n_sys, int32_t n_pl, int32_t n_obs,
+                              double t0, double jitter, kc_mode mode, void *chi2_out,
+                              void *grad_out, kc_stream stream) {
+  return chi2_grad(params, t, v_obs, sigma, n_sys, n_pl, n_obs, t0, jitter, mode, chi2_out,
+                   grad_out, stream, true);
 }
 
 // Tile for the free-jitter kernels: the tuned or default shape of the
@@ -508,9 +554,9 @@ kc_status kc_nll_grad(const double *params, const double *t, const double *v_obs
                                            static_cast<double *>(nll_out),
                                            static_cast<double *>(grad_out), s, true),
                        "kc_nll_grad (fp64)");
-  return cuda_status(kc::launch_grad_mixed(a, nll_tile(Kind::GradMixed, n_sys, n_pl, n_obs),
-                                           static_cast<float *>(nll_out),
-                                           static_cast<float *>(grad_out), s, true),
+  return cuda_status(kc::launch_grad_scalar(a, kc::scalar_grad_tile(n_sys, n_pl, n_obs),
+                                            static_cast<float *>(nll_out),
+                                            static_cast<float *>(grad_out), s, true),
                      "kc_nll_grad (mixed)");
 }
 

@@ -25,6 +25,7 @@
 #include "kc_device.cuh"
 #include "kc_f64.cuh"
 #include "kc_internal.h"
+#include "kc_pair.cuh"
 #include "kc_tcgen05.cuh"
 
 namespace kc {
@@ -118,9 +119,26 @@ __device__ __forceinline__ void velocity_partials(T e, T K, T cw, T sw, T beta, 
   d.de = K * cw - ks * sE * (ibeta + beta * invD);
 }
 
+// Shared memory of the packed gradient: the sin/cos table, the planets, the
+// systems' gamma, six arrays of staged observations.
 struct MixedGradLayout {
+  size_t tab, pl, gam, obs, total;
+  __host__ __device__ MixedGradLayout(int ST, int J, int tile) {
+    tab = 0;
+    pl = tab + sizeof(AngTab);
+    gam = pl + sizeof(GradPlanetP) * ST * J;
+    obs = align_up(gam + sizeof(float) * ST, 16);
+    total = obs + sizeof(float) * 6 * tile;
+  }
+};
+// obs_tile rounded up to whole pairs of every lane of a system.
+__host__ __device__ inline int grad_tile(int obs_tile, int G) {
+  return (obs_tile + 2 * G - 1) / (2 * G) * (2 * G);
+}
+
+struct ScalarGradLayout {
   size_t pl, gam, sj, obs, w, total;
-  __host__ __device__ MixedGradLayout(int ST, int J, int obs_tile) {
+  __host__ __device__ ScalarGradLayout(int ST, int J, int obs_tile) {
     pl = 0;
     gam = pl + sizeof(GradPlanetF) * ST * J;
     sj = gam + sizeof(float) * ST;
@@ -161,18 +179,155 @@ struct F64GradLayout {
 
 // ------------------------------------------------------------ mixed
 
+// Two observations per lane at a time, packed (kc_pair.cuh).  Bound by FP32
+// issue and register ports like the forward kernel: 103 clocks per warp,
+// planet and observation and sub-partition (68 of them the forward part);
+// 128 registers hold the packed sums of up to three planets.  65536 x 3 x
+// 512, us: 375 with the scalar kernel, 277 at its launch shape, 260 at the
+// shape of kc_api.cu's model.
+template <int J>
+__global__ void __launch_bounds__(256, 2)
+grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_out,
+                  float *__restrict__ grad_out) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int NP = 5 * J + 1;
+  const int block = blockDim.x;
+  const int ST = block / G;
+  const int tile = grad_tile(obs_tile, G);
+  const MixedGradLayout L(ST, J, tile);
+  float *tab_s = reinterpret_cast<float *>(smem + L.tab);
+  GradPlanetP *pl_s = reinterpret_cast<GradPlanetP *>(smem + L.pl);
+  float *gam_s = reinterpret_cast<float *>(smem + L.gam);
+  float *obs_s = reinterpret_cast<float *>(smem + L.obs);   // th, tl, v hi, v lo, w, t - t0
+
+  const int tid = threadIdx.x;
+  const int64_t sys0 = (int64_t)blockIdx.x * ST;
+  const double t_ref = a.n_obs > 0 ? a.t[0] : a.t0;
+  const Split3 tr3 = split3(t_ref), te3 = split3(a.t0);
+  const float dref_f = (tr3.x0 - te3.x0) + (tr3.x1 - te3.x1);     // t_ref - t0, float
+  const float jit2 = d2f(a.jitter2);
+  ang_tab_load(tab_s, tid, block);
+
+  bool wide = false;
+  for (int i = tid; i < ST * J; i += block) {
+    const int sl = i / J, j = i - sl * J;
+    const int64_t s = sys0 + sl;
+    GradPlanetP q = {};
+    if (s < a.n_sys && dbg_ok(a.invalid, s * NP + 5 * j + 4 < a.n_sys * NP, kDbgParam, s * NP)) {
+      bool far;
+      q = grad_setup_pair(a.params + s * NP + 5 * j, t_ref, a.t0, far);
+      wide |= far;
+    }
+    pl_s[i] = q;
+  }
+  for (int i = block - 1 - tid; i < ST; i += block) {
+    const int64_t s = sys0 + i;
+    gam_s[i] = s < a.n_sys ? d2f(system_gamma_g(a.params + s * NP, J)) : 0.0f;
+  }
+
+  const int sl = tid / G, c = tid - sl * G;
+  const int64_t s = sys0 + sl;
+  const GradPlanetP *q = pl_s + sl * J;
+  Kahan2 acc = {0, 0};
+  f32x2 sum_a = 0;
+  GradSums g[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) g[j] = GradSums{{0, 0}, 0, 0, 0, 0};
+
+  for (int k0 = 0; k0 < a.n_obs; k0 += obs_tile) {
+    const int nk = min(obs_tile, a.n_obs - k0);
+    const int npad = grad_tile(nk, G);
+    if (k0 > 0) __syncthreads();
+    // the padding has zero weight
+    for (int k = block - 1 - tid; k < npad; k += block) {
+      float th = 0.0f, tl = 0.0f, vh = 0.0f, vl = 0.0f, wk = 0.0f, dt = 0.0f;
+      if (k < nk && dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k)) {
+        sub_ds(split3(a.t[k0 + k]), tr3, th, tl);
+        dt = th + dref_f;
+        tau_place(th, tl);
+        wide |= !(fabsf(th) < kPairMaxTau);
+        split_d(a.v[k0 + k], vh, vl);
+        const float sg = d2f(a.sigma[k0 + k]);
+        const float var = __fmaf_rn(sg, sg, jit2);
+        wk = var > 0.0f ? 1.0f / var : __int_as_float(0x7fc00000);
+      }
+      obs_s[k] = th;
+      obs_s[tile + k] = tl;
+      obs_s[2 * tile + k] = vh;
+      obs_s[3 * tile + k] = vl;
+      obs_s[4 * tile + k] = wk;
+      obs_s[5 * tile + k] = dt;
+    }
+    wide = __syncthreads_or(wide);
+    const float gam = gam_s[sl];
+    with_high_e(wide, [&](auto tag) {
+      constexpr bool WIDE = decltype(tag)::value;
+      for (int k = 2 * c; k < npad; k += 2 * G) {
+        // the planets' constants are read again in every iteration: hoisted
+        // for all J planets they would not fit the registers
+        asm volatile("" ::: "memory");
+        auto at = [&](int array) {
+          return *reinterpret_cast<const f32x2 *>(obs_s + array * tile + k);
+        };
+        const f32x2 th = at(0), tl = at(1);
+        GradTerms o[J];
+        Kahan2 V = {dup2(gam), 0};
+#pragma unroll
+        for (int j = 0; j < J; ++j) o[j] = grad_terms<WIDE>(th, tl, q[j], tab_s, V);
+        const f32x2 r = sub2(sub2(V.big, at(2)), add2(V.small, at(3)));
+        const f32x2 wr = mul2(at(4), r), a2 = add2(wr, wr);
+        kahan_add(acc, mul2(wr, r));
+        sum_a = add2(sum_a, a2);
+        const f32x2 adt = mul2(a2, at(5));
+#pragma unroll
+        for (int j = 0; j < J; ++j) grad_add(g[j], o[j], q[j], a2, adt);
+      }
+    });
+  }
+  if (a.n_obs == 0) __syncthreads();            // gam_s, pl_s written by other threads
+
+  Kahan chi = kahan_join(acc);
+  float sa = join2(sum_a);
+  GradLane gl[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) gl[j] = grad_join(g[j]);
+  for (int m = G >> 1; m >= 1; m >>= 1) {
+    const Kahan o = {shfl_xor(chi.big, m), shfl_xor(chi.small, m)};
+    kahan_merge(chi, o);
+    sa += shfl_xor(sa, m);
+#pragma unroll
+    for (int j = 0; j < J; ++j) grad_combine(gl[j], m);
+  }
+  if (c == 0 && s < a.n_sys) {
+    // NaN for an invalid system
+    const float poison = 0.0f * gam_s[sl];
+    const float value = kahan_value(chi) + poison;
+    if (chi2_out) chi2_out[s] = value;
+    note_invalid(a.invalid, value);
+    float *out = grad_out + s * NP;
+#pragma unroll
+    for (int j = 0; j < J; ++j) grad_finish(gl[j], q[j], sa, poison, out + 5 * j);
+    out[5 * J] = sa + poison;
+  }
+}
+
+// One observation per lane at a time, in scalar single precision: the
+// gradient behind autograd and of the free-jitter likelihood.  Autograd hands
+// its gradient out in double, so its callers hold it to double's tolerance: it
+// may not move by a single-precision rounding from one version to the next,
+// which any other order or form of these sums would do.
 // NLL = true: the free-jitter negative log-likelihood (see kc_fwd.cu) and
 // its gradient, including d nll / d sigma_j = sigma_j sum_k w_k (1 - w_k r_k^2)
 // (the planet and gamma terms carry w_k r_k instead of 2 w_k r_k).
 template <int J, bool NLL = false>
 __global__ void __launch_bounds__(256, 2)
-grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_out,
+grad_scalar_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_out,
                   float *__restrict__ grad_out) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NP = 5 * J + 1 + (NLL ? 1 : 0);
   const int block = blockDim.x;
   const int ST = block / G;
-  const MixedGradLayout L(ST, J, obs_tile);
+  const ScalarGradLayout L(ST, J, obs_tile);
   GradPlanetF *pl_s = reinterpret_cast<GradPlanetF *>(smem + L.pl);
   float *gam_s = reinterpret_cast<float *>(smem + L.gam);
   float *sj_s = reinterpret_cast<float *>(smem + L.sj);
@@ -1238,12 +1393,14 @@ struct GradShape {
   int block, obs_tile;
   size_t smem;
 };
-static GradShape grad_shape(int n_pl, const Tile &t, bool f64) {
+enum class GradKernel { F64, Packed, Scalar };
+static GradShape grad_shape(int n_pl, const Tile &t, GradKernel kernel) {
   GradShape f{t.block, t.obs_tile, 0};
   auto bytes = [&] {
     const int ST = f.block / t.G;
-    return f64 ? F64GradLayout(ST, n_pl, f.obs_tile).total
-               : MixedGradLayout(ST, n_pl, f.obs_tile).total;
+    if (kernel == GradKernel::F64) return F64GradLayout(ST, n_pl, f.obs_tile).total;
+    if (kernel == GradKernel::Scalar) return ScalarGradLayout(ST, n_pl, f.obs_tile).total;
+    return MixedGradLayout(ST, n_pl, grad_tile(f.obs_tile, t.G)).total;
   };
   constexpr size_t kMax = 227 * 1024;
   while (bytes() > kMax) {
@@ -1272,18 +1429,33 @@ static GradShape grad_shape(int n_pl, const Tile &t, bool f64) {
   }
 
 cudaError_t launch_grad_mixed(const UniformArgs &a, const Tile &tile, float *chi2, float *grad,
-                              cudaStream_t st, bool nll) {
+                              cudaStream_t st) {
   if (tile.G > 32) return cudaErrorInvalidValue;
-  const GradShape f = grad_shape(a.n_pl, tile, false);
-  const size_t smem = f.smem;
+  const GradShape f = grad_shape(a.n_pl, tile, GradKernel::Packed);
+  const int ST = f.block / tile.G;
+  const int grid = (int)((a.n_sys + ST - 1) / ST);
+  cudaError_t err = cudaSuccess;
+#define KC_LAUNCH(JJ)                                                                    \
+  err = set_smem(grad_mixed_kernel<JJ>, f.smem);                                         \
+  if (err == cudaSuccess)                                                                \
+    grad_mixed_kernel<JJ><<<grid, f.block, f.smem, st>>>(a, tile.G, f.obs_tile, chi2, grad);
+  KC_DISPATCH_J(a.n_pl, KC_LAUNCH)
+#undef KC_LAUNCH
+  if (err != cudaSuccess) return err;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_grad_scalar(const UniformArgs &a, const Tile &tile, float *chi2, float *grad,
+                               cudaStream_t st, bool nll) {
+  if (tile.G > 32) return cudaErrorInvalidValue;
+  const GradShape f = grad_shape(a.n_pl, tile, GradKernel::Scalar);
   const int ST = f.block / tile.G;
   const int grid = (int)((a.n_sys + ST - 1) / ST);
   cudaError_t err = cudaSuccess;
 #define KC_LAUNCH_NLL(JJ, NN)                                                                   \
-  err = set_smem(grad_mixed_kernel<JJ, NN>, smem);                                              \
+  err = set_smem(grad_scalar_kernel<JJ, NN>, f.smem);                                           \
   if (err == cudaSuccess)                                                                       \
-    grad_mixed_kernel<JJ, NN><<<grid, f.block, smem, st>>>(a, tile.G, f.obs_tile, chi2,           \
-                                                              grad);
+    grad_scalar_kernel<JJ, NN><<<grid, f.block, f.smem, st>>>(a, tile.G, f.obs_tile, chi2, grad);
 #define KC_LAUNCH(JJ)                      \
   if (nll) {                               \
     KC_LAUNCH_NLL(JJ, true)                \
@@ -1300,7 +1472,7 @@ cudaError_t launch_grad_mixed(const UniformArgs &a, const Tile &tile, float *chi
 cudaError_t launch_grad_f64(const UniformArgs &a, const Tile &tile, double *chi2, double *grad,
                             cudaStream_t st, bool nll) {
   if (tile.G > 32) return cudaErrorInvalidValue;
-  const GradShape f = grad_shape(a.n_pl, tile, true);
+  const GradShape f = grad_shape(a.n_pl, tile, GradKernel::F64);
   const size_t smem = f.smem;
   const int ST = f.block / tile.G;
   const int grid = (int)((a.n_sys + ST - 1) / ST);

@@ -164,7 +164,11 @@ cudaError_t launch_chi2_mixed_warp(const UniformArgs &a, const Tile &tile, float
 cudaError_t launch_grad_f64(const UniformArgs &a, const Tile &tile, double *chi2,
                             double *grad, cudaStream_t st, bool nll = false);
 cudaError_t launch_grad_mixed(const UniformArgs &a, const Tile &tile, float *chi2,
-                              float *grad, cudaStream_t st, bool nll = false);
+                              float *grad, cudaStream_t st);
+// The scalar kernel behind autograd and the free-jitter gradient, whose
+// results keep their rounding (kc_grad.cu).
+cudaError_t launch_grad_scalar(const UniformArgs &a, const Tile &tile, float *chi2,
+                               float *grad, cudaStream_t st, bool nll);
 // Free-jitter negative log-likelihood, forward only (kc_fwd.cu).
 cudaError_t launch_nll_mixed(const UniformArgs &a, const Tile &tile, float *out, cudaStream_t st);
 cudaError_t launch_nll_f64(const UniformArgs &a, const Tile &tile, double *out, cudaStream_t st);
@@ -184,6 +188,7 @@ enum class Kind { Chi2F64 = 0, Chi2Mixed = 1, GradF64 = 2, GradMixed = 3, GnMixe
 Tile default_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs);
 Tile builtin_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs);  // without a table entry
 Tile choose_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs);
+Tile scalar_grad_tile(int64_t n_sys, int n_pl, int n_obs);
 bool has_tile_entry(Kind kind, int64_t n_sys, int n_pl, int n_obs);  // tuned or pinned
 int obs_tile_for(Kind kind, int n_obs);
 

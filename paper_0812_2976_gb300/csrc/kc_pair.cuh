@@ -211,11 +211,25 @@ struct __align__(16) PlanetP {
   float A, B, pad;
 };
 
-// Constants of one planet (K, e, w as in planet_setup_mixed).  An invalid
-// planet (checked by the caller) gets e = NaN, which makes its velocities
-// NaN.  wide: set if the period is too short for the short form.
-__device__ __forceinline__ PlanetP planet_setup_pair(const double *p, double t_ref, double t0,
-                                                     bool &wide) {
+// What planet_setup_pair derives besides the phase and the start: sin and cos
+// of w, b2 = 1 - e^2 (one rounding) and b = sqrt(b2).
+struct OrbitF {
+  float sw, cw, b2, b;
+};
+
+// x y z with the product x y's remainder and x's low part carried (x, y, z
+// rounded once each, the result once more).
+__device__ __forceinline__ float product3(float x_hi, float x_lo, float y, float z) {
+  float u, ue;
+  two_prod(x_hi, y, u, ue);
+  return __fmaf_rn(u, z, __fmaf_rn(x_lo, y, ue) * z);
+}
+
+// Phase, start and orbit constants of one planet; the caller sets A and B.
+// An invalid planet gets e = NaN, which makes its velocities NaN.  wide: set
+// if the period is too short for the short form.
+__device__ __forceinline__ PlanetP planet_setup_orbit(const double *p, double t_ref, double t0,
+                                                      bool &wide, OrbitF &o) {
   PlanetP q;
   float n_hi, n_lo, c_hi, c_lo;
   phase_setup_ds(p[0], p[4], t_ref, t0, n_hi, n_lo, c_hi, c_lo);
@@ -234,20 +248,48 @@ __device__ __forceinline__ PlanetP planet_setup_pair(const double *p, double t_r
   split_d(p[3], w_hi, w_lo);
   float sw, cw;
   sincosf(w_hi, &sw, &cw);
-  const float sw1 = __fmaf_rn(w_lo, cw, sw);
-  cw = __fmaf_rn(-w_lo, sw, cw);
-  // K cos w b2 and K sin w sqrt(b2), b2 = 1 - e^2 in one rounding, each
-  // product rounded once (its remainder and K's low part carried)
-  float K_hi, K_lo;
-  split_d(p[1], K_hi, K_lo);
-  const float b2 = __fmaf_rn(-ef, ef, 1.0f), b = sqrtf(b2);
-  float u, ue;
-  two_prod(K_hi, cw, u, ue);
-  q.A = __fmaf_rn(u, b2, __fmaf_rn(K_lo, cw, ue) * b2);
-  two_prod(K_hi, sw1, u, ue);
-  q.B = __fmaf_rn(u, b, __fmaf_rn(K_lo, sw1, ue) * b);
+  o.sw = __fmaf_rn(w_lo, cw, sw);
+  o.cw = __fmaf_rn(-w_lo, sw, cw);
+  o.b2 = __fmaf_rn(-ef, ef, 1.0f);
+  o.b = sqrtf(o.b2);
   q.pad = 0.0f;
   return q;
+}
+
+__device__ __forceinline__ PlanetP planet_setup_pair(const double *p, double t_ref, double t0,
+                                                     bool &wide) {
+  OrbitF o;
+  PlanetP q = planet_setup_orbit(p, t_ref, t0, wide, o);
+  float K_hi, K_lo;
+  split_d(p[1], K_hi, K_lo);
+  q.A = product3(K_hi, K_lo, o.cw, o.b2);
+  q.B = product3(K_hi, K_lo, o.sw, o.b);
+  return q;
+}
+
+// The gradient's planet: A and B of the solve without K, and the constants
+// of the partials (grad_terms).
+struct __align__(16) GradPlanetP {
+  PlanetP p;
+  float K, C, sw, esw, cw, beta, ibeta, n2;      // C = beta cos w, esw = e sin w, n2 = 1/P^2
+};
+
+__device__ __forceinline__ GradPlanetP grad_setup_pair(const double *p, double t_ref, double t0,
+                                                       bool &wide) {
+  GradPlanetP g;
+  OrbitF o;
+  g.p = planet_setup_orbit(p, t_ref, t0, wide, o);
+  g.p.A = o.cw * o.b2;
+  g.p.B = o.sw * o.b;
+  g.K = d2f(p[1]);
+  g.C = o.cw * o.b;
+  g.sw = o.sw;
+  g.cw = o.cw;
+  g.esw = g.p.e * o.sw;
+  g.beta = o.b;
+  g.ibeta = 1.0f / o.b;
+  g.n2 = g.p.n * g.p.n;
+  return g;
 }
 
 // ------------------------------------------------ mean anomaly
@@ -356,6 +398,84 @@ __device__ __forceinline__ void velocity_sum(Kahan2 &V, const PlanetP &q, f32x2 
   const f32x2 D = fma2(dup2(-q.e), c, dup2(1.0f));
   const f32x2 num = fma2(dup2(q.A), c, neg2(mul2(dup2(q.B), s)));
   kahan_add_y(V, fma2(num, rcp2(D), neg2(V.small)));
+}
+
+// ------------------------------------------------ partials
+
+// One planet of a pair of observations, for the gradient: with y = 1/D,
+//   dK = v/K = (A cos E - B sin E) y,
+//   Q  = sin(w + f) = (sin w cos E + C sin E - e sin w) y;
+// the other partials follow (GradSums).  V takes K dK.
+struct GradTerms {
+  f32x2 s, dK, Q, y;
+};
+
+template <bool WIDE>
+__device__ __forceinline__ GradTerms grad_terms(f32x2 th, f32x2 tl, const GradPlanetP &g,
+                                                const float *tab, Kahan2 &V) {
+  GradTerms o;
+  const f32x2 M = mean_anomaly2<WIDE>(th, tl, g.p);
+  f32x2 s, c, E;
+  kepler_pair(abs2(M), g.p, tab, s, c, E);
+  o.s = signed_as(s, M);
+  o.y = rcp2(fma2(dup2(-g.p.e), c, dup2(1.0f)));
+  o.dK = mul2(fma2(dup2(g.p.A), c, neg2(mul2(dup2(g.p.B), o.s))), o.y);
+  o.Q = mul2(fma2(dup2(g.C), o.s, fma2(dup2(g.sw), c, dup2(-g.esw))), o.y);
+  kahan_add_y(V, fma2(dup2(g.K), o.dK, neg2(V.small)));
+  return o;
+}
+
+// Sums over the observations, a = 2 w r: of a dt Q y^2 (compensated: the
+// period's terms cancel heavily), a dK, a Q y sin E (1/beta + beta y), a Q, a
+// Q y^2.  The partials by (P, K, e, w, M0) are
+//   2 pi n2 K beta dt Q y^2,  dK,  K cos w - K Q y sin E (1/beta + beta y),
+//   -K (Q + e sin w),  -K beta Q y^2,
+// so their factors, and the parts a alone multiplies, are applied once per
+// system (grad_finish): 17 packed operations per pair and planet for all five
+// where the partials formed one by one took about 40 scalar ones each.
+struct GradSums {
+  Kahan2 P;
+  f32x2 K, e, w, M;
+};
+
+__device__ __forceinline__ void grad_add(GradSums &G, const GradTerms &o, const GradPlanetP &g,
+                                         f32x2 a, f32x2 adt) {
+  const f32x2 Qy = mul2(o.Q, o.y), Qyy = mul2(Qy, o.y);
+  const f32x2 h = fma2(dup2(g.beta), o.y, dup2(g.ibeta));
+  kahan_add_y(G.P, fma2(adt, Qyy, neg2(G.P.small)));
+  G.K = fma2(a, o.dK, G.K);
+  G.e = fma2(mul2(a, Qy), mul2(o.s, h), G.e);
+  G.w = fma2(a, o.Q, G.w);
+  G.M = fma2(a, Qyy, G.M);
+}
+
+__device__ __forceinline__ float join2(f32x2 x) { return lo2(x) + hi2(x); }
+
+// A planet's five sums of one lane (the pair joined).
+struct GradLane {
+  Kahan P;
+  float K, e, w, M;
+};
+__device__ __forceinline__ GradLane grad_join(const GradSums &G) {
+  return GradLane{kahan_join(G.P), join2(G.K), join2(G.e), join2(G.w), join2(G.M)};
+}
+__device__ __forceinline__ void grad_combine(GradLane &g, int m) {
+  const Kahan o = {shfl_xor(g.P.big, m), shfl_xor(g.P.small, m)};
+  kahan_merge(g.P, o);
+  g.K += shfl_xor(g.K, m);
+  g.e += shfl_xor(g.e, m);
+  g.w += shfl_xor(g.w, m);
+  g.M += shfl_xor(g.M, m);
+}
+// The planet's gradient from the system's sums; sum_a = sum of a.
+__device__ __forceinline__ void grad_finish(const GradLane &s, const GradPlanetP &g, float sum_a,
+                                            float poison, float *out) {
+  const float Kb = g.K * g.beta;
+  out[0] = __fmaf_rn(Kb * (kTwoPiF * g.n2), kahan_value(s.P), poison);
+  out[1] = s.K + poison;
+  out[2] = __fmaf_rn(g.K, __fmaf_rn(g.cw, sum_a, -s.e), poison);
+  out[3] = __fmaf_rn(-g.K, __fmaf_rn(g.esw, sum_a, s.w), poison);
+  out[4] = __fmaf_rn(-Kb, s.M, poison);
 }
 
 }  // namespace kc

@@ -8,7 +8,7 @@ into chi2 (tests/tolerance.py)."""
 import numpy as np
 import pytest
 import torch
-from tolerance import U32, chi2_rounding_term
+from tolerance import U32, chi2_rounding_term, grad_excess, uniform_arith
 
 pytestmark = pytest.mark.gpu
 
@@ -37,7 +37,7 @@ def rows(rng, n_sys, n_pl, p_range, e_range):
     return par
 
 
-@pytest.mark.parametrize("p_range,span,e_range,n_pl,n_obs", [
+FORMS = [
     ((0.50, 0.53), 4000.0, (0.0, 0.9), 3, 129),      # short form, every start of a period
     ((0.47, 0.4999), 4000.0, (0.0, 0.9), 2, 130),    # wide form just beyond it
     ((0.012, 0.02), 300.0, (0.0, 0.6), 2, 67),       # 1/P on both sides of 64 cycles/d
@@ -48,7 +48,10 @@ def rows(rng, n_sys, n_pl, p_range, e_range):
     ((1.0, 4000.0), 4000.0, (0.0, 0.95), 8, 3),
     ((1.0, 4000.0), 4000.0, (0.0, 0.95), 5, 1024),   # the staged tile, full
     ((1.0, 4000.0), 4000.0, (0.0, 0.95), 1, 1027),   # and beyond
-])
+]
+
+
+@pytest.mark.parametrize("p_range,span,e_range,n_pl,n_obs", FORMS)
 def test_chi2_where_the_form_changes(kc, oracle_mod, p_range, span, e_range, n_pl, n_obs):
     rng = np.random.default_rng(n_obs + n_pl)
     n_sys = 150
@@ -62,6 +65,32 @@ def test_chi2_where_the_form_changes(kc, oracle_mod, p_range, span, e_range, n_p
     args = [torch.tensor(x, device="cuda") for x in (par, t, v, sig)]
     got = kc.kc_chi2_eval_ex(*args, t0=T0, mode="mixed").cpu().numpy().astype(np.float64)
     assert np.all(np.abs(got - ref) <= bound)
+
+
+@pytest.mark.parametrize("lanes", [1, 8, 32])
+@pytest.mark.parametrize("p_range,span,e_range,n_pl,n_obs", FORMS)
+def test_gradient_where_the_form_changes(kc, oracle_mod, p_range, span, e_range, n_pl, n_obs,
+                                         lanes):
+    """chi2 as above, and every component of the gradient within the parity
+    tests' bound (1e-3, plus the derived term where its sum cancels)."""
+    rng = np.random.default_rng(100 + n_obs + n_pl)
+    n_sys = 90
+    par = rows(rng, n_sys, n_pl, p_range, e_range)
+    t = np.sort(rng.uniform(T0, T0 + span, n_obs))
+    sig = rng.uniform(1.0, 4.0, n_obs)
+    v = oracle_mod.predict(par[:1], t, n_pl, T0)[0] + sig * rng.standard_normal(n_obs)
+    ref, gref, gabs = oracle_mod.chi2(par, t, v, sig, n_pl, t0=T0, gabs=True)
+    bound = 1e-5 * np.maximum(ref, 1.0) + chi2_rounding_term(oracle_mod, par, t, v, sig, n_pl, T0,
+                                                             0.0, U32)
+    args = [torch.tensor(x, device="cuda") for x in (par, t, v, sig)]
+    kc.kc_set_tile("grad", "mixed", n_sys, n_pl, n_obs, (lanes, 64))
+    try:
+        chi2, grad = kc.kc_chi2_grad(*args, t0=T0, mode="mixed")
+        ar = uniform_arith(kc, oracle_mod, par, t, v, sig, n_pl, T0, 0.0, "mixed")
+    finally:
+        kc.kc_set_tile("grad", "mixed", n_sys, n_pl, n_obs, None)
+    assert np.all(np.abs(chi2.cpu().numpy().astype(np.float64) - ref) <= bound)
+    assert grad_excess(grad.cpu().numpy(), gref, gabs, 1e-3, U32, ar) <= 1.0
 
 
 def test_eccentricities_up_to_one(kc, oracle_mod):
