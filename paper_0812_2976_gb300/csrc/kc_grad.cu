@@ -20,6 +20,7 @@
 //   dV/dgamma = 1.
 // Each system is handled by G <= 32 consecutive threads (one warp segment),
 // combined by shuffles.
+#include <algorithm>
 #include <cmath>
 
 #include "kc_device.cuh"
@@ -653,6 +654,9 @@ grad_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ chi2_ou
 constexpr int kGnWarps = 4;      // mixed: systems (warps) per CTA
 constexpr int kGnWarpsD = 2;     // FP64
 constexpr int kGnObsTile = 256;
+constexpr int kGnAhead = 4;      // systems a warp of a pair kernel sets up together
+constexpr int kTcObsTile = 512;  // observations the pair kernels stage at a time
+constexpr int kGnRows = 64;      // observations per batch of the pair kernels: two per lane
 
 __host__ __device__ constexpr int gn_np(int J) { return 5 * J + 1; }
 __host__ __device__ constexpr int gn_mt(int J) { return (gn_np(J) + 15) / 16; }
@@ -661,6 +665,7 @@ __host__ __device__ constexpr int gn_nt(int J) { return (gn_np(J) + 7) / 8; }
 // which is 4 mod 16 pairs, so that with the column swizzle below the 64-bit
 // row writes and fragment loads of each half-warp hit 32 different banks.
 __host__ __device__ constexpr int gn_row2(int J) { return gn_mt(J) * 16 + 4; }
+
 
 struct GnMixedLayout {
   size_t pl, gam, obs, w, u, total;
@@ -671,6 +676,17 @@ struct GnMixedLayout {
     w = obs + sizeof(float4) * obs_tile;
     u = align_up(w + sizeof(float4) * obs_tile, 16);
     total = align_up(u + sizeof(float2) * kGnWarps * 32 * gn_row2(J), 16);
+  }
+};
+
+struct GnPairLayout {
+  size_t tab, pl, obs, u, total;
+  __host__ __device__ GnPairLayout(int J, int obs_tile) {
+    tab = 0;
+    pl = tab + sizeof(AngTab);
+    obs = align_up(pl + sizeof(GradPlanetP) * kGnWarps * kGnAhead * J, 16);
+    u = align_up(obs + sizeof(float) * 5 * obs_tile, 16);
+    total = align_up(u + sizeof(float2) * kGnWarps * kGnRows * gn_row2(J), 16);
   }
 };
 
@@ -704,49 +720,6 @@ __device__ __forceinline__ float2 tf32_pair(float x) {
   return make_float2(hi, lo);
 }
 
-// One observation of the Gauss-Newton pass for the lane: its chi2 and
-// gradient terms are added to acc, gP, g, and its row u = sqrt(w) J written
-// to urow.  A lane past the batch's end evaluates a valid observation with
-// weight 0, so all lanes run the same instructions.
-template <int J>
-__device__ __forceinline__ void gn_obs(const float4 &o, const float4 &wt, bool live, float gam,
-                                       const GradPlanetF (&qr)[J], Kahan &acc, Kahan (&gP)[J],
-                                       float (&g)[5 * J + 1], float (&urow)[5 * J + 1]) {
-  float sEj[J], cEj[J];
-  Kahan V = {0.0f, 0.0f};
-#pragma unroll
-  for (int j = 0; j < J; ++j) {
-    const PlanetF &p = qr[j].base;
-    const float M = mean_anomaly_mixed(o.x, o.y, p);
-    kepler_f32_h(M, p.e, qr[j].m, sEj[j], cEj[j]);
-    kahan_add(V, velocity_mixed(p, sEj[j], cEj[j]));
-  }
-  const float r = __fadd_rn(__fsub_rn(V.big, o.z), __fsub_rn(gam, __fadd_rn(V.small, o.w)));
-  const float wk = live ? wt.x : 0.0f, wr = wk * r, a2 = 2.0f * wr;
-  kahan_add(acc, wr * r);
-  const float sw = live ? wt.z : 0.0f;
-#pragma unroll
-  for (int j = 0; j < J; ++j) {
-    const GradPlanetF &qj = qr[j];
-    Partials<float> d;
-    const float invD = rcp_fast(__fmaf_rn(-qj.base.e, cEj[j], 1.0f));
-    velocity_partials(qj.base.e, qj.K, qj.cw, qj.sw, qj.beta, qj.ibeta, sEj[j], cEj[j], invD, d);
-    d.dP = d.dM * (-kTwoPiF * wt.y * qj.n2);
-    kahan_add(gP[j], a2 * d.dP);
-    g[5 * j + 1] = fmaf(a2, d.dK, g[5 * j + 1]);
-    g[5 * j + 2] = fmaf(a2, d.de, g[5 * j + 2]);
-    g[5 * j + 3] = fmaf(a2, d.dw, g[5 * j + 3]);
-    g[5 * j + 4] = fmaf(a2, d.dM, g[5 * j + 4]);
-    urow[5 * j + 0] = sw * d.dP;
-    urow[5 * j + 1] = sw * d.dK;
-    urow[5 * j + 2] = sw * d.de;
-    urow[5 * j + 3] = sw * d.dw;
-    urow[5 * j + 4] = sw * d.dM;
-  }
-  g[5 * J] += a2;
-  urow[5 * J] = sw;
-}
-
 // D = A B + D for one 16 x 8 tile, A 16 x 8 (row), B 8 x 8 (col), TF32.
 __device__ __forceinline__ void mma_tf32(float (&d)[4], const unsigned (&a)[4],
                                          const unsigned (&b)[2]) {
@@ -755,6 +728,124 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const unsigned (&a)[4],
       "{%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// The observations of one tile staged for the Gauss-Newton kernels: five
+// arrays of STRIDE floats (th, tl, v hi, v lo, sqrt w), padded with zero weight
+// to whole batches.  Returns whether a time asks for the wide mean anomaly.
+template <int STRIDE>
+__device__ __forceinline__ bool gn_stage(const UniformArgs &a, int k0, int nk, int npad, int tid,
+                                         int nthreads, const Split3 &tr3, float jit2, float *obs) {
+  bool wide = false;
+  for (int k = tid; k < npad; k += nthreads) {
+    float th = 0.0f, tl = 0.0f, vh = 0.0f, vl = 0.0f, wk = 0.0f;
+    if (k < nk && dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k)) {
+      sub_ds(split3(a.t[k0 + k]), tr3, th, tl);
+      tau_place(th, tl);
+      wide |= !(fabsf(th) < kPairMaxTau);
+      split_d(a.v[k0 + k], vh, vl);
+      const float sg = d2f(a.sigma[k0 + k]);
+      const float var = __fmaf_rn(sg, sg, jit2);
+      wk = var > 0.0f ? 1.0f / var : __int_as_float(0x7fc00000);
+    }
+    const float v[5] = {th, tl, vh, vl, sqrtf(wk)};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) obs[i * STRIDE + k] = v[i];
+  }
+  return wide;
+}
+
+// One pair of observations of a lane (columns k, k + 1 of the staged tile):
+// chi2 and gradient sums, and the rows of sqrt(w) J over their factors.
+// dref = t_ref - t0.
+template <int J, int STRIDE, bool WIDE>
+__device__ __forceinline__ void gn_pair(const float *obs, int k, float dref, const GradPlanetP *q,
+                                        const float *tab, float gam, Kahan2 &acc, f32x2 &sum_a,
+                                        GradSums (&g)[J], f32x2 (&u)[5 * J + 1]) {
+  auto at = [&](int array) { return *reinterpret_cast<const f32x2 *>(obs + array * STRIDE + k); };
+  const f32x2 th = at(0), tl = at(1);
+  GradTerms o[J];
+  Kahan2 V = {dup2(gam), 0};
+#pragma unroll
+  for (int j = 0; j < J; ++j) o[j] = grad_terms<WIDE>(th, tl, q[j], tab, V);
+  const f32x2 r = sub2(sub2(V.big, at(2)), add2(V.small, at(3)));
+  const f32x2 sw = at(4), sr = mul2(sw, r), a2 = add2(sr, sr);
+  kahan_add(acc, mul2(sr, sr));
+  sum_a = fma2(a2, sw, sum_a);
+  const f32x2 swdt = mul2(sw, add2(add2(th, tl), dup2(dref)));
+#pragma unroll
+  for (int j = 0; j < J; ++j) gn_add(g[j], o[j], q[j], sw, swdt, a2, u + 5 * j);
+  u[5 * J] = sw;
+}
+
+// A warp's next kGnAhead systems, s0 + i stride, set up together: planet j of
+// system i by lane i J + j into q[i J + j], gamma of system i by lane 16 + i (the
+// lane's return value).  One system's setup is a chain of some 500
+// instructions in J lanes; alone it took a tenth of the time of a system of
+// 3 planets and 512 observations, and half of one of 1 and 256.  wide: bit l
+// set if lane l's planet asks for the wide mean anomaly.
+template <int J>
+__device__ __forceinline__ float gn_setup_ahead(const UniformArgs &a, int64_t s0, int64_t stride,
+                                                int lane, double t_ref, GradPlanetP *q,
+                                                unsigned &wide) {
+  static_assert(kGnAhead * J <= 16, "planets in lanes 0 .. 15, gamma from lane 16");
+  constexpr int NP = 5 * J + 1;
+  bool far = false;
+  float gam = 0.0f;
+  __syncwarp();                                        // the last systems' use of q
+  if (lane < kGnAhead * J) {
+    const int i = lane / J, j = lane - i * J;
+    const int64_t s = s0 + i * stride;
+    GradPlanetP p = {};
+    if (s < a.n_sys && dbg_ok(a.invalid, s * NP + 5 * j + 4 < a.n_sys * NP, kDbgParam, s * NP))
+      p = grad_setup_pair(a.params + s * NP + 5 * j, t_ref, a.t0, far);
+    q[lane] = p;
+  } else if (lane >= 16 && lane < 16 + kGnAhead) {
+    const int64_t s = s0 + (lane - 16) * stride;
+    if (s < a.n_sys) gam = d2f(system_gamma_g(a.params + s * NP, J));
+  }
+  wide = __ballot_sync(0xffffffffu, far);
+  return gam;
+}
+
+// chi2 and gradient of a warp's system: the lanes' sums combined and written.
+// scale: the factors of the rows' columns (gn_scale).
+template <int J>
+__device__ __forceinline__ void gn_write_grad(const UniformArgs &a, int64_t s, int lane,
+                                              float poison, const Kahan2 &acc2, f32x2 sum_a,
+                                              const GradSums (&g)[J], const float *scale,
+                                              float *chi2_out, float *grad_out) {
+  constexpr int NP = 5 * J + 1;
+  Kahan acc = kahan_join(acc2);
+  float sa = join2(sum_a);
+  GradLane gl[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) gl[j] = grad_join(g[j]);
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) {
+    const Kahan o = {shfl_xor(acc.big, m), shfl_xor(acc.small, m)};
+    kahan_merge(acc, o);
+    sa += shfl_xor(sa, m);
+#pragma unroll
+    for (int j = 0; j < J; ++j) grad_combine(gl[j], m);
+  }
+  if (s >= a.n_sys) return;
+  if (lane == 0) {
+    const float value = kahan_value(acc) + poison;
+    if (chi2_out) chi2_out[s] = value;
+    note_invalid(a.invalid, value);
+  }
+  if (grad_out) {
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      const float v[5] = {kahan_value(gl[j].P), gl[j].K, gl[j].e, gl[j].w, gl[j].M};
+#pragma unroll
+      for (int i = 0; i < 5; ++i)
+        if (lane == ((5 * j + i) & 31))
+          grad_out[s * NP + 5 * j + i] = __fmaf_rn(scale[5 * j + i], v[i], poison);
+    }
+    if (lane == ((5 * J) & 31)) grad_out[s * NP + 5 * J] = sa + poison;
+  }
 }
 
 template <int J>
@@ -954,6 +1045,148 @@ gn_mixed_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__
     }
 }
 
+// The pair form (kc_pair.cuh) with mma.sync, n_pl <= 3: the same chi2, bit for
+// bit, as the tcgen05 kernel.  From four planets on its registers (192 to 255)
+// leave too few warps: 20000 x 4 x 256 ran 267 us against 217 for the kernel
+// above, 10000 x 8 x 256 476 against 296.
+template <int J>
+__global__ void __launch_bounds__(kGnWarps * 32)
+gn_pair_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__ grad_out,
+               float *__restrict__ jtj_out) {
+  constexpr int NP = gn_np(J), MT = gn_mt(J), NT = gn_nt(J), ROW2 = gn_row2(J);
+  constexpr int NTRI = NP * (NP + 1) / 2, kTile = kTcObsTile;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const GnPairLayout L(J, kTile);
+  float *tab_s = reinterpret_cast<float *>(smem + L.tab);
+  float *obs_s = reinterpret_cast<float *>(smem + L.obs);
+  float2 *u_all = reinterpret_cast<float2 *>(smem + L.u);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int block = kGnWarps * 32;
+  GradPlanetP *ahead = reinterpret_cast<GradPlanetP *>(smem + L.pl) + warp * kGnAhead * J;
+  const double t_ref = a.n_obs > 0 ? a.t[0] : a.t0;
+  const Split3 tr3 = split3(t_ref), te3 = split3(a.t0);
+  const float dref_f = (tr3.x0 - te3.x0) + (tr3.x1 - te3.x1);     // t_ref - t0
+  const float jit2 = d2f(a.jitter2);
+
+  ang_tab_load(tab_s, tid, block);
+  for (int i = tid; i < kGnWarps * kGnRows * ROW2; i += block)
+    u_all[i] = make_float2(0.0f, 0.0f);                           // incl. padding
+  // observations that fit one tile are staged once for all of the CTA's systems
+  const bool staged_once = a.n_obs <= kTile;
+  bool far = false;
+  if (staged_once)
+    far = gn_stage<kTile>(a, 0, a.n_obs, (a.n_obs + kGnRows - 1) / kGnRows * kGnRows, tid, block,
+                          tr3, jit2, obs_s);
+  far = __syncthreads_or(far);
+
+  // The (hi, lo) pair of element (row r, column c) of U sits at
+  // r * ROW2 + (c ^ ((r >> 2) & 3)): with ROW2 = 4 mod 16 both the row writes
+  // (rows l and 32 + l for lane l) and the fragment loads touch 32 different
+  // banks in each half-warp.
+  float2 *u = u_all + warp * kGnRows * ROW2;
+  const int gid = lane >> 2, tig = lane & 3;
+  const int sw_row = (lane >> 2) & 3;
+
+  // a system per warp; the CTA's warps step together (they share the tile)
+  const int64_t stride = (int64_t)gridDim.x * kGnWarps;
+  int ahead_i = kGnAhead;                              // systems used of those set up
+  unsigned wide_ahead = 0;
+  float gam_ahead = 0.0f;
+  for (int64_t s = (int64_t)blockIdx.x * kGnWarps + warp; s - warp < a.n_sys; s += stride) {
+    if (ahead_i == kGnAhead) {
+      ahead_i = 0;
+      gam_ahead = gn_setup_ahead<J>(a, s, stride, lane, t_ref, ahead, wide_ahead);
+    }
+    const GradPlanetP *q = ahead + ahead_i * J;
+    const float gam = __shfl_sync(0xffffffffu, gam_ahead, 16 + ahead_i);
+    bool wide = far || ((wide_ahead >> (ahead_i * J)) & ((1u << J) - 1u)) != 0u;
+    ++ahead_i;
+    __syncwarp();
+    Kahan2 acc = {0, 0};
+    f32x2 sum_a = 0;
+    GradSums g[J];
+    float C[MT][NT][4];
+#pragma unroll
+    for (int j = 0; j < J; ++j) g[j] = GradSums{{0, 0}, 0, 0, 0, 0};
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) C[mt][nt][i] = 0.0f;
+
+    for (int k0 = 0; k0 < a.n_obs; k0 += kTile) {
+      const int nk = min(kTile, a.n_obs - k0);
+      const int npad = (nk + kGnRows - 1) / kGnRows * kGnRows;
+      if (!staged_once) {
+        __syncthreads();
+        const bool w = gn_stage<kTile>(a, k0, nk, npad, tid, block, tr3, jit2, obs_s);
+        wide |= (bool)__syncthreads_or(w);
+      }
+      for (int kb = 0; kb < npad; kb += kGnRows) {
+        {
+          f32x2 urow[NP];
+          if (wide)
+            gn_pair<J, kTile, true>(obs_s, kb + 2 * lane, dref_f, q, tab_s, gam, acc, sum_a, g,
+                                    urow);
+          else
+            gn_pair<J, kTile, false>(obs_s, kb + 2 * lane, dref_f, q, tab_s, gam, acc, sum_a, g,
+                                     urow);
+#pragma unroll
+          for (int i = 0; i < NP; ++i) {
+            u[lane * ROW2 + (i ^ sw_row)] = tf32_pair(lo2(urow[i]));
+            u[(32 + lane) * ROW2 + (i ^ sw_row)] = tf32_pair(hi2(urow[i]));
+          }
+        }
+        __syncwarp();
+        // H += U^T U: k-steps of 8 rows, as in gn_mixed_kernel
+#pragma unroll
+        for (int ks = 0; ks < kGnRows / 8; ++ks) {
+          const float2 *r0 = u + (ks * 8 + tig) * ROW2;
+          const float2 *r1 = r0 + 4 * ROW2;
+          const int g0 = gid ^ ((2 * ks) & 3), g1 = gid ^ ((2 * ks + 1) & 3);   // row swizzles
+          const float2 x[4] = {r0[g0], r0[g0 + 8], r1[g1], r1[g1 + 8]};
+          static_assert(MT == 1, "n_pl <= 3");
+          unsigned ah[4], al[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            ah[i] = __float_as_uint(x[i].x);
+            al[i] = __float_as_uint(x[i].y);
+          }
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt) {
+            const unsigned bh[2] = {ah[nt], ah[2 + nt]}, bl[2] = {al[nt], al[2 + nt]};
+            mma_tf32(C[0][nt], al, bh);
+            mma_tf32(C[0][nt], ah, bl);
+            mma_tf32(C[0][nt], ah, bh);
+          }
+        }
+        __syncwarp();
+      }
+    }
+
+    float scale[NP];                       // the rows' columns over their factors
+#pragma unroll
+    for (int p = 0; p < NP; ++p) scale[p] = gn_scale(q, J, p);
+    const float poison = 0.0f * gam;                   // NaN for an invalid system
+    gn_write_grad<J>(a, s, lane, poison, acc, sum_a, g, scale, chi2_out, grad_out);
+    if (s < a.n_sys) {
+      float *H = jtj_out + s * NTRI;
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int row = gid + (i >= 2 ? 8 : 0);
+          const int col = 8 * nt + 2 * tig + (i & 1);
+          if (row < NP && col < NP && col >= row)
+            H[tri_index(NP, row, col)] =
+                __fmaf_rn(gn_scale(q, J, row) * gn_scale(q, J, col), C[0][nt][i], poison);
+        }
+    }
+  }
+}
+
 // ---------------------------------------------- Gauss-Newton on tcgen05
 //
 // The same pass with the U^T U update on the fifth-generation tensor cores:
@@ -972,17 +1205,22 @@ gn_mixed_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__
 // TMEM, D1 += hi hi^T and D2 += lo hi^T (two MMAs per K step, not three),
 // give H = D1 + D2 + D2^T in the epilogue.  The four diagonal 16 x 16
 // blocks are kept; 3/4 of the products are cross-system terms that are
-// thrown away.  A batch is 64 observations, two per lane, evaluated side by
-// side (two independent chains per planet for the scheduler); its tile is
-// two 64 x 32 halves.  The order of the observations along K is free (the
+// thrown away.  A batch is 64 observations, two per lane in packed form
+// (kc_pair.cuh); its tile is two 64 x 32 halves.  The columns go in over their
+// per-planet factors (gn_add), which the epilogue applies to H.  The order of the observations along K is free (the
 // sum runs over all of them), so lane l puts its pair at K = 2l and 2l + 1
 // and writes both words of an element with one 8-byte store.
 // One tile suffices: a warp rewrites it only after evaluating the next 64
 // observations, by which time the MMAs that read it have long completed
 // (its lane 0 still waits on the mbarrier their commit arrives on).  A CTA
-// barrier per batch hands the written tile to the issuing thread (on a
-// GB300 this ran 822 us on 65536 x 3 x 512 against 891 us with a "full"
-// mbarrier that let the other warps run a batch ahead of warp 0).  With
+// barrier per batch hands the written tile to the issuing thread (an earlier
+// version ran 822 us on 65536 x 3 x 512 this way against 891 us with a "full"
+// mbarrier that let the other warps run a batch ahead of warp 0).  The CTAs
+// are persistent: the table and the observations are staged once, and a warp
+// sets four of its systems up at a time.  On 65536 x 3 x 512: 732 us with the
+// scalar evaluation, 685 packed, 640 persistent, 619 with the setups
+// together.  Bound by latency: 16 warps per SM (registers, TMEM and shared
+// memory all end there), issue slots 44 % busy.  With
 // M = 64 the accumulator's row r sits in TMEM lane 32 (r / 16) + r % 16, so
 // warp w reads its system's blocks from its own lanes 32 w .. 32 w + 15,
 // columns 16 w .. 16 w + 15 (D1) and 64 + 16 w .. 64 + 16 w + 15 (D2), and
@@ -992,19 +1230,17 @@ gn_mixed_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__
 
 constexpr int kTcHalfBytes = 64 * 32 * 4;       // 64 rows x 32 observations, TF32
 constexpr int kTcBatch = 64;                    // observations per batch
-constexpr int kTcObsTile = 512;                 // observations staged at a time
 constexpr int kTcCols = 128;                    // TMEM columns per CTA: D1, D2
 constexpr uint64_t kTcWaitLimit = 20000000;     // ns an mbarrier wait may take (20 ms)
 
 struct GnTcLayout {
-  size_t u, pl, gam, obs, w, bar, slot, total;
+  size_t u, tab, pl, obs, bar, slot, total;
   __host__ __device__ GnTcLayout(int J) {
     u = 0;                                       // hi halves, then lo halves: 1024-aligned
-    pl = u + 4 * kTcHalfBytes;
-    gam = pl + sizeof(GradPlanetF) * kGnWarps * J;
-    obs = align_up(gam + sizeof(float) * kGnWarps, 16);
-    w = obs + sizeof(float4) * kTcObsTile;
-    bar = align_up(w + sizeof(float4) * kTcObsTile, 8);
+    tab = u + 4 * kTcHalfBytes;
+    pl = tab + sizeof(AngTab);
+    obs = align_up(pl + sizeof(GradPlanetP) * kGnWarps * kGnAhead * J, 16);
+    bar = align_up(obs + sizeof(float) * 5 * kTcObsTile, 8);
     slot = bar + sizeof(uint64_t);
     total = align_up(slot + 16, 16) + 1024;     // 1024 bytes to align the base
   }
@@ -1029,16 +1265,15 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, uint64_
 // an element would move by less than 2^-20 of itself).
 template <int NP>
 __device__ __forceinline__ void gn_tc_store(unsigned char *rows, uint32_t lane_q,
-                                            const float (&ua)[NP], const float (&ub)[NP]) {
+                                            const f32x2 (&u)[NP]) {
   constexpr unsigned kTf32Mask = 0xffffe000u;
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
-    const float ha = __uint_as_float(__float_as_uint(ua[p]) & kTf32Mask);
-    const float hb = __uint_as_float(__float_as_uint(ub[p]) & kTf32Mask);
+    const f32x2 h = pack2(__uint_as_float(__float_as_uint(lo2(u[p])) & kTf32Mask),
+                          __uint_as_float(__float_as_uint(hi2(u[p])) & kTf32Mask));
     const uint32_t off = (p >> 3) * 1024 + (p & 7) * 128 + ((lane_q ^ (p & 7)) << 4);
-    *reinterpret_cast<float2 *>(rows + off) = make_float2(ha, hb);
-    *reinterpret_cast<float2 *>(rows + 2 * kTcHalfBytes + off) =
-        make_float2(__fsub_rn(ua[p], ha), __fsub_rn(ub[p], hb));
+    *reinterpret_cast<f32x2 *>(rows + off) = h;
+    *reinterpret_cast<f32x2 *>(rows + 2 * kTcHalfBytes + off) = sub2(u[p], h);
   }
 }
 
@@ -1055,18 +1290,15 @@ gn_mixed_tc_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restric
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char *smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
   const GnTcLayout L(J);
-  GradPlanetF *pl_s = reinterpret_cast<GradPlanetF *>(smem + L.pl);
-  float *gam_s = reinterpret_cast<float *>(smem + L.gam);
-  float4 *obs_s = reinterpret_cast<float4 *>(smem + L.obs);
-  float4 *wt_s = reinterpret_cast<float4 *>(smem + L.w);
+  float *tab_s = reinterpret_cast<float *>(smem + L.tab);
+  float *obs_s = reinterpret_cast<float *>(smem + L.obs);       // th, tl, v hi, v lo, sqrt w
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem + L.bar);   // commits of the MMAs
   uint32_t *slot = reinterpret_cast<uint32_t *>(smem + L.slot);
   unsigned char *tiles = smem + L.u;
   const uint32_t tiles_a = tc::smem_u32(tiles), bar_a = tc::smem_u32(bar);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t sys0 = (int64_t)blockIdx.x * kGnWarps;
-  const int64_t s = sys0 + warp;
+  GradPlanetP *ahead = reinterpret_cast<GradPlanetP *>(smem + L.pl) + warp * kGnAhead * J;
 
   if (warp == 0) tc::tmem_alloc(tc::smem_u32(slot), kTcCols);
   if (tid == 0) {
@@ -1077,25 +1309,18 @@ gn_mixed_tc_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restric
   const Split3 tr3 = split3(t_ref), te3 = split3(a.t0);
   const float dref_f = (tr3.x0 - te3.x0) + (tr3.x1 - te3.x1);     // t_ref - t0
   const float jit2 = d2f(a.jitter2);
-  for (int i = tid; i < kGnWarps * J; i += kThreads) {
-    const int64_t si = sys0 + i / J;
-    GradPlanetF q = {};
-    if (si < a.n_sys &&
-        dbg_ok(a.invalid, si * NP + 5 * (i % J) + 4 < a.n_sys * NP, kDbgParam, si * NP))
-      q = grad_setup_mixed(a.params + si * NP + 5 * (i % J), t_ref, a.t0);
-    pl_s[i] = q;
-  }
-  for (int i = tid; i < kGnWarps; i += kThreads)
-    gam_s[i] = sys0 + i < a.n_sys ? d2f(system_gamma_g(a.params + (sys0 + i) * NP, J)) : 0.0f;
+  ang_tab_load(tab_s, tid, kThreads);
+  // observations that fit one tile are staged once for all of the CTA's systems
+  const bool staged_once = a.n_obs <= kTcObsTile;
+  bool far = false;
+  if (staged_once)
+    far = gn_stage<kTcObsTile>(a, 0, a.n_obs, (a.n_obs + kTcBatch - 1) / kTcBatch * kTcBatch, tid,
+                               kThreads, tr3, jit2, obs_s);
   tc::fence_before_sync();
-  __syncthreads();
+  far = __syncthreads_or(far);
   tc::fence_after_sync();
   const uint32_t taddr = *slot;
 
-  GradPlanetF qr[J];
-#pragma unroll
-  for (int j = 0; j < J; ++j) qr[j] = pl_s[warp * J + j];
-  const float gam = gam_s[warp];
   // lane l: columns 2 l, 2 l + 1 of the batch, in half l / 16
   const uint32_t lane_q = (uint32_t)(lane & 15) >> 1;
   unsigned char *my_rows = tiles + (lane >> 4) * kTcHalfBytes + 2048 * warp + 8 * (lane & 1);
@@ -1103,121 +1328,117 @@ gn_mixed_tc_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restric
   // start address alone (bits 0-13: the address / 16; the tiles end below
   // 2^18 bytes, so an offset adds without a carry out of the field).
   const uint64_t dtile = tc::desc_kmajor_sw128(tiles_a);
-  Kahan acc = {0.0f, 0.0f};
-  Kahan gP[J];
-  float g[NP];
-#pragma unroll
-  for (int i = 0; i < NP; ++i) g[i] = 0.0f;
-#pragma unroll
-  for (int j = 0; j < J; ++j) gP[j] = Kahan{0.0f, 0.0f};
   uint32_t nb = 0;                                   // batches (commits) so far
   bool ok = true;
 
-  for (int k0 = 0; k0 < a.n_obs; k0 += kTcObsTile) {
-    const int nk = min(kTcObsTile, a.n_obs - k0);
-    __syncthreads();
-    for (int k = tid; k < nk; k += kThreads) {
-      if (!dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k)) continue;
-      float th, tl, vh, vl;
-      sub_ds(split3(a.t[k0 + k]), tr3, th, tl);
-      split_d(a.v[k0 + k], vh, vl);
-      obs_s[k] = make_float4(th, tl, vh, vl);
-      const float sg = d2f(a.sigma[k0 + k]);
-      const float var = __fmaf_rn(sg, sg, jit2);
-      const float wk = var > 0.0f ? 1.0f / var : __int_as_float(0x7fc00000);
-      wt_s[k] = make_float4(wk, th + dref_f, sqrtf(wk), 0.0f);
+  // Four systems at a time, one per warp.  A warp sets its own system up; the
+  // barrier of a batch is the only one the systems share, and the first one
+  // of a group also orders the group's first MMA (which overwrites the
+  // accumulators) after every warp's read of the group before.
+  const int64_t stride = (int64_t)gridDim.x * kGnWarps;
+  int ahead_i = kGnAhead;                            // systems used of those set up
+  unsigned wide_ahead = 0;
+  float gam_ahead = 0.0f;
+  for (int64_t s = (int64_t)blockIdx.x * kGnWarps + warp; s - warp < a.n_sys; s += stride) {
+    if (ahead_i == kGnAhead) {
+      ahead_i = 0;
+      gam_ahead = gn_setup_ahead<J>(a, s, stride, lane, t_ref, ahead, wide_ahead);
     }
-    __syncthreads();
-    for (int kb = 0; kb < nk; kb += kTcBatch) {
-      const int ka = kb + lane, kbb = kb + 32 + lane;
-      const int ia = min(ka, nk - 1), ib = min(kbb, nk - 1);
-      float ua[NP], ub[NP];
-      gn_obs<J>(obs_s[ia], wt_s[ia], ka < nk, gam, qr, acc, gP, g, ua);
-      gn_obs<J>(obs_s[ib], wt_s[ib], kbb < nk, gam, qr, acc, gP, g, ub);
-      if (nb > 0 && ok)                  // the MMAs that read the tile before
-        ok = warp_wait(bar_a, (nb - 1) & 1u, kTcWaitLimit, lane);
-      gn_tc_store<NP>(my_rows, lane_q, ua, ub);
-      tc::fence_proxy_async_smem();
-      __syncthreads();
-      if (tid == 0) {
-        tc::fence_after_sync();
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-          // K step ks: columns 8 ks .. 8 ks + 7 of the batch, in half ks / 4
-          const uint32_t off = ((ks >> 2) * kTcHalfBytes + 32 * (ks & 3)) >> 4;
-          const uint64_t hi = dtile + off, lo = dtile + off + (2 * kTcHalfBytes >> 4);
-          const uint32_t accumulate = (nb | ks) != 0;
-          tc::mma_tf32(taddr, hi, hi, IDESC, accumulate);                 // D1 += hi hi^T
-          tc::mma_tf32(taddr + kTcCols / 2, lo, hi, IDESC, accumulate);   // D2 += lo hi^T
-        }
-        tc::commit(bar_a);
-      }
-      ++nb;
-    }
-  }
-
-  // Every MMA is complete once the last commit's phase is; a longer wait if
-  // a wait gave up before.
-  float h[16];
-  if (nb > 0) {
-    const bool last_ok = warp_wait(bar_a, (nb - 1) & 1u, ok ? kTcWaitLimit : 4 * kTcWaitLimit,
-                                   lane);
-    ok = ok && last_ok;
-    tc::fence_after_sync();
-    const uint32_t blk = taddr + ((uint32_t)(32 * warp) << 16) + 16u * warp;
-    float h2[16];
-    tc::tmem_ld16(blk, h);
-    tc::tmem_ld16(blk + kTcCols / 2, h2);
-    // H = D1 + D2 + D2^T: lane r < 16 holds row r of both blocks; D2's is
-    // transposed through 16 x 17 floats of the warp's own in the staged
-    // observations' shared memory (read by no warp after the last batch's
-    // barrier).
-    float *tr = reinterpret_cast<float *>(obs_s) + warp * 16 * 17;
-    if (lane < 16) {
-#pragma unroll
-      for (int i = 0; i < 16; ++i) tr[lane * 17 + i] = h2[i];
-    }
+    const GradPlanetP *q = ahead + ahead_i * J;
+    const float gam = __shfl_sync(0xffffffffu, gam_ahead, 16 + ahead_i);
+    bool wide = far || ((wide_ahead >> (ahead_i * J)) & ((1u << J) - 1u)) != 0u;
+    ++ahead_i;
     __syncwarp();
-    if (lane < 16) {
+    Kahan2 acc2 = {0, 0};
+    f32x2 sum_a = 0;
+    GradSums g[J];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) h[i] += h2[i] + tr[i * 17 + lane];
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 16; ++i) h[i] = 0.0f;
-  }
+    for (int j = 0; j < J; ++j) g[j] = GradSums{{0, 0}, 0, 0, 0, 0};
+    const uint32_t nb0 = nb;
 
-  for (int m = 16; m >= 1; m >>= 1) {
-    Kahan o = {shfl_xor(acc.big, m), shfl_xor(acc.small, m)};
-    kahan_merge(acc, o);
+    for (int k0 = 0; k0 < a.n_obs; k0 += kTcObsTile) {
+      const int nk = min(kTcObsTile, a.n_obs - k0);
+      const int npad = (nk + kTcBatch - 1) / kTcBatch * kTcBatch;
+      if (!staged_once) {
+        __syncthreads();
+        const bool w = gn_stage<kTcObsTile>(a, k0, nk, npad, tid, kThreads, tr3, jit2, obs_s);
+        wide |= (bool)__syncthreads_or(w);
+      }
+      for (int kb = 0; kb < npad; kb += kTcBatch) {
+        f32x2 u[NP];
+        if (wide)
+          gn_pair<J, kTcObsTile, true>(obs_s, kb + 2 * lane, dref_f, q, tab_s, gam, acc2, sum_a, g,
+                                       u);
+        else
+          gn_pair<J, kTcObsTile, false>(obs_s, kb + 2 * lane, dref_f, q, tab_s, gam, acc2, sum_a,
+                                        g, u);
+        if (nb > 0 && ok)                  // the MMAs that read the tile before
+          ok = warp_wait(bar_a, (nb - 1) & 1u, kTcWaitLimit, lane);
+        gn_tc_store<NP>(my_rows, lane_q, u);
+        tc::fence_proxy_async_smem();
+        tc::fence_before_sync();
+        __syncthreads();
+        if (tid == 0) {
+          tc::fence_after_sync();
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-      Kahan op = {shfl_xor(gP[j].big, m), shfl_xor(gP[j].small, m)};
-      kahan_merge(gP[j], op);
+          for (int ks = 0; ks < 8; ++ks) {
+            // K step ks: columns 8 ks .. 8 ks + 7 of the batch, in half ks / 4
+            const uint32_t off = ((ks >> 2) * kTcHalfBytes + 32 * (ks & 3)) >> 4;
+            const uint64_t hi = dtile + off, lo = dtile + off + (2 * kTcHalfBytes >> 4);
+            const uint32_t accumulate = ((nb - nb0) | ks) != 0;
+            tc::mma_tf32(taddr, hi, hi, IDESC, accumulate);                 // D1 += hi hi^T
+            tc::mma_tf32(taddr + kTcCols / 2, lo, hi, IDESC, accumulate);   // D2 += lo hi^T
+          }
+          tc::commit(bar_a);
+        }
+        ++nb;
+      }
     }
+
+    // Every MMA is complete once the last commit's phase is; a longer wait if
+    // a wait gave up before.
+    float h[16];
+    if (nb > nb0) {
+      const bool last_ok = warp_wait(bar_a, (nb - 1) & 1u, ok ? kTcWaitLimit : 4 * kTcWaitLimit,
+                                     lane);
+      ok = ok && last_ok;
+      tc::fence_after_sync();
+      const uint32_t blk = taddr + ((uint32_t)(32 * warp) << 16) + 16u * warp;
+      float h2[16];
+      tc::tmem_ld16(blk, h);
+      tc::tmem_ld16(blk + kTcCols / 2, h2);
+      // H = D1 + D2 + D2^T: lane r < 16 holds row r of both blocks; D2's is
+      // transposed through 16 x 17 floats of the warp's own 2 KB of the
+      // operand tile (no MMA reads the tile any more, and only this warp
+      // writes there).
+      float *tr = reinterpret_cast<float *>(tiles + 2048 * warp);
+      __syncwarp();
+      if (lane < 16) {
 #pragma unroll
-    for (int i = 0; i < NP; ++i) g[i] += shfl_xor(g[i], m);
-  }
+        for (int i = 0; i < 16; ++i) tr[lane * 17 + i] = h2[i];
+      }
+      __syncwarp();
+      if (lane < 16) {
 #pragma unroll
-  for (int j = 0; j < J; ++j) g[5 * j] = kahan_value(gP[j]);
-  if (s < a.n_sys) {
+        for (int i = 0; i < 16; ++i) h[i] += h2[i] + tr[i * 17 + lane];
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) h[i] = 0.0f;
+    }
+
     // NaN for an invalid system, or where a wait on the tensor cores gave up
     const float poison = ok ? 0.0f * gam : __int_as_float(0x7fc00000);
-    if (lane == 0) {
-      const float value = kahan_value(acc) + poison;
-      if (chi2_out) chi2_out[s] = value;
-      note_invalid(a.invalid, value);
-    }
-    if (grad_out) {
+    float scale[NP];                       // the rows' columns over their factors
 #pragma unroll
-      for (int i = 0; i < NP; ++i)
-        if (lane == (i & 31)) grad_out[s * NP + i] = g[i] + poison;
-    }
-    float *H = jtj_out + s * NTRI;
-    if (lane < NP) {
+    for (int p = 0; p < NP; ++p) scale[p] = gn_scale(q, J, p);
+    gn_write_grad<J>(a, s, lane, poison, acc2, sum_a, g, scale, chi2_out, grad_out);
+    if (s < a.n_sys && lane < NP) {
+      float *H = jtj_out + s * NTRI;
+      const float mine = gn_scale(q, J, lane);
 #pragma unroll
       for (int c = 0; c < NP; ++c)
-        if (c >= lane) H[tri_index(NP, lane, c)] = h[c] + poison;
+        if (c >= lane) H[tri_index(NP, lane, c)] = __fmaf_rn(mine * scale[c], h[c], poison);
     }
   }
 
@@ -1495,6 +1716,26 @@ cudaError_t launch_grad_f64(const UniformArgs &a, const Tile &tile, double *chi2
   return cudaGetLastError();
 }
 
+// The pair form with mma.sync (split 0, n_pl <= 3): persistent, as many CTAs
+// as are resident at once.
+template <int J>
+cudaError_t launch_gn_pair(const UniformArgs &a, void *chi2, void *grad, void *jtj,
+                           cudaStream_t st) {
+  const size_t smem = GnPairLayout(J, kTcObsTile).total;
+  cudaError_t err = set_smem(gn_pair_kernel<J>, smem);
+  if (err != cudaSuccess) return err;
+  int per_sm = 0;
+  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gn_pair_kernel<J>, kGnWarps * 32,
+                                                      smem);
+  if (err != cudaSuccess) return err;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const int64_t groups = (a.n_sys + kGnWarps - 1) / kGnWarps;
+  const int grid = (int)std::min<int64_t>(groups, (int64_t)sm_count() * per_sm);
+  gn_pair_kernel<J><<<grid, kGnWarps * 32, smem, st>>>(a, (float *)chi2, (float *)grad,
+                                                       (float *)jtj);
+  return cudaGetLastError();
+}
+
 // The tcgen05 variant (split 4): n_pl <= 3.  Every resident CTA holds
 // kTcCols TMEM columns, so the launch is refused unless the SM's 512
 // columns cover all CTAs that can be resident at once (an allocation would
@@ -1510,7 +1751,12 @@ cudaError_t launch_gn_tc(const UniformArgs &a, void *chi2, void *grad, void *jtj
                                                       kGnWarps * 32, smem);
   if (err != cudaSuccess) return err;
   if (per_sm < 1 || per_sm * kTcCols > 512) return cudaErrorInvalidConfiguration;
-  const int grid = (int)((a.n_sys + kGnWarps - 1) / kGnWarps);
+  // persistent: the resident CTAs take the groups of four systems in turn.
+  // As many as the SM's TMEM, shared memory and registers hold (the occupancy
+  // query counts one for a kernel that allocates TMEM).
+  const int64_t groups = (a.n_sys + kGnWarps - 1) / kGnWarps;
+  const int fit = std::min(512 / kTcCols, (int)(228 * 1024 / (smem + 1024)));
+  const int grid = (int)std::min<int64_t>(groups, (int64_t)sm_count() * std::max(fit, 1));
   gn_mixed_tc_kernel<J><<<grid, kGnWarps * 32, smem, st>>>(a, (float *)chi2, (float *)grad,
                                                            (float *)jtj);
   return cudaGetLastError();
@@ -1518,8 +1764,8 @@ cudaError_t launch_gn_tc(const UniformArgs &a, void *chi2, void *grad, void *jtj
 
 // Without a tuned entry the mixed Gauss-Newton kernel updates U^T U on
 // tcgen05 where it can (n_pl <= 3): on a GB300, 65536 systems x 3 planets x
-// 512 observations took 822 us against 869 us with mma.sync (whose
-// registers do not leave room for two observations per lane: 958 us).
+// 512 observations take 619 us against 702 us with mma.sync (164 registers),
+// 20000 x 1 x 256 78 against 72.
 int gn_default_variant(int n_pl) { return n_pl <= 3 ? 4 : 0; }
 
 bool gn_variant_ok(int variant, int n_pl) {
@@ -1551,15 +1797,25 @@ cudaError_t launch_gauss_newton(const UniformArgs &a, bool f64, void *chi2, void
 #undef KC_LAUNCH
   } else {
     const int grid = (int)((a.n_sys + kGnWarps - 1) / kGnWarps);
-#define KC_LAUNCH(JJ)                                                                        \
-  {                                                                                          \
-    const size_t smem = GnMixedLayout(JJ, kGnObsTile).total;                                 \
-    err = set_smem(gn_mixed_kernel<JJ>, smem);                                               \
-    if (err == cudaSuccess)                                                                  \
+#define KC_LAUNCH(JJ)                                                                     \
+  {                                                                                       \
+    const size_t smem = GnMixedLayout(JJ, kGnObsTile).total;                              \
+    err = set_smem(gn_mixed_kernel<JJ>, smem);                                            \
+    if (err == cudaSuccess)                                                               \
       gn_mixed_kernel<JJ><<<grid, kGnWarps * 32, smem, st>>>(a, (float *)chi2, (float *)grad, \
-                                                             (float *)jtj);                  \
+                                                             (float *)jtj);               \
   }
-    KC_DISPATCH_J(a.n_pl, KC_LAUNCH)
+    switch (a.n_pl) {
+      case 1: return launch_gn_pair<1>(a, chi2, grad, jtj, st);
+      case 2: return launch_gn_pair<2>(a, chi2, grad, jtj, st);
+      case 3: return launch_gn_pair<3>(a, chi2, grad, jtj, st);
+      case 4: KC_LAUNCH(4) break;
+      case 5: KC_LAUNCH(5) break;
+      case 6: KC_LAUNCH(6) break;
+      case 7: KC_LAUNCH(7) break;
+      case 8: KC_LAUNCH(8) break;
+      default: return cudaErrorInvalidValue;
+    }
 #undef KC_LAUNCH
   }
   if (err != cudaSuccess) return err;

@@ -449,6 +449,41 @@ __device__ __forceinline__ void grad_add(GradSums &G, const GradTerms &o, const 
   G.M = fma2(a, Qyy, G.M);
 }
 
+// The same planet's row of sqrt(w) J for the Gauss-Newton matrix, each column
+// over its per-planet factor (gn_scale), and its gradient sums from the row
+// with a = 2 sqrt(w) r; swdt = sqrt(w) (t - t0).
+__device__ __forceinline__ void gn_add(GradSums &G, const GradTerms &o, const GradPlanetP &g,
+                                       f32x2 sw, f32x2 swdt, f32x2 a, f32x2 *u) {
+  const f32x2 Qy = mul2(o.Q, o.y), Qyy = mul2(Qy, o.y);
+  const f32x2 h = fma2(dup2(g.beta), o.y, dup2(g.ibeta));
+  u[0] = mul2(swdt, Qyy);
+  u[1] = mul2(sw, o.dK);
+  u[2] = mul2(sw, sub2(dup2(g.cw), mul2(Qy, mul2(o.s, h))));
+  u[3] = mul2(sw, add2(o.Q, dup2(g.esw)));
+  u[4] = mul2(sw, Qyy);
+  kahan_add_y(G.P, fma2(a, u[0], neg2(G.P.small)));
+  G.K = fma2(a, u[1], G.K);
+  G.e = fma2(a, u[2], G.e);
+  G.w = fma2(a, u[3], G.w);
+  G.M = fma2(a, u[4], G.M);
+}
+
+// Factor of parameter p (0 .. 5 n_pl) of a system's rows: the columns are (dt
+// Q y^2, dK, cos w - .., Q + e sin w, Q y^2) per planet, then 1.
+__device__ __forceinline__ float gn_scale(const GradPlanetP *q, int J, int p) {
+  const int j = p / 5, i = p - 5 * j;
+  if (j >= J) return 1.0f;
+  const GradPlanetP &g = q[j];
+  const float Kb = g.K * g.beta;
+  switch (i) {
+    case 0: return Kb * (kTwoPiF * g.n2);
+    case 1: return 1.0f;
+    case 2: return g.K;
+    case 3: return -g.K;
+    default: return -Kb;
+  }
+}
+
 __device__ __forceinline__ float join2(f32x2 x) { return lo2(x) + hi2(x); }
 
 // A planet's five sums of one lane (the pair joined).

@@ -125,3 +125,43 @@ def test_times_and_parameters_out_of_range_stay_nan(kc):
     t[50] = np.nan
     assert torch.isnan(run(t)).all()
     kc.kc_last_device_error()                        # leaves the counter at zero
+
+
+@pytest.mark.parametrize("split", [0, 4])
+@pytest.mark.parametrize("n_pl,n_obs,n_sys,span", [
+    (3, 600, 2600, 3000.0),        # several groups of systems per CTA, two staged tiles
+    (2, 512, 5000, 3000.0),        # one full tile, staged once
+    (1, 65, 9000, 30000.0),        # the wide mean anomaly
+])
+def test_gauss_newton_persistent(kc, oracle_mod, split, n_pl, n_obs, n_sys, span):
+    """The pair forms of the Gauss-Newton kernel over several groups per CTA,
+    sampled systems against the oracle: H within 1e-4 of the correlation
+    scale, chi2 and gradient as in the other tests; an invalid system among
+    those set up together."""
+    rng = np.random.default_rng(n_obs + n_sys)
+    par = rows(rng, n_sys, n_pl, (1.0, 3000.0), (0.0, 0.85))
+    par[7, 2] = 1.5
+    t = np.sort(rng.uniform(T0, T0 + span, n_obs))
+    sig = rng.uniform(1.0, 4.0, n_obs)
+    v = rng.normal(0.0, 30.0, n_obs)
+    args = [torch.tensor(x, device="cuda") for x in (par, t, v, sig)]
+    kc.kc_last_device_error()
+    kc.kc_set_tile("gn", "mixed", n_sys, n_pl, n_obs, (32, 128, split))
+    try:
+        chi2, grad, H = [x.cpu().numpy().astype(np.float64)
+                         for x in kc.kc_chi2_gauss_newton(*args, t0=T0)]
+    finally:
+        kc.kc_set_tile("gn", "mixed", n_sys, n_pl, n_obs, None)
+    assert kc.kc_last_device_error() == 1 and np.isnan(chi2[7]) and np.isnan(H[7]).all()
+    idx = np.setdiff1d(np.r_[0:12, rng.choice(n_sys, 60, replace=False), n_sys - 3:n_sys], [7])
+    p = par[idx]
+    ref, gref, gabs = oracle_mod.chi2(p, t, v, sig, n_pl, t0=T0, gabs=True)
+    assert np.all(np.abs(chi2[idx] - ref) <= 1e-5 * np.maximum(ref, 1.0) + chi2_rounding_term(
+        oracle_mod, p, t, v, sig, n_pl, T0, 0.0, U32))
+    ar = uniform_arith(kc, oracle_mod, p, t, v, sig, n_pl, T0, 0.0, "mixed", "gn")
+    assert grad_excess(grad[idx], gref, gabs, 1e-3, U32, ar) <= 1.0
+    n = 5 * n_pl + 1
+    Hr = oracle_mod.unpack_symmetric(oracle_mod.gauss_newton(p, t, sig, n_pl, t0=T0), n)
+    Hg = oracle_mod.unpack_symmetric(H[idx], n)
+    d = np.sqrt(np.diagonal(Hr, axis1=1, axis2=2))
+    assert np.max(np.abs(Hg - Hr) / (d[:, :, None] * d[:, None, :])) <= 1e-4
