@@ -231,9 +231,9 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
   const GradPlanetP *q = pl_s + sl * J;
   Kahan2 acc = {0, 0};
   f32x2 sum_a = 0;
-  GradSums g[J];
+  typename GradSumsFor<J>::type g[J];
 #pragma unroll
-  for (int j = 0; j < J; ++j) g[j] = GradSums{{0, 0}, 0, 0, 0, 0};
+  for (int j = 0; j < J; ++j) g[j] = {{0, 0}, 0, 0, 0, 0};
 
   for (int k0 = 0; k0 < a.n_obs; k0 += obs_tile) {
     const int nk = min(obs_tile, a.n_obs - k0);

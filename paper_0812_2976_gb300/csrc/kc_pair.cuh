@@ -449,6 +449,49 @@ __device__ __forceinline__ void grad_add(GradSums &G, const GradTerms &o, const 
   G.M = fma2(a, Qyy, G.M);
 }
 
+// The same sums with the pair's two halves added one after the other: six
+// registers a planet instead of twelve.  A packed multiply-add of three
+// register pairs reads as many registers as two scalar ones, so it is no
+// faster; from four planets on (where twelve registers a planet spill) the
+// kernels sum this way.
+struct GradSumsS {
+  Kahan P;
+  float K, e, w, M;
+};
+
+__device__ __forceinline__ void add_halves(float &sum, f32x2 a, f32x2 b) {
+  sum = __fmaf_rn(hi2(a), hi2(b), __fmaf_rn(lo2(a), lo2(b), sum));
+}
+
+__device__ __forceinline__ void grad_add(GradSumsS &G, const GradTerms &o, const GradPlanetP &g,
+                                         f32x2 a, f32x2 adt) {
+  const f32x2 Qy = mul2(o.Q, o.y), Qyy = mul2(Qy, o.y);
+  const f32x2 h = fma2(dup2(g.beta), o.y, dup2(g.ibeta));
+  const f32x2 P = mul2(adt, Qyy);
+  kahan_add(G.P, lo2(P));
+  kahan_add(G.P, hi2(P));
+  add_halves(G.K, a, o.dK);
+  add_halves(G.e, mul2(a, Qy), mul2(o.s, h));
+  add_halves(G.w, a, o.Q);
+  add_halves(G.M, a, Qyy);
+}
+
+template <int J>
+struct GradSumsFor {
+  typedef GradSums type;
+};
+#define KC_SCALAR_SUMS(J)   \
+  template <>               \
+  struct GradSumsFor<J> {   \
+    typedef GradSumsS type; \
+  }
+KC_SCALAR_SUMS(4);
+KC_SCALAR_SUMS(5);
+KC_SCALAR_SUMS(6);
+KC_SCALAR_SUMS(7);
+KC_SCALAR_SUMS(8);
+#undef KC_SCALAR_SUMS
+
 // The same planet's row of sqrt(w) J for the Gauss-Newton matrix, each column
 // over its per-planet factor (gn_scale), and its gradient sums from the row
 // with a = 2 sqrt(w) r; swdt = sqrt(w) (t - t0).
@@ -493,6 +536,9 @@ struct GradLane {
 };
 __device__ __forceinline__ GradLane grad_join(const GradSums &G) {
   return GradLane{kahan_join(G.P), join2(G.K), join2(G.e), join2(G.w), join2(G.M)};
+}
+__device__ __forceinline__ GradLane grad_join(const GradSumsS &G) {
+  return GradLane{G.P, G.K, G.e, G.w, G.M};
 }
 __device__ __forceinline__ void grad_combine(GradLane &g, int m) {
   const Kahan o = {shfl_xor(g.P.big, m), shfl_xor(g.P.small, m)};
