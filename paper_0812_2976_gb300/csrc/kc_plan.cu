@@ -49,6 +49,7 @@ struct kc_plan {
   int64_t *d_obs_off = nullptr, *d_par_off = nullptr, *d_order = nullptr;
   int32_t *d_n_pl = nullptr;
   double *d_t_ref = nullptr;
+  int32_t *d_far = nullptr;               // mixed: systems with far times
   void *d_obs_a = nullptr, *d_obs_b = nullptr;
   unsigned long long *d_queue = nullptr;  // kPlanMaxStreams counters
   bool obs_ready = false;
@@ -59,7 +60,7 @@ struct kc_plan {
 
   kc::RaggedDev dev() const {
     return kc::RaggedDev{d_obs_off, d_par_off, d_n_pl, d_order, d_t_ref, n_sys, t0,
-                         kc::invalid_counter(), n_obs, n_par};
+                         kc::invalid_counter(), d_far, n_obs, n_par};
   }
   void drop_graph() {
     for (PlanStream &ps : streams) ps.drop_graph();
@@ -80,7 +81,7 @@ struct kc_plan {
     if (cap_stream) cudaStreamDestroy(cap_stream);
     cap_stream = nullptr;
     for (void *p : {(void *)d_obs_off, (void *)d_par_off, (void *)d_order, (void *)d_n_pl,
-                    (void *)d_t_ref, d_obs_a, d_obs_b, (void *)d_queue})
+                    (void *)d_t_ref, (void *)d_far, d_obs_a, d_obs_b, (void *)d_queue})
       if (p) cudaFree(p);
   }
 };
@@ -226,8 +227,10 @@ kc_status kc_plan_create_ragged(kc_plan **plan, const int64_t *obs_off, const in
   p->n_sys = n_sys;
   p->n_obs = obs_off[n_sys];
   p->n_par = par_off[n_sys];
-  const size_t obs_bytes_a = p->n_obs * (mode == KC_MIXED ? sizeof(float4) : sizeof(kc::ObsR64));
-  const size_t obs_bytes_b = mode == KC_MIXED ? p->n_obs * sizeof(float2) : 0;
+  const size_t pairs = (size_t)kc::ragged_pair(p->n_obs, n_sys) + 1;
+  const size_t obs_bytes_a =
+      mode == KC_MIXED ? pairs * 2 * sizeof(float4) : p->n_obs * sizeof(kc::ObsR64);
+  const size_t obs_bytes_b = mode == KC_MIXED ? pairs * sizeof(float4) : 0;
   cudaError_t e = cudaSuccess;
   auto alloc = [&](void **ptr, size_t bytes) {
     if (e == cudaSuccess) e = cudaMalloc(ptr, bytes > 0 ? bytes : 16);
@@ -237,6 +240,7 @@ kc_status kc_plan_create_ragged(kc_plan **plan, const int64_t *obs_off, const in
   alloc((void **)&p->d_order, sizeof(int64_t) * n_sys);
   alloc((void **)&p->d_n_pl, sizeof(int32_t) * n_sys);
   alloc((void **)&p->d_t_ref, sizeof(double) * n_sys);
+  if (mode == KC_MIXED) alloc((void **)&p->d_far, sizeof(int32_t) * n_sys);
   alloc(&p->d_obs_a, obs_bytes_a);
   alloc(&p->d_obs_b, obs_bytes_b);
   alloc((void **)&p->d_queue, sizeof(unsigned long long) * kPlanMaxStreams);

@@ -16,7 +16,7 @@
 //    for that count;
 //  - the observations, fixed for the plan (Sec. 4.1 treats them as
 //    constants for every model), are converted once per plan to the form the
-//    kernel reads (float pairs for the mixed path).
+//    kernel reads (packed pairs for the mixed path).
 // The per-planet arithmetic is that of the uniform kernels (kc_device.cuh).
 #include <algorithm>
 #include <cmath>
@@ -26,6 +26,7 @@
 #include "kc_device.cuh"
 #include "kc_f64.cuh"
 #include "kc_internal.h"
+#include "kc_pair.cuh"
 #include "kc_ragged.h"
 
 namespace kc {
@@ -59,11 +60,12 @@ __device__ inline double system_gamma_r(const double *p, int J) {
 
 // ------------------------------------------------------------ observation prep
 
-// One warp per system: tau = t - t_ref (t_ref = the system's first
-// observation) and v as float pairs, w = 1/(sigma^2 + jitter^2), t - t0.
+// One warp per system, a lane per pair of observations: tau = t - t_ref (t_ref
+// = the system's first observation) at fixed binary places and v as float
+// pairs, w = 1/(sigma^2 + jitter^2), t - t0.
 __global__ void prep_obs_mixed(RaggedDev d, const double *__restrict__ t,
                                const double *__restrict__ v, const double *__restrict__ sigma,
-                               double jitter2, float4 *__restrict__ oa, float2 *__restrict__ ob,
+                               double jitter2, float4 *__restrict__ oa, float4 *__restrict__ ob,
                                double *__restrict__ t_ref) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -76,17 +78,32 @@ __global__ void prep_obs_mixed(RaggedDev d, const double *__restrict__ t,
     // no FP64 instruction: differences from exact three-float splits
     const Split3 tr3 = split3(tr), te3 = split3(d.t0);
     const float jit2 = d2f(jitter2);
-    for (int64_t k = o0 + lane; k < o1; k += 32) {
-      const Split3 tk = split3(t[k]);
-      float th, tl, vh, vl;
-      sub_ds(tk, tr3, th, tl);
-      split_d(v[k], vh, vl);
-      oa[k] = make_float4(th, tl, vh, vl);
-      const float sg = d2f(sigma[k]);
-      const float var = __fmaf_rn(sg, sg, jit2);
-      ob[k] = make_float2(var > 0.0f ? 1.0f / var : __int_as_float(0x7fc00000),
-                          (tk.x0 - te3.x0) + (tk.x1 - te3.x1));
+    const int64_t pair0 = ragged_pair(o0, s);
+    bool far = false;
+    for (int64_t k = o0 + 2 * lane; k < o1; k += 64) {
+      float th[2], tl[2], vh[2], vl[2], w[2], dt[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        th[i] = tl[i] = vh[i] = vl[i] = w[i] = dt[i] = 0.0f;
+        if (k + i < o1) {
+          const Split3 tk = split3(t[k + i]);
+          sub_ds(tk, tr3, th[i], tl[i]);
+          tau_place(th[i], tl[i]);
+          far |= !(fabsf(th[i]) < kPairMaxTau);
+          split_d(v[k + i], vh[i], vl[i]);
+          const float sg = d2f(sigma[k + i]);
+          const float var = __fmaf_rn(sg, sg, jit2);
+          w[i] = var > 0.0f ? 1.0f / var : __int_as_float(0x7fc00000);
+          dt[i] = (tk.x0 - te3.x0) + (tk.x1 - te3.x1);
+        }
+      }
+      const int64_t p = pair0 + ((k - o0) >> 1);
+      oa[2 * p] = make_float4(th[0], th[1], tl[0], tl[1]);
+      oa[2 * p + 1] = make_float4(vh[0], vh[1], vl[0], vl[1]);
+      ob[p] = make_float4(w[0], w[1], dt[0], dt[1]);
     }
+    const bool any = __any_sync(0xffffffffu, far);
+    if (lane == 0) d.far[s] = any ? 1 : 0;
   }
 }
 
@@ -151,36 +168,10 @@ predict_ragged_kernel(const double *__restrict__ params,
 
 // ------------------------------------------------------------ per-system bodies
 
-struct RPlanetF {
-  PlanetF base;
-  float K, cw, sw, beta, n2, ibeta;   // ibeta = 1/beta
-  StartF m;                           // the e-only constants of Mikkola's start
-};
-
 struct RPlanetD {
   PlanetD base;
   double K, cw, sw, n2, ibeta;
 };
-
-__device__ inline RPlanetF rsetup_mixed(const double *p, double t_ref, double t0, bool grad) {
-  RPlanetF g;
-  g.base = planet_setup_mixed(p, t_ref, t0);
-  g.m = kepler_start_setup(g.base.e);
-  g.K = g.cw = g.sw = g.beta = g.n2 = g.ibeta = 0.0f;
-  if (grad) {
-    float w_hi, w_lo;
-    split_d(p[3], w_hi, w_lo);
-    float sw, cw;
-    sincosf(w_hi, &sw, &cw);
-    g.sw = __fmaf_rn(w_lo, cw, sw);
-    g.cw = __fmaf_rn(-w_lo, sw, cw);
-    g.K = d2f(p[1]);
-    g.beta = sqrtf((1.0f - g.base.e) * (1.0f + g.base.e));
-    g.ibeta = 1.0f / g.beta;
-    g.n2 = g.base.n_hi * g.base.n_hi;
-  }
-  return g;
-}
 
 __device__ inline RPlanetD rsetup_f64(const double *p, double dref, bool grad) {
   RPlanetD g;
@@ -210,93 +201,106 @@ __device__ __forceinline__ void partials_r(T e, T K, T cw, T sw, T beta, T ibeta
   de = K * cw - ks * sE * (ibeta + beta * invD);
 }
 
-template <int J, bool GRAD>
-__device__ __forceinline__ void body_mixed(const RPlanetF *pl, float gam, const float4 *oa,
-                                           const float2 *ob, int64_t o0, int n, int lane,
-                                           float *chi2_out, float *grad_out) {
-  constexpr int NP = 5 * J + 1;
-  Kahan acc = {0.0f, 0.0f};
-  float g[GRAD ? NP : 1];
-  Kahan gP[GRAD ? J : 1];       // compensated d/dP sums (they cancel heavily)
+// The planet constants of a mixed plan: with or without the partials'.
+template <bool GRAD>
+struct RaggedPlanet;
+template <>
+struct RaggedPlanet<true> {
+  typedef GradPlanetP type;
+};
+template <>
+struct RaggedPlanet<false> {
+  typedef PlanetP type;
+};
+
+// One system of J planets and n observations by a warp, a pair of
+// observations per lane at a time (kc_pair.cuh), the next pair loaded while
+// this one is evaluated.
+template <int J, bool GRAD, bool WIDE>
+__device__ __forceinline__ void body_mixed(const typename RaggedPlanet<GRAD>::type *pl, float gam,
+                                           const float *tab, const float4 *oa, const float4 *ob,
+                                           int64_t pair0, int n, int lane, float *chi2_out,
+                                           float *grad_out) {
+  constexpr int JG = GRAD ? J : 1;
+  Kahan2 acc = {0, 0};
+  f32x2 sum_a = 0;
+  typename GradSumsFor<JG>::type g[JG];
 #pragma unroll
-  for (int i = 0; i < (GRAD ? NP : 1); ++i) g[i] = 0.0f;
-#pragma unroll
-  for (int j = 0; j < (GRAD ? J : 1); ++j) gP[j] = Kahan{0.0f, 0.0f};
-  // the next observation is loaded while this one is evaluated
-  float4 o_next = make_float4(0.f, 0.f, 0.f, 0.f);
-  float2 wt_next = make_float2(0.f, 0.f);
-  if (lane < n) {
-    o_next = oa[o0 + lane];
-    wt_next = ob[o0 + lane];
+  for (int j = 0; j < JG; ++j) g[j] = {{0, 0}, 0, 0, 0, 0};
+  const int pairs = (n + 1) >> 1;
+  oa += 2 * pair0;
+  ob += pair0;
+  float4 t_next = make_float4(0.f, 0.f, 0.f, 0.f), v_next = t_next, w_next = t_next;
+  if (lane < pairs) {
+    t_next = oa[2 * lane];
+    v_next = oa[2 * lane + 1];
+    w_next = ob[lane];
   }
-  for (int k = lane; k < n; k += 32) {
-    // Gradient: the planets' constants are read from shared memory again in
-    // every iteration (the empty asm with a memory clobber keeps the
-    // compiler from hoisting them, with the solver's per-planet constants,
-    // into registers for all J planets): no spills at 128 registers, 4 %
-    // faster on the ragged workload.
-    if (GRAD) asm volatile("" ::: "memory");
-    const float4 o = o_next;
-    const float2 wt = wt_next;
-    if (k + 32 < n) {
-      o_next = oa[o0 + k + 32];
-      wt_next = ob[o0 + k + 32];
+  for (int p = lane; p < pairs; p += 32) {
+    // the planets' constants are read from shared memory again in every
+    // iteration instead of being hoisted into registers for all J planets (the
+    // forward kernel spilled 3 KB so: 50000 systems of 16 to 1024 observations
+    // in 287 us against 222)
+    asm volatile("" ::: "memory");
+    const float4 tt = t_next, vv = v_next, ww = w_next;
+    if (p + 32 < pairs) {
+      t_next = oa[2 * (p + 32)];
+      v_next = oa[2 * (p + 32) + 1];
+      w_next = ob[p + 32];
     }
-    float sEj[J], cEj[J];
-    Kahan V = {0.0f, 0.0f};
+    const f32x2 th = pack2(tt.x, tt.y), tl = pack2(tt.z, tt.w);
+    Kahan2 V = {dup2(gam), 0};
+    GradTerms o[JG];
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-      const PlanetF q = pl[j].base;
-      const float M = mean_anomaly_mixed(o.x, o.y, q);
-      kepler_f32_h(M, q.e, pl[j].m, sEj[j], cEj[j]);
-      kahan_add(V, velocity_mixed(q, sEj[j], cEj[j]));
-    }
-    const float r = __fadd_rn(__fsub_rn(V.big, o.z), __fsub_rn(gam, __fadd_rn(V.small, o.w)));
-    const float wr = wt.x * r;
-    kahan_add(acc, wr * r);
-    if (GRAD) {
-      const float a2 = 2.0f * wr;
-#pragma unroll
-      for (int j = 0; j < J; ++j) {
-        const RPlanetF q = pl[j];
-        float dK, dw, dM, de;
-        const float invD = rcp_fast(__fmaf_rn(-q.base.e, cEj[j], 1.0f));
-        partials_r(q.base.e, q.K, q.cw, q.sw, q.beta, q.ibeta, sEj[j], cEj[j], invD, dK, dw,
-                   dM, de);
-        const float dP = dM * (-kTwoPiF * wt.y * q.n2);
-        kahan_add(gP[GRAD ? j : 0], a2 * dP);
-        g[5 * j + 1] = __fmaf_rn(a2, dK, g[5 * j + 1]);
-        g[5 * j + 2] = __fmaf_rn(a2, de, g[5 * j + 2]);
-        g[5 * j + 3] = __fmaf_rn(a2, dw, g[5 * j + 3]);
-        g[5 * j + 4] = __fmaf_rn(a2, dM, g[5 * j + 4]);
+      if constexpr (GRAD) {
+        o[j] = grad_terms<WIDE>(th, tl, pl[j], tab, V);
+      } else {
+        const f32x2 M = mean_anomaly2<WIDE>(th, tl, pl[j]);
+        f32x2 s, c, E;
+        kepler_pair(abs2(M), pl[j], tab, s, c, E);
+        velocity_sum(V, pl[j], signed_as(s, M), c);
       }
-      g[GRAD ? 5 * J : 0] += a2;
+    }
+    const f32x2 r = sub2(sub2(V.big, pack2(vv.x, vv.y)), add2(V.small, pack2(vv.z, vv.w)));
+    const f32x2 wr = mul2(pack2(ww.x, ww.y), r);
+    kahan_add(acc, mul2(wr, r));
+    if constexpr (GRAD) {
+      const f32x2 a2 = add2(wr, wr), adt = mul2(a2, pack2(ww.z, ww.w));
+      sum_a = add2(sum_a, a2);
+#pragma unroll
+      for (int j = 0; j < J; ++j) grad_add(g[j], o[j], pl[j], a2, adt);
     }
   }
+  Kahan chi = kahan_join(acc);
+  float sa = join2(sum_a);
+  GradLane gl[JG];
+#pragma unroll
+  for (int j = 0; j < JG; ++j) gl[j] = grad_join(g[j]);
 #pragma unroll
   for (int m = 16; m >= 1; m >>= 1) {
-    Kahan o = {shfl_xor(acc.big, m), shfl_xor(acc.small, m)};
-    kahan_merge(acc, o);
-    if (GRAD) {
+    const Kahan o = {shfl_xor(chi.big, m), shfl_xor(chi.small, m)};
+    kahan_merge(chi, o);
+    if constexpr (GRAD) {
+      sa += shfl_xor(sa, m);
 #pragma unroll
-      for (int j = 0; j < (GRAD ? J : 1); ++j) {
-        Kahan op = {shfl_xor(gP[j].big, m), shfl_xor(gP[j].small, m)};
-        kahan_merge(gP[j], op);
-      }
-#pragma unroll
-      for (int i = 0; i < (GRAD ? NP : 1); ++i) g[i] += shfl_xor(g[i], m);
+      for (int j = 0; j < JG; ++j) grad_combine(gl[j], m);
     }
   }
-  if (GRAD) {
-#pragma unroll
-    for (int j = 0; j < (GRAD ? J : 1); ++j) g[GRAD ? 5 * j : 0] = kahan_value(gP[j]);
-  }
   if (lane == 0) {
-    const float poison = 0.0f * gam;
-    *chi2_out = kahan_value(acc) + poison;
-    if (GRAD) {
+    float poison = 0.0f * gam;
 #pragma unroll
-      for (int i = 0; i < (GRAD ? NP : 1); ++i) grad_out[i] = g[i] + poison;
+    for (int j = 0; j < J; ++j) {
+      if constexpr (GRAD)
+        poison += 0.0f * pl[j].p.e;
+      else
+        poison += 0.0f * pl[j].e;
+    }
+    *chi2_out = kahan_value(chi) + poison;
+    if constexpr (GRAD) {
+#pragma unroll
+      for (int j = 0; j < JG; ++j) grad_finish(gl[j], pl[j], sa, poison, grad_out + 5 * j);
+      grad_out[5 * J] = sa + poison;
     }
   }
 }
@@ -379,43 +383,100 @@ constexpr int kMaxWarps = 8;   // block <= 256
     default: BODY(8); break;                        \
   }
 
-// Each warp: take the next system from the queue (systems in decreasing
-// order of work), set up its planets (one lane per planet, FP64), evaluate
-// it with 32 lanes over its observations, reduce, write; until the queue is
-// empty.  The queue counter must be zero at launch.
-// Gradient: at most 128 registers, two CTAs of 256 threads per SM; the body
-// then keeps part of its accumulators in local memory, and still runs 1.26x
-// faster than at one CTA per SM (252 registers) on the ragged workload.
-// Forward: at most 80 registers, three CTAs per SM (1.08x over two).
+// Each warp: take the next kAhead systems from the queue (systems in
+// decreasing order of work), set all their planets up at once (lane 8 i + j
+// the planet j of the i-th), evaluate them one after the other with 32 lanes
+// over the observations, reduce, write; until the queue is empty.  The queue
+// counter must be zero at launch.  Taken one at a time, each system would wait
+// for the counter, its descriptors, its parameters and a setup chain of some
+// 500 instructions in J lanes.
+// At most 128 registers, two CTAs of 256 threads per SM.  For the forward
+// kernel three or four (80 or 64 registers) gain up to 6 % on large batches
+// and lose on small ones, where each CTA's table load and the queue count:
+// 50000 systems of 16 to 1024 observations 224 us (two), 222 (three), 210
+// (four); 3000 of them 30, 36, 36; 20000 of 4 to 20 observations 29, 35, 33.
+// Bound by the FP32 pipe's instructions (packed ones take two issue slots) at
+// large sizes.  Measured before, one observation per instruction and a system
+// at a time: forward 50000 systems 310 us, 3000 51, 20000 tiny 31; gradient
+// 50000 systems 439 us (now 322), 200000 1734 (now 1185).
+constexpr int kAhead = 4;
+static_assert(kAhead * KC_MAX_PLANETS == 32, "a lane per planet of the systems taken");
+
 template <bool GRAD>
-__global__ void __launch_bounds__(256, GRAD ? 2 : 3)
-ragged_mixed_kernel(RaggedDev d, const float4 *__restrict__ oa, const float2 *__restrict__ ob,
+__global__ void __launch_bounds__(256, 2)
+ragged_mixed_kernel(RaggedDev d, const float4 *__restrict__ oa, const float4 *__restrict__ ob,
                     const double *__restrict__ params, float *__restrict__ chi2,
                     float *__restrict__ grad, unsigned long long *__restrict__ queue) {
-  __shared__ RPlanetF pl_s[kMaxWarps][KC_MAX_PLANETS];
+  typedef typename RaggedPlanet<GRAD>::type Planet;
+  __shared__ AngTab tab_s;
+  __shared__ Planet pl_s[kMaxWarps][kAhead * KC_MAX_PLANETS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  RPlanetF *pl = pl_s[warp];
+  ang_tab_load(tab_s.s, threadIdx.x, blockDim.x);
+  __syncthreads();
+  const int mine = lane / KC_MAX_PLANETS, mine_j = lane % KC_MAX_PLANETS;
+  // fewer at a time where the queue holds few per warp (300 systems taken four
+  // at a time ran 40 us against 17)
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int take = (int)max((int64_t)1, min((int64_t)kAhead, d.n_sys / (4 * warps)));
   for (;;) {
     unsigned long long idx = 0;
-    if (lane == 0) idx = atomicAdd(queue, 1ull);
+    if (lane == 0) idx = atomicAdd(queue, (unsigned long long)take);
     idx = __shfl_sync(0xffffffffu, idx, 0);
     if (idx >= (unsigned long long)d.n_sys) break;
-    const int64_t s = d.order[idx];
-    if (!dbg_ok(d.invalid, 0 <= s && s < d.n_sys, kDbgOrder, (int64_t)idx)) continue;
-    const int J = d.n_pl[s];
-    const int64_t o0 = d.obs_off[s];
-    if (!ragged_system_ok(d, s, J, o0, d.obs_off[s + 1])) continue;
-    const int n = (int)(d.obs_off[s + 1] - o0);
-    const double *p = params + d.par_off[s];
-    if (lane < J) pl[lane] = rsetup_mixed(p + 5 * lane, d.t_ref[s], d.t0, GRAD);
-    const float gam = d2f(system_gamma_r(p, J));
+    // this lane's system of the ones taken (J = 0: none), and its planet
+    int64_t s = -1, o0 = 0, p0 = 0;
+    int J = 0, n = 0;
+    float gam = 0.0f;
+    bool far = false;
+    if (mine < take && idx + mine < (unsigned long long)d.n_sys) {
+      s = d.order[idx + mine];
+      if (dbg_ok(d.invalid, 0 <= s && s < d.n_sys, kDbgOrder, (int64_t)(idx + mine))) {
+        J = d.n_pl[s];
+        o0 = d.obs_off[s];
+        const int64_t o1 = d.obs_off[s + 1];
+        p0 = d.par_off[s];
+        n = (int)(o1 - o0);
+        if (!ragged_system_ok(d, s, J, o0, o1)) J = 0;
+      }
+    }
+    __syncwarp();                                // the last systems' use of the planets
+    if (mine_j < J) {
+      const double *p = params + p0 + 5 * mine_j;
+      if constexpr (GRAD)
+        pl_s[warp][lane] = grad_setup_pair(p, d.t_ref[s], d.t0, far);
+      else
+        pl_s[warp][lane] = planet_setup_pair(p, d.t_ref[s], d.t0, far);
+      if (mine_j == 0) {
+        const double gd = params[p0 + 5 * J];
+        gam = finite_bits(gd) ? d2f(gd) : __int_as_float(0x7fc00000);
+        far |= d.far[s] != 0;
+      }
+    }
+    const unsigned wide = __ballot_sync(0xffffffffu, far);
     __syncwarp();
-    float *gout = GRAD ? grad + d.par_off[s] : nullptr;
-#define KC_BODY(JJ) body_mixed<JJ, GRAD>(pl, gam, oa, ob, o0, n, lane, chi2 + s, gout)
-    KC_RAGGED_SWITCH(KC_BODY)
+    for (int i = 0; i < take; ++i) {
+      const int from = i * KC_MAX_PLANETS;
+      const int Ji = __shfl_sync(0xffffffffu, J, from);
+      if (Ji == 0) continue;
+      const int64_t si = __shfl_sync(0xffffffffu, s, from);
+      const int64_t oi = __shfl_sync(0xffffffffu, o0, from);
+      const int64_t pi = __shfl_sync(0xffffffffu, p0, from);
+      const int ni = __shfl_sync(0xffffffffu, n, from);
+      const float gi = __shfl_sync(0xffffffffu, gam, from);
+      const Planet *pl = pl_s[warp] + from;
+      const bool wi = ((wide >> from) & 0xffu) != 0u;
+      float *gout = GRAD ? grad + pi : nullptr;
+      const int64_t pair0 = ragged_pair(oi, si);
+      const int J = Ji;
+#define KC_BODY(JJ)                                                                          \
+  if (wi)                                                                                    \
+    body_mixed<JJ, GRAD, true>(pl, gi, tab_s.s, oa, ob, pair0, ni, lane, chi2 + si, gout);   \
+  else                                                                                       \
+    body_mixed<JJ, GRAD, false>(pl, gi, tab_s.s, oa, ob, pair0, ni, lane, chi2 + si, gout)
+      KC_RAGGED_SWITCH(KC_BODY)
 #undef KC_BODY
-    if (lane == 0) note_invalid(d.invalid, chi2[s]);      // lane 0 wrote it
-    __syncwarp();
+      if (lane == 0) note_invalid(d.invalid, chi2[si]);      // lane 0 wrote it
+    }
   }
 }
 
@@ -470,7 +531,7 @@ cudaError_t ragged_prep(const RaggedDev &d, int mode, const double *t, const dou
   if (blocks < 1) blocks = 1;
   if (mode == KC_MIXED)
     prep_obs_mixed<<<(int)blocks, 256, 0, st>>>(d, t, v, sigma, jitter2, (float4 *)obs_a,
-                                                (float2 *)obs_b, t_ref);
+                                                (float4 *)obs_b, t_ref);
   else
     prep_obs_f64<<<(int)blocks, 256, 0, st>>>(d, t, v, sigma, jitter2, (ObsR64 *)obs_a, t_ref);
   return cudaGetLastError();
@@ -504,11 +565,11 @@ cudaError_t ragged_launch(const RaggedDev &d, int mode, bool grad, const void *o
   if (mode == KC_MIXED) {
     if (grad)
       ragged_mixed_kernel<true><<<grid, block, 0, st>>>(d, (const float4 *)obs_a,
-                                                        (const float2 *)obs_b, params,
+                                                        (const float4 *)obs_b, params,
                                                         (float *)chi2, (float *)gradp, queue);
     else
       ragged_mixed_kernel<false><<<grid, block, 0, st>>>(d, (const float4 *)obs_a,
-                                                         (const float2 *)obs_b, params,
+                                                         (const float4 *)obs_b, params,
                                                          (float *)chi2, (float *)gradp, queue);
   } else {
     if (grad)

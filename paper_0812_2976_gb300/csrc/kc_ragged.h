@@ -26,13 +26,24 @@ struct RaggedDev {
   int64_t n_sys;
   double t0;
   unsigned long long *invalid;   // NaN-result counter (kc_last_device_error) or NULL
+  // mixed: nonzero where a time of the system asks for the wide mean anomaly
+  int32_t *far;
   int64_t n_obs_total;           // observations of the plan (obs_off[n_sys])
   int64_t n_par_total;           // packed parameters of the plan (par_off[n_sys])
 };
 
+// The mixed path keeps a system's observations as pairs for the packed
+// evaluation: pair p of system s at ragged_pair(obs_off[s], s) + p, the last
+// one of an odd count completed with zero weight.  The offsets need no array:
+// from one system to the next they grow by at least the pairs it has.
+__host__ __device__ inline int64_t ragged_pair(int64_t obs_off, int64_t s) {
+  return (obs_off + s) >> 1;
+}
+
 // Converts t, v, sigma (device, [obs_off[n_sys]]) to the kernel's form:
-// mixed: obs_a float4 (tau_hi, tau_lo, v_hi, v_lo), obs_b float2 (w, t - t0);
-// fp64: obs_a ObsR64, obs_b unused.  Fills t_ref.
+// mixed, per pair: obs_a two float4 (th, th', tl, tl') and (v_hi, v_hi', v_lo,
+// v_lo'), obs_b one float4 (w, w', t - t0, t' - t0); fp64: obs_a ObsR64, obs_b
+// unused.  Fills t_ref and, mixed, far.
 cudaError_t ragged_prep(const RaggedDev &d, int mode, const double *t, const double *v,
                         const double *sigma, double jitter2, void *obs_a, void *obs_b,
                         double *t_ref, cudaStream_t st);
