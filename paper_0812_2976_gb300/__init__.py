@@ -47,7 +47,9 @@ def _ptr(x: Optional[torch.Tensor]) -> Optional[int]:
 
 def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the raw handle: 0.4 us of host time a call, where building the Stream
+        # object of torch.cuda.current_stream() takes 3 to 4
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if isinstance(stream, torch.cuda.Stream) else int(stream)
 
 
@@ -58,7 +60,7 @@ def _dev_f64(name: str, x: torch.Tensor, dim: int) -> torch.Tensor:
         raise TypeError(f"{name} must be float64")
     if x.dim() != dim:
         raise ValueError(f"{name} must be {dim}-D")
-    return x.contiguous()
+    return x if x.is_contiguous() else x.contiguous()
 
 
 def _out_f32(name: str, x, n: int, device) -> None:
@@ -689,7 +691,9 @@ class _Chi2Fn(torch.autograd.Function):
     @staticmethod
     def backward(ctx, grad_chi2):
         (grad,) = ctx.saved_tensors
-        g = grad.to(torch.float64) * grad_chi2.to(torch.float64)[:, None]
+        # the float64 product widens a float32 gradient itself: the same bits
+        # as a converted copy, one launch and 9 us of host time less
+        g = grad * grad_chi2.to(torch.float64)[:, None]
         return g, None, None, None, None, None, None
 
 
@@ -705,7 +709,7 @@ class _NllFn(torch.autograd.Function):
     @staticmethod
     def backward(ctx, grad_out):
         (grad,) = ctx.saved_tensors
-        return (grad.to(torch.float64) * grad_out.to(torch.float64)[:, None],
+        return (grad * grad_out.to(torch.float64)[:, None],        # as _Chi2Fn's
                 None, None, None, None, None)
 
 

@@ -91,6 +91,8 @@ class KcError(RuntimeError):
 def load() -> ctypes.CDLL:
     """Load libkc.so; raises if it has not been built."""
     global _lib
+    if _lib is not None:          # set once, complete, under the lock
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

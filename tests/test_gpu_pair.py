@@ -165,3 +165,26 @@ def test_gauss_newton_persistent(kc, oracle_mod, split, n_pl, n_obs, n_sys, span
     Hg = oracle_mod.unpack_symmetric(H[idx], n)
     d = np.sqrt(np.diagonal(Hr, axis1=1, axis2=2))
     assert np.max(np.abs(Hg - Hr) / (d[:, :, None] * d[:, None, :])) <= 1e-4
+
+
+@pytest.mark.parametrize("mode", ["mixed", "fp64"])
+def test_backward_is_the_widened_product(kc, mode):
+    """backward scales the kernel's gradient in float64: the bits of widening
+    both factors first, under a strided incoming gradient, and differentiable
+    by it."""
+    rng = np.random.default_rng(5)
+    par = torch.tensor(rows(rng, 33, 2, (2.0, 900.0), (0.0, 0.9)), device="cuda")
+    t = torch.tensor(np.sort(rng.uniform(T0, T0 + 3000.0, 70)), device="cuda")
+    v, sig = torch.zeros_like(t), torch.ones_like(t)
+    p = par.clone().requires_grad_()
+    value = kc.chi2(p, t, v, sig, t0=T0, mode=mode)
+    g = torch.tensor(rng.standard_normal((33, 2)), device="cuda").to(value.dtype)[:, 0]
+    g.requires_grad_()
+    got, = torch.autograd.grad(value, p, g, create_graph=True)
+    _, ref = kc._grad_call("kc_chi2_grad_scalar", par, t, v, sig, T0, 0.0, mode)
+    assert got.dtype == torch.float64
+    assert torch.equal(got, ref.double() * g.detach().double()[:, None])
+    by_g, = torch.autograd.grad(got.sum(), g)
+    want = ref.double().sum(dim=1)
+    assert torch.allclose(by_g.double(), want, rtol=1e-5 if mode == "mixed" else 1e-12,
+                          atol=1e-6 * float(want.abs().max()))
