@@ -374,6 +374,82 @@ __device__ __forceinline__ EvalX solve_x(double tau, float tf, const PlanetX &p)
   return o;
 }
 
+// E of one (M, e) in double, for |M| in [2^-30, 1.02 pi] and 0 <= e <=
+// kEccFast: solve_x's way with M itself and e of every evaluation, and with
+// small E to full relative precision: of sin Ef = S + C b + q, b = Ef - a, the
+// table's doubles take the first two terms, only q (below 2e-6 S and 5e-7 C b)
+// is a float pair.  Five FP64 instructions, where an FP64 Halley step from
+// the single-precision solution took some 16.
+__device__ __forceinline__ double kepler_x(double M, double e) {
+  const unsigned sign = (unsigned)__double2hiint(M) & 0x80000000u;
+  M = xor_sign(M, sign);
+  float eh, el;
+  split_d(e, eh, el);
+  const StartP st = start_constants_fast(eh);
+  const float m = d2f_cut(M), sb = m * st.bs;
+  const float r = start_root(sb, __fmaf_rn(sb, sb, 1.0f)), x = r * r;
+  float pq = __fmaf_rn(x, st.q[4], st.q[3]);
+  pq = __fmaf_rn(x, pq, st.q[2]);
+  pq = __fmaf_rn(x, pq, st.q[1]);
+  pq = __fmaf_rn(x, pq, st.q[0]);
+  const float E0 = __fmaf_rn(r, pq, m);
+  const float kf = __fadd_rn(E0, kF64Round), a = __fsub_rn(kf, kF64Round);
+  const unsigned i = min(__float_as_uint(kf) - __float_as_uint(kF64Round), (unsigned)(kF64TabN - 1));
+  const float4 tf = *reinterpret_cast<const float4 *>(kF64Tab.f[i]);
+  const double2 td = *reinterpret_cast<const double2 *>(kF64Tab.sc[i]);
+  const FF S = {tf.x, tf.y}, C = {tf.z, tf.w};
+  float b = __fsub_rn(E0, a);
+  float Ef;
+  {
+    const float h = -0.5f * b;
+    const float s0 = __fmaf_rn(b, __fmaf_rn(h, S.h, C.h), S.h);
+    const float c0 = __fmaf_rn(b, __fmaf_rn(h, C.h, -S.h), C.h);
+    const float f = __fmaf_rn(-eh, s0, __fsub_rn(E0, m));
+    Ef = __fsub_rn(E0, f * rcp_fast(__fmaf_rn(-eh, c0, 1.0f)));
+  }
+  b = __fsub_rn(Ef, a);
+  // cos b - 1 = m2 and sin b - b = t3 as pairs
+  float b2, b2e, b3, b3e;
+  two_prod(b, b, b2, b2e);
+  FF m2, t3, q;
+  m2.h = -0.5f * b2;
+  m2.l = __fmaf_rn(b2e, -0.5f, b2 * b2 * (1.0f / 24.0f));
+  two_prod(b, b2, b3, b3e);
+  constexpr float kSixth = -1.0f / 6.0f, kSixthLo = (float)(-1.0 / 6.0 - (double)kSixth);
+  two_prod(b3, kSixth, t3.h, t3.l);
+  t3.l = __fmaf_rn(b3, kSixthLo, t3.l);
+  t3.l = __fmaf_rn(__fmaf_rn(b, b2e, b3e), kSixth, t3.l);
+  t3.l = __fmaf_rn(b3 * b2, 1.0f / 120.0f, t3.l);
+  {
+    float w, we, y, ye, err;
+    two_prod(S.h, m2.h, w, we);
+    two_prod(C.h, t3.h, y, ye);
+    two_sum(w, y, q.h, err);
+    float t = __fmaf_rn(S.h, m2.l, we) + ye;
+    t = __fmaf_rn(S.l, m2.h, t);
+    t = __fmaf_rn(C.h, t3.l, t);
+    t = __fmaf_rn(C.l, t3.h, t);
+    fast_two_sum(q.h, t + err, q.h, q.l);
+  }
+  // f(Ef) = (Ef - M) - e S - e (C b + q), as a pair
+  const double R = fma(td.y, f2d_cut(b), pair_d(q.h, q.l));
+  float fh, fl;
+  split_cut(fma(-e, R, fma(-e, td.x, f2d_cut(Ef) - M)), fh, fl);
+  // E = Ef - d, d = f/f' + (f''/2f') d^2
+  float dc, dce, z, ze, err;
+  two_prod(S.h, -b, z, ze);
+  two_sum(z, __fmaf_rn(C.h, m2.h, -S.h * t3.h), dc, dce);
+  FF c1;
+  const FF D = one_minus_e(eh, el, C, FF{dc, dce + ze}, c1);
+  const float ri = rcp_fast(D.h), d0 = fh * ri;
+  float rem = __fmaf_rn(-d0, D.h, fh);
+  rem = __fmaf_rn(-d0, D.l, rem + fl);
+  rem = __fmaf_rn(eh * __fmaf_rn(C.h, b, S.h), 0.5f * d0 * d0, rem);
+  float h, l;
+  two_sum(-d0, -(rem * ri), h, l);
+  return xor_sign(f2d_cut(Ef) + pair_d(h, l), sign);
+}
+
 // V + (vh, vl) += v, v = (A cos E - B sin E)/D: the part at the table's angle
 // on the FP64 pipe, the difference in float pairs.
 __device__ __forceinline__ void velocity_x(const EvalX &o, const PlanetX &p, double &V, float &vh,

@@ -180,12 +180,10 @@ struct StartP {
   float bs, q[5];
 };
 
-__device__ __forceinline__ StartP start_constants(float e) {
+// a = (1 - e)/(4 e + 1/2), sa = sqrt(a) and bs are given.
+__device__ __forceinline__ StartP start_from(float e, float a, float sa, float bs) {
   StartP p;
-  const float r = 1.0f / __fmaf_rn(4.0f, e, 0.5f);
-  const float a = fmaxf((1.0f - e) * r, 1e-8f);      // e rounded up to 1: finite
-  const float sa = sqrtf(a);
-  p.bs = 0.5f * r / (a * sa);
+  p.bs = bs;
   float f = e * sa;
   p.q[0] = 3.0f * f;
   f *= a;
@@ -197,6 +195,20 @@ __device__ __forceinline__ StartP start_constants(float e) {
   f *= a;
   p.q[4] = f * start_fit(e, -0.8390f, 3.4927f, -4.6815f, 2.2459f);
   return p;
+}
+
+__device__ __forceinline__ StartP start_constants(float e) {
+  const float r = 1.0f / __fmaf_rn(4.0f, e, 0.5f);
+  const float a = fmaxf((1.0f - e) * r, 1e-8f);      // e rounded up to 1: finite
+  const float sa = sqrtf(a);
+  return start_from(e, a, sa, 0.5f * r / (a * sa));
+}
+
+// The same for one evaluation (every (M, e) of the Kepler-only solver has its
+// own e): approximate reciprocals; e up to kEccFast.
+__device__ __forceinline__ StartP start_constants_fast(float e) {
+  const float r = rcp_fast(__fmaf_rn(4.0f, e, 0.5f)), a = (1.0f - e) * r, is = rsqrt_fast(a);
+  return start_from(e, a, a * is, 0.5f * r * (is * is * is));
 }
 
 // Phase: n = 1/P rounded; nq its multiple of 2^-17 (n itself above 2^6,
