@@ -555,7 +555,7 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
           } else {
             const EvalX x = solve_x(o.tau, o.tf, p);
             if (want_resid) rmax = fmax(rmax, resid_x(x, p));
-            velocity_x(x, p, r, vh, vl);
+            velocity_x<false>(x, p, r, vh, vl);
           }
         }
         if (!HI) r = add_pair(r, vh, vl);
@@ -607,7 +607,8 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
 // observations of each of the CTA's systems per CTA.  Bound by the FP64 pipe
 // like chi2 (kc_f64.cuh); the planets are set up once per CTA, where one
 // thread per (system, observation) had repeated the setup at every
-// evaluation (512 x 3 x 1000: 305 us, now 38).
+// evaluation (512 x 3 x 1000: 305 us, now 44; 32 without 1/D's correction in
+// FP64, which takes the error from 2.2e-15 to 4e-16 of the velocities' rms).
 constexpr int kPredictBlock = 128;
 constexpr int kPredictMinG = 8;
 
