@@ -184,7 +184,7 @@ __device__ __forceinline__ void warp_tile_sum(const float *th_s, int tile, const
         const f32x2 M = mean_anomaly2<WIDE>(th[i], tl[i], qj);
         const f32x2 m = abs2(M);
         f32x2 s, cE, E;
-        kepler_pair(m, qj, tab, s, cE, E);
+        kepler_pair<false>(m, qj, tab, s, cE, E);
         if (RESID) {
           const f32x2 r = fma2(dup2(-qj.e), s, sub2(E, m));
           const int k = base + (i << (lg + 1));
@@ -248,7 +248,7 @@ chi2_mixed_warp_kernel(UniformArgs a, int lg, int tile, int ntiles, float *__res
   double t0v = 0.0, v0v = 0.0, s0v = 1.0, t1v = 0.0, v1v = 0.0, s1v = 1.0;
   if (has0) { t0v = a.t[ob]; v0v = a.v[ob]; s0v = a.sigma[ob]; }
   if (has1) { t1v = a.t[ob + block]; v1v = a.v[ob + block]; s1v = a.sigma[ob + block]; }
-  ang_tab_load(tab_s, tid, block);
+  ang_tab_load<false>(tab_s, tid, block);
 
   // the reference time's split, needed by the threads that stage
   Split3 tr3 = {0.0f, 0.0f, 0.0f};

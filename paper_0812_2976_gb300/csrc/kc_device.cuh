@@ -797,14 +797,6 @@ __device__ __forceinline__ float velocity_mixed(const PlanetF &q, float sE, floa
   return __fmaf_rn(num, rcp_fast(D), q.C);
 }
 
-// The same velocity with the e cos w term folded: A e = K cos w e = C, so
-// A (cos E - e) - B sin E = A cos E - (B sin E + C), two FMAs.
-__device__ __forceinline__ float velocity_h(const PlanetF &q, float sE, float cE) {
-  const float D = __fmaf_rn(-q.e, cE, 1.0f);
-  const float num = __fmaf_rn(q.A, cE, -__fmaf_rn(q.B, sE, q.C));
-  return __fmaf_rn(num, rcp_fast(D), q.C);
-}
-
 // V + v for one planet (the planet sum's addition inside the last FMA).
 __device__ __forceinline__ double velocity_add_f64(const PlanetD &q, double sE, double cE,
                                                    double V) {

@@ -207,7 +207,7 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
   const Split3 tr3 = split3(t_ref), te3 = split3(a.t0);
   const float dref_f = (tr3.x0 - te3.x0) + (tr3.x1 - te3.x1);     // t_ref - t0, float
   const float jit2 = d2f(a.jitter2);
-  ang_tab_load(tab_s, tid, block);
+  ang_tab_load<true>(tab_s, tid, block);
 
   bool wide = false;
   for (int i = tid; i < ST * J; i += block) {
@@ -1069,7 +1069,7 @@ gn_pair_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__ 
   const float dref_f = (tr3.x0 - te3.x0) + (tr3.x1 - te3.x1);     // t_ref - t0
   const float jit2 = d2f(a.jitter2);
 
-  ang_tab_load(tab_s, tid, block);
+  ang_tab_load<true>(tab_s, tid, block);
   for (int i = tid; i < kGnWarps * kGnRows * ROW2; i += block)
     u_all[i] = make_float2(0.0f, 0.0f);                           // incl. padding
   // observations that fit one tile are staged once for all of the CTA's systems
@@ -1309,7 +1309,7 @@ gn_mixed_tc_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restric
   const Split3 tr3 = split3(t_ref), te3 = split3(a.t0);
   const float dref_f = (tr3.x0 - te3.x0) + (tr3.x1 - te3.x1);     // t_ref - t0
   const float jit2 = d2f(a.jitter2);
-  ang_tab_load(tab_s, tid, kThreads);
+  ang_tab_load<true>(tab_s, tid, kThreads);
   // observations that fit one tile are staged once for all of the CTA's systems
   const bool staged_once = a.n_obs <= kTcObsTile;
   bool far = false;

@@ -125,19 +125,24 @@ constexpr double ang_series(double x, bool cosine) {
   }
   return sum;
 }
-constexpr AngTab make_ang_tab() {
+// vers: 1 - cos in place of cos (= 2 sin^2 of half the angle).
+constexpr AngTab make_ang_tab(bool vers) {
   AngTab t{};
   for (int k = 0; k < kAngTabN; ++k) {
+    const double h = ang_series(k / 512.0, false);
     t.s[k] = (float)ang_series(k / 256.0, false);
-    t.c[k] = (float)ang_series(k / 256.0, true);
+    t.c[k] = vers ? (float)(2.0 * h * h) : (float)ang_series(k / 256.0, true);
   }
   return t;
 }
-static __device__ const __align__(16) AngTab kAngTab = make_ang_tab();
+static __device__ const __align__(16) AngTab kAngTab = make_ang_tab(false);
+static __device__ const __align__(16) AngTab kAngTabV = make_ang_tab(true);
 
 // The CTA's copy in shared memory (16-byte copies; a barrier must follow).
+// VERS: the form kepler_pair<true> takes.
+template <bool VERS>
 __device__ __forceinline__ void ang_tab_load(float *tab, int tid, int nthreads) {
-  const float4 *src = reinterpret_cast<const float4 *>(&kAngTab);
+  const float4 *src = reinterpret_cast<const float4 *>(VERS ? &kAngTabV : &kAngTab);
   for (int i = tid; i < kAngTabN / 2; i += nthreads) reinterpret_cast<float4 *>(tab)[i] = src[i];
 }
 
@@ -220,7 +225,7 @@ struct __align__(16) PlanetP {
   float n, nq, c, nlo2pi;
   float clo2pi, n2pi, e;
   StartP st;
-  float A, B, pad;
+  float A, B, ome;           // ome = 1 - e (gradient only)
 };
 
 // What planet_setup_pair derives besides the phase and the start: sin and cos
@@ -264,7 +269,7 @@ __device__ __forceinline__ PlanetP planet_setup_orbit(const double *p, double t_
   o.cw = __fmaf_rn(-w_lo, sw, cw);
   o.b2 = __fmaf_rn(-ef, ef, 1.0f);
   o.b = sqrtf(o.b2);
-  q.pad = 0.0f;
+  q.ome = 0.0f;
   return q;
 }
 
@@ -283,7 +288,7 @@ __device__ __forceinline__ PlanetP planet_setup_pair(const double *p, double t_r
 // of the partials (grad_terms).
 struct __align__(16) GradPlanetP {
   PlanetP p;
-  float K, C, sw, esw, cw, beta, ibeta, n2;      // C = beta cos w, esw = e sin w, n2 = 1/P^2
+  float K, C, sw, esw, cw, beta, ibeta, swo;     // C = beta cos w, esw = e sin w, swo = (1 - e) sin w
 };
 
 __device__ __forceinline__ GradPlanetP grad_setup_pair(const double *p, double t_ref, double t0,
@@ -291,6 +296,11 @@ __device__ __forceinline__ GradPlanetP grad_setup_pair(const double *p, double t
   GradPlanetP g;
   OrbitF o;
   g.p = planet_setup_orbit(p, t_ref, t0, wide, o);
+  float e_hi, e_lo;
+  split_d(p[2], e_hi, e_lo);
+  g.p.ome = __fsub_rn(__fsub_rn(1.0f, e_hi), e_lo);
+  o.b2 = g.p.ome * (1.0f + g.p.e);
+  o.b = sqrtf(o.b2);
   g.p.A = o.cw * o.b2;
   g.p.B = o.sw * o.b;
   g.K = d2f(p[1]);
@@ -298,9 +308,9 @@ __device__ __forceinline__ GradPlanetP grad_setup_pair(const double *p, double t
   g.sw = o.sw;
   g.cw = o.cw;
   g.esw = g.p.e * o.sw;
+  g.swo = o.sw * g.p.ome;
   g.beta = o.b;
   g.ibeta = 1.0f / o.b;
-  g.n2 = g.p.n * g.p.n;
   return g;
 }
 
@@ -367,6 +377,14 @@ __device__ __forceinline__ unsigned ang_index(float k) {
 // |M| (s, without M's sign), cos E (c) and, for a residual, E.
 // The table's angle a = E0 rounded to 2^-8 is exact in float, and so is b =
 // E0 - a, |b| <= 2^-9: sin b = b and cos b = 1 - b^2/2 to 1.3e-9.
+// VERS: from the table of 1 - cos, c is 1 - cos E and D = (1 - e) + e (1 - cos
+// E), to full relative precision where e is high and E small: the partials take
+// 1/D squared, and cos E rounded near 1 cost them up to 4e-6 there (ragged batches
+// whose gradient norm one such system dominates: 1.6e-6 off, now 5.7e-7; the
+// scalar form 4.6e-7; the geometric mean over 90 batches 0.81 of the scalar
+// form's error).  Two packed additions more: 65536 x 3 x 512 260 us both, 20000 x
+// 6 x 256 90 -> 94.
+template <bool VERS>
 __device__ __forceinline__ void kepler_pair(f32x2 m, const PlanetP &q, const float *tab, f32x2 &s,
                                             f32x2 &c, f32x2 &E) {
   const f32x2 b = mul2(m, dup2(q.st.bs));
@@ -382,18 +400,28 @@ __device__ __forceinline__ void kepler_pair(f32x2 m, const PlanetP &q, const flo
   const f32x2 k = add2(E0, dup2(kAngRound));
   const f32x2 d0 = sub2(E0, sub2(k, dup2(kAngRound)));
   const unsigned i0 = ang_index(lo2(k)), i1 = ang_index(hi2(k));
-  const f32x2 S = pack2(tab[i0], tab[i1]), C = pack2(tab[kAngTabN + i0], tab[kAngTabN + i1]);
+  const f32x2 S = pack2(tab[i0], tab[i1]), T = pack2(tab[kAngTabN + i0], tab[kAngTabN + i1]);
+  const f32x2 C = VERS ? sub2(dup2(1.0f), T) : T;
   const f32x2 h0 = mul2(d0, dup2(-0.5f));
   const f32x2 s0 = fma2(d0, fma2(h0, S, C), S);
-  const f32x2 c0 = fma2(d0, fma2(h0, C, neg2(S)), C);
   // Newton: d = (E0 - e sin E0 - m)/(1 - e cos E0), E = E0 - d
   const f32x2 ne = dup2(-q.e);
   const f32x2 f = fma2(ne, s0, sub2(E0, m));
-  const f32x2 d = mul2(f, rcp2(fma2(ne, c0, dup2(1.0f))));
-  const f32x2 h = mul2(d, dup2(-0.5f));
-  s = fma2(d, neg2(fma2(neg2(h), s0, c0)), s0);
-  c = fma2(d, fma2(h, c0, s0), c0);
-  E = sub2(E0, d);
+  if constexpr (VERS) {
+    const f32x2 v0 = fma2(d0, fma2(neg2(h0), C, S), T), c0 = sub2(dup2(1.0f), v0);
+    const f32x2 d = mul2(f, rcp2(fma2(dup2(q.e), v0, dup2(q.ome))));
+    const f32x2 h = mul2(d, dup2(-0.5f));
+    s = fma2(d, neg2(fma2(neg2(h), s0, c0)), s0);
+    c = fma2(d, neg2(fma2(h, c0, s0)), v0);
+    E = sub2(E0, d);
+  } else {
+    const f32x2 c0 = fma2(d0, fma2(h0, C, neg2(S)), C);
+    const f32x2 d = mul2(f, rcp2(fma2(ne, c0, dup2(1.0f))));
+    const f32x2 h = mul2(d, dup2(-0.5f));
+    s = fma2(d, neg2(fma2(neg2(h), s0, c0)), s0);
+    c = fma2(d, fma2(h, c0, s0), c0);
+    E = sub2(E0, d);
+  }
 }
 
 // x with M's sign (x's own kept: an exclusive or).
@@ -428,11 +456,11 @@ __device__ __forceinline__ GradTerms grad_terms(f32x2 th, f32x2 tl, const GradPl
   GradTerms o;
   const f32x2 M = mean_anomaly2<WIDE>(th, tl, g.p);
   f32x2 s, c, E;
-  kepler_pair(abs2(M), g.p, tab, s, c, E);
+  kepler_pair<true>(abs2(M), g.p, tab, s, c, E);      // c = 1 - cos E
   o.s = signed_as(s, M);
-  o.y = rcp2(fma2(dup2(-g.p.e), c, dup2(1.0f)));
-  o.dK = mul2(fma2(dup2(g.p.A), c, neg2(mul2(dup2(g.p.B), o.s))), o.y);
-  o.Q = mul2(fma2(dup2(g.C), o.s, fma2(dup2(g.sw), c, dup2(-g.esw))), o.y);
+  o.y = rcp2(fma2(dup2(g.p.e), c, dup2(g.p.ome)));
+  o.dK = mul2(fma2(dup2(-g.p.A), c, fma2(dup2(-g.p.B), o.s, dup2(g.p.A))), o.y);
+  o.Q = mul2(fma2(dup2(g.C), o.s, fma2(dup2(-g.sw), c, dup2(g.swo))), o.y);
   kahan_add_y(V, fma2(dup2(g.K), o.dK, neg2(V.small)));
   return o;
 }
@@ -440,7 +468,7 @@ __device__ __forceinline__ GradTerms grad_terms(f32x2 th, f32x2 tl, const GradPl
 // Sums over the observations, a = 2 w r: of a dt Q y^2 (compensated: the
 // period's terms cancel heavily), a dK, a Q y sin E (1/beta + beta y), a Q, a
 // Q y^2.  The partials by (P, K, e, w, M0) are
-//   2 pi n2 K beta dt Q y^2,  dK,  K cos w - K Q y sin E (1/beta + beta y),
+//   2 pi n^2 K beta dt Q y^2,  dK,  K cos w - K Q y sin E (1/beta + beta y),
 //   -K (Q + e sin w),  -K beta Q y^2,
 // so their factors, and the parts a alone multiplies, are applied once per
 // system (grad_finish): 17 packed operations per pair and planet for all five
@@ -531,7 +559,7 @@ __device__ __forceinline__ float gn_scale(const GradPlanetP *q, int J, int p) {
   const GradPlanetP &g = q[j];
   const float Kb = g.K * g.beta;
   switch (i) {
-    case 0: return Kb * (kTwoPiF * g.n2);
+    case 0: return Kb * (kTwoPiF * (g.p.n * g.p.n));
     case 1: return 1.0f;
     case 2: return g.K;
     case 3: return -g.K;
@@ -564,7 +592,7 @@ __device__ __forceinline__ void grad_combine(GradLane &g, int m) {
 __device__ __forceinline__ void grad_finish(const GradLane &s, const GradPlanetP &g, float sum_a,
                                             float poison, float *out) {
   const float Kb = g.K * g.beta;
-  out[0] = __fmaf_rn(Kb * (kTwoPiF * g.n2), kahan_value(s.P), poison);
+  out[0] = __fmaf_rn(Kb * (kTwoPiF * (g.p.n * g.p.n)), kahan_value(s.P), poison);
   out[1] = s.K + poison;
   out[2] = __fmaf_rn(g.K, __fmaf_rn(g.cw, sum_a, -s.e), poison);
   out[3] = __fmaf_rn(-g.K, __fmaf_rn(g.esw, sum_a, s.w), poison);

@@ -258,7 +258,7 @@ __device__ __forceinline__ void body_mixed(const typename RaggedPlanet<GRAD>::ty
       } else {
         const f32x2 M = mean_anomaly2<WIDE>(th, tl, pl[j]);
         f32x2 s, c, E;
-        kepler_pair(abs2(M), pl[j], tab, s, c, E);
+        kepler_pair<false>(abs2(M), pl[j], tab, s, c, E);
         velocity_sum(V, pl[j], signed_as(s, M), c);
       }
     }
@@ -398,7 +398,7 @@ constexpr int kMaxWarps = 8;   // block <= 256
 // Bound by the FP32 pipe's instructions (packed ones take two issue slots) at
 // large sizes.  Measured before, one observation per instruction and a system
 // at a time: forward 50000 systems 310 us, 3000 51, 20000 tiny 31; gradient
-// 50000 systems 439 us (now 322), 200000 1734 (now 1185).
+// 50000 systems 440 us (now 339), 200000 1734.
 constexpr int kAhead = 4;
 static_assert(kAhead * KC_MAX_PLANETS == 32, "a lane per planet of the systems taken");
 
@@ -411,7 +411,7 @@ ragged_mixed_kernel(RaggedDev d, const float4 *__restrict__ oa, const float4 *__
   __shared__ AngTab tab_s;
   __shared__ Planet pl_s[kMaxWarps][kAhead * KC_MAX_PLANETS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  ang_tab_load(tab_s.s, threadIdx.x, blockDim.x);
+  ang_tab_load<GRAD>(tab_s.s, threadIdx.x, blockDim.x);
   __syncthreads();
   const int mine = lane / KC_MAX_PLANETS, mine_j = lane % KC_MAX_PLANETS;
   // fewer at a time where the queue holds few per warp (300 systems taken four
