@@ -45,8 +45,8 @@ FP32_LANES_PER_SM = 128
 ROTATE_BYTES = 256 << 20
 FALLBACK_SM_MHZ = 2070.0
 
-# Algorithmic FP32 work of one planet-observation evaluation of the mixed
-# path, in FLOPs (FMA = 2, add/mul = 1; MUFU sin/cos/rcp and integer or
+# Algorithmic FP32 work of one planet-observation evaluation of the scalar
+# mixed kernels (the tile kernels, the likelihood, the scalar adjoint), in FLOPs (FMA = 2, add/mul = 1; MUFU sin/cos/rcp and integer or
 # select operations not counted), from the algorithm as implemented:
 #   double-single mean anomaly 18 (its low part formed already scaled by
 #   2 pi), Mikkola's starting value 18 (its per-planet constants and the
@@ -60,8 +60,7 @@ MEAN_ANOMALY_FLOPS = 18
 
 
 def mixed_flops_per_eval(n_pl: int, warp: bool = False) -> float:
-    """FLOPs per evaluation of the mixed chi2 kernels (the tile kernels and
-    the warp-per-system kernel run the same per-evaluation arithmetic)."""
+    """FLOPs per evaluation of the scalar mixed chi2 kernels."""
     return MEAN_ANOMALY_FLOPS + KEPLER_MIXED_FLOPS + 8 + 4 + 10.0 / n_pl
 
 
@@ -98,7 +97,40 @@ def gn_tensor_flops_per_obs(n_pl: int, split: int) -> float:
     return tiles * 3 * 16 * 8 * 2          # per observation (K = 1 of each 8-deep step)
 
 
-# FP64 path, FP64 FLOPs per planet-observation evaluation (FMA = 2), from its
+# The packed kernels (the warp-per-system chi2, kc_chi2_grad's adjoint, the
+# Gauss-Newton kernel up to three planets, the ragged kernel) per evaluation:
+# mean anomaly 13, start 17, tabulated sin/cos 12, Newton step and its update
+# 15, velocity and planet Kahan sum 10, and per observation the residual and
+# the compensated square 9.  The adjoint: 59 up to the update (1 - cos E beside
+# cos E), 1/D and the two terms the partials are made of 17, five sums 19, and per
+# observation 12.
+def pair_flops_per_eval(n_pl: int) -> float:
+    return 13 + 17 + 12 + 15 + 10 + 9.0 / n_pl
+
+
+def pair_grad_flops_per_eval(n_pl: int) -> float:
+    return 59 + 17 + 19 + 12.0 / n_pl
+
+
+def chi2_flops_per_eval(n_pl: int, tile) -> float:
+    return pair_flops_per_eval(n_pl) if tile[2] == 3 else mixed_flops_per_eval(n_pl)
+
+
+def gauss_newton_flops_per_eval(n_pl: int) -> float:
+    """The row of U as gn_flops_per_eval, on the adjoint that n_pl takes."""
+    grad = pair_grad_flops_per_eval(n_pl) if n_pl <= 3 else grad_flops_per_eval(n_pl)
+    return grad + 5 + 1.0 / n_pl
+
+
+# FP64 FLOPs the FP64 chi2 kernel executes per evaluation: phase 3, f(E) 4,
+# velocity at the tabulated angle 5, and per observation 5; the rest of the
+# evaluation runs in float expansions.
+def f64_flops_per_eval(n_pl: int) -> float:
+    return 3 + 4 + 5 + 5.0 / n_pl
+
+
+# The same evaluation with every leading term in FP64 (the form the ragged and
+# the Gauss-Newton FP64 kernels keep), FP64 FLOPs (FMA = 2), from its
 # algorithm: mean anomaly 6 (tau/P minus its integer part in one FMA, the
 # offset, the removal of the nearest integer, the scaled FMA; the integer
 # parts and the low part of the phase in single precision), table-driven
@@ -218,7 +250,7 @@ def grid_sweep_throughput(kc, synth, dev, stream, args):
     evals = w.n_sys * w.n_pl * w.n_obs
     val = evals / sec
     tile = kc.kc_get_tile("chi2", "mixed", w.n_sys, w.n_pl, w.n_obs)
-    fpe = mixed_flops_per_eval(w.n_pl, warp=tile[2] == 3)
+    fpe = chi2_flops_per_eval(w.n_pl, tile)
     peak = 2 * FP32_LANES_PER_SM * sm_count() * sm_mhz_for_peaks() * 1e6 / 1e12
     out = {"value": val, "unit": "planet-obs evals/s", "ms_per_step": 1e3 * sec,
            "n_sys": w.n_sys, "roofline_frac": val * fpe / 1e12 / peak,
@@ -277,10 +309,12 @@ def gradient_throughput(kc, synth, dev, stream, args):
         out["cpu_baseline"] = oracle_subset(w, 16384, grad=True)
     out["roofline_alu"] = {
         "peak": peak, "unit": "TFLOP/s",
-        "chi2_grad_frac": out["chi2_grad"] * grad_flops_per_eval(w.n_pl) / 1e12 / peak,
+        "chi2_grad_frac": out["chi2_grad"] * pair_grad_flops_per_eval(w.n_pl) / 1e12 / peak,
         "nll_grad_frac": out["nll_grad"] * grad_flops_per_eval(w.n_pl) / 1e12 / peak,
-        "gauss_newton_frac": out["gauss_newton"] * gn_flops_per_eval(w.n_pl) / 1e12 / peak,
-        "flops_per_eval": {"grad": grad_flops_per_eval(w.n_pl), "gauss_newton": gn_flops_per_eval(w.n_pl)},
+        "gauss_newton_frac": out["gauss_newton"] * gauss_newton_flops_per_eval(w.n_pl) / 1e12 / peak,
+        "flops_per_eval": {"grad": pair_grad_flops_per_eval(w.n_pl),
+                           "nll_grad": grad_flops_per_eval(w.n_pl),
+                           "gauss_newton": gauss_newton_flops_per_eval(w.n_pl)},
         "gauss_newton_tensor_tflops": out["gauss_newton"] / w.n_pl * gn_tensor_flops_per_obs(
             w.n_pl, kc.kc_get_tile("gn", "mixed", w.n_sys, w.n_pl, w.n_obs)[2]) / 1e12}
     # the two ways of adding U^T U, side by side
@@ -774,13 +808,13 @@ def run_kc(args):
         # pipe probe, x 2 FLOP x SMs x maximum SM clock
         f64_rate = kc.kc_measure_pipe_rate("fp64", stream=stream)
         f32_rate = kc.kc_measure_pipe_rate("fp32", stream=stream)
+        f64_fpe = f64_flops_per_eval(w.n_pl)
         f64_peak = 2 * f64_rate * sm_count() * sm_mhz_for_peaks() * 1e6 / 1e12
         extras["fp64"] = {"value": f64_val, "unit": "planet-obs evals/s",
                           "ms_per_step": 1e3 * f_s / len(f_ev),
-                          "roofline": {"bound": "fp64", "achieved": f64_val * F64_FLOPS_PER_EVAL
-                                       / 1e12, "peak": f64_peak, "unit": "TFLOP/s",
-                                       "frac": f64_val * F64_FLOPS_PER_EVAL / 1e12 / f64_peak,
-                                       "flops_per_eval": F64_FLOPS_PER_EVAL,
+                          "roofline": {"bound": "fp64", "achieved": f64_val * f64_fpe / 1e12, "peak": f64_peak, "unit": "TFLOP/s",
+                                       "frac": f64_val * f64_fpe / 1e12 / f64_peak,
+                                       "flops_per_eval": f64_fpe,
                                        "peak_basis": f"measured DFMA rate {f64_rate:.2f} per SM "
                                                      f"per clock x 2 FLOP x {sm_count()} SMs x max SM clock"}}
         extras["pipe_rates_per_sm_clock"] = {"fp32_fma": f32_rate, "fp64_fma": f64_rate}
@@ -794,8 +828,7 @@ def run_kc(args):
     pk, pk_kind = peaks()
     sm_mhz = pk.get("sm_max_mhz", FALLBACK_SM_MHZ)
     peak_tflops = 2 * FP32_LANES_PER_SM * sm_count() * sm_mhz * 1e6 / 1e12
-    warp = tile[2] == 3
-    flops = mixed_flops_per_eval(w.n_pl, warp) * evals
+    flops = chi2_flops_per_eval(w.n_pl, tile) * evals
     achieved = flops / (t_sum / args.steps) / 1e12          # one GPU's launch
     traffic = (DRAM_BYTES_PER_LAUNCH.get((args.config, args.n_sys, tuple(tile)))
                if world == 1 else None)
@@ -804,7 +837,7 @@ def run_kc(args):
                 "kernel": mixed_kernel_name(w.n_pl, tile),
                 "peak_basis": f"FP32 FMA pipe: {sm_count()} SMs x {FP32_LANES_PER_SM} lanes x 2 FLOP "
                               f"x {sm_mhz:.0f} MHz ({pk_kind} max SM clock)",
-                "flops_per_eval": mixed_flops_per_eval(w.n_pl, warp)}
+                "flops_per_eval": chi2_flops_per_eval(w.n_pl, tile)}
 
     if rank != 0:
         return
@@ -966,8 +999,8 @@ def ragged_measure(kc, synth, dev, stream, flush, args, world=1, rank=0, compact
     # ALU roofline of the persistent kernel: every system at its own n_pl
     n_obs_s = np.diff(np.asarray(w.obs_off)).astype(np.float64)
     npl_s = np.asarray(w.n_pl).astype(np.float64)
-    per_planet = (grad_flops_per_eval(1) - 12.0) if want_grad else (mixed_flops_per_eval(1) - 10.0)
-    per_obs = 12.0 if want_grad else 10.0
+    per_obs = 12.0 if want_grad else 9.0
+    per_planet = (pair_grad_flops_per_eval(1) if want_grad else pair_flops_per_eval(1)) - per_obs
     flops_step = float(np.sum(n_obs_s * (npl_s * per_planet + per_obs)))
     peak = 2 * FP32_LANES_PER_SM * sm_count() * sm_mhz_for_peaks() * 1e6 / 1e12
     achieved = flops_step / (t_sum / args.steps) / 1e12
