@@ -20,11 +20,11 @@
 //    float-pair difference;
 //  - v = N/D with N = A cos E - B sin E: N at the table's angle by two FP64
 //    operations, times 1/D (a float pair assembled into a double on the
-//    integer pipe) onto the planet sum, and the difference of N in float pairs, summed compensated and
-//    added to V once per observation.
+//    integer pipe) onto the planet sum, and the difference of N in float
+//    pairs, summed compensated and added to V once per observation.
 //
-// FP64 instructions per evaluation: 7, and 4 per observation (before: 33 and
-// 3).  Error of v, in units of K, against 64-bit mantissas in an emulation
+// FP64 instructions per evaluation: 7 (11 where 1/D is corrected, velocity_x),
+// and 4 per observation (before: 33 and 3).  Error of v, in units of K, against 64-bit mantissas in an emulation
 // (rms over 2.6e5 draws; P in 1 .. 4000 d, 4000 d of observations), with
 // the form of one FP64 Halley step and one FP64 Newton step for 1/D in
 // brackets: e < 0.3 1.5e-15 (5.4e-15), 0.3 .. 0.8 1.8e-15 (4.4e-15), 0.8 ..
@@ -452,19 +452,24 @@ __device__ __forceinline__ double kepler_x(double M, double e) {
 
 // V + (vh, vl) += v, v = (A cos E - B sin E)/D: the part at the table's angle
 // on the FP64 pipe, the difference in float pairs.
-// FINE: 1/D corrected once in FP64 (four instructions more).  The pair's 48
-// bits are what limits v: the error of model velocities, 2.2e-15 of their rms
-// with the pair and 2.1e-15 to 2.5e-15 in the form before it, is 3e-16 to 7e-16
-// so.  In chi2 it averages out (4e-16 without it).
-template <bool FINE>
-__device__ __forceinline__ void velocity_x(const EvalX &o, const PlanetX &p, double &V, float &vh,
-                                           float &vl) {
+// fine: 1/D corrected once in FP64 (four instructions more), for planets above
+// kEccFine and for model velocities.  The pair's 48 bits of D, relative to D = 1
+// - e cos E, are what limits v: the error of model velocities was 2.2e-15 of
+// their rms with the pair (2.1e-15 to 2.5e-15 in the form before it) and is
+// 3e-16 to 7e-16 so; that of chi2 with all e in 0.85 .. 0.95 was 2.5e-15 (1.35e-15
+// before it) and is 6.6e-16.  At lower e it averages out in chi2 (e in 0.1 .. 0.4:
+// 3.6e-16, 1.9e-15 before).  The vote makes it a branch (a
+// predicated FP64 instruction takes the pipe's time all the same).
+constexpr float kEccFine = 0.6f;
+__device__ __forceinline__ void velocity_x(const EvalX &o, const PlanetX &p, bool fine, double &V,
+                                           float &vh, float &vl) {
   const double N = fma(xor_sign(p.B, o.sign ^ 0x80000000u), o.S, p.A * o.C);
   double y = pair_d(o.y.h, o.y.l);
-  if (FINE) {
+  if (__any_sync(__activemask(), fine)) {
     float h, l;
     two_sum(o.dc.h, o.dc.l, h, l);
-    y = fma(y, fma(-fma(-p.e, o.C + pair_d(h, l), 1.0), y, 1.0), y);
+    const double yf = fma(y, fma(-fma(-p.e, o.C + pair_d(h, l), 1.0), y, 1.0), y);
+    y = fine ? yf : y;
   }
   V = fma(N, y, V);
   const float Bh = xor_sign(p.Bh, o.sign), Bl = xor_sign(p.Bl, o.sign);
@@ -531,7 +536,7 @@ __device__ __forceinline__ double model_velocity(double tau, const PlanetX *q, i
       double sE, cE, res;
       V = eval_high(tau, tf, q[j], V, sE, cE, res);
     } else {
-      velocity_x<true>(solve_x(tau, tf, q[j]), q[j], V, vh, vl);
+      velocity_x(solve_x(tau, tf, q[j]), q[j], true, V, vh, vl);
     }
   }
   return HI ? V : add_pair(V, vh, vl);

@@ -555,7 +555,7 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
           } else {
             const EvalX x = solve_x(o.tau, o.tf, p);
             if (want_resid) rmax = fmax(rmax, resid_x(x, p));
-            velocity_x<false>(x, p, r, vh, vl);
+            velocity_x(x, p, p.eh > kEccFine, r, vh, vl);
           }
         }
         if (!HI) r = add_pair(r, vh, vl);
