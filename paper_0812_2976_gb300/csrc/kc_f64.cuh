@@ -24,12 +24,13 @@
 //    pairs, summed compensated and added to V once per observation.
 //
 // FP64 instructions per evaluation: 7 (11 where 1/D is corrected, velocity_x),
-// and 4 per observation (before: 33 and 3).  Error of v, in units of K, against 64-bit mantissas in an emulation
-// (rms over 2.6e5 draws; P in 1 .. 4000 d, 4000 d of observations), with
-// the form of one FP64 Halley step and one FP64 Newton step for 1/D in
-// brackets: e < 0.3 1.5e-15 (5.4e-15), 0.3 .. 0.8 1.8e-15 (4.4e-15), 0.8 ..
-// 0.95 2.9e-15 (2.6e-15).  Valid for e <= kEccFast; above it the kernels
-// take kepler_f64<true>.
+// and 4 per observation (before: 33 and 3).  Error of v without that
+// correction, in units of K, against 64-bit mantissas in an emulation (rms over
+// 2.6e5 draws; P in 1 .. 4000 d, 4000 d of observations), with the form of one
+// FP64 Halley step and one FP64 Newton step for 1/D in brackets: e < 0.3 1.5e-15
+// (5.4e-15), 0.3 .. 0.8 1.8e-15 (4.4e-15), 0.8 .. 0.95 2.9e-15 (2.6e-15: hence the
+// correction).  Valid for e <= kEccFast; above it the kernels take
+// kepler_f64<true>.
 #pragma once
 
 #include "kc_device.cuh"
