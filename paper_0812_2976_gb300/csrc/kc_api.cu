@@ -10,6 +10,7 @@
 #include <mutex>
 #include <string>
 #include <tuple>
+#include <utility>
 #include <vector>
 
 #include "kc_internal.h"
@@ -105,6 +106,24 @@ int sm_count() {
   }
   g_sm_count[dev] = n;
   return n;
+}
+
+namespace {
+std::mutex g_smem_mu;
+std::map<std::pair<int, const void *>, size_t> g_smem_limit;   // set so far
+}  // namespace
+
+cudaError_t raise_smem_limit(const void *kernel, size_t bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;    // allowed without the attribute
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(g_smem_mu);
+  size_t &limit = g_smem_limit[{dev, kernel}];
+  if (bytes <= limit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) limit = bytes;
+  return e;
 }
 
 unsigned long long *invalid_counter() {

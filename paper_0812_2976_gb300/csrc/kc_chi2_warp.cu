@@ -388,8 +388,10 @@ const void *warp_kernel_for(int J, int variant) {
   return nullptr;
 }
 
-// CTAs of the kernel resident per SM (occupancy API), per device, planet
-// count, block and shared-memory size; 0 when the shape does not fit.
+// CTAs of the kernel resident per SM (occupancy API), remembered per device,
+// planet count, block and shared-memory size; 0 when the shape does not fit.
+// The shared-memory limit is not remembered here: it belongs to the kernel, not
+// to a size.
 std::mutex g_occ_mu;
 std::map<std::tuple<int, int, int, size_t>, int> g_occ;
 
@@ -399,21 +401,19 @@ int blocks_per_sm(int J, int variant, int block, size_t smem) {
     cudaGetLastError();
     return 1;                                    // no device: shapes stay valid
   }
+  const void *fn = warp_kernel_for(J, variant);
+  if (!fn) return 0;
+  if (raise_smem_limit(fn, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
   const auto key = std::make_tuple(dev * 16 + J, block, variant, smem);
   {
     std::lock_guard<std::mutex> lk(g_occ_mu);
     auto it = g_occ.find(key);
     if (it != g_occ.end()) return it->second;
   }
-  const void *fn = warp_kernel_for(J, variant);
   int n = 0;
-  if (!fn) return 0;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, block, smem) != cudaSuccess) {
     cudaGetLastError();
     n = 0;

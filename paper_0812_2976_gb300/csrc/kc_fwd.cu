@@ -792,8 +792,7 @@ kepler_f32_kernel(const float *__restrict__ M, const float *__restrict__ e, int6
 
 template <typename Kern>
 cudaError_t set_smem(Kern k, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  return raise_smem_limit(reinterpret_cast<const void *>(k), bytes);
 }
 
 int grid_for(int64_t n_sys, int ST) { return (int)((n_sys + ST - 1) / ST); }

@@ -1601,8 +1601,7 @@ gn_f64_kernel(UniformArgs a, double *__restrict__ chi2_out, double *__restrict__
 
 template <typename Kern>
 cudaError_t set_smem(Kern k, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  return raise_smem_limit(reinterpret_cast<const void *>(k), bytes);
 }
 
 }  // namespace

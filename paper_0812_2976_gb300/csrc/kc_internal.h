@@ -113,6 +113,12 @@ __device__ __forceinline__ bool dbg_ok(unsigned long long *words, bool ok, Debug
 // (kc_api.cu); freed with cudaFreeAsync on the same stream.
 cudaError_t scratch_alloc(void **ptr, size_t bytes, cudaStream_t st);
 
+// Lets a kernel (a __global__ function's address) be launched with `bytes` of
+// dynamic shared memory on the current device (kc_api.cu).  The limit belongs
+// to the kernel, for every thread and stream, and setting a smaller one lowers
+// it: so it is only ever raised.
+cudaError_t raise_smem_limit(const void *kernel, size_t bytes);
+
 // Forward chi2 (kc_fwd.cu).  launch_chi2_mixed_prepared runs the split
 // variant on caller-provided scratch of mixed_scratch_bytes() bytes (256-byte
 // aligned).
