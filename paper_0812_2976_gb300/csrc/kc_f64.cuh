@@ -142,6 +142,12 @@ __device__ __forceinline__ double pair_d(float h, float l) {
   const unsigned hi = (b >> 3) + 0x38000000u + (sum < lo ? 1u : 0u);
   return __hiloint2double((int)(hi | sign), (int)sum);
 }
+// pair_d for a pair that may be no number: NaN where h is infinite or NaN.
+__device__ __forceinline__ double pair_or_nan(float h, float l) {
+  const double d = pair_d(h, l);
+  const bool none = (__float_as_uint(h) & 0x7f800000u) == 0x7f800000u;
+  return __hiloint2double(none ? 0x7ff80000 : __double2hiint(d), __double2loint(d));
+}
 __device__ __forceinline__ double xor_sign(double x, unsigned sign) {
   return __hiloint2double(__double2hiint(x) ^ (int)sign, __double2loint(x));
 }
@@ -281,7 +287,10 @@ __device__ __forceinline__ EvalX solve_x(double tau, float tf, const PlanetX &p)
   o.sign = (unsigned)__double2hiint(u) & 0x80000000u;
   u = xor_sign(u, o.sign);
   o.u = u;
-  o.lo2pi = xor_sign(tf * p.inv_P_lo2pi, o.sign);
+  // n 0: NaN for a time or phase that is none (or beyond float's range).  The
+  // conversions below turn it into some number; from here it reaches every float
+  // pair of the solution, and pair_or_nan hands it on.
+  o.lo2pi = xor_sign(__fmaf_rn(n, 0.0f, __fmul_rn(tf, p.inv_P_lo2pi)), o.sign);
   // single-precision solve
   const float m = d2f_cut(u) * kTwoPiF;
   const float sb = m * p.st.bs;
@@ -490,11 +499,11 @@ __device__ __forceinline__ void velocity_x(const EvalX &o, const PlanetX &p, boo
   vl += err + we;
 }
 
-// V + (vh, vl) for a compensated pair.
+// V + (vh, vl) for a compensated pair (NaN where a time was).
 __device__ __forceinline__ double add_pair(double V, float vh, float vl) {
   float h, l;
   two_sum(vh, vl, h, l);
-  return V + pair_d(h, l);
+  return V + pair_or_nan(h, l);
 }
 
 // sin E (with M's sign), cos E and 1/D in double, the reciprocal's pair (48
@@ -507,7 +516,7 @@ __device__ __forceinline__ void solved_d(const EvalX &o, double e, double &sE, d
   sE = xor_sign(o.S + pair_d(h, l), o.sign);
   two_sum(o.dc.h, o.dc.l, h, l);
   cE = o.C + pair_d(h, l);
-  y = pair_d(o.y.h, o.y.l);
+  y = pair_or_nan(o.y.h, o.y.l);
   y = fma(y, fma(-fma(-e, cE, 1.0), y, 1.0), y);
 }
 
