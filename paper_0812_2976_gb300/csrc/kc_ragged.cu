@@ -127,7 +127,8 @@ __global__ void prep_obs_f64(RaggedDev d, const double *__restrict__ t,
 }
 
 // FP64 model velocities of a ragged batch, one warp per system, its planets
-// set up once by the first lanes.
+// set up once by the first lanes, KC_MAX_PLANETS of them at a time: the counts
+// are device data that no host check sees, and nothing else here limits them.
 __global__ void __launch_bounds__(256)
 predict_ragged_kernel(const double *__restrict__ params,
                                       const int64_t *__restrict__ par_off,
@@ -146,23 +147,27 @@ predict_ragged_kernel(const double *__restrict__ params,
     if (o1 <= o0) continue;
     const int J = n_pl[s];
     // the caller's arrays (no totals known here): ordered offsets, a planet
-    // count in range
     if (!dbg_ok(words, o0 >= 0 && par_off[s] >= 0, kDbgObsOff, s) ||
-        !dbg_ok(words, J >= 1 && J <= KC_MAX_PLANETS, kDbgPlanets, s))
+        !dbg_ok(words, J >= 1, kDbgPlanets, s))
       continue;
     const double *p = params + par_off[s];
     const double tr = t[o0];
     const double gam = system_gamma_r(p, J);
-    __syncwarp();
-    if (lane < J) {
-      double sw, cw, beta;
-      pl[lane] = planet_setup_x(p + 5 * lane, tr - t0, sw, cw, beta);
+    for (int j0 = 0; j0 == 0 || j0 < J; j0 += KC_MAX_PLANETS) {
+      const int n = min(J - j0, KC_MAX_PLANETS);
+      __syncwarp();
+      if (lane < n) {
+        double sw, cw, beta;
+        pl[lane] = planet_setup_x(p + 5 * (j0 + lane), tr - t0, sw, cw, beta);
+      }
+      __syncwarp();
+      const bool hi = any_high_e(lane < n && pl[lane].e > (double)kEccFast);
+      for (int64_t k = o0 + lane; k < o1; k += 32) {
+        const double V = j0 == 0 ? gam : v_out[k];       // the lane's own sum so far
+        v_out[k] = hi ? model_velocity<true>(t[k] - tr, pl, n, V)
+                      : model_velocity<false>(t[k] - tr, pl, n, V);
+      }
     }
-    __syncwarp();
-    const bool hi = any_high_e(lane < J && pl[lane].e > (double)kEccFast);
-    for (int64_t k = o0 + lane; k < o1; k += 32)
-      v_out[k] = hi ? model_velocity<true>(t[k] - tr, pl, J, gam)
-                    : model_velocity<false>(t[k] - tr, pl, J, gam);
   }
 }
 
