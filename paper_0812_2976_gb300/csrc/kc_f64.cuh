@@ -281,9 +281,13 @@ __device__ __forceinline__ EvalX solve_x(double tau, float tf, const PlanetX &p)
   // n + c0 lies within 0.5 + 2^-23 |tau/P| of 0 (the table covers 0.528)
   const float n = rintf(__fmaf_rn(tf, p.inv_P_f, p.c0f));
   double u = fma(tau, p.inv_P, -f2d(n)) + p.c0;
-  // (a vote, so that the usual case skips the FP64 work instead of
-  // predicating it)
-  if (__any_sync(__activemask(), fabsf(n) > 1e5f)) u -= f2d(rintf(d2f(u)));
+  // (a vote, so that the usual case skips the FP64 work instead of predicating
+  // it; the value is each lane's own, so that no lane's bits hang on the others)
+  const bool wrap = fabsf(n) > 1e5f;
+  if (__any_sync(__activemask(), wrap)) {
+    const double w = u - f2d(rintf(d2f(u)));
+    u = wrap ? w : u;
+  }
   o.sign = (unsigned)__double2hiint(u) & 0x80000000u;
   u = xor_sign(u, o.sign);
   o.u = u;
@@ -534,7 +538,8 @@ __device__ __forceinline__ double eval_high(double tau, float tf, const PlanetX 
 }
 
 // The model velocity gamma + sum_j v_j at tau.  HI: a planet of the system (or
-// of the warp) lies above kEccFast.
+// of the warp) lies above kEccFast; each planet takes the form of its own
+// eccentricity.
 template <bool HI>
 __device__ __forceinline__ double model_velocity(double tau, const PlanetX *q, int J, double gam) {
   const float tf = d2f(tau);
@@ -542,14 +547,14 @@ __device__ __forceinline__ double model_velocity(double tau, const PlanetX *q, i
   float vh = 0.0f, vl = 0.0f;
 #pragma unroll 1
   for (int j = 0; j < J; ++j) {
-    if (HI) {
+    if (HI && q[j].e > (double)kEccFast) {
       double sE, cE, res;
       V = eval_high(tau, tf, q[j], V, sE, cE, res);
     } else {
       velocity_x(solve_x(tau, tf, q[j]), q[j], true, V, vh, vl);
     }
   }
-  return HI ? V : add_pair(V, vh, vl);
+  return add_pair(V, vh, vl);
 }
 
 // |E - M - e sin E| of the solution, in double.

@@ -548,7 +548,7 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
 #pragma unroll 1
         for (int j = 0; j < J; ++j) {
           const PlanetX &p = q[j];
-          if (HI) {
+          if (HI && p.e > (double)kEccFast) {
             double sE, cE, res;
             r = eval_high(o.tau, o.tf, p, r, sE, cE, res);
             if (want_resid) rmax = fmax(rmax, res);
@@ -558,7 +558,7 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
             velocity_x(x, p, p.eh > kEccFine, r, vh, vl);
           }
         }
-        if (!HI) r = add_pair(r, vh, vl);
+        r = add_pair(r, vh, vl);
         if (NLL) {
           const double var = o.w + s2_s[sl];
           const double wk = var > 0.0 ? 1.0 / var : __longlong_as_double(0x7ff8000000000000ll);

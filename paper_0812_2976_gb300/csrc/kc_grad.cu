@@ -562,7 +562,7 @@ grad_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ chi2_ou
         for (int j = 0; j < J; ++j) {
           const GradPlanetX &p = q[j];
           double cE;
-          if (HI) {
+          if (HI && p.base.e > (double)kEccFast) {
             double res;
             eval_high(o.tau, o.tf, p.base, 0.0, sE[j], cE, res);
             y[j] = 1.0 / fma(-p.base.e, cE, 1.0);

@@ -1,0 +1,53 @@
+"""A system's results do not depend on the systems it is evaluated with: the
+bits of a row are the same beside rows of phases past 1e5 periods and of e >
+0.95 as beside ordinary ones, at the same launch shape."""
+import numpy as np
+import pytest
+import torch
+from test_gpu_pair import T0, rows
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kc():
+    import paper_0812_2976_gb300 as kc
+    from paper_0812_2976_gb300 import build
+    build.build()
+    kc._lib.load()
+    return kc
+
+
+def two_batches(n_pl, p_range, e_range, plain=(1.0, 3000.0), n_sys=512, n_obs=200):
+    """Rows of which every third is ordinary in both batches; the others are
+    ordinary in the first and drawn from the given ranges in the second."""
+    rng = np.random.default_rng(n_pl)
+    plain = rows(rng, n_sys, n_pl, plain, (0.0, 0.93))
+    mixed = plain.copy()
+    odd = np.arange(n_sys) % 3 != 0
+    mixed[odd] = rows(rng, int(odd.sum()), n_pl, p_range, e_range)
+    t = np.sort(rng.uniform(T0, T0 + 4000.0, n_obs))
+    v, s = rng.normal(0.0, 30.0, n_obs), rng.uniform(1.0, 4.0, n_obs)
+    put = lambda x: torch.tensor(x, device="cuda")  # noqa: E731
+    return put(plain), put(mixed), [put(x) for x in (t, v, s)], ~torch.tensor(odd)
+
+
+ODD = [((0.004, 0.02), (0.0, 0.9), (0.05, 0.1)),      # 1e5 periods and more; up to 8e4
+       ((1.0, 3000.0), (0.951, 0.99), (1.0, 3000.0))]
+
+
+@pytest.mark.parametrize("p_range,e_range,ordinary", ODD)
+@pytest.mark.parametrize("n_pl", [1, 3, 5])
+def test_double_precision(kc, n_pl, p_range, e_range, ordinary):
+    plain, mixed, obs, same = two_batches(n_pl, p_range, e_range, ordinary)
+    for kernel in ("chi2", "grad"):
+        kc.kc_set_tile(kernel, "fp64", 512, n_pl, 200, (4, 64))
+    try:
+        for fn in (lambda p: (kc.kc_chi2_eval_ex(p, *obs, t0=T0, mode="fp64"),),
+                   lambda p: kc.kc_chi2_grad(p, *obs, t0=T0, mode="fp64"),
+                   lambda p: (kc.kc_rv_predict(p, obs[0][:9].contiguous(), t0=T0),)):
+            for a, b in zip(fn(plain), fn(mixed)):
+                assert torch.equal(a.cpu()[same], b.cpu()[same])
+    finally:
+        for kernel in ("chi2", "grad"):
+            kc.kc_set_tile(kernel, "fp64", 512, n_pl, 200, None)
