@@ -674,10 +674,9 @@ __device__ inline float reduce_pi<float>(float M) {
 }
 
 // One (M, e) per thread and iteration, five FP64 instructions each (kepler_x)
-// where every lane of the warp has 0 <= e <= kEccFast and |M| <= 1.02 pi above
-// 2^-30 (the leading words compared, on the integer pipe); otherwise the whole
-// warp takes the form with two FP64 quartic steps, which costs some 2000 clocks
-// a warp.  2^24 elements, e <= 0.95: 1070 -> 260 us, bound by issue (memory: 60
+// where 0 <= e <= kEccFast and |M| <= 1.02 pi above 2^-30 (the leading words
+// compared, on the integer pipe); the other elements of a warp take the form with
+// two FP64 quartic steps, which costs it some 2000 clocks.  2^24 elements, e <= 0.95: 1070 -> 260 us, bound by issue (memory: 60
 // us); e < 0.999: 617 -> 569 us for 2^22.  Error against 64-bit mantissas, 4e5
 // draws with |M| from 1e-8: rms 9.10e-17 -> 9.05e-17, largest relative 3.6e-15
 // both.
@@ -696,10 +695,10 @@ __global__ void kepler_f64_kernel(const double *__restrict__ M, const double *__
     const double ei = e[i];
     double Mi = M[i];
     if (((unsigned)__double2hiint(Mi) & 0x7fffffffu) > 0x400921fau) Mi = reduce_pi(Mi);
-    if (any_high_e(!kepler_x_takes(Mi, ei), __activemask()))
-      E[i] = kepler_f64<true>(Mi, ei, s, c);
-    else
+    if (kepler_x_takes(Mi, ei))
       E[i] = kepler_x(Mi, ei);
+    else
+      E[i] = kepler_f64<true>(Mi, ei, s, c);
   }
 }
 
@@ -744,11 +743,21 @@ __device__ __forceinline__ f32x2 kepler_f32x2(f32x2 M, f32x2 e) {
   return pack2(copysignf(lo2(E), lo2(M)), copysignf(hi2(E), hi2(M)));
 }
 
+// Two reduced (M, e), each by the form of its own e: kepler_f32 outside [0, 1).
+__device__ __forceinline__ f32x2 kepler_any2(float m0, float m1, float e0, float e1) {
+  const f32x2 r = kepler_f32x2(pack2(m0, m1), pack2(e0, e1));
+  float x = lo2(r), y = hi2(r), s, c;
+  if (__float_as_uint(e0) >= 0x3f800000u) x = kepler_f32(m0, e0, s, c);   // the bits of 1.0f
+  if (__float_as_uint(e1) >= 0x3f800000u) y = kepler_f32(m1, e1, s, c);
+  return pack2(x, y);
+}
+
 // Four (M, e) per thread and iteration when the three arrays are 16-byte
 // aligned: float4 streaming loads and stores (the data are touched once) and
 // two packed solves in flight per thread.  Where one of the four M lies beyond
-// pi all are reduced; where one e lies outside [0, 1) all take kepler_f32.  The
-// rest (or everything, unaligned) one element per thread.
+// pi all are reduced (which leaves the others as they are); an e outside [0, 1)
+// takes kepler_f32.  The rest (or everything, unaligned) two elements per
+// iteration, with the same bits.
 // At 12 bytes an element memory alone takes 29 to 31 us for 2^24 elements; the
 // scalar form's 69 instructions an element issued for 33 of its 38.9 us.
 // Packed: 44 instructions, 34.9 us; the wait for memory is hidden by warps, so
@@ -765,9 +774,8 @@ __device__ __forceinline__ float4 kepler_f32_x4(float4 m, float4 ee) {
     const f32x2 b = kepler_f32x2(pack2(m.z, m.w), pack2(ee.z, ee.w));
     return make_float4(lo2(a), hi2(a), lo2(b), hi2(b));
   }
-  float s, c;
-  return make_float4(kepler_f32(m.x, ee.x, s, c), kepler_f32(m.y, ee.y, s, c),
-                     kepler_f32(m.z, ee.z, s, c), kepler_f32(m.w, ee.w, s, c));
+  const f32x2 a = kepler_any2(m.x, m.y, ee.x, ee.y), b = kepler_any2(m.z, m.w, ee.z, ee.w);
+  return make_float4(lo2(a), hi2(a), lo2(b), hi2(b));
 }
 
 __global__ void __launch_bounds__(256, 8)
@@ -784,9 +792,11 @@ kepler_f32_kernel(const float *__restrict__ M, const float *__restrict__ e, int6
   for (int64_t i = tid; i < n4; i += stride) {
     __stcs(E4 + i, kepler_f32_x4(__ldcs(M4 + i), __ldcs(e4 + i)));
   }
-  for (int64_t i = 4 * n4 + tid; i < n; i += stride) {
-    float s, c;
-    E[i] = kepler_f32(reduce_pi(M[i]), e[i], s, c);
+  for (int64_t i = 4 * n4 + tid; i < n; i += 2 * stride) {
+    const int64_t j = i + stride < n ? i + stride : i;
+    const f32x2 r = kepler_any2(reduce_pi(M[i]), reduce_pi(M[j]), e[i], e[j]);
+    E[i] = lo2(r);
+    if (j != i) E[j] = hi2(r);
   }
 }
 

@@ -1,6 +1,8 @@
 """A system's results do not depend on the systems it is evaluated with: the
 bits of a row are the same beside rows of phases past 1e5 periods and of e >
-0.95 as beside ordinary ones, at the same launch shape."""
+0.95 as beside ordinary ones, at the same launch shape; and an element of a
+Kepler solve's beside elements that need the other solver, and wherever it lies
+in memory."""
 import numpy as np
 import pytest
 import torch
@@ -51,3 +53,24 @@ def test_double_precision(kc, n_pl, p_range, e_range, ordinary):
     finally:
         for kernel in ("chi2", "grad"):
             kc.kc_set_tile(kernel, "fp64", 512, n_pl, 200, None)
+
+
+@pytest.mark.parametrize("mode", ["fp64", "mixed"])
+def test_kepler_solve(kc, mode):
+    rng = np.random.default_rng(2)
+    kind = np.float64 if mode == "fp64" else np.float32
+    M = rng.uniform(-3.1, 3.1, 4096).astype(kind)
+    e = rng.uniform(0.0, 0.94, 4096).astype(kind)
+    M2, e2 = M.copy(), e.copy()
+    e2[1::7], M2[3::7], e2[5::7] = 0.98, 1e-12, -0.0
+    same = np.ones(4096, bool)
+    same[1::7] = same[3::7] = same[5::7] = False
+    a, b = (kc.kc_kepler_solve(torch.tensor(x, device="cuda"), torch.tensor(y, device="cuda"),
+                               mode=mode).cpu().numpy() for x, y in ((M, e), (M2, e2)))
+    assert np.array_equal(a[same], b[same])
+    # nor on where in memory an element lies
+    shifted = [torch.tensor(np.concatenate([[0], x]).astype(kind), device="cuda")[1:]
+               for x in (M, e)]
+    assert np.array_equal(kc.kc_kepler_solve(*shifted, mode=mode).cpu().numpy(), a)
+    odd = [torch.tensor(x[:4093], device="cuda") for x in (M, e)]
+    assert np.array_equal(kc.kc_kepler_solve(*odd, mode=mode).cpu().numpy(), a[:4093])
