@@ -159,13 +159,23 @@ __device__ __forceinline__ float xor_sign(float x, unsigned sign) {
 
 // inv_P, c0, e, A, B as in PlanetD (A and B the velocity constants of the
 // E-form); their float pairs, 1/P and 2 pi times its low part in single
-// precision, and the start's constants (start_constants).
+// precision, and the start's constants (start_constants).  high: the velocity
+// takes the form without float expansions (eval_high).
 struct __align__(8) PlanetX {
   double inv_P, c0, e, A, B;
   float inv_P_f, inv_P_lo2pi, c0f;
   StartP st;
-  float eh, el, Ah, Al, Bh, Bl, pad;
+  float eh, el, Ah, Al, Bh, Bl;
+  int high;
 };
+
+// Whether the velocity's differences, of 1e-3 K and less, fit the float pairs:
+// |K| in [2^-30, 2^100) or zero (leading words compared).  Below it pair_d drops
+// bits (2^-84 absolute), above it the pairs overflow.
+__device__ __forceinline__ bool amplitude_fits(double K) {
+  const unsigned h = (unsigned)__double2hiint(K) & 0x7fffffffu;
+  return h - 0x3e100000u < 0x46300000u - 0x3e100000u || K == 0.0;
+}
 
 // sin and cos of any finite w from the table: w - 2 pi k in three FP64
 // FMAs (2 pi as two doubles; k below 2^30, else the library's sincos), then
@@ -226,6 +236,7 @@ __device__ __forceinline__ PlanetX planet_setup_x(const double *p, double dref, 
   split_d(e, q.eh, q.el);
   split_d(q.A, q.Ah, q.Al);
   split_d(q.B, q.Bh, q.Bl);
+  q.high = e > (double)kEccFast || !amplitude_fits(K);
   q.st = start_constants(q.eh);
   return q;
 }
@@ -503,11 +514,13 @@ __device__ __forceinline__ void velocity_x(const EvalX &o, const PlanetX &p, boo
   vl += err + we;
 }
 
-// V + (vh, vl) for a compensated pair (NaN where a time was).
+// V + (vh, vl) for a compensated pair (NaN where a time was; a zero pair, whose
+// pair_d is 2^-127, adds nothing).
 __device__ __forceinline__ double add_pair(double V, float vh, float vl) {
   float h, l;
   two_sum(vh, vl, h, l);
-  return V + pair_or_nan(h, l);
+  const double d = pair_or_nan(h, l);
+  return V + __hiloint2double(h == 0.0f ? 0 : __double2hiint(d), __double2loint(d));
 }
 
 // sin E (with M's sign), cos E and 1/D in double, the reciprocal's pair (48
@@ -538,8 +551,7 @@ __device__ __forceinline__ double eval_high(double tau, float tf, const PlanetX 
 }
 
 // The model velocity gamma + sum_j v_j at tau.  HI: a planet of the system (or
-// of the warp) lies above kEccFast; each planet takes the form of its own
-// eccentricity.
+// of the warp) is a `high` one; each planet takes its own form.
 template <bool HI>
 __device__ __forceinline__ double model_velocity(double tau, const PlanetX *q, int J, double gam) {
   const float tf = d2f(tau);
@@ -547,7 +559,7 @@ __device__ __forceinline__ double model_velocity(double tau, const PlanetX *q, i
   float vh = 0.0f, vl = 0.0f;
 #pragma unroll 1
   for (int j = 0; j < J; ++j) {
-    if (HI && q[j].e > (double)kEccFast) {
+    if (HI && q[j].high) {
       double sE, cE, res;
       V = eval_high(tau, tf, q[j], V, sE, cE, res);
     } else {

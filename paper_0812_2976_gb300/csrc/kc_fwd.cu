@@ -538,7 +538,7 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
     const PlanetX *q = pl_s + sl * J;
     bool hi = false;
 #pragma unroll
-    for (int j = 0; j < J; ++j) hi = hi || q[j].e > (double)kEccFast;
+    for (int j = 0; j < J; ++j) hi = hi || q[j].high;
     with_high_e(any_high_e(hi), [&](auto tag) {
       constexpr bool HI = decltype(tag)::value;
       for (int k = c; k < nk; k += G) {
@@ -548,7 +548,7 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
 #pragma unroll 1
         for (int j = 0; j < J; ++j) {
           const PlanetX &p = q[j];
-          if (HI && p.e > (double)kEccFast) {
+          if (HI && p.high) {
             double sE, cE, res;
             r = eval_high(o.tau, o.tf, p, r, sE, cE, res);
             if (want_resid) rmax = fmax(rmax, res);
@@ -642,7 +642,7 @@ rv_predict_kernel(const double *__restrict__ params, const double *__restrict__ 
   const int64_t s = sys0 + sl;
   const PlanetX *q = pl_s + sl * J;
   bool hi = false;
-  for (int j = 0; j < J; ++j) hi = hi || q[j].e > (double)kEccFast;
+  for (int j = 0; j < J; ++j) hi = hi || q[j].high;
   const double gam = s < n_sys ? gam_s[sl] : 0.0;
   with_high_e(any_high_e(hi), [&](auto tag) {
     constexpr bool HI = decltype(tag)::value;

@@ -161,7 +161,7 @@ predict_ragged_kernel(const double *__restrict__ params,
         pl[lane] = planet_setup_x(p + 5 * (j0 + lane), tr - t0, sw, cw, beta);
       }
       __syncwarp();
-      const bool hi = any_high_e(lane < n && pl[lane].e > (double)kEccFast);
+      const bool hi = any_high_e(lane < n && pl[lane].high);
       for (int64_t k = o0 + lane; k < o1; k += 32) {
         const double V = j0 == 0 ? gam : v_out[k];       // the lane's own sum so far
         v_out[k] = hi ? model_velocity<true>(t[k] - tr, pl, n, V)
