@@ -607,18 +607,21 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
 // observations of each of the CTA's systems per CTA.  Bound by the FP64 pipe
 // like chi2 (kc_f64.cuh); the planets are set up once per CTA, where one
 // thread per (system, observation) had repeated the setup at every
-// evaluation (512 x 3 x 1000: 305 us, now 44; 32 without 1/D's correction in
-// FP64, which takes the error from 2.2e-15 to 4e-16 of the velocities' rms).
+// evaluation (512 x 3 x 1000: 305 us, now 43; 32 without 1/D's correction in
+// FP64, which takes the error from 2.2e-15 to 4e-16 of the velocities' rms).  G
+// is the power of two that n_obs fills, down to one thread per system: every lane
+// evaluates (275996 systems of 5 planets above e = 0.95 at a single time: 358 us,
+// 2060 with 8 threads per system, 444 with the setup per evaluation).
 constexpr int kPredictBlock = 128;
-constexpr int kPredictMinG = 8;
 
 __global__ void __launch_bounds__(kPredictBlock)
 rv_predict_kernel(const double *__restrict__ params, const double *__restrict__ t, int64_t n_sys,
                   int J, int n_obs, double t0, int G, int chunk, int chunks,
                   double *__restrict__ v_out) {
-  __shared__ PlanetX pl_s[kPredictBlock / kPredictMinG * KC_MAX_PLANETS];
-  __shared__ double gam_s[kPredictBlock / kPredictMinG];
+  extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, ST = kPredictBlock / G;
+  PlanetX *pl_s = reinterpret_cast<PlanetX *>(smem);
+  double *gam_s = reinterpret_cast<double *>(pl_s + ST * J);
   const int npar = 5 * J + 1;
   const int64_t group = blockIdx.x / chunks;
   const int k0 = (int)(blockIdx.x - group * chunks) * chunk, k1 = min(n_obs, k0 + chunk);
@@ -1077,8 +1080,11 @@ cudaError_t launch_nll_f64(const UniformArgs &a, const Tile &tile, double *out, 
 
 cudaError_t launch_rv_predict(const double *params, const double *t, int64_t n_sys, int n_pl,
                               int n_obs, double t0, double *v_out, cudaStream_t st) {
-  int G = kPredictMinG;
+  int G = 1;
   while (G < kPredictBlock && G < n_obs) G <<= 1;
+  const size_t smem = (sizeof(PlanetX) * n_pl + sizeof(double)) * (kPredictBlock / G);
+  const cudaError_t err = set_smem(rv_predict_kernel, smem);
+  if (err != cudaSuccess) return err;
   const int64_t groups = (n_sys + kPredictBlock / G - 1) / (kPredictBlock / G);
   // up to eight observations per thread share a CTA's setup, as long as the
   // CTAs still fill the SMs four times over
@@ -1086,7 +1092,7 @@ cudaError_t launch_rv_predict(const double *params, const double *t, int64_t n_s
   while (per > 1 && groups * ((n_obs + per * G - 1) / (per * G)) < (int64_t)sm_count() * 4) per /= 2;
   const int chunk = per * G, chunks = (n_obs + chunk - 1) / chunk;
   if (groups * chunks > 0x7fffffff) return cudaErrorInvalidConfiguration;
-  rv_predict_kernel<<<(unsigned)(groups * chunks), kPredictBlock, 0, st>>>(
+  rv_predict_kernel<<<(unsigned)(groups * chunks), kPredictBlock, smem, st>>>(
       params, t, n_sys, n_pl, n_obs, t0, G, chunk, chunks, v_out);
   return cudaGetLastError();
 }
