@@ -30,8 +30,9 @@
 //    the planets over it: a planet's constants (PlanetP, computed once per
 //    (system, planet)) are read from shared memory once per chunk, and the
 //    chunk's Kepler solves are independent chains for the scheduler.
-//  - A CTA whose planets or times leave the short mean anomaly's range takes
-//    the wide one for all its systems (kc_pair.cuh).
+//  - A CTA with a period or a time outside the short mean anomaly's range takes
+//    the wide one for all its systems (kc_pair.cuh); a far time has the planets and
+//    the staged times made plain pairs.
 //  - The lanes of a system combine their compensated sums with TwoSum
 //    shuffles, and the warps of a system (G > 32) through a few words of
 //    shared memory; no atomics, no scratch memory.  Splitting a system over
@@ -102,11 +103,14 @@ __device__ __forceinline__ bool setup_item(int i, int spr, int64_t sys0, int64_t
                                            const double (&p)[5], double t_ref, double t0,
                                            PlanetP *pl_s, float *gam_s, unsigned long long *dbg) {
   if (!dbg_ok(dbg, i < spr * (J + 1), kDbgSmem, i)) return false;
-  bool wide = false;
+  bool brief = false;
   if (i < spr * J) {
     const int64_t s = sys0 + i / J;
     PlanetP q = {};
-    if (s < n_sys) q = planet_setup_pair(p, t_ref, t0, wide);
+    if (s < n_sys) {
+      q = planet_setup_pair(p, t_ref, t0, false);
+      brief = short_period(q);
+    }
     pl_s[i] = q;
   } else {
     const int sl = i - spr * J;
@@ -114,7 +118,7 @@ __device__ __forceinline__ bool setup_item(int i, int spr, int64_t sys0, int64_t
     if (sys0 + sl < n_sys) g = finite_bits(p[0]) ? d2f(p[0]) : __int_as_float(0x7fc00000);
     gam_s[sl] = g;
   }
-  return wide;
+  return brief;
 }
 
 // The item's parameters.  DEMC: the launch evaluates DE-MC proposals; with
@@ -153,12 +157,15 @@ __device__ __forceinline__ void load_item(int i, int spr, int64_t sys0, const Un
 
 // The thread's observations of one staged tile: npad (whole chunks), nk of
 // them real.  The thread takes kChunk observations at a time as kChunk / 2
-// packed pairs.
+// packed pairs.  WIDE and t != NULL: the times as plain pairs, from t (n_obs of
+// them, the tile's first one at k0).
 template <int J, bool RESID, bool WIDE>
 __device__ __forceinline__ void warp_tile_sum(const float *th_s, int tile, const PlanetP *q,
                                               const float *tab, float gam, int c, int lg,
                                               int npad, int nk, Kahan2 &acc, float &rmax,
-                                              unsigned long long *dbg) {
+                                              unsigned long long *dbg,
+                                              const double *t = nullptr, int k0 = 0,
+                                              int n_obs = 0) {
   constexpr int kPairs = kChunk / 2;
   const int step = kChunk << lg;
   for (int base = 2 * c; base < npad; base += step) {
@@ -170,6 +177,8 @@ __device__ __forceinline__ void warp_tile_sum(const float *th_s, int tile, const
       const float *o = th_s + base + (i << (lg + 1));
       th[i] = *reinterpret_cast<const f32x2 *>(o);
       tl[i] = *reinterpret_cast<const f32x2 *>(o + tile);
+      if (WIDE && t != nullptr)
+        plain_times(t, k0 + base + (i << (lg + 1)), n_obs, th[i], tl[i]);
       V[i].big = dup2(gam);
       V[i].small = 0;
     }
@@ -178,7 +187,7 @@ __device__ __forceinline__ void warp_tile_sum(const float *th_s, int tile, const
     // 2^20-system sweep; all four at once spill: 2171)
 #pragma unroll 2
     for (int j = 0; j < J; ++j) {
-      const PlanetP qj = q[j];
+      const PlanetP &qj = q[j];
 #pragma unroll
       for (int i = 0; i < kPairs; ++i) {
         const f32x2 M = mean_anomaly2<WIDE>(th[i], tl[i], qj);
@@ -207,6 +216,157 @@ __device__ __forceinline__ void warp_tile_sum(const float *th_s, int tile, const
   }
 }
 
+// Observation k of a staged tile: tau = t - t_ref as (th, tl) and v as float
+// pairs, w = 1/(sigma^2 + jitter^2); the padding up to whole chunks has zero
+// weight (and tau = v = 0).  plain: tau stays as it is (kc_pair.cuh).  Returns
+// whether the time is a far one.
+__device__ __forceinline__ bool stage_obs(float *obs_s, int tile, int k, bool real, double t,
+                                          double v, double sigma, const Split3 &tr3, float jit2,
+                                          bool plain, unsigned long long *dbg) {
+  if (!dbg_ok(dbg, k < tile, kDbgSmem, k)) return false;
+  float th = 0.0f, tl = 0.0f, vh = 0.0f, vl = 0.0f, wk = 0.0f;
+  if (real) {
+    sub_ds(split3(t), tr3, th, tl);
+    if (!plain) tau_place(th, tl);
+    split_d(v, vh, vl);
+    const float sg = d2f(sigma);
+    const float var = __fmaf_rn(sg, sg, jit2);
+    wk = var > 0.0f ? 1.0f / var : __int_as_float(0x7fc00000);
+  }
+  obs_s[k] = th;
+  obs_s[tile + k] = tl;
+  obs_s[2 * tile + k] = vh;
+  obs_s[3 * tile + k] = vl;
+  obs_s[4 * tile + k] = wk;
+  return far_time(th);
+}
+
+// The CTA's shared memory.
+template <int J>
+struct WarpSmem {
+  float *tab, *gam, *obs, *red;
+  PlanetP *pl;
+  __device__ __forceinline__ WarpSmem(unsigned char *smem, int spr, int tile, int nwarps) {
+    const WarpLayout L(spr, J, tile, nwarps);
+    tab = reinterpret_cast<float *>(smem + L.tab);
+    pl = reinterpret_cast<PlanetP *>(smem + L.pl);
+    gam = reinterpret_cast<float *>(smem + L.gam);
+    obs = reinterpret_cast<float *>(smem + L.obs);
+    red = reinterpret_cast<float *>(smem + L.red);
+  }
+};
+
+// The CTA's systems, one per G lanes, once the first tile is staged: all tiles'
+// sums, their combination, the results.  poison: NaN for an invalid system.  WIDE:
+// plain and te as in wide_systems.  The short and the wide form part before
+// it and do not meet again: joined after each tile, the wide body's registers cost
+// the short one's 1 to 4 %.
+template <int J, bool RESID, bool DEMC, bool WIDE>
+__device__ __forceinline__ void systems(const UniformArgs &a, unsigned char *smem, int lg, int tile,
+                                        int ntiles, float *out, float *resid_out, bool plain,
+                                        const double *te, float gam,
+                                        float poison) {
+  const int block = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G = 1 << lg, spr = block >> lg, step = G * kChunk;
+  const WarpSmem<J> m(smem, spr, tile, block >> 5);
+  int slot = tid >> lg;
+  if (!dbg_ok(a.invalid, slot < spr, kDbgSmem, slot)) slot = 0;
+  const int c = tid & (G - 1);                   // the thread's place in its system
+  const int64_t s = (int64_t)blockIdx.x * spr + slot;
+  const PlanetP *q = m.pl + slot * J;
+  Kahan2 acc2 = {0, 0};
+  float rmax = 0.0f;
+
+  for (int t = 0; t < ntiles; ++t) {
+    const int k0 = t * tile;
+    const int nk = min(tile, a.n_obs - k0);
+    const int npad = round_up_pow2(nk, step);
+    if (t > 0) {
+      __syncthreads();
+      const Split3 tr3 = split3(a.t[0]);
+      const float jit2 = d2f(a.jitter2);
+      for (int k = tid; k < npad; k += block) {
+        const bool real = k < nk && dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k);
+        stage_obs(m.obs, tile, k, real, real ? a.t[k0 + k] : 0.0, real ? a.v[k0 + k] : 0.0,
+                  real ? a.sigma[k0 + k] : 1.0, tr3, jit2, plain, a.invalid);
+      }
+      __syncthreads();
+    }
+    if constexpr (WIDE)
+      warp_tile_sum<J, RESID, true>(m.obs, tile, q, m.tab, gam, c, lg, npad, nk, acc2, rmax,
+                                    a.invalid, te, k0, a.n_obs);
+    else
+      warp_tile_sum<J, RESID, false>(m.obs, tile, q, m.tab, gam, c, lg, npad, nk, acc2, rmax,
+                                     a.invalid);
+  }
+  Kahan acc = kahan_join(acc2);
+
+  // combine the system's lanes within each of its warps (G a power of two)
+  for (int d = (G < 32 ? G : 32) >> 1; d >= 1; d >>= 1) {
+    Kahan o = {shfl_xor(acc.big, d), shfl_xor(acc.small, d)};
+    kahan_merge(acc, o);
+    if (RESID) rmax = fmaxf(rmax, shfl_xor(rmax, d));
+  }
+  if (G > 32) {
+    // then its G / 32 warps, in warp order, through shared memory (lg is
+    // the same for the whole CTA, so every thread reaches the barrier)
+    float *red_s = m.red;
+    if (lane == 0) {
+      red_s[3 * warp] = acc.big;
+      red_s[3 * warp + 1] = acc.small;
+      red_s[3 * warp + 2] = rmax;
+    }
+    __syncthreads();
+    if (c == 0) {
+      for (int w = warp + 1; w < warp + (G >> 5); ++w) {
+        if (!dbg_ok(a.invalid, w < (block >> 5), kDbgSmem, w)) break;
+        const Kahan o = {red_s[3 * w], red_s[3 * w + 1]};
+        kahan_merge(acc, o);
+        rmax = fmaxf(rmax, red_s[3 * w + 2]);
+      }
+    }
+  }
+  if (c == 0 && s < a.n_sys) {
+    const float value = kahan_value(acc) + poison;   // NaN survives n_obs == 0
+    out[s] = value;
+    note_invalid(a.invalid, value);
+    if (RESID) resid_out[s] = rmax;
+    // the proposals this CTA formed are visible here after the barrier
+    if (DEMC) demc_accept<5 * J + 1>(a, s, value);
+  }
+}
+
+// The systems of a CTA with a period or a time outside the short mean anomaly's
+// range; far: one of the thread's times is.  All threads of the CTA call it.
+template <int J, bool RESID, bool DEMC>
+__device__ __forceinline__ void wide_systems(const UniformArgs &a, unsigned char *smem, int lg,
+                                             int tile, int ntiles, float *out, float *resid_out,
+                                             bool far, float gam, float poison) {
+  const int block = blockDim.x, tid = threadIdx.x, spr = block >> lg;
+  const int64_t sys0 = (int64_t)blockIdx.x * spr;
+  const WarpSmem<J> m(smem, spr, tile, block >> 5);
+  const bool plain = __syncthreads_or(far);
+  if (plain) {
+    // the planets and the first tile's times as plain pairs
+    for (int i = tid; i < spr * J; i += block) {
+      const int64_t at = (sys0 + i / J) * (5 * J + 1) + 5 * (i % J);
+      if (sys0 + i / J < a.n_sys && dbg_ok(a.invalid, at < a.n_sys * (5 * J + 1), kDbgParam, at))
+        planet_plain(m.pl[i], a.params[at]);
+    }
+    const Split3 tr3 = split3(a.t[0]);
+    for (int k = tid; k < min(tile, a.n_obs); k += block)
+      sub_ds(split3(a.t[k]), tr3, m.obs[k], m.obs[tile + k]);
+    __syncthreads();
+  }
+  int slot = tid >> lg;
+  if (!dbg_ok(a.invalid, slot < spr, kDbgSmem, slot)) slot = 0;
+  float n_max = 0.0f;                            // the system's shortest period
+#pragma unroll
+  for (int j = 0; j < J; ++j) n_max = fmaxf(n_max, m.pl[slot * J + j].n);
+  systems<J, RESID, DEMC, true>(a, smem, lg, tile, ntiles, out, resid_out, plain,
+                                n_max > kPairExactFreq ? a.t : nullptr, gam, poison);
+}
+
 // RESID: also the per-system max Kepler residual.  DEMC: the batch is a
 // DE-MC step's proposals (a.demc): formed in the prologue, Metropolis
 // decision in the epilogue; plain evaluations contain neither.
@@ -220,14 +380,12 @@ chi2_mixed_warp_kernel(UniformArgs a, int lg, int tile, int ntiles, float *__res
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int block = blockDim.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const int G = 1 << lg;
   const int spr = block >> lg;                   // systems of this CTA
-  const WarpLayout L(spr, J, tile, block >> 5);
-  float *tab_s = reinterpret_cast<float *>(smem + L.tab);
-  PlanetP *pl_s = reinterpret_cast<PlanetP *>(smem + L.pl);
-  float *gam_s = reinterpret_cast<float *>(smem + L.gam);
-  float *obs_s = reinterpret_cast<float *>(smem + L.obs);
+  const WarpSmem<J> m(smem, spr, tile, block >> 5);
+  float *tab_s = m.tab, *gam_s = m.gam, *obs_s = m.obs;
+  PlanetP *pl_s = m.pl;
 
   const int64_t sys0 = (int64_t)blockIdx.x * spr;
   const int nitems = spr * (J + 1);
@@ -252,31 +410,9 @@ chi2_mixed_warp_kernel(UniformArgs a, int lg, int tile, int ntiles, float *__res
 
   // the reference time's split, needed by the threads that stage
   Split3 tr3 = {0.0f, 0.0f, 0.0f};
-  if (ob < npad0 || ntiles > 1) tr3 = split3(t_ref);
+  if (ob < npad0) tr3 = split3(t_ref);
   const float jit2 = d2f(a.jitter2);
-  // tau = t - t_ref as (th, tl) and v as float pairs, w = 1/(sigma^2 +
-  // jitter^2); the padding up to whole chunks has zero weight (and tau = v =
-  // 0).  Returns whether the time asks for the wide mean anomaly.
-  auto convert = [&](int k, bool real, double t, double v, double sigma) {
-    if (!dbg_ok(a.invalid, k < tile, kDbgSmem, k)) return false;
-    float th = 0.0f, tl = 0.0f, vh = 0.0f, vl = 0.0f, wk = 0.0f;
-    if (real) {
-      sub_ds(split3(t), tr3, th, tl);
-      tau_place(th, tl);
-      split_d(v, vh, vl);
-      const float sg = d2f(sigma);
-      const float var = __fmaf_rn(sg, sg, jit2);
-      wk = var > 0.0f ? 1.0f / var : __int_as_float(0x7fc00000);
-    }
-    obs_s[k] = th;
-    obs_s[tile + k] = tl;
-    obs_s[2 * tile + k] = vh;
-    obs_s[3 * tile + k] = vl;
-    obs_s[4 * tile + k] = wk;
-    return !(fabsf(th) < kPairMaxTau);
-  };
-
-  bool wide = false;
+  bool far = false, wide = false;
   if (tid < nitems)
     wide = setup_item<J>(tid, spr, sys0, a.n_sys, p, t_ref, a.t0, pl_s, gam_s, a.invalid);
   for (int i = tid + block; i < nitems; i += block) {       // more items than threads
@@ -284,83 +420,29 @@ chi2_mixed_warp_kernel(UniformArgs a, int lg, int tile, int ntiles, float *__res
     load_item<J, DEMC>(i, spr, sys0, a, q);
     wide |= setup_item<J>(i, spr, sys0, a.n_sys, q, t_ref, a.t0, pl_s, gam_s, a.invalid);
   }
-  if (ob < npad0) wide |= convert(ob, has0, t0v, v0v, s0v);
-  if (ob + block < npad0) wide |= convert(ob + block, has1, t1v, v1v, s1v);
+  if (ob < npad0)
+    far |= stage_obs(obs_s, tile, ob, has0, t0v, v0v, s0v, tr3, jit2, false, a.invalid);
+  if (ob + block < npad0)
+    far |= stage_obs(obs_s, tile, ob + block, has1, t1v, v1v, s1v, tr3, jit2, false, a.invalid);
   for (int k = ob + 2 * block; k < npad0; k += block) {
     const bool real = k < nk0 && dbg_ok(a.invalid, k < a.n_obs, kDbgObs, k);
-    wide |= convert(k, real, real ? a.t[k] : 0.0, real ? a.v[k] : 0.0, real ? a.sigma[k] : 1.0);
+    far |= stage_obs(obs_s, tile, k, real, real ? a.t[k] : 0.0, real ? a.v[k] : 0.0,
+                     real ? a.sigma[k] : 1.0, tr3, jit2, false, a.invalid);
   }
-  wide = __syncthreads_or(wide);
+  if (ntiles > 1) far |= far_later(a.t, tile, a.n_obs);
+  wide = __syncthreads_or(wide || far);
 
-  // ---- the CTA's systems, one per G lanes ----
   int slot = tid >> lg;
   if (!dbg_ok(a.invalid, slot < spr, kDbgSmem, slot)) slot = 0;
-  const int c = tid & (G - 1);                   // the thread's place in its system
-  const int64_t s = sys0 + slot;
-  const PlanetP *q = pl_s + slot * J;
   const float gam = gam_s[slot];
   float poison = 0.0f * gam;                     // NaN for an invalid system
 #pragma unroll
-  for (int j = 0; j < J; ++j) poison += 0.0f * q[j].e;
-  Kahan2 acc2 = {0, 0};
-  float rmax = 0.0f;
-
-  for (int t = 0; t < ntiles; ++t) {
-    const int k0 = t * tile;
-    const int nk = min(tile, a.n_obs - k0);
-    const int npad = round_up_pow2(nk, step);
-    if (t > 0) {
-      __syncthreads();
-      bool far = false;
-      for (int k = tid; k < npad; k += block) {
-        const bool real = k < nk && dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k);
-        far |= convert(k, real, real ? a.t[k0 + k] : 0.0, real ? a.v[k0 + k] : 0.0,
-                       real ? a.sigma[k0 + k] : 1.0);
-      }
-      wide |= (bool)__syncthreads_or(far);
-    }
-    if (wide)
-      warp_tile_sum<J, RESID, true>(obs_s, tile, q, tab_s, gam, c, lg, npad, nk, acc2, rmax,
-                                    a.invalid);
-    else
-      warp_tile_sum<J, RESID, false>(obs_s, tile, q, tab_s, gam, c, lg, npad, nk, acc2, rmax,
-                                     a.invalid);
-  }
-  Kahan acc = kahan_join(acc2);
-
-  // combine the system's lanes within each of its warps (G a power of two)
-  for (int m = (G < 32 ? G : 32) >> 1; m >= 1; m >>= 1) {
-    Kahan o = {shfl_xor(acc.big, m), shfl_xor(acc.small, m)};
-    kahan_merge(acc, o);
-    if (RESID) rmax = fmaxf(rmax, shfl_xor(rmax, m));
-  }
-  if (G > 32) {
-    // then its G / 32 warps, in warp order, through shared memory (lg is
-    // the same for the whole CTA, so every thread reaches the barrier)
-    float *red_s = reinterpret_cast<float *>(smem + L.red);
-    if (lane == 0) {
-      red_s[3 * warp] = acc.big;
-      red_s[3 * warp + 1] = acc.small;
-      red_s[3 * warp + 2] = rmax;
-    }
-    __syncthreads();
-    if (c == 0) {
-      for (int w = warp + 1; w < warp + (G >> 5); ++w) {
-        if (!dbg_ok(a.invalid, w < (block >> 5), kDbgSmem, w)) break;
-        const Kahan o = {red_s[3 * w], red_s[3 * w + 1]};
-        kahan_merge(acc, o);
-        rmax = fmaxf(rmax, red_s[3 * w + 2]);
-      }
-    }
-  }
-  if (c == 0 && s < a.n_sys) {
-    const float value = kahan_value(acc) + poison;   // NaN survives n_obs == 0
-    out[s] = value;
-    note_invalid(a.invalid, value);
-    if (RESID) resid_out[s] = rmax;
-    // the proposals this CTA formed are visible here after the barrier
-    if (DEMC) demc_accept<5 * J + 1>(a, s, value);
-  }
+  for (int j = 0; j < J; ++j) poison += 0.0f * pl_s[slot * J + j].e;
+  if (wide)
+    wide_systems<J, RESID, DEMC>(a, smem, lg, tile, ntiles, out, resid_out, far, gam, poison);
+  else
+    systems<J, RESID, DEMC, false>(a, smem, lg, tile, ntiles, out, resid_out, false, nullptr,
+                                   gam, poison);
 }
 
 // Variants: 0 plain, 1 with the Kepler residual, 2 DE-MC step.

@@ -713,6 +713,21 @@ __device__ __forceinline__ void phase_setup_ds(double P, double M0, double t_ref
   fast_two_sum(sc, __fadd_rn(__fadd_rn(t_small, ml), se), c_hi, c_lo);
 }
 
+// 1/P alone, as phase_setup_ds forms it.
+__device__ __forceinline__ void frequency_ds(double P, float &n_hi, float &n_lo) {
+  const Split3 Ps = split3(P);
+  if (!(Ps.x0 >= 0x1p-20f && Ps.x0 <= 0x1p40f)) {
+    float c_hi, c_lo;
+    phase_setup_wide(P, 0.0, 0.0, 0.0, n_hi, n_lo, c_hi, c_lo);
+    return;
+  }
+  const float r = rcp_fast(Ps.x0);
+  float pr, pre;
+  two_prod(Ps.x0, r, pr, pre);
+  const float x = __fmaf_rn(-Ps.x1, r, __fsub_rn(__fsub_rn(1.0f, pr), pre));
+  fast_two_sum(r, r * __fmaf_rn(x, x, x), n_hi, n_lo);
+}
+
 // Single-precision constants of one planet for the mixed path.
 // t_ref: the reference time the observation times are taken from; t0: the
 // epoch of M0.

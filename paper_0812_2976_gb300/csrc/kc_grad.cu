@@ -209,15 +209,14 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
   const float jit2 = d2f(a.jitter2);
   ang_tab_load<true>(tab_s, tid, block);
 
-  bool wide = false;
+  bool wide = false, plain = false;
   for (int i = tid; i < ST * J; i += block) {
     const int sl = i / J, j = i - sl * J;
     const int64_t s = sys0 + sl;
     GradPlanetP q = {};
     if (s < a.n_sys && dbg_ok(a.invalid, s * NP + 5 * j + 4 < a.n_sys * NP, kDbgParam, s * NP)) {
-      bool far;
-      q = grad_setup_pair(a.params + s * NP + 5 * j, t_ref, a.t0, far);
-      wide |= far;
+      q = grad_setup_pair(a.params + s * NP + 5 * j, t_ref, a.t0, false);
+      wide |= short_period(q.p);
     }
     pl_s[i] = q;
   }
@@ -226,27 +225,18 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
     gam_s[i] = s < a.n_sys ? d2f(system_gamma_g(a.params + s * NP, J)) : 0.0f;
   }
 
-  const int sl = tid / G, c = tid - sl * G;
-  const int64_t s = sys0 + sl;
-  const GradPlanetP *q = pl_s + sl * J;
-  Kahan2 acc = {0, 0};
-  f32x2 sum_a = 0;
-  typename GradSumsFor<J>::type g[J];
-#pragma unroll
-  for (int j = 0; j < J; ++j) g[j] = {{0, 0}, 0, 0, 0, 0};
-
-  for (int k0 = 0; k0 < a.n_obs; k0 += obs_tile) {
-    const int nk = min(obs_tile, a.n_obs - k0);
-    const int npad = grad_tile(nk, G);
-    if (k0 > 0) __syncthreads();
-    // the padding has zero weight
+  // the tile that starts at k0; the padding has zero weight; plain: the times
+  // stay as they are.  Returns whether one is a far one.
+  auto stage = [&](int k0) {
+    const int nk = min(obs_tile, a.n_obs - k0), npad = grad_tile(nk, G);
+    bool far = false;
     for (int k = block - 1 - tid; k < npad; k += block) {
       float th = 0.0f, tl = 0.0f, vh = 0.0f, vl = 0.0f, wk = 0.0f, dt = 0.0f;
       if (k < nk && dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k)) {
         sub_ds(split3(a.t[k0 + k]), tr3, th, tl);
         dt = th + dref_f;
-        tau_place(th, tl);
-        wide |= !(fabsf(th) < kPairMaxTau);
+        if (!plain) tau_place(th, tl);
+        far |= far_time(th);
         split_d(a.v[k0 + k], vh, vl);
         const float sg = d2f(a.sigma[k0 + k]);
         const float var = __fmaf_rn(sg, sg, jit2);
@@ -259,10 +249,53 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
       obs_s[4 * tile + k] = wk;
       obs_s[5 * tile + k] = dt;
     }
-    wide = __syncthreads_or(wide);
+    return far;
+  };
+  bool far = stage(0);
+  if (a.n_obs > obs_tile) far |= far_later(a.t, obs_tile, a.n_obs);
+  wide = __syncthreads_or(wide || far);
+
+  const int sl = tid / G, c = tid - sl * G;
+  const int64_t s = sys0 + sl;
+  const GradPlanetP *q = pl_s + sl * J;
+
+  // all tiles' sums, their combination, the results (compiled twice from here on,
+  // so that the short form keeps its registers)
+  with_high_e(wide, [&](auto tag) {
+    constexpr bool WIDE = decltype(tag)::value;
+    bool exact = false;
+    if (WIDE) {
+      plain = __syncthreads_or(far);
+      if (plain) {
+        // the planets and the first tile's times as plain pairs
+        for (int i = tid; i < ST * J; i += block) {
+          const int64_t at = (sys0 + i / J) * NP + 5 * (i % J);
+          if (sys0 + i / J < a.n_sys && dbg_ok(a.invalid, at < a.n_sys * NP, kDbgParam, at))
+            planet_plain(pl_s[i].p, a.params[at]);
+        }
+        for (int k = tid; k < min(obs_tile, a.n_obs); k += block)
+          sub_ds(split3(a.t[k]), tr3, obs_s[k], obs_s[tile + k]);
+        __syncthreads();
+      }
+      float n_max = 0.0f;                        // the system's shortest period
+#pragma unroll
+      for (int j = 0; j < J; ++j) n_max = fmaxf(n_max, q[j].p.n);
+      exact = n_max > kPairExactFreq;
+    }
     const float gam = gam_s[sl];
-    with_high_e(wide, [&](auto tag) {
-      constexpr bool WIDE = decltype(tag)::value;
+    Kahan2 acc = {0, 0};
+    f32x2 sum_a = 0;
+    typename GradSumsFor<J>::type g[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) g[j] = {{0, 0}, 0, 0, 0, 0};
+
+    for (int k0 = 0; k0 < a.n_obs; k0 += obs_tile) {
+      if (k0 > 0) {
+        __syncthreads();
+        stage(k0);
+        __syncthreads();
+      }
+      const int npad = grad_tile(min(obs_tile, a.n_obs - k0), G);
       for (int k = 2 * c; k < npad; k += 2 * G) {
         // the planets' constants are read again in every iteration: hoisted
         // for all J planets they would not fit the registers
@@ -270,7 +303,8 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
         auto at = [&](int array) {
           return *reinterpret_cast<const f32x2 *>(obs_s + array * tile + k);
         };
-        const f32x2 th = at(0), tl = at(1);
+        f32x2 th = at(0), tl = at(1);
+        if (WIDE && exact) plain_times(a.t, k0 + k, a.n_obs, th, tl);
         GradTerms o[J];
         Kahan2 V = {dup2(gam), 0};
 #pragma unroll
@@ -283,33 +317,32 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
 #pragma unroll
         for (int j = 0; j < J; ++j) grad_add(g[j], o[j], q[j], a2, adt);
       }
-    });
-  }
-  if (a.n_obs == 0) __syncthreads();            // gam_s, pl_s written by other threads
+    }
 
-  Kahan chi = kahan_join(acc);
-  float sa = join2(sum_a);
-  GradLane gl[J];
+    Kahan chi = kahan_join(acc);
+    float sa = join2(sum_a);
+    GradLane gl[J];
 #pragma unroll
-  for (int j = 0; j < J; ++j) gl[j] = grad_join(g[j]);
-  for (int m = G >> 1; m >= 1; m >>= 1) {
-    const Kahan o = {shfl_xor(chi.big, m), shfl_xor(chi.small, m)};
-    kahan_merge(chi, o);
-    sa += shfl_xor(sa, m);
+    for (int j = 0; j < J; ++j) gl[j] = grad_join(g[j]);
+    for (int m = G >> 1; m >= 1; m >>= 1) {
+      const Kahan o = {shfl_xor(chi.big, m), shfl_xor(chi.small, m)};
+      kahan_merge(chi, o);
+      sa += shfl_xor(sa, m);
 #pragma unroll
-    for (int j = 0; j < J; ++j) grad_combine(gl[j], m);
-  }
-  if (c == 0 && s < a.n_sys) {
-    // NaN for an invalid system
-    const float poison = 0.0f * gam_s[sl];
-    const float value = kahan_value(chi) + poison;
-    if (chi2_out) chi2_out[s] = value;
-    note_invalid(a.invalid, value);
-    float *out = grad_out + s * NP;
+      for (int j = 0; j < J; ++j) grad_combine(gl[j], m);
+    }
+    if (c == 0 && s < a.n_sys) {
+      // NaN for an invalid system
+      const float poison = 0.0f * gam_s[sl];
+      const float value = kahan_value(chi) + poison;
+      if (chi2_out) chi2_out[s] = value;
+      note_invalid(a.invalid, value);
+      float *out = grad_out + s * NP;
 #pragma unroll
-    for (int j = 0; j < J; ++j) grad_finish(gl[j], q[j], sa, poison, out + 5 * j);
-    out[5 * J] = sa + poison;
-  }
+      for (int j = 0; j < J; ++j) grad_finish(gl[j], q[j], sa, poison, out + 5 * j);
+      out[5 * J] = sa + poison;
+    }
+  });
 }
 
 // One observation per lane at a time, in scalar single precision: the
@@ -732,17 +765,19 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const unsigned (&a)[4],
 
 // The observations of one tile staged for the Gauss-Newton kernels: five
 // arrays of STRIDE floats (th, tl, v hi, v lo, sqrt w), padded with zero weight
-// to whole batches.  Returns whether a time asks for the wide mean anomaly.
+// to whole batches.  plain: the times stay as they are.  Returns whether one is
+// a far one.
 template <int STRIDE>
 __device__ __forceinline__ bool gn_stage(const UniformArgs &a, int k0, int nk, int npad, int tid,
-                                         int nthreads, const Split3 &tr3, float jit2, float *obs) {
-  bool wide = false;
+                                         int nthreads, const Split3 &tr3, float jit2, bool plain,
+                                         float *obs) {
+  bool far = false;
   for (int k = tid; k < npad; k += nthreads) {
     float th = 0.0f, tl = 0.0f, vh = 0.0f, vl = 0.0f, wk = 0.0f;
     if (k < nk && dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k)) {
       sub_ds(split3(a.t[k0 + k]), tr3, th, tl);
-      tau_place(th, tl);
-      wide |= !(fabsf(th) < kPairMaxTau);
+      if (!plain) tau_place(th, tl);
+      far |= far_time(th);
       split_d(a.v[k0 + k], vh, vl);
       const float sg = d2f(a.sigma[k0 + k]);
       const float var = __fmaf_rn(sg, sg, jit2);
@@ -752,18 +787,53 @@ __device__ __forceinline__ bool gn_stage(const UniformArgs &a, int k0, int nk, i
 #pragma unroll
     for (int i = 0; i < 5; ++i) obs[i * STRIDE + k] = v[i];
   }
-  return wide;
+  return far;
+}
+
+// What the Gauss-Newton kernels know before their first system: whether any time
+// is a far one (then the times and every 1/P are plain pairs), the observations
+// staged where they fit one tile.  Contains barriers.
+template <int TILE, int ROWS>
+__device__ __forceinline__ bool gn_prepare(const UniformArgs &a, bool staged_once, int tid,
+                                           int nthreads, const Split3 &tr3, float jit2,
+                                           float *obs) {
+  const int npad = (a.n_obs + ROWS - 1) / ROWS * ROWS;
+  bool far = false;
+  if (staged_once) {
+    far = gn_stage<TILE>(a, 0, a.n_obs, npad, tid, nthreads, tr3, jit2, false, obs);
+  } else {
+    for (int k = tid; k < a.n_obs; k += nthreads) {
+      float th, tl;
+      sub_ds(split3(a.t[k]), tr3, th, tl);
+      tau_place(th, tl);
+      far |= far_time(th);
+    }
+  }
+  far = __syncthreads_or(far);
+  if (far && staged_once) {
+    for (int k = tid; k < a.n_obs; k += nthreads)
+      sub_ds(split3(a.t[k]), tr3, obs[k], obs[TILE + k]);
+    __syncthreads();
+  }
+  return far;
 }
 
 // One pair of observations of a lane (columns k, k + 1 of the staged tile):
 // chi2 and gradient sums, and the rows of sqrt(w) J over their factors.
-// dref = t_ref - t0.
+// dref = t_ref - t0; k0: the tile's first observation.
 template <int J, int STRIDE, bool WIDE>
-__device__ __forceinline__ void gn_pair(const float *obs, int k, float dref, const GradPlanetP *q,
+__device__ __forceinline__ void gn_pair(const UniformArgs &a, const float *obs, int k0, int k,
+                                        float dref, const GradPlanetP *q,
                                         const float *tab, float gam, Kahan2 &acc, f32x2 &sum_a,
                                         GradSums (&g)[J], f32x2 (&u)[5 * J + 1]) {
   auto at = [&](int array) { return *reinterpret_cast<const f32x2 *>(obs + array * STRIDE + k); };
-  const f32x2 th = at(0), tl = at(1);
+  f32x2 th = at(0), tl = at(1);
+  if (WIDE) {
+    float n_max = 0.0f;
+#pragma unroll
+    for (int j = 0; j < J; ++j) n_max = fmaxf(n_max, q[j].p.n);
+    if (n_max > kPairExactFreq) plain_times(a.t, k0 + k, a.n_obs, th, tl);
+  }
   GradTerms o[J];
   Kahan2 V = {dup2(gam), 0};
 #pragma unroll
@@ -786,25 +856,27 @@ __device__ __forceinline__ void gn_pair(const float *obs, int k, float dref, con
 // set if lane l's planet asks for the wide mean anomaly.
 template <int J>
 __device__ __forceinline__ float gn_setup_ahead(const UniformArgs &a, int64_t s0, int64_t stride,
-                                                int lane, double t_ref, GradPlanetP *q,
-                                                unsigned &wide) {
+                                                int lane, double t_ref, bool plain,
+                                                GradPlanetP *q, unsigned &wide) {
   static_assert(kGnAhead * J <= 16, "planets in lanes 0 .. 15, gamma from lane 16");
   constexpr int NP = 5 * J + 1;
-  bool far = false;
+  bool brief = false;
   float gam = 0.0f;
   __syncwarp();                                        // the last systems' use of q
   if (lane < kGnAhead * J) {
     const int i = lane / J, j = lane - i * J;
     const int64_t s = s0 + i * stride;
     GradPlanetP p = {};
-    if (s < a.n_sys && dbg_ok(a.invalid, s * NP + 5 * j + 4 < a.n_sys * NP, kDbgParam, s * NP))
-      p = grad_setup_pair(a.params + s * NP + 5 * j, t_ref, a.t0, far);
+    if (s < a.n_sys && dbg_ok(a.invalid, s * NP + 5 * j + 4 < a.n_sys * NP, kDbgParam, s * NP)) {
+      p = grad_setup_pair(a.params + s * NP + 5 * j, t_ref, a.t0, plain);
+      brief = short_period(p.p);
+    }
     q[lane] = p;
   } else if (lane >= 16 && lane < 16 + kGnAhead) {
     const int64_t s = s0 + (lane - 16) * stride;
     if (s < a.n_sys) gam = d2f(system_gamma_g(a.params + s * NP, J));
   }
-  wide = __ballot_sync(0xffffffffu, far);
+  wide = __ballot_sync(0xffffffffu, brief);
   return gam;
 }
 
@@ -1074,11 +1146,7 @@ gn_pair_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__ 
     u_all[i] = make_float2(0.0f, 0.0f);                           // incl. padding
   // observations that fit one tile are staged once for all of the CTA's systems
   const bool staged_once = a.n_obs <= kTile;
-  bool far = false;
-  if (staged_once)
-    far = gn_stage<kTile>(a, 0, a.n_obs, (a.n_obs + kGnRows - 1) / kGnRows * kGnRows, tid, block,
-                          tr3, jit2, obs_s);
-  far = __syncthreads_or(far);
+  const bool plain = gn_prepare<kTile, kGnRows>(a, staged_once, tid, block, tr3, jit2, obs_s);
 
   // The (hi, lo) pair of element (row r, column c) of U sits at
   // r * ROW2 + (c ^ ((r >> 2) & 3)): with ROW2 = 4 mod 16 both the row writes
@@ -1096,11 +1164,11 @@ gn_pair_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__ 
   for (int64_t s = (int64_t)blockIdx.x * kGnWarps + warp; s - warp < a.n_sys; s += stride) {
     if (ahead_i == kGnAhead) {
       ahead_i = 0;
-      gam_ahead = gn_setup_ahead<J>(a, s, stride, lane, t_ref, ahead, wide_ahead);
+      gam_ahead = gn_setup_ahead<J>(a, s, stride, lane, t_ref, plain, ahead, wide_ahead);
     }
     const GradPlanetP *q = ahead + ahead_i * J;
     const float gam = __shfl_sync(0xffffffffu, gam_ahead, 16 + ahead_i);
-    bool wide = far || ((wide_ahead >> (ahead_i * J)) & ((1u << J) - 1u)) != 0u;
+    const bool wide = plain || ((wide_ahead >> (ahead_i * J)) & ((1u << J) - 1u)) != 0u;
     ++ahead_i;
     __syncwarp();
     Kahan2 acc = {0, 0};
@@ -1121,18 +1189,18 @@ gn_pair_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__ 
       const int npad = (nk + kGnRows - 1) / kGnRows * kGnRows;
       if (!staged_once) {
         __syncthreads();
-        const bool w = gn_stage<kTile>(a, k0, nk, npad, tid, block, tr3, jit2, obs_s);
-        wide |= (bool)__syncthreads_or(w);
+        gn_stage<kTile>(a, k0, nk, npad, tid, block, tr3, jit2, plain, obs_s);
+        __syncthreads();
       }
       for (int kb = 0; kb < npad; kb += kGnRows) {
         {
           f32x2 urow[NP];
           if (wide)
-            gn_pair<J, kTile, true>(obs_s, kb + 2 * lane, dref_f, q, tab_s, gam, acc, sum_a, g,
-                                    urow);
+            gn_pair<J, kTile, true>(a, obs_s, k0, kb + 2 * lane, dref_f, q, tab_s, gam, acc,
+                                    sum_a, g, urow);
           else
-            gn_pair<J, kTile, false>(obs_s, kb + 2 * lane, dref_f, q, tab_s, gam, acc, sum_a, g,
-                                     urow);
+            gn_pair<J, kTile, false>(a, obs_s, k0, kb + 2 * lane, dref_f, q, tab_s, gam, acc,
+                                     sum_a, g, urow);
 #pragma unroll
           for (int i = 0; i < NP; ++i) {
             u[lane * ROW2 + (i ^ sw_row)] = tf32_pair(lo2(urow[i]));
@@ -1312,12 +1380,9 @@ gn_mixed_tc_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restric
   ang_tab_load<true>(tab_s, tid, kThreads);
   // observations that fit one tile are staged once for all of the CTA's systems
   const bool staged_once = a.n_obs <= kTcObsTile;
-  bool far = false;
-  if (staged_once)
-    far = gn_stage<kTcObsTile>(a, 0, a.n_obs, (a.n_obs + kTcBatch - 1) / kTcBatch * kTcBatch, tid,
-                               kThreads, tr3, jit2, obs_s);
   tc::fence_before_sync();
-  far = __syncthreads_or(far);
+  const bool plain =
+      gn_prepare<kTcObsTile, kTcBatch>(a, staged_once, tid, kThreads, tr3, jit2, obs_s);
   tc::fence_after_sync();
   const uint32_t taddr = *slot;
 
@@ -1342,11 +1407,11 @@ gn_mixed_tc_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restric
   for (int64_t s = (int64_t)blockIdx.x * kGnWarps + warp; s - warp < a.n_sys; s += stride) {
     if (ahead_i == kGnAhead) {
       ahead_i = 0;
-      gam_ahead = gn_setup_ahead<J>(a, s, stride, lane, t_ref, ahead, wide_ahead);
+      gam_ahead = gn_setup_ahead<J>(a, s, stride, lane, t_ref, plain, ahead, wide_ahead);
     }
     const GradPlanetP *q = ahead + ahead_i * J;
     const float gam = __shfl_sync(0xffffffffu, gam_ahead, 16 + ahead_i);
-    bool wide = far || ((wide_ahead >> (ahead_i * J)) & ((1u << J) - 1u)) != 0u;
+    const bool wide = plain || ((wide_ahead >> (ahead_i * J)) & ((1u << J) - 1u)) != 0u;
     ++ahead_i;
     __syncwarp();
     Kahan2 acc2 = {0, 0};
@@ -1361,17 +1426,17 @@ gn_mixed_tc_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restric
       const int npad = (nk + kTcBatch - 1) / kTcBatch * kTcBatch;
       if (!staged_once) {
         __syncthreads();
-        const bool w = gn_stage<kTcObsTile>(a, k0, nk, npad, tid, kThreads, tr3, jit2, obs_s);
-        wide |= (bool)__syncthreads_or(w);
+        gn_stage<kTcObsTile>(a, k0, nk, npad, tid, kThreads, tr3, jit2, plain, obs_s);
+        __syncthreads();
       }
       for (int kb = 0; kb < npad; kb += kTcBatch) {
         f32x2 u[NP];
         if (wide)
-          gn_pair<J, kTcObsTile, true>(obs_s, kb + 2 * lane, dref_f, q, tab_s, gam, acc2, sum_a, g,
-                                       u);
+          gn_pair<J, kTcObsTile, true>(a, obs_s, k0, kb + 2 * lane, dref_f, q, tab_s, gam, acc2,
+                                       sum_a, g, u);
         else
-          gn_pair<J, kTcObsTile, false>(obs_s, kb + 2 * lane, dref_f, q, tab_s, gam, acc2, sum_a,
-                                        g, u);
+          gn_pair<J, kTcObsTile, false>(a, obs_s, k0, kb + 2 * lane, dref_f, q, tab_s, gam, acc2,
+                                        sum_a, g, u);
         if (nb > 0 && ok)                  // the MMAs that read the tile before
           ok = warp_wait(bar_a, (nb - 1) & 1u, kTcWaitLimit, lane);
         gn_tc_store<NP>(my_rows, lane_q, u);

@@ -149,8 +149,14 @@ __device__ __forceinline__ void ang_tab_load(float *tab, int tid, int nthreads) 
 // ------------------------------------------------ observation times
 
 // tau = th + tl with th a multiple of 2^-6 d (or tau_hi itself from 2^17 d
-// on, whose last place is no finer) and |tl| <= 2^-7 d.
+// on, whose last place is no finer) and |tl| <= 2^-7 d, rounded to 2^-32 d and
+// finer (err: what it lost).
 constexpr float kTauPlace = 64.0f;
+__device__ __forceinline__ void tau_place(float &hi, float &lo, float &err) {
+  const float th = fabsf(hi) < 131072.0f ? rintf(hi * kTauPlace) * (1.0f / kTauPlace) : hi;
+  two_sum(__fsub_rn(hi, th), lo, lo, err);
+  hi = th;
+}
 __device__ __forceinline__ void tau_place(float &hi, float &lo) {
   const float th = fabsf(hi) < 131072.0f ? rintf(hi * kTauPlace) * (1.0f / kTauPlace) : hi;
   lo = __fadd_rn(__fsub_rn(hi, th), lo);
@@ -158,10 +164,45 @@ __device__ __forceinline__ void tau_place(float &hi, float &lo) {
 }
 
 // Limits of the short form of the mean anomaly (mean_anomaly_pair): 1/P up
-// to 2 cycles/d, |tau| below 2^14 d (45 years).  Beyond them a CTA takes
-// mean_anomaly_wide for all its systems.
+// to 2 cycles/d, |tau| below 2^14 d (45 years).  Beyond them the wide form
+// runs, and what the binary places would lose is kept:
+//  - a time beyond the limit: every time stays the plain pair (tau_hi, tau_lo),
+//    and every 1/P (n_hi, n_lo) (planet_plain).  Placed, 1/P is known to 2^-42
+//    cycles/d: 4.5e-7 rad (rms) in M at P = 3000 d and 1e6 d, 2e-4 where times
+//    and periods are given in seconds;
+//  - 1/P above the limit: that planet keeps the plain pair;
+//  - 1/P above kPairExactFreq: the system's times are read as plain pairs.
+//    Placed, they are known to 2^-33 d: 6.5e-7 rad at P = 1e-3 d (6e-9 at the
+//    limit).
+// So M is within 2e-7 rad (4e-8 to 8e-8 rms) wherever |tau/P| < 2^22.
 constexpr float kPairMaxFreq = 2.0f;
+constexpr float kPairExactFreq = 16.0f;
 constexpr float kPairMaxTau = 16384.0f;
+
+__device__ __forceinline__ bool far_time(float th) { return !(fabsf(th) < kPairMaxTau); }
+
+// Whether one of the thread's times beyond the first tile is a far one (out of
+// line: few batches have more than one tile).
+static __device__ __noinline__ bool far_later(const double *t, int tile, int n_obs) {
+  bool far = false;
+  for (int k = tile + threadIdx.x; k < n_obs; k += blockDim.x)
+    far |= !(fabs(t[k] - t[0]) < (double)kPairMaxTau);
+  return far;
+}
+
+// Observations k and k + 1 of t (n of them; the padding has tau = 0) as plain
+// pairs, for the rare systems of the last case: one FP64 subtraction each, on a pipe
+// that is idle otherwise (65536 x 4 x 256 with P in 0.001 .. 0.01 d: 188 us; the
+// float expansions of the staging, 100 instructions, took 239).
+__device__ __forceinline__ void plain_times(const double *t, int k, int n, f32x2 &th,
+                                            f32x2 &tl) {
+  const double t_ref = t[0];
+  float ah, al, bh, bl;
+  split_d(k < n ? t[k] - t_ref : 0.0, ah, al);
+  split_d(k + 1 < n ? t[k + 1] - t_ref : 0.0, bh, bl);
+  th = pack2(ah, bh);
+  tl = pack2(al, bl);
+}
 
 // ------------------------------------------------ per-planet constants
 
@@ -216,9 +257,9 @@ __device__ __forceinline__ StartP start_constants_fast(float e) {
   return start_from(e, a, a * is, 0.5f * r * (is * is * is));
 }
 
-// Phase: n = 1/P rounded; nq its multiple of 2^-17 (n itself above 2^6,
-// whose last place is no finer), nlo the rest; c a multiple of 2^-23, clo the
-// rest, both low parts and n2pi times 2 pi.  Start: st, above.
+// Phase: n = 1/P rounded; nq its multiple of 2^-17 (n itself in a plain pair),
+// nlo the rest; c a multiple of 2^-23, clo the rest, both low parts and n2pi
+// times 2 pi.  Start: st, above.
 // Velocity: v = (A cos E - B sin E)/(1 - e cos E), A = K cos w (1 - e^2),
 // B = K sqrt(1 - e^2) sin w.
 struct __align__(16) PlanetP {
@@ -242,22 +283,24 @@ __device__ __forceinline__ float product3(float x_hi, float x_lo, float y, float
   return __fmaf_rn(u, z, __fmaf_rn(x_lo, y, ue) * z);
 }
 
+// Whether a planet's period is too short for the short form.
+__device__ __forceinline__ bool short_period(const PlanetP &q) { return !(q.n <= kPairMaxFreq); }
+
 // Phase, start and orbit constants of one planet; the caller sets A and B.
-// An invalid planet gets e = NaN, which makes its velocities NaN.  wide: set
-// if the period is too short for the short form.
+// An invalid planet gets e = NaN, which makes its velocities NaN.  plain: 1/P
+// as a plain pair whatever its size.
 __device__ __forceinline__ PlanetP planet_setup_orbit(const double *p, double t_ref, double t0,
-                                                      bool &wide, OrbitF &o) {
+                                                      bool plain, OrbitF &o) {
   PlanetP q;
   float n_hi, n_lo, c_hi, c_lo;
   phase_setup_ds(p[0], p[4], t_ref, t0, n_hi, n_lo, c_hi, c_lo);
   constexpr float kPlaceN = 131072.0f, kPlaceC = 8388608.0f;          // 2^17, 2^23
   q.n = n_hi;
-  q.nq = n_hi < 64.0f ? rintf(n_hi * kPlaceN) * (1.0f / kPlaceN) : n_hi;
+  q.nq = n_hi <= kPairMaxFreq && !plain ? rintf(n_hi * kPlaceN) * (1.0f / kPlaceN) : n_hi;
   q.nlo2pi = __fadd_rn(__fsub_rn(n_hi, q.nq), n_lo) * kTwoPiF;
   q.c = rintf(c_hi * kPlaceC) * (1.0f / kPlaceC);
   q.clo2pi = __fadd_rn(__fsub_rn(c_hi, q.c), c_lo) * kTwoPiF;
   q.n2pi = n_hi * kTwoPiF;
-  wide = !(n_hi <= kPairMaxFreq);
   const float ef = d2f(p[2]);
   q.e = planet_valid(p[0], p[1], p[2], p[3], p[4]) ? ef : __int_as_float(0x7fc00000);
   q.st = start_constants(q.e);
@@ -274,14 +317,22 @@ __device__ __forceinline__ PlanetP planet_setup_orbit(const double *p, double t_
 }
 
 __device__ __forceinline__ PlanetP planet_setup_pair(const double *p, double t_ref, double t0,
-                                                     bool &wide) {
+                                                     bool plain) {
   OrbitF o;
-  PlanetP q = planet_setup_orbit(p, t_ref, t0, wide, o);
+  PlanetP q = planet_setup_orbit(p, t_ref, t0, plain, o);
   float K_hi, K_lo;
   split_d(p[1], K_hi, K_lo);
   q.A = product3(K_hi, K_lo, o.cw, o.b2);
   q.B = product3(K_hi, K_lo, o.sw, o.b);
   return q;
+}
+
+// 1/P of a planet that is set up, made a plain pair (a far time is known only
+// after the setup).
+__device__ __forceinline__ void planet_plain(PlanetP &q, double P) {
+  float n_lo;
+  frequency_ds(P, q.nq, n_lo);
+  q.nlo2pi = n_lo * kTwoPiF;
 }
 
 // The gradient's planet: A and B of the solve without K, and the constants
@@ -292,10 +343,10 @@ struct __align__(16) GradPlanetP {
 };
 
 __device__ __forceinline__ GradPlanetP grad_setup_pair(const double *p, double t_ref, double t0,
-                                                       bool &wide) {
+                                                       bool plain) {
   GradPlanetP g;
   OrbitF o;
-  g.p = planet_setup_orbit(p, t_ref, t0, wide, o);
+  g.p = planet_setup_orbit(p, t_ref, t0, plain, o);
   float e_hi, e_lo;
   split_d(p[2], e_hi, e_lo);
   g.p.ome = __fsub_rn(__fsub_rn(1.0f, e_hi), e_lo);
@@ -330,28 +381,33 @@ __device__ __forceinline__ f32x2 mean_anomaly_pair(f32x2 th, f32x2 tl, const Pla
   return fma2(u, dup2(kTwoPiF), lo);
 }
 
-// One observation at any period and time the double-single phase covers
-// (|tau/P| < 2^22): tau as the float pair of its leading 48 bits, the
-// product's FMA remainder kept, every part wrapped before the sum.
-__device__ __forceinline__ float mean_anomaly_wide(float th, float tl, const PlanetP &q) {
-  const float hi = __fadd_rn(th, tl);
-  const float lo = __fsub_rn(tl, __fsub_rn(hi, th));
-  const float p = __fmul_rn(hi, q.nq);
-  const float pe = __fmaf_rn(hi, q.nq, -p);
-  float lc = __fmaf_rn(lo, q.n, pe);
-  lc = __fadd_rn(lc, __fmaf_rn(hi, q.nlo2pi, q.clo2pi) * (float)kInvTwoPi);
-  lc = __fsub_rn(lc, round_small(lc));
-  float u = __fadd_rn(__fsub_rn(p, round_small(p)), q.c);
-  u = __fsub_rn(u, round_small(u));
-  u = __fsub_rn(u, round_small(__fadd_rn(u, lc)));
-  return __fmaf_rn(u, kTwoPiF, lc * kTwoPiF);
+__device__ __forceinline__ f32x2 round2(f32x2 x) {
+  return sub2(add2(x, dup2(kRoundMagic)), dup2(kRoundMagic));
+}
+
+// M at any period and time the double-single phase covers (|tau/P| < 2^22): tau
+// as the float pair of its leading 48 bits, the product's FMA remainder and the
+// sum's TwoSum remainder kept, every part wrapped before the last sum, 2 pi with
+// its own low part.  |M| <= 1.0001 pi.
+__device__ __forceinline__ f32x2 mean_anomaly_wide(f32x2 th, f32x2 tl, const PlanetP &q) {
+  const f32x2 hi = add2(th, tl), lo = sub2(tl, sub2(hi, th));
+  const f32x2 n = dup2(q.nq), p = mul2(hi, n), pe = fma2(hi, n, neg2(p));
+  f32x2 lc = fma2(lo, dup2(q.n), pe);
+  lc = fma2(fma2(hi, dup2(q.nlo2pi), dup2(q.clo2pi)), dup2((float)kInvTwoPi), lc);
+  lc = sub2(lc, round2(lc));
+  const f32x2 f = sub2(p, round2(p)), c = dup2(q.c);
+  f32x2 u = add2(f, c);
+  const f32x2 v = sub2(u, f);
+  lc = add2(lc, add2(sub2(f, sub2(u, v)), sub2(c, v)));
+  u = sub2(u, round2(u));
+  u = sub2(u, round2(add2(u, lc)));
+  constexpr float kTwoPiLo = (float)(kTwoPi - (double)kTwoPiF);
+  return fma2(u, dup2(kTwoPiF), fma2(u, dup2(kTwoPiLo), mul2(lc, dup2(kTwoPiF))));
 }
 
 template <bool WIDE>
 __device__ __forceinline__ f32x2 mean_anomaly2(f32x2 th, f32x2 tl, const PlanetP &q) {
-  if (WIDE)
-    return pack2(mean_anomaly_wide(lo2(th), lo2(tl), q), mean_anomaly_wide(hi2(th), hi2(tl), q));
-  return mean_anomaly_pair(th, tl, q);
+  return WIDE ? mean_anomaly_wide(th, tl, q) : mean_anomaly_pair(th, tl, q);
 }
 
 // ------------------------------------------------ Kepler's equation

@@ -50,6 +50,7 @@ struct kc_plan {
   int32_t *d_n_pl = nullptr;
   double *d_t_ref = nullptr;
   int32_t *d_far = nullptr;               // mixed: systems with far times
+  float2 *d_err = nullptr;                // mixed: see RaggedDev::tau_err
   void *d_obs_a = nullptr, *d_obs_b = nullptr;
   unsigned long long *d_queue = nullptr;  // kPlanMaxStreams counters
   bool obs_ready = false;
@@ -60,7 +61,7 @@ struct kc_plan {
 
   kc::RaggedDev dev() const {
     return kc::RaggedDev{d_obs_off, d_par_off, d_n_pl, d_order, d_t_ref, n_sys, t0,
-                         kc::invalid_counter(), d_far, n_obs, n_par};
+                         kc::invalid_counter(), d_far, d_err, n_obs, n_par};
   }
   void drop_graph() {
     for (PlanStream &ps : streams) ps.drop_graph();
@@ -81,7 +82,8 @@ struct kc_plan {
     if (cap_stream) cudaStreamDestroy(cap_stream);
     cap_stream = nullptr;
     for (void *p : {(void *)d_obs_off, (void *)d_par_off, (void *)d_order, (void *)d_n_pl,
-                    (void *)d_t_ref, (void *)d_far, d_obs_a, d_obs_b, (void *)d_queue})
+                    (void *)d_t_ref, (void *)d_far, (void *)d_err, d_obs_a, d_obs_b,
+                    (void *)d_queue})
       if (p) cudaFree(p);
   }
 };
@@ -240,7 +242,10 @@ kc_status kc_plan_create_ragged(kc_plan **plan, const int64_t *obs_off, const in
   alloc((void **)&p->d_order, sizeof(int64_t) * n_sys);
   alloc((void **)&p->d_n_pl, sizeof(int32_t) * n_sys);
   alloc((void **)&p->d_t_ref, sizeof(double) * n_sys);
-  if (mode == KC_MIXED) alloc((void **)&p->d_far, sizeof(int32_t) * n_sys);
+  if (mode == KC_MIXED) {
+    alloc((void **)&p->d_far, sizeof(int32_t) * n_sys);
+    alloc((void **)&p->d_err, sizeof(float2) * pairs);
+  }
   alloc(&p->d_obs_a, obs_bytes_a);
   alloc(&p->d_obs_b, obs_bytes_b);
   alloc((void **)&p->d_queue, sizeof(unsigned long long) * kPlanMaxStreams);

@@ -79,17 +79,24 @@ __global__ void prep_obs_mixed(RaggedDev d, const double *__restrict__ t,
     const Split3 tr3 = split3(tr), te3 = split3(d.t0);
     const float jit2 = d2f(jitter2);
     const int64_t pair0 = ragged_pair(o0, s);
-    bool far = false;
+    // a far time leaves all of the system's as plain pairs
+    bool seen = false;
+    for (int64_t k = o0 + lane; k < o1; k += 32) {
+      float th, tl;
+      sub_ds(split3(t[k]), tr3, th, tl);
+      tau_place(th, tl);
+      seen |= far_time(th);
+    }
+    const bool far = __any_sync(0xffffffffu, seen);
     for (int64_t k = o0 + 2 * lane; k < o1; k += 64) {
-      float th[2], tl[2], vh[2], vl[2], w[2], dt[2];
+      float th[2], tl[2], vh[2], vl[2], w[2], dt[2], err[2];
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        th[i] = tl[i] = vh[i] = vl[i] = w[i] = dt[i] = 0.0f;
+        th[i] = tl[i] = vh[i] = vl[i] = w[i] = dt[i] = err[i] = 0.0f;
         if (k + i < o1) {
           const Split3 tk = split3(t[k + i]);
           sub_ds(tk, tr3, th[i], tl[i]);
-          tau_place(th[i], tl[i]);
-          far |= !(fabsf(th[i]) < kPairMaxTau);
+          if (!far) tau_place(th[i], tl[i], err[i]);
           split_d(v[k + i], vh[i], vl[i]);
           const float sg = d2f(sigma[k + i]);
           const float var = __fmaf_rn(sg, sg, jit2);
@@ -101,9 +108,9 @@ __global__ void prep_obs_mixed(RaggedDev d, const double *__restrict__ t,
       oa[2 * p] = make_float4(th[0], th[1], tl[0], tl[1]);
       oa[2 * p + 1] = make_float4(vh[0], vh[1], vl[0], vl[1]);
       ob[p] = make_float4(w[0], w[1], dt[0], dt[1]);
+      d.tau_err[p] = make_float2(err[0], err[1]);
     }
-    const bool any = __any_sync(0xffffffffu, far);
-    if (lane == 0) d.far[s] = any ? 1 : 0;
+    if (lane == 0) d.far[s] = far ? 1 : 0;
   }
 }
 
@@ -220,11 +227,12 @@ struct RaggedPlanet<false> {
 
 // One system of J planets and n observations by a warp, a pair of
 // observations per lane at a time (kc_pair.cuh), the next pair loaded while
-// this one is evaluated.
+// this one is evaluated.  WIDE and err != NULL: the times completed to plain
+// pairs by the plan's tau_err.
 template <int J, bool GRAD, bool WIDE>
 __device__ __forceinline__ void body_mixed(const typename RaggedPlanet<GRAD>::type *pl, float gam,
                                            const float *tab, const float4 *oa, const float4 *ob,
-                                           int64_t pair0, int n, int lane, float *chi2_out,
+                                           const float2 *err, int64_t pair0, int n, int lane, float *chi2_out,
                                            float *grad_out) {
   constexpr int JG = GRAD ? J : 1;
   Kahan2 acc = {0, 0};
@@ -253,7 +261,15 @@ __device__ __forceinline__ void body_mixed(const typename RaggedPlanet<GRAD>::ty
       v_next = oa[2 * (p + 32) + 1];
       w_next = ob[p + 32];
     }
-    const f32x2 th = pack2(tt.x, tt.y), tl = pack2(tt.z, tt.w);
+    f32x2 th = pack2(tt.x, tt.y), tl = pack2(tt.z, tt.w);
+    if (WIDE && err != nullptr) {
+      const float2 e = err[pair0 + p];
+      float h0, l0, h1, l1;
+      two_sum(tt.x, tt.z, h0, l0);
+      two_sum(tt.y, tt.w, h1, l1);
+      th = pack2(h0, h1);
+      tl = pack2(l0 + e.x, l1 + e.y);
+    }
     Kahan2 V = {dup2(gam), 0};
     GradTerms o[JG];
 #pragma unroll
@@ -432,7 +448,7 @@ ragged_mixed_kernel(RaggedDev d, const float4 *__restrict__ oa, const float4 *__
     int64_t s = -1, o0 = 0, p0 = 0;
     int J = 0, n = 0;
     float gam = 0.0f;
-    bool far = false;
+    bool wide_me = false, exact_me = false;
     if (mine < take && idx + mine < (unsigned long long)d.n_sys) {
       s = d.order[idx + mine];
       if (dbg_ok(d.invalid, 0 <= s && s < d.n_sys, kDbgOrder, (int64_t)(idx + mine))) {
@@ -447,17 +463,24 @@ ragged_mixed_kernel(RaggedDev d, const float4 *__restrict__ oa, const float4 *__
     __syncwarp();                                // the last systems' use of the planets
     if (mine_j < J) {
       const double *p = params + p0 + 5 * mine_j;
-      if constexpr (GRAD)
+      const bool far = d.far[s] != 0;
+      const PlanetP *mine_p;
+      if constexpr (GRAD) {
         pl_s[warp][lane] = grad_setup_pair(p, d.t_ref[s], d.t0, far);
-      else
+        mine_p = &pl_s[warp][lane].p;
+      } else {
         pl_s[warp][lane] = planet_setup_pair(p, d.t_ref[s], d.t0, far);
+        mine_p = &pl_s[warp][lane];
+      }
+      wide_me = far || short_period(*mine_p);
+      exact_me = !far && !(mine_p->n <= kPairExactFreq);
       if (mine_j == 0) {
         const double gd = params[p0 + 5 * J];
         gam = finite_bits(gd) ? d2f(gd) : __int_as_float(0x7fc00000);
-        far |= d.far[s] != 0;
       }
     }
-    const unsigned wide = __ballot_sync(0xffffffffu, far);
+    const unsigned wide = __ballot_sync(0xffffffffu, wide_me);
+    const unsigned exact = __ballot_sync(0xffffffffu, exact_me);
     __syncwarp();
     for (int i = 0; i < take; ++i) {
       const int from = i * KC_MAX_PLANETS;
@@ -470,14 +493,17 @@ ragged_mixed_kernel(RaggedDev d, const float4 *__restrict__ oa, const float4 *__
       const float gi = __shfl_sync(0xffffffffu, gam, from);
       const Planet *pl = pl_s[warp] + from;
       const bool wi = ((wide >> from) & 0xffu) != 0u;
+      const float2 *err = ((exact >> from) & 0xffu) != 0u ? d.tau_err : nullptr;
       float *gout = GRAD ? grad + pi : nullptr;
       const int64_t pair0 = ragged_pair(oi, si);
       const int J = Ji;
 #define KC_BODY(JJ)                                                                          \
   if (wi)                                                                                    \
-    body_mixed<JJ, GRAD, true>(pl, gi, tab_s.s, oa, ob, pair0, ni, lane, chi2 + si, gout);   \
+    body_mixed<JJ, GRAD, true>(pl, gi, tab_s.s, oa, ob, err, pair0, ni, lane, chi2 + si,     \
+                               gout);                                                        \
   else                                                                                       \
-    body_mixed<JJ, GRAD, false>(pl, gi, tab_s.s, oa, ob, pair0, ni, lane, chi2 + si, gout)
+    body_mixed<JJ, GRAD, false>(pl, gi, tab_s.s, oa, ob, nullptr, pair0, ni, lane,           \
+                                chi2 + si, gout)
       KC_RAGGED_SWITCH(KC_BODY)
 #undef KC_BODY
       if (lane == 0) note_invalid(d.invalid, chi2[si]);      // lane 0 wrote it

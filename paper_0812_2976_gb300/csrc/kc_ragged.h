@@ -26,8 +26,10 @@ struct RaggedDev {
   int64_t n_sys;
   double t0;
   unsigned long long *invalid;   // NaN-result counter (kc_last_device_error) or NULL
-  // mixed: nonzero where a time of the system asks for the wide mean anomaly
+  // mixed: nonzero where a time of the system is a far one (its times are plain
+  // pairs then); per pair of observations, what tl lost to its binary place
   int32_t *far;
+  float2 *tau_err;
   int64_t n_obs_total;           // observations of the plan (obs_off[n_sys])
   int64_t n_par_total;           // packed parameters of the plan (par_off[n_sys])
 };
@@ -43,7 +45,7 @@ __host__ __device__ inline int64_t ragged_pair(int64_t obs_off, int64_t s) {
 // Converts t, v, sigma (device, [obs_off[n_sys]]) to the kernel's form:
 // mixed, per pair: obs_a two float4 (th, th', tl, tl') and (v_hi, v_hi', v_lo,
 // v_lo'), obs_b one float4 (w, w', t - t0, t' - t0); fp64: obs_a ObsR64, obs_b
-// unused.  Fills t_ref and, mixed, far.
+// unused.  Fills t_ref and, mixed, far and tau_err.
 cudaError_t ragged_prep(const RaggedDev &d, int mode, const double *t, const double *v,
                         const double *sigma, double jitter2, void *obs_a, void *obs_b,
                         double *t_ref, cudaStream_t st);
