@@ -30,9 +30,10 @@
 //    the planets over it: a planet's constants (PlanetP, computed once per
 //    (system, planet)) are read from shared memory once per chunk, and the
 //    chunk's Kepler solves are independent chains for the scheduler.
-//  - A CTA with a period or a time outside the short mean anomaly's range takes
-//    the wide one for all its systems (kc_pair.cuh); a far time has the planets and
-//    the staged times made plain pairs.
+//  - A CTA with a period or a time outside the short mean anomaly's range runs
+//    the wide body (kc_pair.cuh), in which a system without either still takes
+//    the short form; the first far time has the planets and the staged times made
+//    plain pairs.
 //  - The lanes of a system combine their compensated sums with TwoSum
 //    shuffles, and the warps of a system (G > 32) through a few words of
 //    shared memory; no atomics, no scratch memory.  Splitting a system over
@@ -157,13 +158,13 @@ __device__ __forceinline__ void load_item(int i, int spr, int64_t sys0, const Un
 
 // The thread's observations of one staged tile: npad (whole chunks), nk of
 // them real.  The thread takes kChunk observations at a time as kChunk / 2
-// packed pairs.  WIDE and t != NULL: the times as plain pairs, from t (n_obs of
-// them, the tile's first one at k0).
+// packed pairs.  WIDE: form as in kc_pair.cuh; with t != NULL the times as plain
+// pairs, from t (n_obs of them, the tile's first one at k0).
 template <int J, bool RESID, bool WIDE>
 __device__ __forceinline__ void warp_tile_sum(const float *th_s, int tile, const PlanetP *q,
                                               const float *tab, float gam, int c, int lg,
                                               int npad, int nk, Kahan2 &acc, float &rmax,
-                                              unsigned long long *dbg,
+                                              unsigned long long *dbg, MeanForm form = {},
                                               const double *t = nullptr, int k0 = 0,
                                               int n_obs = 0) {
   constexpr int kPairs = kChunk / 2;
@@ -190,7 +191,7 @@ __device__ __forceinline__ void warp_tile_sum(const float *th_s, int tile, const
       const PlanetP &qj = q[j];
 #pragma unroll
       for (int i = 0; i < kPairs; ++i) {
-        const f32x2 M = mean_anomaly2<WIDE>(th[i], tl[i], qj);
+        const f32x2 M = mean_anomaly2<WIDE>(th[i], tl[i], qj, form);
         const f32x2 m = abs2(M);
         f32x2 s, cE, E;
         kepler_pair<false>(m, qj, tab, s, cE, E);
@@ -258,13 +259,13 @@ struct WarpSmem {
 
 // The CTA's systems, one per G lanes, once the first tile is staged: all tiles'
 // sums, their combination, the results.  poison: NaN for an invalid system.  WIDE:
-// plain and te as in wide_systems.  The short and the wide form part before
+// plain, form and te as in wide_systems.  The short and the wide form part before
 // it and do not meet again: joined after each tile, the wide body's registers cost
 // the short one's 1 to 4 %.
 template <int J, bool RESID, bool DEMC, bool WIDE>
 __device__ __forceinline__ void systems(const UniformArgs &a, unsigned char *smem, int lg, int tile,
                                         int ntiles, float *out, float *resid_out, bool plain,
-                                        const double *te, float gam,
+                                        MeanForm form, const double *te, float gam,
                                         float poison) {
   const int block = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = 1 << lg, spr = block >> lg, step = G * kChunk;
@@ -294,7 +295,7 @@ __device__ __forceinline__ void systems(const UniformArgs &a, unsigned char *sme
     }
     if constexpr (WIDE)
       warp_tile_sum<J, RESID, true>(m.obs, tile, q, m.tab, gam, c, lg, npad, nk, acc2, rmax,
-                                    a.invalid, te, k0, a.n_obs);
+                                    a.invalid, form, te, k0, a.n_obs);
     else
       warp_tile_sum<J, RESID, false>(m.obs, tile, q, m.tab, gam, c, lg, npad, nk, acc2, rmax,
                                      a.invalid);
@@ -363,7 +364,10 @@ __device__ __forceinline__ void wide_systems(const UniformArgs &a, unsigned char
   float n_max = 0.0f;                            // the system's shortest period
 #pragma unroll
   for (int j = 0; j < J; ++j) n_max = fmaxf(n_max, m.pl[slot * J + j].n);
-  systems<J, RESID, DEMC, true>(a, smem, lg, tile, ntiles, out, resid_out, plain,
+  MeanForm form;
+  form.brief = !plain && n_max <= kPairMaxFreq;
+  form.some = __any_sync(0xffffffffu, form.brief);
+  systems<J, RESID, DEMC, true>(a, smem, lg, tile, ntiles, out, resid_out, plain, form,
                                 n_max > kPairExactFreq ? a.t : nullptr, gam, poison);
 }
 
@@ -441,7 +445,7 @@ chi2_mixed_warp_kernel(UniformArgs a, int lg, int tile, int ntiles, float *__res
   if (wide)
     wide_systems<J, RESID, DEMC>(a, smem, lg, tile, ntiles, out, resid_out, far, gam, poison);
   else
-    systems<J, RESID, DEMC, false>(a, smem, lg, tile, ntiles, out, resid_out, false, nullptr,
+    systems<J, RESID, DEMC, false>(a, smem, lg, tile, ntiles, out, resid_out, false, {}, nullptr,
                                    gam, poison);
 }
 

@@ -263,6 +263,7 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
   // so that the short form keeps its registers)
   with_high_e(wide, [&](auto tag) {
     constexpr bool WIDE = decltype(tag)::value;
+    MeanForm form;
     bool exact = false;
     if (WIDE) {
       plain = __syncthreads_or(far);
@@ -280,6 +281,8 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
       float n_max = 0.0f;                        // the system's shortest period
 #pragma unroll
       for (int j = 0; j < J; ++j) n_max = fmaxf(n_max, q[j].p.n);
+      form.brief = !plain && n_max <= kPairMaxFreq;
+      form.some = __any_sync(0xffffffffu, form.brief);
       exact = n_max > kPairExactFreq;
     }
     const float gam = gam_s[sl];
@@ -308,7 +311,7 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
         GradTerms o[J];
         Kahan2 V = {dup2(gam), 0};
 #pragma unroll
-        for (int j = 0; j < J; ++j) o[j] = grad_terms<WIDE>(th, tl, q[j], tab_s, V);
+        for (int j = 0; j < J; ++j) o[j] = grad_terms<WIDE>(th, tl, q[j], tab_s, V, form);
         const f32x2 r = sub2(sub2(V.big, at(2)), add2(V.small, at(3)));
         const f32x2 wr = mul2(at(4), r), a2 = add2(wr, wr);
         kahan_add(acc, mul2(wr, r));

@@ -405,9 +405,23 @@ __device__ __forceinline__ f32x2 mean_anomaly_wide(f32x2 th, f32x2 tl, const Pla
   return fma2(u, dup2(kTwoPiF), fma2(u, dup2(kTwoPiLo), mul2(lc, dup2(kTwoPiF))));
 }
 
+// The form of a wide body's lane: `brief` if its system takes the short form all
+// the same, `some` (for the warp) if any lane's does.  So a system's bits do not
+// hang on the others of its warp, which run the rest of the solve together.
+struct MeanForm {
+  bool some = false, brief = false;
+};
+
 template <bool WIDE>
-__device__ __forceinline__ f32x2 mean_anomaly2(f32x2 th, f32x2 tl, const PlanetP &q) {
-  return WIDE ? mean_anomaly_wide(th, tl, q) : mean_anomaly_pair(th, tl, q);
+__device__ __forceinline__ f32x2 mean_anomaly2(f32x2 th, f32x2 tl, const PlanetP &q,
+                                               MeanForm form = {}) {
+  if (!WIDE) return mean_anomaly_pair(th, tl, q);
+  f32x2 M = mean_anomaly_wide(th, tl, q);
+  if (form.some) {
+    const f32x2 m = mean_anomaly_pair(th, tl, q);
+    M = form.brief ? m : M;
+  }
+  return M;
 }
 
 // ------------------------------------------------ Kepler's equation
@@ -508,9 +522,10 @@ struct GradTerms {
 
 template <bool WIDE>
 __device__ __forceinline__ GradTerms grad_terms(f32x2 th, f32x2 tl, const GradPlanetP &g,
-                                                const float *tab, Kahan2 &V) {
+                                                const float *tab, Kahan2 &V,
+                                                MeanForm form = {}) {
   GradTerms o;
-  const f32x2 M = mean_anomaly2<WIDE>(th, tl, g.p);
+  const f32x2 M = mean_anomaly2<WIDE>(th, tl, g.p, form);
   f32x2 s, c, E;
   kepler_pair<true>(abs2(M), g.p, tab, s, c, E);      // c = 1 - cos E
   o.s = signed_as(s, M);

@@ -1,8 +1,8 @@
 """A system's results do not depend on the systems it is evaluated with: the
-bits of a row are the same beside rows of phases past 1e5 periods and of e >
-0.95 as beside ordinary ones, at the same launch shape; and an element of a
-Kepler solve's beside elements that need the other solver, and wherever it lies
-in memory."""
+bits of a row are the same beside rows of short periods, of phases past 1e5
+periods and of e > 0.95 as beside ordinary ones, at the same launch shape; and
+an element of a Kepler solve's beside elements that need the other solver, and
+wherever it lies in memory."""
 import numpy as np
 import pytest
 import torch
@@ -53,6 +53,24 @@ def test_double_precision(kc, n_pl, p_range, e_range, ordinary):
     finally:
         for kernel in ("chi2", "grad"):
             kc.kc_set_tile(kernel, "fp64", 512, n_pl, 200, None)
+
+
+@pytest.mark.parametrize("n_pl", [1, 3])
+@pytest.mark.parametrize("split", [0, 4])
+def test_mixed_short_periods(kc, n_pl, split):
+    plain, mixed, obs, same = two_batches(n_pl, (0.01, 0.4), (0.0, 0.9))
+    kc.kc_set_tile("chi2", "mixed", 512, n_pl, 200, (8, 128, 3))
+    kc.kc_set_tile("grad", "mixed", 512, n_pl, 200, (4, 128))
+    kc.kc_set_tile("gn", "mixed", 512, n_pl, 200, (32, 128, split))
+    try:
+        for fn in (lambda p: (kc.kc_chi2_eval_ex(p, *obs, t0=T0, mode="mixed"),),
+                   lambda p: kc.kc_chi2_grad(p, *obs, t0=T0, mode="mixed"),
+                   lambda p: kc.kc_chi2_gauss_newton(p, *obs, t0=T0)):
+            for a, b in zip(fn(plain), fn(mixed)):
+                assert torch.equal(a.cpu()[same], b.cpu()[same])
+    finally:
+        for kernel in ("chi2", "grad", "gn"):
+            kc.kc_set_tile(kernel, "mixed", 512, n_pl, 200, None)
 
 
 @pytest.mark.parametrize("mode", ["fp64", "mixed"])
