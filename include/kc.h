@@ -124,10 +124,11 @@ kc_status kc_chi2_grad(const double *params, const double *t,
                        double jitter, kc_mode mode, void *chi2_out,
                        void *grad_out, kc_stream stream);
 
-/* The same, KC_MIXED by the scalar one-observation kernel: its sums keep
+/* The same, KC_MIXED by the scalar one-observation kernel: at one launch
+ * shape (the built-in one unless the size is tuned or pinned) its sums keep
  * their form and order from version to version, for a caller that hands the
- * gradient on in double (autograd does) and so may not see it move by a
- * single-precision rounding.  KC_FP64: kc_chi2_grad. */
+ * gradient on in double (autograd does).  They carry single precision all the
+ * same.  KC_FP64: kc_chi2_grad. */
 kc_status kc_chi2_grad_scalar(const double *params, const double *t,
                               const double *v_obs, const double *sigma,
                               int64_t n_sys, int32_t n_pl, int32_t n_obs,
@@ -372,8 +373,11 @@ typedef enum kc_kernel {
 
 /* Tiles are looked up by (kernel, mode, n_pl, power-of-two bucket of n_sys,
  * power-of-two bucket of n_obs, SM count of the current device) in a
- * process-wide table; a missing entry uses a built-in heuristic.  kc_set_tile (tile == NULL removes the entry)
- * and kc_get_tile (the tile that would be used) act on that table. */
+ * process-wide table; a missing entry uses a built-in heuristic.  kc_set_tile
+ * (tile == NULL removes the entry) and kc_get_tile (the tile that would be used)
+ * act on that table.  KC_KERNEL_GRAD with KC_MIXED: kc_set_tile also sets the
+ * shape of the scalar gradient (kc_chi2_grad_scalar, kc_nll_grad), and
+ * kc_autotune times that kernel by itself and keeps its own fastest. */
 kc_status kc_set_tile(kc_kernel kernel, kc_mode mode, int64_t n_sys,
                       int32_t n_pl, int32_t n_obs, const kc_tile *tile);
 kc_status kc_get_tile(kc_kernel kernel, kc_mode mode, int64_t n_sys,

@@ -247,7 +247,7 @@ static Tile even_tile(Kind kind, int64_t n_sys, int n_obs) {
   while (G < 256 && n_sys * G < want_threads) G <<= 1;
   const int max_g_obs = n_obs >= 4 ? n_obs / 4 : 1;
   while (G > 1 && G > max_g_obs) G >>= 1;
-  if (kind == Kind::GradMixed && G > 32) G = 32;
+  if (kind == Kind::GradScalar && G > 32) G = 32;
   if (G < 4) G = 4;
   t.G = G;
   t.obs_tile = obs_tile_for(kind, n_obs);
@@ -326,14 +326,6 @@ Tile choose_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs) {
     }
   }
   return builtin_tile(kind, n_sys, n_pl, n_obs);
-}
-
-// The scalar gradient's shape: the gradient's table entry, else the rule its
-// results were always summed by (the order of a sum shows in its rounding).
-Tile scalar_grad_tile(int64_t n_sys, int n_pl, int n_obs) {
-  if (has_tile_entry(Kind::GradMixed, n_sys, n_pl, n_obs))
-    return choose_tile(Kind::GradMixed, n_sys, n_pl, n_obs);
-  return even_tile(Kind::GradMixed, n_sys, n_obs);
 }
 
 }  // namespace kc
@@ -487,7 +479,7 @@ static kc_status chi2_grad(const double *params, const double *t, const double *
                        "kc_chi2_grad (fp64)");
   }
   if (scalar)
-    return cuda_status(kc::launch_grad_scalar(a, kc::scalar_grad_tile(n_sys, n_pl, n_obs),
+    return cuda_status(kc::launch_grad_scalar(a, kc::choose_tile(Kind::GradScalar, n_sys, n_pl, n_obs),
                                               static_cast<float *>(chi2_out),
                                               static_cast<float *>(grad_out), s, false),
                        "kc_chi2_grad_scalar");
@@ -583,7 +575,7 @@ kc_status kc_nll_grad(const double *params, const double *t, const double *v_obs
                                            static_cast<double *>(nll_out),
                                            static_cast<double *>(grad_out), s, true),
                        "kc_nll_grad (fp64)");
-  return cuda_status(kc::launch_grad_scalar(a, kc::scalar_grad_tile(n_sys, n_pl, n_obs),
+  return cuda_status(kc::launch_grad_scalar(a, kc::choose_tile(Kind::GradScalar, n_sys, n_pl, n_obs),
                                             static_cast<float *>(nll_out),
                                             static_cast<float *>(grad_out), s, true),
                      "kc_nll_grad (mixed)");
@@ -728,16 +720,19 @@ kc_status kc_set_tile(kc_kernel kernel, kc_mode mode, int64_t n_sys, int32_t n_p
                       const kc_tile *tile) {
   if (!kernel_ok(kernel, mode) || n_sys < 0 || n_obs < 0 || n_pl < 1 || n_pl > KC_MAX_PLANETS)
     return fail(KC_ERR_ARG, "kc_set_tile: bad kernel, mode or sizes");
-  const kc::TileKey key = kc::key_of(kind_of(kernel, mode), n_sys, n_pl, n_obs);
-  std::lock_guard<std::mutex> lk(kc::g_tile_mu);
-  if (!tile) {
-    kc::g_tiles.erase(key);
-    return ok();
-  }
-  if (!tile_ok(kernel, mode, *tile)) return fail(KC_ERR_ARG, "kc_set_tile: inadmissible tile");
-  if (kernel == KC_KERNEL_GN && !kc::gn_variant_ok(tile->split, n_pl))
+  if (tile && !tile_ok(kernel, mode, *tile))
+    return fail(KC_ERR_ARG, "kc_set_tile: inadmissible tile");
+  if (tile && kernel == KC_KERNEL_GN && !kc::gn_variant_ok(tile->split, n_pl))
     return fail(KC_ERR_ARG, "kc_set_tile: the tcgen05 Gauss-Newton variant needs n_pl <= 3");
-  kc::g_tiles[key] = Tile{tile->threads_per_system, tile->block, 0, tile->split};
+  const Kind kind = kind_of(kernel, mode);
+  std::lock_guard<std::mutex> lk(kc::g_tile_mu);
+  for (Kind k : {kind, kind == Kind::GradMixed ? Kind::GradScalar : kind}) {
+    const kc::TileKey key = kc::key_of(k, n_sys, n_pl, n_obs);
+    if (tile)
+      kc::g_tiles[key] = Tile{tile->threads_per_system, tile->block, 0, tile->split};
+    else
+      kc::g_tiles.erase(key);
+  }
   return ok();
 }
 
@@ -763,7 +758,6 @@ kc_status kc_autotune(const double *params, const double *t, const double *v_obs
   if (!kernel_ok(kernel, mode)) return fail(KC_ERR_ARG, "kc_autotune: bad kernel or mode");
   if (n_sys == 0) return fail(KC_ERR_ARG, "kc_autotune: empty problem");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const kc::Kind kind = kind_of(kernel, mode);
   const size_t elem = mode == KC_FP64 ? sizeof(double) : sizeof(float);
   const size_t npar = 5 * (size_t)n_pl + 1;
   void *chi = nullptr, *grad = nullptr, *jtj = nullptr;
@@ -782,26 +776,20 @@ kc_status kc_autotune(const double *params, const double *t, const double *v_obs
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   UniformArgs a{params, t, v_obs, sigma, n_sys, n_pl, n_obs, 0.0, 0.0, kc::invalid_counter()};
-  auto launch = [&](const Tile &tile) -> cudaError_t {
+  auto launch = [&](Kind kind, const Tile &tile) -> cudaError_t {
     switch (kind) {
       case kc::Kind::Chi2F64: return kc::launch_chi2_f64(a, tile, (double *)chi, nullptr, s);
       case kc::Kind::Chi2Mixed: return kc::launch_chi2_mixed(a, tile, (float *)chi, nullptr, s);
       case kc::Kind::GradF64: return kc::launch_grad_f64(a, tile, (double *)chi, (double *)grad, s);
       case kc::Kind::GradMixed:
         return kc::launch_grad_mixed(a, tile, (float *)chi, (float *)grad, s);
+      case kc::Kind::GradScalar:
+        return kc::launch_grad_scalar(a, tile, (float *)chi, (float *)grad, s, false);
       case kc::Kind::GnMixed:
         return kc::launch_gauss_newton(a, false, chi, grad, jtj, s, tile.split);
     }
     return cudaErrorInvalidValue;
   };
-  float best_t = 1e30f;
-  Tile best_tile = kc::builtin_tile(kind, n_sys, n_pl, n_obs);
-  best_tile.obs_tile = kc::obs_tile_for(kind, n_obs);
-  // the built-in tile is kept unless a candidate beats it by 1 % (shapes
-  // within timing noise of each other would otherwise trade places from
-  // one run to the next)
-  float builtin_t = 1e30f;
-  const Tile builtin = best_tile;
   const char *env = getenv("KC_AUTOTUNE_VERBOSE");     // candidate timings to stderr
   const bool verbose = env && env[0] == '1';
   cudaError_t err = cudaSuccess;
@@ -831,49 +819,66 @@ kc_status kc_autotune(const double *params, const double *t, const double *v_obs
   for (int G : {8, 16, 32, 64, 128})
     for (int W = 4; W <= 32 && kernel == KC_KERNEL_CHI2; ++W)
       if ((32 * W) % G == 0) cands.push_back(kc_tile{G, 32 * W, 3});
-  for (const kc_tile &cand : cands) {
-    const int G = cand.threads_per_system, B = cand.block, split = cand.split;
-    if (!tile_ok(kernel, mode, cand)) continue;
-    if (n_obs > 0 && G > n_obs && split != 3 && kernel != KC_KERNEL_GN) continue;
-    if (split == 2 && G / 32 > (n_obs + 31) / 32) continue;   // chunks of >= 32 obs
-    if (split == 3 && !kc::warp_lanes_fit(G, n_obs)) continue;  // >= 4 obs per lane
-    Tile tile{G, B, kc::obs_tile_for(kind, n_obs), split};
-    err = launch(tile);                       // warm-up (and smem attribute)
-    if (err == cudaErrorInvalidConfiguration && split >= 3) {
-      err = cudaSuccess;                      // does not fit on an SM: nothing launched
-      continue;
+  // the fastest candidate for one kernel; the built-in tile is kept unless a
+  // candidate beats it by 1 % (shapes within timing noise of each other would
+  // otherwise trade places from one run to the next)
+  auto tune = [&](Kind kind, Tile &best_tile, float &best_t) {
+    best_t = 1e30f;
+    best_tile = kc::builtin_tile(kind, n_sys, n_pl, n_obs);
+    best_tile.obs_tile = kc::obs_tile_for(kind, n_obs);
+    float builtin_t = 1e30f;
+    const Tile builtin = best_tile;
+    for (const kc_tile &cand : cands) {
+      const int G = cand.threads_per_system, B = cand.block, split = cand.split;
+      if (!tile_ok(kernel, mode, cand)) continue;
+      if (n_obs > 0 && G > n_obs && split != 3 && kernel != KC_KERNEL_GN) continue;
+      if (split == 2 && G / 32 > (n_obs + 31) / 32) continue;   // chunks of >= 32 obs
+      if (split == 3 && !kc::warp_lanes_fit(G, n_obs)) continue;  // >= 4 obs per lane
+      Tile tile{G, B, kc::obs_tile_for(kind, n_obs), split};
+      err = launch(kind, tile);                       // warm-up (and smem attribute)
+      if (err == cudaErrorInvalidConfiguration && split >= 3) {
+        err = cudaSuccess;                      // does not fit on an SM: nothing launched
+        continue;
+      }
+      if (err != cudaSuccess) break;
+      // per launch: the mean of four launches back to back (as a caller
+      // evaluating batch after batch runs them: launches that overlap their
+      // neighbours' start and end are credited for it), the best of three
+      constexpr int kBackToBack = 4;
+      float tmin = 1e30f;
+      for (int rep = 0; rep < 3 && err == cudaSuccess; ++rep) {
+        cudaEventRecord(e0, s);
+        for (int i = 0; i < kBackToBack && err == cudaSuccess; ++i) err = launch(kind, tile);
+        cudaEventRecord(e1, s);
+        cudaEventSynchronize(e1);
+        float ms = 0.0f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        ms /= kBackToBack;
+        tmin = ms < tmin ? ms : tmin;
+      }
+      if (err != cudaSuccess) break;
+      if (verbose)
+        fprintf(stderr, "kc_autotune: kind %d n_sys %lld G %3d block %3d split %d: %9.2f us\n",
+                (int)kind, (long long)n_sys, G, B, split, 1e3 * tmin);
+      if (tile.G == builtin.G && tile.block == builtin.block && tile.split == builtin.split)
+        builtin_t = tmin;
+      if (tmin < best_t) {
+        best_t = tmin;
+        best_tile = tile;
+      }
     }
-    if (err != cudaSuccess) break;
-    // per launch: the mean of four launches back to back (as a caller
-    // evaluating batch after batch runs them: launches that overlap their
-    // neighbours' start and end are credited for it), the best of three
-    constexpr int kBackToBack = 4;
-    float tmin = 1e30f;
-    for (int rep = 0; rep < 3 && err == cudaSuccess; ++rep) {
-      cudaEventRecord(e0, s);
-      for (int i = 0; i < kBackToBack && err == cudaSuccess; ++i) err = launch(tile);
-      cudaEventRecord(e1, s);
-      cudaEventSynchronize(e1);
-      float ms = 0.0f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      ms /= kBackToBack;
-      tmin = ms < tmin ? ms : tmin;
+    if (builtin_t < 1e30f && best_t > 0.99f * builtin_t) {
+      best_t = builtin_t;
+      best_tile = builtin;
     }
-    if (err != cudaSuccess) break;
-    if (verbose)
-      fprintf(stderr, "kc_autotune: kind %d n_sys %lld G %3d block %3d split %d: %9.2f us\n",
-              (int)kind, (long long)n_sys, G, B, split, 1e3 * tmin);
-    if (tile.G == builtin.G && tile.block == builtin.block && tile.split == builtin.split)
-      builtin_t = tmin;
-    if (tmin < best_t) {
-      best_t = tmin;
-      best_tile = tile;
-    }
-  }
-  if (builtin_t < 1e30f && best_t > 0.99f * builtin_t) {
-    best_t = builtin_t;
-    best_tile = builtin;
-  }
+  };
+  const Kind kind = kind_of(kernel, mode);
+  Tile best_tile, scalar_tile;
+  float best_t = 1e30f, scalar_t = 1e30f;
+  tune(kind, best_tile, best_t);
+  // autograd and the free-jitter gradient run another kernel
+  if (kind == Kind::GradMixed && err == cudaSuccess)
+    tune(Kind::GradScalar, scalar_tile, scalar_t);
   cudaFreeAsync(chi, s);
   if (grad) cudaFreeAsync(grad, s);
   if (jtj) cudaFreeAsync(jtj, s);
@@ -884,6 +889,8 @@ kc_status kc_autotune(const double *params, const double *t, const double *v_obs
   {
     std::lock_guard<std::mutex> lk(kc::g_tile_mu);
     kc::g_tiles[kc::key_of(kind, n_sys, n_pl, n_obs)] = best_tile;
+    if (kind == Kind::GradMixed)
+      kc::g_tiles[kc::key_of(Kind::GradScalar, n_sys, n_pl, n_obs)] = scalar_tile;
   }
   if (best) {
     best->threads_per_system = best_tile.G;

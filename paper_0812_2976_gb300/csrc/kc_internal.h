@@ -190,11 +190,14 @@ cudaError_t launch_kepler_f32(const float *M, const float *e, int64_t n, float *
 size_t smem_chi2_mixed(int n_pl, const Tile &tile);
 
 // Launch shape for a problem (kc_api.cu): the tuned table, else a heuristic.
-enum class Kind { Chi2F64 = 0, Chi2Mixed = 1, GradF64 = 2, GradMixed = 3, GnMixed = 4 };
+// GradScalar: the scalar gradient kernel (autograd, free jitter), tuned and pinned
+// together with GradMixed but timed by itself.
+enum class Kind {
+  Chi2F64 = 0, Chi2Mixed = 1, GradF64 = 2, GradMixed = 3, GnMixed = 4, GradScalar = 5
+};
 Tile default_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs);
 Tile builtin_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs);  // without a table entry
 Tile choose_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs);
-Tile scalar_grad_tile(int64_t n_sys, int n_pl, int n_obs);
 bool has_tile_entry(Kind kind, int64_t n_sys, int n_pl, int n_obs);  // tuned or pinned
 int obs_tile_for(Kind kind, int n_obs);
 
