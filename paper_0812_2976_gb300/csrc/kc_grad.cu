@@ -775,45 +775,53 @@ __device__ __forceinline__ bool gn_stage(const UniformArgs &a, int k0, int nk, i
                                          int nthreads, const Split3 &tr3, float jit2, bool plain,
                                          float *obs) {
   bool far = false;
-  for (int k = tid; k < npad; k += nthreads) {
-    float th = 0.0f, tl = 0.0f, vh = 0.0f, vl = 0.0f, wk = 0.0f;
-    if (k < nk && dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k)) {
-      sub_ds(split3(a.t[k0 + k]), tr3, th, tl);
-      if (!plain) tau_place(th, tl);
-      far |= far_time(th);
-      split_d(a.v[k0 + k], vh, vl);
-      const float sg = d2f(a.sigma[k0 + k]);
-      const float var = __fmaf_rn(sg, sg, jit2);
-      wk = var > 0.0f ? 1.0f / var : __int_as_float(0x7fc00000);
-    }
-    const float v[5] = {th, tl, vh, vl, sqrtf(wk)};
+  // four observations' loads in flight: a tile is staged again for every four
+  // systems where the observations exceed it
+  for (int k4 = tid; k4 < npad; k4 += 4 * nthreads) {
+    double t[4], v[4], sigma[4];
+    bool real[4];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) obs[i * STRIDE + k] = v[i];
+    for (int i = 0; i < 4; ++i) {
+      const int k = k4 + i * nthreads;
+      real[i] = k < nk && dbg_ok(a.invalid, k0 + k < a.n_obs, kDbgObs, k0 + k);
+      t[i] = real[i] ? a.t[k0 + k] : 0.0;
+      v[i] = real[i] ? a.v[k0 + k] : 0.0;
+      sigma[i] = real[i] ? a.sigma[k0 + k] : 1.0;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = k4 + i * nthreads;
+      if (k >= npad) break;
+      float th = 0.0f, tl = 0.0f, vh = 0.0f, vl = 0.0f, wk = 0.0f;
+      if (real[i]) {
+        sub_ds(split3(t[i]), tr3, th, tl);
+        if (!plain) tau_place(th, tl);
+        far |= far_time(th);
+        split_d(v[i], vh, vl);
+        const float sg = d2f(sigma[i]);
+        const float var = __fmaf_rn(sg, sg, jit2);
+        wk = var > 0.0f ? 1.0f / var : __int_as_float(0x7fc00000);
+      }
+      const float o[5] = {th, tl, vh, vl, sqrtf(wk)};
+#pragma unroll
+      for (int j = 0; j < 5; ++j) obs[j * STRIDE + k] = o[j];
+    }
   }
   return far;
 }
 
-// What the Gauss-Newton kernels know before their first system: whether any time
-// is a far one (then the times and every 1/P are plain pairs), the observations
-// staged where they fit one tile.  Contains barriers.
+// The observations staged where they fit one tile, before the first system: as
+// plain pairs if any time is a far one, which it returns.  Contains barriers.
 template <int TILE, int ROWS>
 __device__ __forceinline__ bool gn_prepare(const UniformArgs &a, bool staged_once, int tid,
                                            int nthreads, const Split3 &tr3, float jit2,
                                            float *obs) {
   const int npad = (a.n_obs + ROWS - 1) / ROWS * ROWS;
   bool far = false;
-  if (staged_once) {
+  if (staged_once)
     far = gn_stage<TILE>(a, 0, a.n_obs, npad, tid, nthreads, tr3, jit2, false, obs);
-  } else {
-    for (int k = tid; k < a.n_obs; k += nthreads) {
-      float th, tl;
-      sub_ds(split3(a.t[k]), tr3, th, tl);
-      tau_place(th, tl);
-      far |= far_time(th);
-    }
-  }
   far = __syncthreads_or(far);
-  if (far && staged_once) {
+  if (far) {
     for (int k = tid; k < a.n_obs; k += nthreads)
       sub_ds(split3(a.t[k]), tr3, obs[k], obs[TILE + k]);
     __syncthreads();
@@ -881,6 +889,22 @@ __device__ __forceinline__ float gn_setup_ahead(const UniformArgs &a, int64_t s0
   }
   wide = __ballot_sync(0xffffffffu, brief);
   return gam;
+}
+
+// The planets of the warp's kGnAhead systems made plain pairs: the first far time
+// of a series longer than a tile is met with the planets set up.
+template <int J>
+__device__ __forceinline__ void gn_ahead_plain(const UniformArgs &a, int64_t s0, int64_t stride,
+                                               int lane, GradPlanetP *q) {
+  constexpr int NP = 5 * J + 1;
+  __syncwarp();
+  if (lane < kGnAhead * J) {
+    const int i = lane / J, j = lane - i * J;
+    const int64_t s = s0 + i * stride;
+    if (s < a.n_sys && dbg_ok(a.invalid, s * NP + 5 * j < a.n_sys * NP, kDbgParam, s * NP))
+      planet_plain(q[lane].p, a.params[s * NP + 5 * j]);
+  }
+  __syncwarp();
 }
 
 // chi2 and gradient of a warp's system: the lanes' sums combined and written.
@@ -1149,7 +1173,7 @@ gn_pair_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__ 
     u_all[i] = make_float2(0.0f, 0.0f);                           // incl. padding
   // observations that fit one tile are staged once for all of the CTA's systems
   const bool staged_once = a.n_obs <= kTile;
-  const bool plain = gn_prepare<kTile, kGnRows>(a, staged_once, tid, block, tr3, jit2, obs_s);
+  bool plain = gn_prepare<kTile, kGnRows>(a, staged_once, tid, block, tr3, jit2, obs_s);
 
   // The (hi, lo) pair of element (row r, column c) of U sits at
   // r * ROW2 + (c ^ ((r >> 2) & 3)): with ROW2 = 4 mod 16 both the row writes
@@ -1171,7 +1195,7 @@ gn_pair_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__ 
     }
     const GradPlanetP *q = ahead + ahead_i * J;
     const float gam = __shfl_sync(0xffffffffu, gam_ahead, 16 + ahead_i);
-    const bool wide = plain || ((wide_ahead >> (ahead_i * J)) & ((1u << J) - 1u)) != 0u;
+    bool wide = plain || ((wide_ahead >> (ahead_i * J)) & ((1u << J) - 1u)) != 0u;
     ++ahead_i;
     __syncwarp();
     Kahan2 acc = {0, 0};
@@ -1192,8 +1216,24 @@ gn_pair_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restrict__ 
       const int npad = (nk + kGnRows - 1) / kGnRows * kGnRows;
       if (!staged_once) {
         __syncthreads();
-        gn_stage<kTile>(a, k0, nk, npad, tid, block, tr3, jit2, plain, obs_s);
-        __syncthreads();
+        const bool far = gn_stage<kTile>(a, k0, nk, npad, tid, block, tr3, jit2, plain, obs_s);
+        if (__syncthreads_or(far) && !plain) {
+          // the first far time: these systems again from the first tile
+          plain = wide = true;
+          gn_ahead_plain<J>(a, s - (ahead_i - 1) * stride, stride, lane, ahead);
+          acc = Kahan2{0, 0};
+          sum_a = 0;
+#pragma unroll
+          for (int j = 0; j < J; ++j) g[j] = GradSums{{0, 0}, 0, 0, 0, 0};
+#pragma unroll
+          for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) C[mt][nt][i] = 0.0f;
+          k0 = -kTile;
+          continue;
+        }
       }
       for (int kb = 0; kb < npad; kb += kGnRows) {
         {
@@ -1384,7 +1424,7 @@ gn_mixed_tc_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restric
   // observations that fit one tile are staged once for all of the CTA's systems
   const bool staged_once = a.n_obs <= kTcObsTile;
   tc::fence_before_sync();
-  const bool plain =
+  bool plain =
       gn_prepare<kTcObsTile, kTcBatch>(a, staged_once, tid, kThreads, tr3, jit2, obs_s);
   tc::fence_after_sync();
   const uint32_t taddr = *slot;
@@ -1414,7 +1454,7 @@ gn_mixed_tc_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restric
     }
     const GradPlanetP *q = ahead + ahead_i * J;
     const float gam = __shfl_sync(0xffffffffu, gam_ahead, 16 + ahead_i);
-    const bool wide = plain || ((wide_ahead >> (ahead_i * J)) & ((1u << J) - 1u)) != 0u;
+    bool wide = plain || ((wide_ahead >> (ahead_i * J)) & ((1u << J) - 1u)) != 0u;
     ++ahead_i;
     __syncwarp();
     Kahan2 acc2 = {0, 0};
@@ -1422,15 +1462,28 @@ gn_mixed_tc_kernel(UniformArgs a, float *__restrict__ chi2_out, float *__restric
     GradSums g[J];
 #pragma unroll
     for (int j = 0; j < J; ++j) g[j] = GradSums{{0, 0}, 0, 0, 0, 0};
-    const uint32_t nb0 = nb;
+    uint32_t nb0 = nb;
 
     for (int k0 = 0; k0 < a.n_obs; k0 += kTcObsTile) {
       const int nk = min(kTcObsTile, a.n_obs - k0);
       const int npad = (nk + kTcBatch - 1) / kTcBatch * kTcBatch;
       if (!staged_once) {
         __syncthreads();
-        gn_stage<kTcObsTile>(a, k0, nk, npad, tid, kThreads, tr3, jit2, plain, obs_s);
-        __syncthreads();
+        const bool far =
+            gn_stage<kTcObsTile>(a, k0, nk, npad, tid, kThreads, tr3, jit2, plain, obs_s);
+        if (__syncthreads_or(far) && !plain) {
+          // the first far time: these systems again from the first tile (whose
+          // first MMA overwrites the accumulators)
+          plain = wide = true;
+          gn_ahead_plain<J>(a, s - (ahead_i - 1) * stride, stride, lane, ahead);
+          acc2 = Kahan2{0, 0};
+          sum_a = 0;
+#pragma unroll
+          for (int j = 0; j < J; ++j) g[j] = GradSums{{0, 0}, 0, 0, 0, 0};
+          nb0 = nb;
+          k0 = -kTcObsTile;
+          continue;
+        }
       }
       for (int kb = 0; kb < npad; kb += kTcBatch) {
         f32x2 u[NP];
@@ -1830,9 +1883,13 @@ cudaError_t launch_gn_tc(const UniformArgs &a, void *chi2, void *grad, void *jtj
 }
 
 // Without a tuned entry the mixed Gauss-Newton kernel updates U^T U on
-// tcgen05 where it can (n_pl <= 3): on a GB300, 65536 systems x 3 planets x
-// 512 observations take 619 us against 702 us with mma.sync (164 registers),
-// 20000 x 1 x 256 78 against 72.
+// tcgen05 where it can (n_pl <= 3): 65536 systems x 3 planets x 512 observations
+// take 617 us against 713 with mma.sync, 20000 x 2 x 400 147 against 164.  One
+// planet's evaluation is too short to hide the hand-off to the tensor core, and
+// from some 128 observations on mma.sync is the faster there (65536 x 1 x 512 367
+// against 412 us, 20000 x 1 x 256 74 against 78); but its H is three times as far
+// off (2.9e-6 against 9.4e-7 of sqrt(H_pp H_qq) at 300 observations, rms, 8.9e-6
+// against 2.8e-6 at 900), so it is taken only where it is asked for.
 int gn_default_variant(int n_pl) { return n_pl <= 3 ? 4 : 0; }
 
 bool gn_variant_ok(int variant, int n_pl) {

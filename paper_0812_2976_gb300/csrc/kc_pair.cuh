@@ -181,12 +181,14 @@ constexpr float kPairMaxTau = 16384.0f;
 
 __device__ __forceinline__ bool far_time(float th) { return !(fabsf(th) < kPairMaxTau); }
 
-// Whether one of the thread's times beyond the first tile is a far one (out of
-// line: few batches have more than one tile).
-static __device__ __noinline__ bool far_later(const double *t, int tile, int n_obs) {
+// Whether one of the thread's times from the first-th on is a far one (out of line:
+// few batches have more than one tile).
+static __device__ __noinline__ bool far_later(const double *t, int first, int n_obs) {
+  const double t_ref = t[0];
   bool far = false;
-  for (int k = tile + threadIdx.x; k < n_obs; k += blockDim.x)
-    far |= !(fabs(t[k] - t[0]) < (double)kPairMaxTau);
+#pragma unroll 4
+  for (int k = first + threadIdx.x; k < n_obs; k += blockDim.x)
+    far |= !(fabs(t[k] - t_ref) < (double)kPairMaxTau);
   return far;
 }
 
