@@ -264,9 +264,21 @@ Tile default_tile(Kind kind, int64_t n_sys, int n_pl, int n_obs) {
     // other even counts two halves of them, so fewer systems share a warp there
     // (100000 x 4 x 40: 116.7 us with 2 lanes a system, 80.3 with 8, the scalar
     // kernel 94.7; 50000 x 4 x 100: 86.4 with 4, 72.1 with 8; 200000 x 2 x 30:
-    // 87.9 with 1, 61.4 with 4, the scalar kernel 74.3).
+    // 87.9 with 1, 61.4 with 4, the scalar kernel 74.3).  Half as many lanes where
+    // the observations are few, and no more than there are pairs of them: a lane
+    // without observations costs as much as the conflicts (108155 x 8 x 12: 174.7
+    // with 8, 137.7 with 4; 60000 x 4 x 20: 43.7, 39.4; 100000 x 2 x 12: 28.7 with 4,
+    // 22.5 with 2, but 60000 x 6 x 23: 47.1 with 4, 61.1 with 2; 153930 x 2 x 2: 34.8
+    // with 4, 21.6 with 1).
     Tile t = model_tile(kCostGradMixed, kind, n_sys, n_pl, n_obs);
-    t.G = std::max(t.G, n_pl % 4 == 0 ? 8 : n_pl % 2 == 0 ? 4 : 1);
+    int least = 1;
+    if (n_pl % 4 == 0) least = n_obs >= 48 ? 8 : 4;
+    else if (n_pl % 2 == 0) least = n_obs >= 24 || n_pl > 2 ? 4 : 2;
+    while (least > 1 && least >= n_obs) least >>= 1;
+    if (t.G < least) {
+      t.G = least;
+      t.block = 128;
+    }
     return t;
   }
   return even_tile(kind, n_sys, n_obs);
