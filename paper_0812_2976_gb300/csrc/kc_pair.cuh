@@ -522,12 +522,9 @@ struct GradTerms {
   f32x2 s, dK, Q, y;
 };
 
-template <bool WIDE>
-__device__ __forceinline__ GradTerms grad_terms(f32x2 th, f32x2 tl, const GradPlanetP &g,
-                                                const float *tab, Kahan2 &V,
-                                                MeanForm form = {}) {
+__device__ __forceinline__ GradTerms grad_terms_at(f32x2 M, const GradPlanetP &g,
+                                                   const float *tab, Kahan2 &V) {
   GradTerms o;
-  const f32x2 M = mean_anomaly2<WIDE>(th, tl, g.p, form);
   f32x2 s, c, E;
   kepler_pair<true>(abs2(M), g.p, tab, s, c, E);      // c = 1 - cos E
   o.s = signed_as(s, M);
@@ -536,6 +533,13 @@ __device__ __forceinline__ GradTerms grad_terms(f32x2 th, f32x2 tl, const GradPl
   o.Q = mul2(fma2(dup2(g.C), o.s, fma2(dup2(-g.sw), c, dup2(g.swo))), o.y);
   kahan_add_y(V, fma2(dup2(g.K), o.dK, neg2(V.small)));
   return o;
+}
+
+template <bool WIDE>
+__device__ __forceinline__ GradTerms grad_terms(f32x2 th, f32x2 tl, const GradPlanetP &g,
+                                                const float *tab, Kahan2 &V,
+                                                MeanForm form = {}) {
+  return grad_terms_at(mean_anomaly2<WIDE>(th, tl, g.p, form), g, tab, V);
 }
 
 // Sums over the observations, a = 2 w r: of a dt Q y^2 (compensated: the

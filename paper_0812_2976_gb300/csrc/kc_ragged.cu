@@ -227,13 +227,20 @@ struct RaggedPlanet<false> {
 
 // One system of J planets and n observations by a warp, a pair of
 // observations per lane at a time (kc_pair.cuh), the next pair loaded while
-// this one is evaluated.  WIDE and err != NULL: the times completed to plain
-// pairs by the plan's tau_err.
+// this one is evaluated.  wide: the wide mean anomaly; with err != NULL the times
+// completed to plain pairs by the plan's tau_err.
+// The gradient has one body for both forms, a branch for the warp in front of the
+// mean anomalies (of half the planets at a time: fewer registers): with a body of
+// each, warps of both forms on an SM waited for instructions (5227 systems of 137 to
+// 1099 observations, half of them with P < 0.5 d: 139 us, now 75; 50000 of 16 to
+// 512: 460, 250; one form only, 50000 of 16 to 1024: 335, 342).  The forward bodies
+// are short enough for two (50000 of 16 to 1024: 220 us, 227 with one; the mixture
+// 63 and 47).
 template <int J, bool GRAD, bool WIDE>
 __device__ __forceinline__ void body_mixed(const typename RaggedPlanet<GRAD>::type *pl, float gam,
                                            const float *tab, const float4 *oa, const float4 *ob,
-                                           const float2 *err, int64_t pair0, int n, int lane, float *chi2_out,
-                                           float *grad_out) {
+                                           const float2 *err, bool wide, int64_t pair0, int n,
+                                           int lane, float *chi2_out, float *grad_out) {
   constexpr int JG = GRAD ? J : 1;
   Kahan2 acc = {0, 0};
   f32x2 sum_a = 0;
@@ -262,7 +269,7 @@ __device__ __forceinline__ void body_mixed(const typename RaggedPlanet<GRAD>::ty
       w_next = ob[p + 32];
     }
     f32x2 th = pack2(tt.x, tt.y), tl = pack2(tt.z, tt.w);
-    if (WIDE && err != nullptr) {
+    if ((GRAD || WIDE) && err != nullptr) {
       const float2 e = err[pair0 + p];
       float h0, l0, h1, l1;
       two_sum(tt.x, tt.z, h0, l0);
@@ -272,11 +279,25 @@ __device__ __forceinline__ void body_mixed(const typename RaggedPlanet<GRAD>::ty
     }
     Kahan2 V = {dup2(gam), 0};
     GradTerms o[JG];
+    if constexpr (GRAD) {
+      constexpr int H = J > 3 ? (J + 1) / 2 : J;
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-      if constexpr (GRAD) {
-        o[j] = grad_terms<WIDE>(th, tl, pl[j], tab, V);
-      } else {
+      for (int j0 = 0; j0 < J; j0 += H) {
+        f32x2 M[H];
+        if (wide) {
+#pragma unroll
+          for (int j = 0; j < H && j0 + j < J; ++j) M[j] = mean_anomaly_wide(th, tl, pl[j0 + j].p);
+        } else {
+#pragma unroll
+          for (int j = 0; j < H && j0 + j < J; ++j) M[j] = mean_anomaly_pair(th, tl, pl[j0 + j].p);
+        }
+#pragma unroll
+        for (int j = 0; j < H && j0 + j < J; ++j)
+          o[j0 + j] = grad_terms_at(M[j], pl[j0 + j], tab, V);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
         const f32x2 M = mean_anomaly2<WIDE>(th, tl, pl[j]);
         f32x2 s, c, E;
         kepler_pair<false>(abs2(M), pl[j], tab, s, c, E);
@@ -500,12 +521,12 @@ ragged_mixed_kernel(RaggedDev d, const float4 *__restrict__ oa, const float4 *__
       float *gout = GRAD ? grad + pi : nullptr;
       const int64_t pair0 = ragged_pair(oi, si);
       const int J = Ji;
-#define KC_BODY(JJ)                                                                          \
-  if (wi)                                                                                    \
-    body_mixed<JJ, GRAD, true>(pl, gi, tab_s.s, oa, ob, err, pair0, ni, lane, chi2 + si,     \
-                               gout);                                                        \
-  else                                                                                       \
-    body_mixed<JJ, GRAD, false>(pl, gi, tab_s.s, oa, ob, nullptr, pair0, ni, lane,           \
+#define KC_BODY(JJ)                                                                        \
+  if (wi && !GRAD)                                                                         \
+    body_mixed<JJ, GRAD, true>(pl, gi, tab_s.s, oa, ob, err, wi, pair0, ni, lane,          \
+                               chi2 + si, gout);                                           \
+  else                                                                                     \
+    body_mixed<JJ, GRAD, false>(pl, gi, tab_s.s, oa, ob, err, wi, pair0, ni, lane,         \
                                 chi2 + si, gout)
       KC_RAGGED_SWITCH(KC_BODY)
 #undef KC_BODY
