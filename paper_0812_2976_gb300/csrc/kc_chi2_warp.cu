@@ -293,7 +293,8 @@ __device__ __forceinline__ void systems(const UniformArgs &a, unsigned char *sme
       }
       __syncthreads();
     }
-    if constexpr (WIDE)
+    // (a warp of short-form systems alone in a wide CTA)
+    if (WIDE && !form.all)
       warp_tile_sum<J, RESID, true>(m.obs, tile, q, m.tab, gam, c, lg, npad, nk, acc2, rmax,
                                     a.invalid, form, te, k0, a.n_obs);
     else
@@ -367,6 +368,7 @@ __device__ __forceinline__ void wide_systems(const UniformArgs &a, unsigned char
   MeanForm form;
   form.brief = !plain && n_max <= kPairMaxFreq;
   form.some = __any_sync(0xffffffffu, form.brief);
+  form.all = __all_sync(0xffffffffu, form.brief);
   systems<J, RESID, DEMC, true>(a, smem, lg, tile, ntiles, out, resid_out, plain, form,
                                 n_max > kPairExactFreq ? a.t : nullptr, gam, poison);
 }

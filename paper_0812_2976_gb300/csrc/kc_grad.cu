@@ -283,6 +283,7 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
       for (int j = 0; j < J; ++j) n_max = fmaxf(n_max, q[j].p.n);
       form.brief = !plain && n_max <= kPairMaxFreq;
       form.some = __any_sync(0xffffffffu, form.brief);
+      form.all = __all_sync(0xffffffffu, form.brief);
       exact = n_max > kPairExactFreq;
     }
     const float gam = gam_s[sl];
@@ -299,27 +300,31 @@ grad_mixed_kernel(UniformArgs a, int G, int obs_tile, float *__restrict__ chi2_o
         __syncthreads();
       }
       const int npad = grad_tile(min(obs_tile, a.n_obs - k0), G);
-      for (int k = 2 * c; k < npad; k += 2 * G) {
-        // the planets' constants are read again in every iteration: hoisted
-        // for all J planets they would not fit the registers
-        asm volatile("" ::: "memory");
-        auto at = [&](int array) {
-          return *reinterpret_cast<const f32x2 *>(obs_s + array * tile + k);
-        };
-        f32x2 th = at(0), tl = at(1);
-        if (WIDE && exact) plain_times(a.t, k0 + k, a.n_obs, th, tl);
-        GradTerms o[J];
-        Kahan2 V = {dup2(gam), 0};
+      // (a warp of short-form systems alone in a wide CTA takes the short body)
+      with_high_e(WIDE && !form.all, [&](auto body) {
+        constexpr bool W = decltype(body)::value;
+        for (int k = 2 * c; k < npad; k += 2 * G) {
+          // the planets' constants are read again in every iteration: hoisted
+          // for all J planets they would not fit the registers
+          asm volatile("" ::: "memory");
+          auto at = [&](int array) {
+            return *reinterpret_cast<const f32x2 *>(obs_s + array * tile + k);
+          };
+          f32x2 th = at(0), tl = at(1);
+          if (W && exact) plain_times(a.t, k0 + k, a.n_obs, th, tl);
+          GradTerms o[J];
+          Kahan2 V = {dup2(gam), 0};
 #pragma unroll
-        for (int j = 0; j < J; ++j) o[j] = grad_terms<WIDE>(th, tl, q[j], tab_s, V, form);
-        const f32x2 r = sub2(sub2(V.big, at(2)), add2(V.small, at(3)));
-        const f32x2 wr = mul2(at(4), r), a2 = add2(wr, wr);
-        kahan_add(acc, mul2(wr, r));
-        sum_a = add2(sum_a, a2);
-        const f32x2 adt = mul2(a2, at(5));
+          for (int j = 0; j < J; ++j) o[j] = grad_terms<W>(th, tl, q[j], tab_s, V, form);
+          const f32x2 r = sub2(sub2(V.big, at(2)), add2(V.small, at(3)));
+          const f32x2 wr = mul2(at(4), r), a2 = add2(wr, wr);
+          kahan_add(acc, mul2(wr, r));
+          sum_a = add2(sum_a, a2);
+          const f32x2 adt = mul2(a2, at(5));
 #pragma unroll
-        for (int j = 0; j < J; ++j) grad_add(g[j], o[j], q[j], a2, adt);
-      }
+          for (int j = 0; j < J; ++j) grad_add(g[j], o[j], q[j], a2, adt);
+        }
+      });
     }
 
     Kahan chi = kahan_join(acc);

@@ -408,10 +408,11 @@ __device__ __forceinline__ f32x2 mean_anomaly_wide(f32x2 th, f32x2 tl, const Pla
 }
 
 // The form of a wide body's lane: `brief` if its system takes the short form all
-// the same, `some` (for the warp) if any lane's does.  So a system's bits do not
-// hang on the others of its warp, which run the rest of the solve together.
+// the same, `some` and `all` (for the warp) if any lane's or every lane's does.  So
+// a system's bits do not hang on the others of its warp, which run the rest of the
+// solve together.
 struct MeanForm {
-  bool some = false, brief = false;
+  bool some = false, all = false, brief = false;
 };
 
 template <bool WIDE>
