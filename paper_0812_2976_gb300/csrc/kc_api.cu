@@ -205,7 +205,14 @@ static Tile model_tile(const TileCost &m, Kind kind, int64_t n_sys, int n_pl, in
   Tile best{32, 128, 0};
   double best_cost = 1e300;
   int levels = 0;
+  // A planet above e = 0.95 takes its warp some 5000 clocks an evaluation: with few
+  // lanes per system one such system in every warp holds the others up.  From 128
+  // observations on a warp per system costs nothing otherwise (FP64 chi2, us at the
+  // model's own choice and so: 31298 x 1 x 639 610, 525, with e up to 0.99 1951, 686;
+  // 25557 x 3 x 182 358, 302 and 1273, 413; 9308 x 1 x 938 256, 245 and 775, 372).
+  const int least = kind == Kind::Chi2F64 && n_obs >= 128 ? 32 : 1;
   for (int G = 1; G <= m.max_g && (G == 1 || G < 2 * n_obs); G <<= 1, ++levels) {
+    if (G < least) continue;
     for (int B = m.min_block; B <= 256; B *= 2) {
       if (G > B) continue;
       const int W = B / 32, ST = B / G;
