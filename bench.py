@@ -46,8 +46,9 @@ ROTATE_BYTES = 256 << 20
 FALLBACK_SM_MHZ = 2070.0
 
 # Algorithmic FP32 work of one planet-observation evaluation of the scalar
-# mixed kernels (the tile kernels, the likelihood, the scalar adjoint), in FLOPs (FMA = 2, add/mul = 1; MUFU sin/cos/rcp and integer or
-# select operations not counted), from the algorithm as implemented:
+# mixed kernels (the tile kernels, the likelihood, the scalar adjoint), in FLOPs
+# (FMA = 2, add/mul = 1; MUFU sin/cos/rcp and integer or select operations not
+# counted), from the algorithm as implemented:
 #   double-single mean anomaly 18 (its low part formed already scaled by
 #   2 pi), Mikkola's starting value 18 (its per-planet constants and the
 #   MUFU square root, logarithm, exponential and reciprocals not counted),
@@ -60,7 +61,8 @@ MEAN_ANOMALY_FLOPS = 18
 
 
 def mixed_flops_per_eval(n_pl: int, warp: bool = False) -> float:
-    """FLOPs per evaluation of the scalar mixed chi2 kernels."""
+    """FLOPs per evaluation of the scalar mixed chi2 kernels (warp: no effect; the
+    warp-per-system kernel's count is pair_flops_per_eval)."""
     return MEAN_ANOMALY_FLOPS + KEPLER_MIXED_FLOPS + 8 + 4 + 10.0 / n_pl
 
 
