@@ -9,11 +9,11 @@
 // velocity.  Everything else is a small correction to a tabulated value:
 //
 //  - the single-precision solve (kc_pair.cuh's start, one Newton step) gives
-//    Ef within about 4e-7 of the root; a, the multiple of 2^-9 rad nearest to
+//    Ef within about 4e-7 of the root (|M| < 1.04 pi, solve_x); a, the multiple of 2^-9 rad nearest to
 //    its start, has sin a and cos a in a table as doubles and as float pairs;
-//  - sin and cos of a + b (b = Ef - a exact in float, |b| < 1.8e-3) and of
-//    the corrected E differ from them by less than 2e-3, so a float pair (48
-//    bits) holds the difference to 1e-17: rotation, Newton's correction and
+//  - sin and cos of a + b (b = Ef - a exact in float, |b| < 1.8e-3 for |M| <= pi,
+//    2.4e-3 just beyond) and of the corrected E differ from them by less than
+//    3e-3, so a float pair (48 bits) holds the difference to 1e-17: rotation, Newton's correction and
 //    the update run in float expansions (products with their FMA remainders,
 //    sums by TwoSum);
 //  - f(Ef) takes two FP64 FMAs, (Ef - 2 pi u) - e sin a, minus e times the
@@ -29,8 +29,9 @@
 // 2.6e5 draws; P in 1 .. 4000 d, 4000 d of observations), with the form of one
 // FP64 Halley step and one FP64 Newton step for 1/D in brackets: e < 0.3 1.5e-15
 // (5.4e-15), 0.3 .. 0.8 1.8e-15 (4.4e-15), 0.8 .. 0.95 2.9e-15 (2.6e-15: hence the
-// correction).  Valid for e <= kEccFast; above it the kernels take two FP64
-// quartic steps (kepler_high).
+// correction).  Valid for e <= kEccFast and amplitudes a float pair holds
+// (amplitude_fits); a planet outside takes two FP64 quartic steps and an FP64
+// velocity (PlanetX::high, eval_high), beside the others of its system.
 #pragma once
 
 #include "kc_device.cuh"
@@ -288,8 +289,9 @@ struct EvalX {
 
 __device__ __forceinline__ EvalX solve_x(double tau, float tf, const PlanetX &p) {
   EvalX o;
-  // phase: n is the integer nearest to it in single precision, so u = tau/P -
-  // n + c0 lies within 0.5 + 2^-23 |tau/P| of 0 (the table covers 0.528)
+  // phase: n is the integer nearest to it in single precision (three roundings),
+  // so u = tau/P - n + c0 lies within 0.5 + 1.5 2^-23 |tau/P| of 0: 0.518 without
+  // the wrap below (the table covers 0.528)
   const float n = rintf(__fmaf_rn(tf, p.inv_P_f, p.c0f));
   double u = fma(tau, p.inv_P, -f2d(n)) + p.c0;
   // (a vote, so that the usual case skips the FP64 work instead of predicating
@@ -402,7 +404,7 @@ __device__ __forceinline__ EvalX solve_x(double tau, float tf, const PlanetX &p)
 // E of one (M, e) in double, for |M| in [2^-30, 1.02 pi] and 0 <= e <=
 // kEccFast: solve_x's way with M itself and e of every evaluation, and with
 // small E to full relative precision: of sin Ef = S + C b + q, b = Ef - a, the
-// table's doubles take the first two terms, only q (below 2e-6 S and 5e-7 C b)
+// table's doubles take the first two terms, only q (below 2.1e-6 S and 7e-7 C b)
 // is a float pair.  Five FP64 instructions, where an FP64 Halley step from
 // the single-precision solution took some 16.
 __device__ __forceinline__ double kepler_x(double M, double e) {

@@ -17,9 +17,9 @@
 //    that their product is a multiple of 2^-23 cycles and its difference
 //    from the nearest integer of the phase is exact in one FMA;
 //  - Mikkola's cubic start with its quintic correction replaced by a
-//    degree-four fit (below): within 8e-4 rad of the root instead of
-//    3.6e-3, which lets one Newton step (4 operations) stand for Halley's
-//    (9);
+//    degree-four fit (below): within 8e-4 rad of the root (1.37e-3 just past
+//    pi) instead of 3.6e-3, which lets one Newton step (4 operations) stand
+//    for Halley's (9);
 //  - sin/cos of the start from a table at multiples of 2^-8 rad in shared
 //    memory and a rotation by the remainder (8 operations instead of 15);
 //  - the velocity as (A cos E - B sin E)/(1 - e cos E) with its last product
@@ -104,7 +104,7 @@ __device__ __forceinline__ Kahan kahan_join(const Kahan2 &k) {
 // ------------------------------------------------ sin/cos table
 
 // sin and cos at k 2^-8 rad, k = 0 .. 1023, rounded to float: 8 KB.  The start
-// of the solve lies in [0, 1.04 pi), below 3.3.  A power of two of entries,
+// of the solve lies in [0, 1.04 pi], below 3.3.  A power of two of entries,
 // so that the index of any start (NaN included, for an invalid planet) is
 // masked into the table.  Two arrays, not (sin, cos) words: two 4-byte
 // gathers land in the halves of the packed registers, where one 8-byte
@@ -215,10 +215,12 @@ __device__ __forceinline__ void plain_times(const double *t, int k, int n, f32x2
 // -0.078 s^5/(1 + e)), sin E is taken as s (3 + c1 x + c2 x^2 + c3 x^3 +
 // c4 x^4), x = s^2, with c1 .. c4 cubics in e fitted to keep the error of
 // ONE NEWTON STEP small (weighted least squares with the weights iterated
-// towards the largest error, kepler_start_fit.py): the start is within 8e-4
-// rad, the step within 5.1e-9 rad of the root for every 0 <= e < 1 and |M|
-// <= 1.02 pi (as Halley's step from the quintic correction).  Scaled
-// to s' = z - 1/z: E0 = M + s' (q0 + q1 x' + .. + q4 x'^4), q_i = e c_i
+// towards the largest error, kepler_start_fit.py, which fits up to |M| = 1.02 pi
+// and checks beyond).  For every 0 <= e < 1, in exact arithmetic: for |M| <= pi
+// the start is within 8e-4 rad and the step within 5.1e-9 rad of the root (as
+// Halley's step from the quintic correction), up to 1.02 pi within 1.06e-3 and
+// 5.1e-9, up to 1.038 pi, where the short mean anomaly ends, within 1.37e-3 and
+// 1.7e-8.  Scaled to s' = z - 1/z: E0 = M + s' (q0 + q1 x' + .. + q4 x'^4), q_i = e c_i
 // a^(i + 1/2).
 __device__ __forceinline__ float start_fit(float e, float k0, float k1, float k2, float k3) {
   return __fmaf_rn(e, __fmaf_rn(e, __fmaf_rn(e, k3, k2), k1), k0);
@@ -369,11 +371,13 @@ __device__ __forceinline__ GradPlanetP grad_setup_pair(const double *p, double t
 
 // ------------------------------------------------ mean anomaly
 
-// M of two observations, |M| <= 1.02 pi.  k is the integer nearest to the
-// phase (up to tl n <= 2^-6 cycles); th nq is a multiple of 2^-23 and its
-// distance from k below 2, so the FMA is exact, and so is the sum with c.
-// The low parts (below 0.1 cycles) add three roundings near 2^-26 rad and
-// the final FMA one: 2.1e-7 rad at worst, 6.9e-8 rms.
+// M of two observations, |M| < 1.038 pi.  k is the integer nearest to the phase
+// without tl n, up to 2^-6 cycles (1/P = 2, |tl| = 2^-7 d), without 1/P's low part,
+// up to 2^-10, and rounded to float, up to 2^-9 (both at |tau/P| = 2^15): |phase -
+// k| < 0.519 cycles; th nq is a multiple of 2^-23 and its distance from k below
+// 2, so the FMA is exact, and so is the sum with c.  The low parts (below 0.1
+// cycles) add three roundings near 2^-26 rad and the final FMA one: 2.1e-7 rad
+// at worst, 6.9e-8 rms.
 __device__ __forceinline__ f32x2 mean_anomaly_pair(f32x2 th, f32x2 tl, const PlanetP &q) {
   const f32x2 magic = dup2(kRoundMagic);
   const f32x2 y = fma2(th, dup2(q.n), dup2(q.c));
@@ -428,10 +432,6 @@ __device__ __forceinline__ f32x2 mean_anomaly2(f32x2 th, f32x2 tl, const PlanetP
 }
 
 // ------------------------------------------------ Kepler's equation
-
-__device__ __forceinline__ float abs_bits(float x) {
-  return fabsf(x);
-}
 
 // s' = z - 1/z of the start for one |M|.  1/z is the exponential of the
 // negated logarithm: ex2 runs at twice the rate of rcp (4 clocks per warp
@@ -504,7 +504,7 @@ __device__ __forceinline__ f32x2 signed_as(f32x2 x, f32x2 M) {
   return pack2(__uint_as_float(a), __uint_as_float(b));
 }
 
-__device__ __forceinline__ f32x2 abs2(f32x2 x) { return pack2(abs_bits(lo2(x)), abs_bits(hi2(x))); }
+__device__ __forceinline__ f32x2 abs2(f32x2 x) { return pack2(fabsf(lo2(x)), fabsf(hi2(x))); }
 
 // V += v with sin E already signed.
 __device__ __forceinline__ void velocity_sum(Kahan2 &V, const PlanetP &q, f32x2 s, f32x2 c) {

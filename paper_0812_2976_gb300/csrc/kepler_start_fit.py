@@ -8,8 +8,10 @@ c_i cubics in e.  One Newton step from E0 errs by (E0 - E)^2 e sin E /
 (2 (1 - e cos E)) to leading order, so the fit minimises the largest
 |E0 - E| sqrt(e sin E / (1 - e cos E)) over a grid of (M, e) by least squares
 with weights moved towards the largest error.  Prints the 4 x 4 coefficients
-(rows c1 .. c4, columns powers of e) and the Newton step's largest error with
-them rounded to four places (about 5e-9 rad).  numpy only, under a minute.
+(rows c1 .. c4, columns powers of e) and, with them rounded to four places, the
+largest error of the start and of the Newton step for |M| up to pi, to the fit's
+end and to what the kernels' mean anomalies reach (1.038 pi in kc_pair.cuh, 1.057
+pi in kc_f64.cuh).  numpy only, under a minute.
 """
 import numpy as np
 
@@ -37,15 +39,18 @@ def cubic_root(M, e):
     return sa * (z - 1.0 / z)
 
 
-def newton_error(coef):
-    worst = 0.0
+def errors(coef, top):
+    """Largest error of the start and of the Newton step for 0 < M <= top."""
+    M = np.concatenate([MEAN[MEAN <= top], np.linspace(0.9 * top, top, 400)])
+    start = step = 0.0
     for e in ECC:
-        s = cubic_root(MEAN, e)
+        s, root = cubic_root(M, e), eccentric(M, e)
         c = [np.polyval(row[::-1], e) for row in coef]
-        E = MEAN + e * s * (3.0 + sum(k * s ** (2 * i + 2) for i, k in enumerate(c)))
-        E1 = E - (E - e * np.sin(E) - MEAN) / (1.0 - e * np.cos(E))
-        worst = max(worst, float(np.abs(E1 - eccentric(MEAN, e)).max()))
-    return worst
+        E = M + e * s * (3.0 + sum(k * s ** (2 * i + 2) for i, k in enumerate(c)))
+        E1 = E - (E - e * np.sin(E) - M) / (1.0 - e * np.cos(E))
+        start = max(start, float(np.abs(E - root).max()))
+        step = max(step, float(np.abs(E1 - root).max()))
+    return start, step
 
 
 def fit(iterations=150):
@@ -72,4 +77,6 @@ def fit(iterations=150):
 if __name__ == "__main__":
     coef = np.round(fit(), 4)
     print(coef)
-    print("largest error of the Newton step: %.2e rad" % newton_error(coef))
+    for top in (1.0, 1.02, 1.038, 1.057):
+        print("|M| <= %.3f pi: largest error of the start %.2e rad, of the Newton step %.2e"
+              % (top, *errors(coef, top * np.pi)))
