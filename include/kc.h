@@ -38,6 +38,13 @@
  *    every device loop has a fixed trip count.  Each system whose result
  *    comes out NaN also adds one to a per-device counter read (and reset)
  *    by kc_last_device_error.
+ *  - A system's result depends on its own parameters, the observations and the
+ *    launch shape alone (which follows the batch's sizes and the tile table),
+ *    never on the other systems of the batch: in two batches of one shape the
+ *    same row gives the same bits.  Two shapes may differ in the last bits of
+ *    the sums.  kc_kepler_solve's elements do not even depend on the shape.
+ *  - Times and periods share one unit (days); other units give the same
+ *    accuracy while |t - t_ref|/P stays below 2^22.
  *  - n_sys == 0 is a no-op.  n_obs == 0 gives chi2 = 0 (NaN if invalid).
  *  - Calls are thread-safe; concurrent calls on different streams do not
  *    share device memory, with one exception: every call of
@@ -124,11 +131,12 @@ kc_status kc_chi2_grad(const double *params, const double *t,
                        double jitter, kc_mode mode, void *chi2_out,
                        void *grad_out, kc_stream stream);
 
-/* The same, KC_MIXED by the scalar one-observation kernel: at one launch
- * shape (the built-in one unless the size is tuned or pinned) its sums keep
- * their form and order from version to version, for a caller that hands the
- * gradient on in double (autograd does).  They carry single precision all the
- * same.  KC_FP64: kc_chi2_grad. */
+/* The same, KC_MIXED by the scalar one-observation kernel (the one of
+ * kc_nll_grad), which the Python binding's autograd function calls: another
+ * order of the same sums, slower than kc_chi2_grad.  Its results carry single
+ * precision like kc_chi2_grad's, whatever type they are handed on in, and their
+ * last bits depend on the launch shape (the built-in one unless the size is
+ * tuned or pinned).  KC_FP64: kc_chi2_grad. */
 kc_status kc_chi2_grad_scalar(const double *params, const double *t,
                               const double *v_obs, const double *sigma,
                               int64_t n_sys, int32_t n_pl, int32_t n_obs,
@@ -262,9 +270,13 @@ kc_status kc_rv_predict_ragged(const double *params, const int64_t *par_off,
                                const int64_t *obs_off, int64_t n_sys, double t0,
                                double *v_out, kc_stream stream);
 
-/* Elementwise Kepler solve with the same device solver the chi2 kernels use
- * (Sec. 4.3): E_out[i] with E - e sin E = M for M[i] in any range and
- * 0 <= e[i] < 1.  KC_FP64: M, e, E_out are double.  KC_MIXED: float.
+/* Elementwise Kepler solve (Sec. 4.3): E_out[i] with E - e sin E = M for M[i]
+ * in any range and 0 <= e[i] < 1.  KC_FP64: M, e, E_out are double, the solver
+ * of the chi2 kernels (a single-precision solution corrected in float pairs)
+ * for e <= 0.95 and two quartic steps in double above.  KC_MIXED: float,
+ * Mikkola's start and one Halley step (the chi2 kernels take a fitted start,
+ * whose constants are set up once per planet, and a Newton step); the root is
+ * the same within float rounding.
  * E_out is reduced to the branch of M reduced to [-pi, pi]. */
 kc_status kc_kepler_solve(const void *M, const void *e, int64_t n,
                           kc_mode mode, void *E_out, kc_stream stream);
@@ -275,7 +287,8 @@ kc_status kc_kepler_solve(const void *M, const void *e, int64_t n,
  * own observations, evaluated by one persistent kernel that takes whole
  * systems from a device work queue (longest first) and is replayed as a CUDA
  * graph.  The observations are fixed for the plan (as the paper treats them,
- * Sec. 4.1); the parameters change from run to run.
+ * Sec. 4.1); the parameters change from run to run.  A system's result depends
+ * on its own parameters and observations alone.
  *   obs_off [n_sys+1] host int64: system s owns observations
  *                     obs_off[s] .. obs_off[s+1] (obs_off[0] == 0,
  *                     non-decreasing; empty systems allowed).
@@ -283,7 +296,8 @@ kc_status kc_kepler_solve(const void *M, const void *e, int64_t n,
  * Parameters are packed: system s's 5*n_pl[s]+1 values (same layout as the
  * uniform calls) follow those of system s-1.  The plan copies the
  * descriptors to the current device and owns that memory, the converted
- * observations and its work queue until kc_plan_destroy.  Creation
+ * observations (28 B each for KC_MIXED, 32 B for KC_FP64) and its work queue
+ * until kc_plan_destroy.  Creation
  * allocates and synchronises; KC_ERR_NOMEM if the device is out of memory. */
 typedef struct kc_plan kc_plan;
 

@@ -9,14 +9,17 @@
 // two-observation form of kc_pair.cuh, laid out for the SMs rather than for
 // a tile.  Bound by FP32 issue and register ports (68 clocks per warp,
 // planet and observation and sub-partition in steady state).  Measured, us
-// per launch, before (scalar form) and now: 2^20 x 4 x 256 3224 -> 2014, 4096
-// x 4 x 256 back to back 14.3 -> 11.2, 300 x 3 x 101 5.9 -> 4.3.
+// per launch, before (scalar form) and now: 2^20 x 4 x 256 3224 -> 1977, 4096
+// x 4 x 256 back to back 14.3 -> 11.2, 300 x 3 x 101 5.9 -> 4.3; 65536 x 4 x 256
+// with ordinary periods 191 -> 127, with 1, 10 and 100 % of the planets below half
+// a day 142, 163 and 166, with a time beyond 2^14 d 169, with periods of 0.001 ..
+// 0.01 d 188.
 //
 //  - A CTA of W warps evaluates W * 32 / G systems (one round).  The host
 //    picks G and W by a cost model (pick_warp_tile) so that the CTAs land
-//    evenly on the SMs and share their staging (for 4096 systems, 27 warps per CTA: one CTA and 27 systems on
-//    every SM, where tiles of 16 systems leave some SMs with 32 and others
-//    with 16).  Larger batches run many waves; the hardware then overlaps
+//    evenly on the SMs and share their staging (for 4096 systems, 27 warps per
+//    CTA: one CTA and 27 systems on every SM, where tiles of 16 systems leave
+//    some SMs with 32 and others with 16).  Larger batches run many waves; the hardware then overlaps
 //    one CTA's prologue with the work of the others on its SM.
 //  - Prologue: every global load (the reference time, this thread's
 //    observation and its planet's parameters) is issued before any of them
@@ -32,8 +35,9 @@
 //    chunk's Kepler solves are independent chains for the scheduler.
 //  - A CTA with a period or a time outside the short mean anomaly's range runs
 //    the wide body (kc_pair.cuh), in which a system without either still takes
-//    the short form; the first far time has the planets and the staged times made
-//    plain pairs.
+//    the short form (a warp of such systems the short body); the first far time
+//    has the planets and the staged times made plain pairs.  So a system's bits
+//    hang on its own planets, the observations and the launch shape alone.
 //  - The lanes of a system combine their compensated sums with TwoSum
 //    shuffles, and the warps of a system (G > 32) through a few words of
 //    shared memory; no atomics, no scratch memory.  Splitting a system over
@@ -45,10 +49,10 @@
 //    (griddepcontrol.launch_dependents), so that a following batch's CTAs
 //    are placed on the SMs as this grid's CTAs exit instead of after the
 //    whole grid has completed (back-to-back 4096 x 4 x 256 batches: 14.0 us
-//    each instead of 16.4 us, with the scalar body).  The launch asks for it only outside stream
-//    capture: as programmatic edges in the DE-MC driver's graph (4096
-//    chains, halves of 2048) it cost a quarter of the generations per
-//    second (2.36e4 against 3.12e4), where back-to-back launches of 1024 to
+//    each instead of 16.4 us, with the scalar body).  The launch asks for it
+//    only outside stream capture: as programmatic edges in the DE-MC driver's
+//    graph (4096 chains, halves of 2048) it cost a quarter of the generations
+//    per second (2.36e4 against 3.12e4), where back-to-back launches of 1024 to
 //    4096 systems gained 2.7-2.9 us each.
 #include <algorithm>
 #include <map>

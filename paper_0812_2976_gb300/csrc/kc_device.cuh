@@ -32,9 +32,8 @@ constexpr float kTwoPiF = 6.28318530717958647692f;
 // Eccentricity up to which one double-precision step suffices (the
 // workloads draw e <= 0.95): above it the single-precision seed's error
 // grows like 1e-7 / (1 - e cos E) near pericentre and the double-precision
-// solve takes two steps.  Kernels choose once per warp (any_high_e), so
-// that the usual case keeps one straight-line body with no branch per
-// planet.
+// solve takes two steps, for that planet alone.  A warp without such a planet
+// runs a copy of its loop that has no branch per planet (any_high_e).
 constexpr float kEccFast = 0.95f;
 
 // ------------------------------------------------ conversions (integer pipe)
@@ -401,9 +400,9 @@ __device__ __forceinline__ float kepler_f32(float M, float e, float &sE, float &
   return kepler_f32_h(M, e, kepler_start_consts(e), sE, cE);
 }
 
-// Warp-uniform choice of the double-precision solver's HI variant: true if
-// any lane holds an eccentricity above kEccFast.  All lanes of `mask` must
-// call it.
+// Warp-uniform choice of the double-precision loops' HI variant, which tells the
+// planets above kEccFast from the others: true if any lane holds one.  All lanes
+// of `mask` must call it.
 __device__ __forceinline__ bool any_high_e(bool mine, unsigned mask = 0xffffffffu) {
   return __any_sync(mask, mine) != 0;
 }

@@ -608,7 +608,8 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
 // like chi2 (kc_f64.cuh); the planets are set up once per CTA, where one
 // thread per (system, observation) had repeated the setup at every
 // evaluation (512 x 3 x 1000: 305 us, now 43; 32 without 1/D's correction in
-// FP64, which takes the error from 2.2e-15 to 4e-16 of the velocities' rms).  G
+// FP64, which takes the error from 2.2e-15 to 4e-16 of the velocities' rms; every
+// e above 0.95: 289, now 234).  G
 // is the power of two that n_obs fills, down to one thread per system: every lane
 // evaluates (275996 systems of 5 planets above e = 0.95 at a single time: 358 us,
 // 2060 with 8 threads per system, 444 with the setup per evaluation).
@@ -679,8 +680,10 @@ __device__ inline float reduce_pi<float>(float M) {
 // One (M, e) per thread and iteration, five FP64 instructions each (kepler_x)
 // where 0 <= e <= kEccFast and |M| <= 1.02 pi above 2^-30 (the leading words
 // compared, on the integer pipe); the other elements of a warp take the form with
-// two FP64 quartic steps, which costs it some 2000 clocks.  2^24 elements, e <= 0.95: 1070 -> 260 us, bound by issue (memory: 60
-// us); e < 0.999: 617 -> 569 us for 2^22.  Error against 64-bit mantissas, 4e5
+// two FP64 quartic steps, which costs it some 2000 clocks.  2^24 elements, e <=
+// 0.95: 1070 -> 260 us, bound by issue and the FP64 pipe (memory: 60 us); 2^22
+// with e < 0.999: 616 -> 576, with one |M| below 2^-30 in a hundred 270 -> 134.
+// Error against 64-bit mantissas, 4e5
 // draws with |M| from 1e-8: rms 9.10e-17 -> 9.05e-17, largest relative 3.6e-15
 // both.
 __device__ __forceinline__ bool kepler_x_takes(double M, double e) {
@@ -765,7 +768,8 @@ __device__ __forceinline__ f32x2 kepler_any2(float m0, float m1, float e0, float
 // scalar form's 69 instructions an element issued for 33 of its 38.9 us.
 // Packed: 44 instructions, 34.9 us; the wait for memory is hidden by warps, so
 // 32 registers for 64 warps per SM (40 registers: 37.0; loads one iteration
-// ahead: 36.8 to 39; sin and cos from a table in shared memory: 39.3).
+// ahead: 36.8 to 39; sin and cos from a table in shared memory: 39.3).  Unaligned
+// arrays 67 -> 47 us.
 __device__ __forceinline__ float4 kepler_f32_x4(float4 m, float4 ee) {
   constexpr float kPi = 3.14159265f;
   if (!(fabsf(m.x) <= kPi && fabsf(m.y) <= kPi && fabsf(m.z) <= kPi && fabsf(m.w) <= kPi))
