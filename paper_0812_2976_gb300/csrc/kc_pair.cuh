@@ -174,7 +174,7 @@ __device__ __forceinline__ void tau_place(float &hi, float &lo) {
 //  - 1/P above kPairExactFreq: the system's times are read as plain pairs.
 //    Placed, they are known to 2^-33 d: 6.5e-7 rad at P = 1e-3 d (6e-9 at the
 //    limit).
-// So M is within 2e-7 rad (4e-8 to 8e-8 rms) wherever |tau/P| < 2^22.
+// So M is within 2.1e-7 rad (4e-8 to 8e-8 rms) wherever |tau/P| < 2^22.
 constexpr float kPairMaxFreq = 2.0f;
 constexpr float kPairExactFreq = 16.0f;
 constexpr float kPairMaxTau = 16384.0f;
