@@ -758,6 +758,14 @@ __device__ __forceinline__ f32x2 kepler_any2(float m0, float m1, float e0, float
   return pack2(x, y);
 }
 
+// The same for four, for the rare group with an e outside [0, 1).  Out of line, as
+// kepler_rest: in the kernel their registers and code cost the main loop 1 us of
+// 36.6 (2^24 elements, arrays larger than L2).
+static __device__ __noinline__ float4 kepler_any4(float4 m, float4 ee) {
+  const f32x2 a = kepler_any2(m.x, m.y, ee.x, ee.y), b = kepler_any2(m.z, m.w, ee.z, ee.w);
+  return make_float4(lo2(a), hi2(a), lo2(b), hi2(b));
+}
+
 // Four (M, e) per thread and iteration when the three arrays are 16-byte
 // aligned: float4 streaming loads and stores (the data are touched once) and
 // two packed solves in flight per thread.  Where one of the four M lies beyond
@@ -766,7 +774,7 @@ __device__ __forceinline__ f32x2 kepler_any2(float m0, float m1, float e0, float
 // iteration, with the same bits.
 // At 12 bytes an element memory alone takes 29 to 31 us for 2^24 elements; the
 // scalar form's 69 instructions an element issued for 33 of its 38.9 us.
-// Packed: 44 instructions, 34.9 us; the wait for memory is hidden by warps, so
+// Packed: 44 instructions, 34.8 us; the wait for memory is hidden by warps, so
 // 32 registers for 64 warps per SM (40 registers: 37.0; loads one iteration
 // ahead: 36.8 to 39; sin and cos from a table in shared memory: 39.3).  Unaligned
 // arrays 67 -> 47 us.
@@ -781,8 +789,18 @@ __device__ __forceinline__ float4 kepler_f32_x4(float4 m, float4 ee) {
     const f32x2 b = kepler_f32x2(pack2(m.z, m.w), pack2(ee.z, ee.w));
     return make_float4(lo2(a), hi2(a), lo2(b), hi2(b));
   }
-  const f32x2 a = kepler_any2(m.x, m.y, ee.x, ee.y), b = kepler_any2(m.z, m.w, ee.z, ee.w);
-  return make_float4(lo2(a), hi2(a), lo2(b), hi2(b));
+  return kepler_any4(m, ee);
+}
+
+// Elements i, i + stride, .. two at a time.
+static __device__ __noinline__ void kepler_rest(const float *M, const float *e, int64_t i,
+                                                int64_t n, int64_t stride, float *E) {
+  for (; i < n; i += 2 * stride) {
+    const int64_t j = i + stride < n ? i + stride : i;
+    const f32x2 r = kepler_any2(reduce_pi(M[i]), reduce_pi(M[j]), e[i], e[j]);
+    E[i] = lo2(r);
+    if (j != i) E[j] = hi2(r);
+  }
 }
 
 __global__ void __launch_bounds__(256, 8)
@@ -799,12 +817,7 @@ kepler_f32_kernel(const float *__restrict__ M, const float *__restrict__ e, int6
   for (int64_t i = tid; i < n4; i += stride) {
     __stcs(E4 + i, kepler_f32_x4(__ldcs(M4 + i), __ldcs(e4 + i)));
   }
-  for (int64_t i = 4 * n4 + tid; i < n; i += 2 * stride) {
-    const int64_t j = i + stride < n ? i + stride : i;
-    const f32x2 r = kepler_any2(reduce_pi(M[i]), reduce_pi(M[j]), e[i], e[j]);
-    E[i] = lo2(r);
-    if (j != i) E[j] = hi2(r);
-  }
+  if (4 * n4 + tid < n) kepler_rest(M, e, 4 * n4 + tid, n, stride, E);
 }
 
 template <typename Kern>
