@@ -230,12 +230,16 @@ struct RaggedPlanet<false> {
 // this one is evaluated.  wide: the wide mean anomaly; with err != NULL the times
 // completed to plain pairs by the plan's tau_err.
 // The gradient has one body for both forms, a branch for the warp in front of the
-// mean anomalies (of half the planets at a time: fewer registers): with a body of
-// each, warps of both forms on an SM waited for instructions (5227 systems of 137 to
-// 1099 observations, half of them with P < 0.5 d: 139 us, now 75; 50000 of 16 to
-// 512: 460, 250; one form only, 50000 of 16 to 1024: 335, 342).  The forward bodies
-// are short enough for two (50000 of 16 to 1024: 220 us, 227 with one; the mixture
-// 63 and 47).
+// mean anomalies of three planets at a time: with a body of each, warps of both
+// forms on an SM waited for instructions.  us with two bodies, with one, all periods
+// above half a day and half of the systems with a shorter one: 50000 systems of 16
+// to 1024 observations 336, 337 and 720, 391; 6000 of 16 to 512 38.1, 40.9 and 87,
+// 44; 5000 of 100 to 1000 58, 58 and 138, 67; 20000 of 4 to 20 43.1, 39.5 and 53,
+// 42.  (Half of the planets at a time, with the times completed outside the branch,
+// it ran 47 us at 6000 and 69 at 5000; both bodies kept, with the one for both
+// forms taken by all systems once one asks for it, 358 and 461 at 50000.)  The
+// forward bodies are short enough for two (50000 of 16 to 1024: 220 us, 227 with
+// one; the mixture 63 and 47).
 template <int J, bool GRAD, bool WIDE>
 __device__ __forceinline__ void body_mixed(const typename RaggedPlanet<GRAD>::type *pl, float gam,
                                            const float *tab, const float4 *oa, const float4 *ob,
@@ -269,22 +273,24 @@ __device__ __forceinline__ void body_mixed(const typename RaggedPlanet<GRAD>::ty
       w_next = ob[p + 32];
     }
     f32x2 th = pack2(tt.x, tt.y), tl = pack2(tt.z, tt.w);
-    if ((GRAD || WIDE) && err != nullptr) {
+    auto complete = [&]() {
       const float2 e = err[pair0 + p];
       float h0, l0, h1, l1;
       two_sum(tt.x, tt.z, h0, l0);
       two_sum(tt.y, tt.w, h1, l1);
       th = pack2(h0, h1);
       tl = pack2(l0 + e.x, l1 + e.y);
-    }
+    };
+    if (!GRAD && WIDE && err != nullptr) complete();
     Kahan2 V = {dup2(gam), 0};
     GradTerms o[JG];
     if constexpr (GRAD) {
-      constexpr int H = J > 3 ? (J + 1) / 2 : J;
+      constexpr int H = J > 3 ? 3 : J;
 #pragma unroll
       for (int j0 = 0; j0 < J; j0 += H) {
         f32x2 M[H];
         if (wide) {
+          if (j0 == 0 && err != nullptr) complete();
 #pragma unroll
           for (int j = 0; j < H && j0 + j < J; ++j) M[j] = mean_anomaly_wide(th, tl, pl[j0 + j].p);
         } else {
