@@ -19,8 +19,9 @@
 //    picks G and W by a cost model (pick_warp_tile) so that the CTAs land
 //    evenly on the SMs and share their staging (for 4096 systems, 27 warps per
 //    CTA: one CTA and 27 systems on every SM, where tiles of 16 systems leave
-//    some SMs with 32 and others with 16).  Larger batches run many waves; the hardware then overlaps
-//    one CTA's prologue with the work of the others on its SM.
+//    some SMs with 32 and others with 16).  Larger batches run many waves; the
+//    hardware then overlaps one CTA's prologue with the work of the others on
+//    its SM.
 //  - Prologue: every global load (the reference time, this thread's
 //    observation and its planet's parameters) is issued before any of them
 //    is used, so the CTA waits for memory once.

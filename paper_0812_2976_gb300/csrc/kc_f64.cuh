@@ -9,13 +9,14 @@
 // velocity.  Everything else is a small correction to a tabulated value:
 //
 //  - the single-precision solve (kc_pair.cuh's start, one Newton step) gives
-//    Ef within about 4e-7 of the root (|M| < 1.04 pi, solve_x); a, the multiple of 2^-9 rad nearest to
-//    its start, has sin a and cos a in a table as doubles and as float pairs;
+//    Ef within about 4e-7 of the root (|M| < 1.04 pi, solve_x); a, the multiple
+//    of 2^-9 rad nearest to its start, has sin a and cos a in a table as doubles
+//    and as float pairs;
 //  - sin and cos of a + b (b = Ef - a exact in float, |b| < 1.8e-3 for |M| <= pi,
 //    2.4e-3 just beyond) and of the corrected E differ from them by less than
-//    3e-3, so a float pair (48 bits) holds the difference to 1e-17: rotation, Newton's correction and
-//    the update run in float expansions (products with their FMA remainders,
-//    sums by TwoSum);
+//    3e-3, so a float pair (48 bits) holds the difference to 1e-17: rotation,
+//    Newton's correction and the update run in float expansions (products with
+//    their FMA remainders, sums by TwoSum);
 //  - f(Ef) takes two FP64 FMAs, (Ef - 2 pi u) - e sin a, minus e times the
 //    float-pair difference;
 //  - v = N/D with N = A cos E - B sin E: N at the table's angle by two FP64

@@ -609,10 +609,10 @@ chi2_f64_kernel(UniformArgs a, int G, int obs_tile, double *__restrict__ out,
 // thread per (system, observation) had repeated the setup at every
 // evaluation (512 x 3 x 1000: 305 us, now 43; 32 without 1/D's correction in
 // FP64, which takes the error from 2.2e-15 to 4e-16 of the velocities' rms; every
-// e above 0.95: 289, now 234).  G
-// is the power of two that n_obs fills, down to one thread per system: every lane
-// evaluates (275996 systems of 5 planets above e = 0.95 at a single time: 358 us,
-// 2060 with 8 threads per system, 444 with the setup per evaluation).
+// e above 0.95: 289, now 234).  G is the power of two that n_obs fills, down to
+// one thread per system: every lane evaluates (275996 systems of 5 planets above
+// e = 0.95 at a single time: 358 us, 2060 with 8 threads per system, 444 with the
+// setup per evaluation).
 constexpr int kPredictBlock = 128;
 
 __global__ void __launch_bounds__(kPredictBlock)
@@ -683,9 +683,8 @@ __device__ inline float reduce_pi<float>(float M) {
 // two FP64 quartic steps, which costs it some 2000 clocks.  2^24 elements, e <=
 // 0.95: 1070 -> 260 us, bound by issue and the FP64 pipe (memory: 60 us); 2^22
 // with e < 0.999: 616 -> 576, with one |M| below 2^-30 in a hundred 270 -> 134.
-// Error against 64-bit mantissas, 4e5
-// draws with |M| from 1e-8: rms 9.10e-17 -> 9.05e-17, largest relative 3.6e-15
-// both.
+// Error against 64-bit mantissas, 4e5 draws with |M| from 1e-8: rms 9.10e-17 ->
+// 9.05e-17, largest relative 3.6e-15 both.
 __device__ __forceinline__ bool kepler_x_takes(double M, double e) {
   constexpr unsigned kEcc = 0x3fee6666u;               // leading word of kEccFast
   constexpr unsigned kMin = 0x3e100000u, kMax = 0x40099999u;        // of 2^-30, 3.19999

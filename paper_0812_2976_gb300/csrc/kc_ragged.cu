@@ -446,7 +446,7 @@ constexpr int kMaxWarps = 8;   // block <= 256
 // Bound by the FP32 pipe's instructions (packed ones take two issue slots) at
 // large sizes.  Measured before, one observation per instruction and a system
 // at a time: forward 50000 systems 310 us, 3000 51, 20000 tiny 31; gradient
-// 50000 systems 440 us (now 339), 200000 1734.
+// 50000 systems 440 us (now 337), 200000 1734 (now 1186).
 constexpr int kAhead = 4;
 static_assert(kAhead * KC_MAX_PLANETS == 32, "a lane per planet of the systems taken");
 
